@@ -9,6 +9,7 @@
 // once per gradient and decoded by every later adjoint-type solve (Sec. 3, Sec. 4).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstdio>
@@ -17,6 +18,7 @@
 #include <vector>
 
 #include "../../include/aewave.h"
+#include "aew_brick.h"
 #include "aew_codec.cuh"
 #include "aew_internal.cuh"
 #include "aew_pca.h"
@@ -108,6 +110,15 @@ struct aew_handle {
   // the source's spatial weights on the z-faces of a (2 src_r + 1)^3 box (point: {1})
   float* src_w = nullptr;
   int src_r = 0;
+  // grids that fit the SMs run their time loops on chip (aew_brick.h): the cut, the halo
+  // exchange buffer with its running tag, and dt s^n of the default and of a given wavelet
+  bool brick = false;
+  aew::BrickPlan bp;
+  unsigned char* halo = nullptr;
+  uint32_t halo_tag = 0;
+  float* dts = nullptr;
+  float* dts_given = nullptr;
+  size_t dts_cap = 0;
   Codec* codec = nullptr;
   std::vector<void*> allocs;
   size_t bytes = 0;
@@ -155,6 +166,8 @@ double ricker(double t, double f0, double t0) {
 }
 
 cudaStream_t S(void* s) { return static_cast<cudaStream_t>(s); }
+
+float* drow(aew_handle* h, float* d, int n);
 
 size_t nblocks_of(const aew_handle* h) {
   return (size_t)(h->cfg.nx / 8) * (h->cfg.ny / 8) * (h->cfg.nz / 8);
@@ -293,9 +306,129 @@ int adj_step_x(aew_handle* h, int n, float* const in[4], float* const out[4],
   return AEW_OK;
 }
 
+// ---------------------------------------------------------------------------------
+// On-chip time loops (aew_brick.h): many steps per launch
+// ---------------------------------------------------------------------------------
+// dt s^n, n = 0 .. nt - 1, on the device: the default wavelet's, or wav's [count]
+int wavelet_on_device(aew_handle* h, const float* wav, size_t count, const float** out,
+                      cudaStream_t s) {
+  if (!wav) {
+    *out = h->dts;
+    return AEW_OK;
+  }
+  if (h->dts_cap < count) {
+    float* p = nullptr;
+    if (!dalloc(h, &p, count)) return fail(h, AEW_E_NOMEM, "wavelet buffer");
+    h->dts_given = p;   // a smaller buffer stays with the handle until it is destroyed
+    h->dts_cap = count;
+    h->stats.device_bytes = h->bytes + aew::codec_device_bytes(h->codec);
+  }
+  std::vector<float> d(count);
+  for (size_t n = 0; n < count; ++n) d[n] = (float)(h->dt * (double)wav[n]);
+  AEW_CK(cudaMemcpyAsync(h->dts_given, d.data(), count * sizeof(float), cudaMemcpyHostToDevice, s));
+  AEW_CK(cudaStreamSynchronize(s));   // d is on this stack
+  *out = h->dts_given;
+  return AEW_OK;
+}
+
+// forward steps without options: in (null: the zero state) -> out (null: not kept), with
+// dts[0 ..] (null: no source) and receiver rows from d_row on (null: none)
+aew::BrickFwd brick_fwd_args(aew_handle* h, float* const in[4], float* const out[4], int nsteps,
+                             const float* dts, float* d_row) {
+  aew::BrickFwd a{};
+  a.m = h->m;
+  if (in) {
+    a.e = in[0];
+    a.vx = in[1];
+    a.vy = in[2];
+    a.vz = in[3];
+  }
+  if (out) {
+    a.e1 = out[0];
+    a.vx1 = out[1];
+    a.vy1 = out[2];
+    a.vz1 = out[3];
+  }
+  a.nx = h->cfg.nx;
+  a.ny = h->cfg.ny;
+  a.nz = h->cfg.nz;
+  a.dth = h->dth;
+  a.nsteps = nsteps;
+  a.dts = dts;
+  a.si = h->cfg.src[0];
+  a.sj = h->cfg.src[1];
+  a.sk = dts ? h->cfg.src[2] : -1;
+  a.src_w = h->src_w;
+  a.sr = h->src_r;
+  a.krec = d_row ? h->krec : -1;
+  a.rec_map = h->rec_map;
+  a.d_out = d_row;
+  a.nrow = h->nrow;
+  a.ef_first = nsteps;
+  return a;
+}
+
+int brick_fwd(aew_handle* h, const aew::BrickFwd& a, cudaStream_t s) {
+  AEW_CK(aew::launch_brick_fwd(a, h->bp, h->halo, &h->halo_tag, aew::codec_err_flag(h->codec), s));
+  ++h->stats.kernel_launches;
+  return AEW_OK;
+}
+
+// incremental steps n0 .. n0 + nsteps - 1 reading e^{n0 + k} at ef (or ef16) + k C
+aew::BrickFwd brick_incr_args(aew_handle* h, float* const in[4], float* const out[4], int n0,
+                              int nsteps, const float* ef, const uint16_t* ef16, float* d_row) {
+  aew::BrickFwd a = brick_fwd_args(h, in, out, nsteps, nullptr, d_row);
+  a.ef_first = n0 == 0 ? 1 : 0;   // e^0 = 0: no extra source
+  a.dm = h->dm;
+  a.ef = ef;
+  a.ef16 = ef16;
+  return a;
+}
+
+// reverse steps n0, n0 - 1, .., n0 - nsteps + 1: in (null: the zero state) -> out (null: not
+// kept); en (or en16): e^{n0}, the earlier states at - C each
+int brick_adj(aew_handle* h, int n0, int nsteps, float* const in[4], float* const out[4],
+              const float* resid, const float* en, const uint16_t* en16, cudaStream_t s) {
+  aew::BrickAdj a{};
+  a.m = h->m;
+  if (in) {
+    a.mu = in[0];
+    a.lx = in[1];
+    a.ly = in[2];
+    a.lz = in[3];
+  }
+  if (out) {
+    a.mu1 = out[0];
+    a.lx1 = out[1];
+    a.ly1 = out[2];
+    a.lz1 = out[3];
+  }
+  a.nx = h->cfg.nx;
+  a.ny = h->cfg.ny;
+  a.nz = h->cfg.nz;
+  a.dth = h->dth;
+  a.nsteps = nsteps;
+  a.en = en;
+  a.en16 = en16;
+  a.en_steps = en || en16 ? (n0 - nsteps + 1 == 0 ? nsteps - 1 : nsteps) : 0;   // e^0 = 0
+  a.resid = (resid && h->nrow) ? resid + (size_t)(n0 + 1) * h->nrow : nullptr;
+  a.nrow = h->nrow;
+  a.krec = h->krec;
+  a.rec_map = h->rec_map;
+  a.acc32 = h->acc32;
+  a.acc64 = h->acc64;
+  a.W = h->cfg.accum_window;
+  a.w0 = (h->cfg.nt - 1 - n0) % a.W;
+  a.last = n0 - nsteps + 1 == 0;
+  AEW_CK(aew::launch_brick_adj(a, h->bp, h->halo, &h->halo_tag, aew::codec_err_flag(h->codec), s));
+  ++h->stats.kernel_launches;
+  return AEW_OK;
+}
+
 // reverse step n: (lam, mu) in ad[cur] -> ad[cur ^ 1]
 int adj_step(aew_handle* h, int n, int cur, const float* resid, const float* en,
              cudaStream_t s) {
+  if (h->brick) return brick_adj(h, n, 1, h->ad[cur], h->ad[cur ^ 1], resid, en, nullptr, s);
   return adj_step_x(h, n, h->ad[cur], h->ad[cur ^ 1], resid, en, h->acc32, h->acc64, nullptr,
                     nullptr, nullptr, s);
 }
@@ -435,8 +568,40 @@ int ae_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
 // ---------------------------------------------------------------------------------
 // Gradient drivers
 // ---------------------------------------------------------------------------------
+int adjoint_full(aew_handle* h, const float* resid, cudaStream_t s) {
+  const int nt = h->cfg.nt;
+  int rc, cur = 0;
+  if (h->brick) {
+    AEW_CK(cudaMemsetAsync(h->acc64, 0, h->C * sizeof(double), s));
+    return brick_adj(h, nt - 1, nt, nullptr, nullptr, resid,
+                     nt > 1 ? h->estore + (size_t)(nt - 1) * h->C : nullptr, nullptr, s);
+  }
+  if ((rc = begin_adjoint(h, s))) return rc;
+  for (int n = nt - 1; n >= 0; --n) {
+    const float* en = n > 0 ? h->estore + (size_t)n * h->C : nullptr;
+    if ((rc = adj_step(h, n, cur, resid, en, s))) return rc;
+    cur ^= 1;
+  }
+  return AEW_OK;
+}
+
 int gradient_full(aew_handle* h, const float* d_obs, const float* wav, cudaStream_t s) {
   const int nt = h->cfg.nt;
+  if (h->brick) {
+    AEW_CK(cudaMemsetAsync(h->estore, 0, h->C * sizeof(float), s));
+    AEW_CK(cudaMemsetAsync(h->d, 0, h->nrow * sizeof(float), s));
+    aew::BrickFwd a = brick_fwd_args(h, nullptr, nullptr, nt, h->dts, drow(h, h->d, 1));
+    a.hist = h->estore + h->C;
+    a.nhist = nt - 1;
+    int rc = brick_fwd(h, a, s);
+    if (rc) return rc;
+    if ((rc = residual_and_misfit(h, d_obs, s))) return rc;
+    if ((rc = misfit_gate(h, s))) return rc;
+    if ((rc = adjoint_full(h, h->R, s))) return rc;
+    h->stats.forward_steps = nt;
+    h->stats.adjoint_steps = nt;
+    return AEW_OK;
+  }
   float* vb[2][3] = {{h->st[0][1], h->st[0][2], h->st[0][3]},
                      {h->st[1][1], h->st[1][2], h->st[1][3]}};
   for (int i = 0; i < 3; ++i) AEW_CK(cudaMemsetAsync(vb[0][i], 0, h->C * sizeof(float), s));
@@ -453,13 +618,7 @@ int gradient_full(aew_handle* h, const float* d_obs, const float* wav, cudaStrea
   int rc = residual_and_misfit(h, d_obs, s);
   if (rc) return rc;
   if ((rc = misfit_gate(h, s))) return rc;
-  if ((rc = begin_adjoint(h, s))) return rc;
-  int cur = 0;
-  for (int n = nt - 1; n >= 0; --n) {
-    const float* en = n > 0 ? h->estore + (size_t)n * h->C : nullptr;
-    if ((rc = adj_step(h, n, cur, h->R, en, s))) return rc;
-    cur ^= 1;
-  }
+  if ((rc = adjoint_full(h, h->R, s))) return rc;
   h->stats.forward_steps = nt;
   h->stats.adjoint_steps = nt;
   return AEW_OK;
@@ -493,6 +652,22 @@ int run_revolve(aew_handle* h, const float* d_obs, const float* resid, const flo
     switch (act.op) {
       case aew::kOpAdvance: {
         const bool to_slot = a + 1 < plan.size() && plan[a + 1].op == aew::kOpStore;
+        if (h->brick && act.arg > 0) {
+          float* out[4];
+          if (to_slot) slot(plan[a + 1].arg, out);
+          const bool direct = to_slot && out[0] != live[0];   // never onto the state it reads
+          const int out_buf = direct ? -1 : (live_buf == 0 ? 1 : 0);
+          for (int i = 0; !direct && i < 4; ++i) out[i] = h->st[out_buf][i];
+          rc = brick_fwd(h, brick_fwd_args(h, live[0] == h->zst[0] ? nullptr : live, out, act.arg,
+                                           h->dts + live_n,
+                                           gradient ? drow(h, h->d, live_n + 1) : nullptr), s);
+          if (rc) return rc;
+          for (int i = 0; i < 4; ++i) live[i] = out[i];
+          live_buf = out_buf;
+          live_n += act.arg;
+          fwd += act.arg;
+          break;
+        }
         for (int k = 0; k < act.arg; ++k) {
           float* out[4];
           int out_buf;
@@ -540,7 +715,11 @@ int run_revolve(aew_handle* h, const float* d_obs, const float* resid, const flo
           float* out[4];
           const int ob = live_buf == 0 ? 1 : 0;
           for (int i = 0; i < 4; ++i) out[i] = h->st[ob][i];
-          rc = fwd_step(h, live_n, live, out, wav, drow(h, h->d, live_n + 1), s);
+          if (h->brick)
+            rc = brick_fwd(h, brick_fwd_args(h, live[0] == h->zst[0] ? nullptr : live, nullptr, 1,
+                                             h->dts + live_n, drow(h, h->d, live_n + 1)), s);
+          else
+            rc = fwd_step(h, live_n, live, out, wav, drow(h, h->d, live_n + 1), s);
           if (rc) return rc;
           ++fwd;
           if ((rc = residual_and_misfit(h, d_obs, s))) return rc;
@@ -605,7 +784,7 @@ int encode_window(aew_handle* h, int tb, cudaStream_t s) {
   const bool mm = aew::codec_minmax(h->codec);
   cudaError_t e = aew::codec_encode_window(h->codec, h->xt[tb & 1], h->vmx + (size_t)tb * nv,
                                            (long long)nv, h->lat + (size_t)tb * nv * h->cfg.n_lat,
-                                           h->ovf, s, h->overlap_ctas,
+                                           h->ovf, s, h->brick ? 0 : h->overlap_ctas,
                                            mm ? h->wmn + (size_t)tb * nv : nullptr,
                                            mm ? h->wr + (size_t)tb * nv : nullptr);
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_encode_window");
@@ -620,7 +799,8 @@ int decode_window(aew_handle* h, int tb, cudaStream_t s, bool bf16 = false) {
   const bool mm = aew::codec_minmax(h->codec);
   cudaError_t e = aew::codec_decode_window(h->codec, h->lat + (size_t)tb * nv * h->cfg.n_lat,
                                            h->vmx + (size_t)tb * nv, h->cfg.nx, h->cfg.ny,
-                                           h->cfg.nz, h->edt[tb & 1], s, h->overlap_ctas,
+                                           h->cfg.nz, h->edt[tb & 1], s,
+                                           h->brick ? 0 : h->overlap_ctas,
                                            mm ? h->wmn + (size_t)tb * nv : nullptr,
                                            mm ? h->wr + (size_t)tb * nv : nullptr, bf16);
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_decode_window");
@@ -646,6 +826,17 @@ const uint16_t* window_e16(aew_handle* h, int n) {
 int time_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
   const int nt = h->cfg.nt, W = nwin_of(h), T = aew::kTSteps;
   int rc;
+  if (h->brick) {   // the on-chip loops fill the GPU: decode and sweep each window in turn
+    AEW_CK(cudaMemsetAsync(h->acc64, 0, h->C * sizeof(double), s));
+    for (int tb = W - 1, cur = 0; tb >= 0; --tb, cur ^= 1) {
+      if ((rc = decode_window(h, tb, s, true))) return rc;
+      const int n0 = std::min(nt - 1, T * tb + T - 1);
+      if ((rc = brick_adj(h, n0, n0 - T * tb + 1, tb == W - 1 ? nullptr : h->ad[cur],
+                          tb > 0 ? h->ad[cur ^ 1] : nullptr, resid, nullptr, window_e16(h, n0), s)))
+        return rc;
+    }
+    return AEW_OK;
+  }
   if ((rc = begin_adjoint(h, s))) return rc;
   if ((rc = join(h, s, h->side, h->ev_sync))) return rc;
   if ((rc = decode_window(h, W - 1, h->side, true))) return rc;
@@ -679,11 +870,38 @@ int gradient_ae_time(aew_handle* h, const float* d_obs, const float* wav, cudaSt
   const int nt = h->cfg.nt, W = nwin_of(h), T = aew::kTSteps;
   const size_t nv = nvec_of(h), wbytes = nv * aew::kNIn * sizeof(uint16_t);
   int rc;
-  if ((rc = zero_state(h, h->st[0], s))) return rc;
   AEW_CK(cudaMemsetAsync(h->vmx, 0, (size_t)W * nv * sizeof(unsigned), s));
   AEW_CK(cudaMemsetAsync(h->xt[0], 0, wbytes, s));   // slot 0 of window 0 is e^0 = 0
   AEW_CK(cudaMemsetAsync(h->ovf, 0, sizeof(int), s));
   AEW_CK(cudaMemsetAsync(h->d, 0, h->nrow * sizeof(float), s));
+  if (h->brick) {   // the on-chip loops fill the GPU: run and encode each window in turn
+    // window tb's states m = T tb .. min(T tb + T, nt) - 1 come from steps m - 1; the last
+    // launch also runs step nt - 1, whose state nt is not stored
+    for (int tb = 0, cur = 0, n = 0; tb < W; ++tb, cur ^= 1) {
+      const int m1 = std::min(T * tb + T, nt);   // one past the window's last state
+      if (T * tb + T > nt) AEW_CK(cudaMemsetAsync(h->xt[tb & 1], 0, wbytes, s));   // tail 0
+      const int steps = (tb == W - 1 ? nt : m1 - 1) - n;
+      if (steps > 0) {
+        aew::BrickFwd a = brick_fwd_args(h, n ? h->st[cur] : nullptr,
+                                         tb < W - 1 ? h->st[cur ^ 1] : nullptr, steps, h->dts + n,
+                                         drow(h, h->d, n + 1));
+        a.npack = m1 - 1 - n;
+        a.tpack = h->xt[tb & 1];
+        a.vmax = h->vmx + (size_t)tb * nv;
+        a.tslot = n + 1 - T * tb;
+        if ((rc = brick_fwd(h, a, s))) return rc;
+        n += steps;
+      }
+      if ((rc = encode_window(h, tb, s))) return rc;
+    }
+    if ((rc = residual_and_misfit(h, d_obs, s))) return rc;
+    if ((rc = misfit_gate(h, s))) return rc;
+    if ((rc = time_adjoint_sweep(h, h->R, s))) return rc;
+    h->stats.forward_steps = nt;
+    h->stats.adjoint_steps = nt;
+    return AEW_OK;
+  }
+  if ((rc = zero_state(h, h->st[0], s))) return rc;
   if ((rc = join(h, s, h->side, h->ev_sync))) return rc;
   auto window_done = [&](int tb) -> int {
     AEW_CK(cudaEventRecord(h->ev_a[tb & 1], s));
@@ -766,6 +984,13 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
   int cur = 0;
   if (h->cfg.storage == AEW_FULL) {
     AEW_CK(cudaMemsetAsync(h->desto, 0, h->C * sizeof(float), s));
+    if (h->brick) {
+      aew::BrickFwd a = brick_incr_args(h, nullptr, nullptr, 0, nt, h->estore, nullptr,
+                                        drow(h, h->dd, 1));
+      a.hist = h->desto + h->C;
+      a.nhist = nt - 1;
+      return brick_fwd(h, a, s);
+    }
     for (int n = 0; n < nt; ++n) {
       float* in[4] = {h->desto + (size_t)n * h->C, h->ad[cur][1], h->ad[cur][2], h->ad[cur][3]};
       float* eo = n + 1 < nt ? h->desto + (size_t)(n + 1) * h->C : h->ad[cur ^ 1][0];
@@ -1123,6 +1348,22 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
     ok = ok && cudaEventCreateWithFlags(&h->ev_sync, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&h->ev_sync2, cudaEventDisableTiming) == cudaSuccess;
   }
+  // on-chip time loops where the grid fits; a z-chunk depth set by hand asks for the
+  // streaming kernels it belongs to
+  if (ok && !getenv("AEW_STENCIL_KC_FWD") && !getenv("AEW_STENCIL_KC_ADJ")) {
+    int sms = 0, coop = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
+    h->brick = coop && aew::brick_plan(c.nx, c.ny, c.nz, sms, &h->bp);
+    if (h->brick) {
+      const size_t nb = aew::brick_halo_bytes(c.nx, h->bp);
+      std::vector<float> dts(nt);
+      for (size_t n = 0; n < nt; ++n) dts[n] = (float)(h->dt * (double)h->wav[n]);
+      ok = dalloc(h, &h->halo, nb) && cudaMemset(h->halo, 0, nb) == cudaSuccess &&
+           dalloc(h, &h->dts, nt) &&
+           cudaMemcpy(h->dts, dts.data(), nt * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+    }
+  }
   if (!ok) {
     g_create_err = "device allocation failed (" + std::to_string(h->bytes) + " bytes held)";
     aew_destroy(h);
@@ -1208,9 +1449,15 @@ int aew_forward(aew_handle* h, const float* c_dev, const float* wavelet_host, fl
   int rc = prepare_c(h, c_dev, s);
   if (rc) return rc;
   h->have_grad = false;  // m changed: stored history no longer matches
+  if (d_dev && h->nrow) AEW_CK(cudaMemsetAsync(d_dev, 0, h->nrow * sizeof(float), s));
+  if (h->brick) {
+    const float* dts = nullptr;
+    if ((rc = wavelet_on_device(h, wavelet_host, (size_t)h->cfg.nt, &dts, s))) return rc;
+    return brick_fwd(h, brick_fwd_args(h, nullptr, nullptr, h->cfg.nt, dts,
+                                       d_dev ? drow(h, d_dev, 1) : nullptr), s);
+  }
   const float* wav = wav_or_default(h, wavelet_host);
   if ((rc = zero_state(h, h->st[0], s))) return rc;
-  if (d_dev && h->nrow) AEW_CK(cudaMemsetAsync(d_dev, 0, h->nrow * sizeof(float), s));
   int cur = 0;
   for (int n = 0; n < h->cfg.nt; ++n) {
     rc = fwd_step(h, n, h->st[cur], h->st[cur ^ 1], wav, d_dev ? drow(h, d_dev, n + 1) : nullptr,
@@ -1254,6 +1501,14 @@ int aew_propagate(aew_handle* h, const float* c_dev, float* const state_dev[4], 
   float* tmp[4] = {h->st[0][0], h->st[0][1], h->st[0][2], h->st[0][3]};
   float* bufs[2][4] = {{state_dev[0], state_dev[1], state_dev[2], state_dev[3]},
                        {tmp[0], tmp[1], tmp[2], tmp[3]}};
+  if (h->brick && nsteps > 0) {
+    const float* dts = nullptr;
+    if (wavelet_host && (rc = wavelet_on_device(h, wavelet_host, (size_t)nsteps, &dts, s))) return rc;
+    if ((rc = brick_fwd(h, brick_fwd_args(h, bufs[0], bufs[1], nsteps, dts,
+                                          d_dev ? drow(h, d_dev, 1) : nullptr), s)))
+      return rc;
+    return copy_state(h, bufs[0], bufs[1], s);
+  }
   std::vector<float> w(wavelet_host ? (size_t)nsteps + (size_t)n0 : 0, 0.f);
   for (int k = 0; wavelet_host && k < nsteps; ++k) w[(size_t)n0 + k] = wavelet_host[k];
   int cur = 0;
@@ -1341,10 +1596,30 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
   const int nt = h->cfg.nt;
   int rc;
   // incremental state in ad[] buffers (free until the incremental adjoint)
-  if ((rc = zero_state(h, h->ad[0], s))) return rc;
   if (h->nrow) AEW_CK(cudaMemsetAsync(dd_out, 0, h->nrow * sizeof(float), s));
   int cur = 0, fcur = 0;
   *fwd = 0;
+  if (h->brick && h->cfg.storage == AEW_FULL) {
+    *fwd = nt;
+    return brick_fwd(h, brick_incr_args(h, nullptr, nullptr, 0, nt, h->estore, nullptr,
+                                        drow(h, dd_out, 1)), s);
+  }
+  if (h->brick && h->cfg.storage == AEW_AE && h->tcodec) {
+    const int W = nwin_of(h), T = aew::kTSteps;
+    *fwd = nt;
+    for (int tb = 0; tb < W; ++tb, cur ^= 1) {
+      if ((rc = decode_window(h, tb, s, true))) return rc;
+      const int n = T * tb;
+      const uint16_t* e16 = reinterpret_cast<const uint16_t*>(h->edt[tb & 1]);
+      if ((rc = brick_fwd(h, brick_incr_args(h, tb ? h->ad[cur] : nullptr,
+                                             tb < W - 1 ? h->ad[cur ^ 1] : nullptr, n,
+                                             std::min(T, nt - n), nullptr, e16,
+                                             drow(h, dd_out, n + 1)), s)))
+        return rc;
+    }
+    return AEW_OK;
+  }
+  if ((rc = zero_state(h, h->ad[0], s))) return rc;
   if (h->cfg.storage == AEW_REVOLVE && (rc = zero_state(h, h->st[0], s))) return rc;
   const bool ae = h->cfg.storage == AEW_AE;
   if (ae && h->tcodec) {
@@ -1399,14 +1674,26 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
     }
     if (h->cfg.storage == AEW_REVOLVE) {
       if (n > 0) {  // lockstep forward recompute: state n from state n-1
-        rc = fwd_step(h, n - 1, h->st[fcur], h->st[fcur ^ 1], h->wav.data(), nullptr, s);
+        if (h->brick)
+          rc = brick_fwd(h, brick_fwd_args(h, h->st[fcur], h->st[fcur ^ 1], 1, h->dts + n - 1,
+                                           nullptr), s);
+        else
+          rc = fwd_step(h, n - 1, h->st[fcur], h->st[fcur ^ 1], h->wav.data(), nullptr, s);
         if (rc) return rc;
         fcur ^= 1;
         ++*fwd;
         en = h->st[fcur][0];
       }
     }
-    if ((rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], en, drow(h, dd_out, n + 1), s))) return rc;
+    if (h->brick && h->cfg.storage == AEW_REVOLVE) {
+      rc = n == 0 ? brick_fwd(h, brick_fwd_args(h, h->ad[cur], h->ad[cur ^ 1], 1, nullptr,
+                                                drow(h, dd_out, 1)), s)
+                  : brick_fwd(h, brick_incr_args(h, h->ad[cur], h->ad[cur ^ 1], n, 1, en, nullptr,
+                                                 drow(h, dd_out, n + 1)), s);
+    } else {
+      rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], en, drow(h, dd_out, n + 1), s);
+    }
+    if (rc) return rc;
     if (ae) AEW_CK(cudaEventRecord(h->ev_a[n & 1], s));
     cur ^= 1;
     ++*fwd;
@@ -1452,7 +1739,6 @@ int aew_hessvec(aew_handle* h, const float* dc_dev, float* hdc_dev, void* stream
   long long fwd = 0;
   if ((rc = incremental_forward(h, h->dd, s, &fwd))) return rc;
   // incremental adjoint: the adjoint solve with residual dd (row 0 unused)
-  const int nt = h->cfg.nt;
   if (h->cfg.storage == AEW_REVOLVE) {
     long long f2 = 0;
     if ((rc = run_revolve(h, nullptr, h->dd, h->wav.data(), false, s, &f2))) return rc;
@@ -1460,14 +1746,8 @@ int aew_hessvec(aew_handle* h, const float* dc_dev, float* hdc_dev, void* stream
   } else if (h->cfg.storage == AEW_AE) {
     if ((rc = h->tcodec ? time_adjoint_sweep(h, h->dd, s) : ae_adjoint_sweep(h, h->dd, s)))
       return rc;
-  } else {
-    if ((rc = begin_adjoint(h, s))) return rc;
-    int acur = 0;
-    for (int n = nt - 1; n >= 0; --n) {
-      const float* en = n > 0 ? h->estore + (size_t)n * h->C : nullptr;
-      if ((rc = adj_step(h, n, acur, h->dd, en, s))) return rc;
-      acur ^= 1;
-    }
+  } else if ((rc = adjoint_full(h, h->dd, s))) {
+    return rc;
   }
   h->stats.hvp_forward_steps = fwd;
   if (aew::codec_take_error(h->codec, s))
@@ -1829,7 +2109,8 @@ int aew_profile_steps(aew_handle* h, const float* c_dev, int kind, int nsteps, d
                       nullptr, nullptr, h->xt[0], (n + 1) % T, h->vmx);
         break;
       case 2:
-        rc = adj_step(h, nt - 1 - n, cur, h->R, h->st[0][0], s);
+        rc = adj_step_x(h, nt - 1 - n, h->ad[cur], h->ad[cur ^ 1], h->R, h->st[0][0], h->acc32,
+                        h->acc64, nullptr, nullptr, nullptr, s);
         break;
       case 3:
         rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], h->st[0][0], nullptr, s);

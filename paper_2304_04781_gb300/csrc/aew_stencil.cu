@@ -36,6 +36,7 @@
 
 #include "aew_gemm.cuh"
 #include "aew_internal.cuh"
+#include "aew_stencil.cuh"
 #include "aew_tc.cuh"
 
 namespace aew {
@@ -104,79 +105,6 @@ __device__ __forceinline__ void tma3(uint32_t dst, const CUtensorMap* map, int x
       "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(mbar)
       : "memory");
-}
-
-__device__ __forceinline__ void st4(float* p, size_t i, float4 v) {
-  *reinterpret_cast<float4*>(p + i) = v;
-}
-__device__ __forceinline__ float& comp(float4& v, int c) {
-  return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w));
-}
-__device__ __forceinline__ float4 z4() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-// the source's force on the z-faces of the 4 nodes (k, y, i0 .. i0 + 3): dts times the
-// spread weight of each face inside the source box (a point source: the one face, 1)
-__device__ __forceinline__ void add_source(float4& v, int k, int y, int i0, const FwdStep& a) {
-  if (a.sk < 0) return;
-  const int W = 2 * a.sr + 1;
-  const int dk = k - a.sk + a.sr, dy = y - a.sj + a.sr;
-  if ((unsigned)dk >= (unsigned)W || (unsigned)dy >= (unsigned)W) return;
-  const float* w = a.src_w + ((size_t)dk * W + dy) * W;
-#pragma unroll
-  for (int d = 0; d < 4; ++d) {
-    const int dx = i0 + d - a.si + a.sr;
-    if ((unsigned)dx < (unsigned)W) comp(v, d) = fmaf(a.dts, __ldg(w + dx), comp(v, d));
-  }
-}
-// The m e products are plain multiplies; the face updates below subtract them with
-// __fsub_rn, which the compiler never merges with a multiply, so every face is
-// fma(dth, round(m_hi e_hi) - round(m_lo e_lo), v) wherever it is computed: by its
-// owner, or recomputed at a chunk's first plane or by the neighbouring lane.  (Left to
-// the compiler, a subtraction could absorb one product into an FMA at one site and not
-// at another, and the results then depended in the last bit on the z-chunk depth.)
-__device__ __forceinline__ float4 mul4(float4 a, float4 b) {
-  return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
-}
-__device__ __forceinline__ float4 fma4(float4 a, float4 b, float4 c) {
-  return make_float4(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y), fmaf(a.z, b.z, c.z),
-                     fmaf(a.w, b.w, c.w));
-}
-// 1 / s for a block maximum m >= 0 given as float bits, equal to
-// gemm::block_inv_scale(m) (s = 2^max(e, -100), m = f 2^e with f in [0.5, 1); 0 for
-// m = 0) but from the exponent field: e = biased - 126 for normal m, and subnormal m
-// falls under the clamp.  Maxima of 2^126 and above take the library path.
-__device__ __forceinline__ float inv_scale_bits(uint32_t mb) {
-  const int eb = (int)(mb >> 23);
-  if (mb == 0u) return 0.f;
-  if (eb >= 253) return gemm::block_inv_scale(__uint_as_float(mb));
-  const int e = max(eb - 126, gemm::kExpMin);
-  return __uint_as_float((uint32_t)(127 - e) << 23);
-}
-__device__ __forceinline__ float hmax4(float4 a) {
-  return fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w)));
-}
-__device__ __forceinline__ uint32_t pack2bf(float a, float b) {
-  __nv_bfloat162 t = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&t);
-}
-// face update v' = v + dth (hi - lo), the difference rounded on its own (see above)
-__device__ __forceinline__ float fupd(float dth, float hi, float lo, float v) {
-  return fmaf(dth, __fsub_rn(hi, lo), v);
-}
-__device__ __forceinline__ float4 fupd4(float dth, float4 hi, float4 lo, float4 v) {
-  return make_float4(fupd(dth, hi.x, lo.x, v.x), fupd(dth, hi.y, lo.y, v.y),
-                     fupd(dth, hi.z, lo.z, v.z), fupd(dth, hi.w, lo.w, v.w));
-}
-// lam' = (lam + inj) + dth (mu - mu_hi)
-__device__ __forceinline__ float lupd(float dth, float mu_hi, float mu, float l) {
-  return fmaf(dth, mu - mu_hi, l);
-}
-__device__ __forceinline__ float4 lupd4(float dth, float4 hi, float4 lo, float4 l) {
-  return make_float4(lupd(dth, hi.x, lo.x, l.x), lupd(dth, hi.y, lo.y, l.y),
-                     lupd(dth, hi.z, lo.z, l.z), lupd(dth, hi.w, lo.w, l.w));
-}
-
-__device__ __forceinline__ bool sticky_error(const int* err) {
-  return err && *reinterpret_cast<const volatile int*>(err) != 0;
 }
 
 // Ring bookkeeping shared by both kernels: the CTA stages planes p0 = kbeg - 1 .. pn =
@@ -317,7 +245,7 @@ __global__ void __launch_bounds__(NTHR, (INCR || PACK) ? 2 : 3)
     const uint8_t* sc = r.at(kbeg);
     vzl = fupd4(dth, me_at<INCR, EFB>(sc, qE), me_at<INCR, EFB>(sb, qE),
                 reinterpret_cast<const float4*>(sb + FwdLayout::VZ)[qO]);
-    add_source(vzl, kbeg - 1, y, i0, a);
+    add_source(vzl, kbeg - 1, y, i0, a, a.dts);
   }
 
   const int NBx = nx >> 3, NBy = ny >> 3;
@@ -406,7 +334,7 @@ __global__ void __launch_bounds__(NTHR, (INCR || PACK) ? 2 : 3)
     // z-faces
     float4 vz1 = fupd4(dth, me_n, me_c, vz_c);
     if (k == nz - 1) vz1 = z4();
-    add_source(vz1, k, y, i0, a);
+    add_source(vz1, k, y, i0, a, a.dts);
     // strain update on interior nodes
     float4 e1;
     e1.x = fmaf(dth, ((vx1.x - vxl) + (vy1.x - vyl.x)) + (vz1.x - vzl.x), e_c.x);
@@ -727,8 +655,7 @@ __global__ void __launch_bounds__(NTHR, 2)
       // dJ/dm += dt e^n q
       const float4 g = mul4(en4, dq);
       if (mode & kAccLast) {
-        float4 s = g;
-        if (fl.w) s = make_float4(w_c.x + g.x, w_c.y + g.y, w_c.z + g.z, w_c.w + g.w);
+        const float4 s = fl.w ? fma4(en4, dq, w_c) : g;
         a64lo.x += (double)s.x;
         a64lo.y += (double)s.y;
         a64hi.x += (double)s.z;
@@ -739,7 +666,7 @@ __global__ void __launch_bounds__(NTHR, 2)
       } else if (mode & kAccFirst) {
         st4(a.acc32, i, g);
       } else {
-        st4(a.acc32, i, make_float4(w_c.x + g.x, w_c.y + g.y, w_c.z + g.z, w_c.w + g.w));
+        st4(a.acc32, i, fma4(en4, dq, w_c));
       }
     }
     lzl = lz1;
