@@ -6,8 +6,7 @@
 // block b = (bz*NBy + by)*NBx + bx.  Each field of each block is divided by its
 // power-of-two scale s_{b,f} = 2^max(e, -100), m 2^e (m in [1/2, 1)) the block's max |f|
 // (exact in BF16).  Inside the gradient the forward step packs and normalises the
-// vectors itself; the entry points here pack a given state (pack_raw_kernel, then
-// normalise_kernel).
+// vectors itself; the entry points here pack a given state (pack_state_kernel).
 //
 // Encoder: A = normalised BF16 block vectors, times W1 (2048 x 512) -> +b1, GELU -> H
 // (BF16), times W2 (512 x n_lat) -> +b2 -> FP16 latent.  Decoder: latent (FP16) times W3
@@ -358,94 +357,121 @@ bool ensure_H(Codec* c, size_t rows) {
 // ---------------------------------------------------------------------------------
 // Algorithm 1 packing: BF16 normalised block vectors
 // ---------------------------------------------------------------------------------
-// Raw BF16 block vectors of a grid state and the per-block, per-field maxima of |f|.
-// One thread per float4 of a grid row: consecutive threads read consecutive x
-// (coalesced) and write 8-byte pieces; the two threads of a block row combine their
-// maxima by shuffle before the atomicMax.
-__global__ void pack_raw_kernel(const float* f0, const float* f1, const float* f2,
-                                const float* f3, int nx, int ny, int NBx, int NBy,
-                                long long nblk, unsigned* bmax, uint16_t* out) {
-  const int xq_n = nx >> 2;
-  const long long total = nblk / NBx * 256LL * xq_n;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long iters = (total + stride - 1) / stride;
-  for (long long q = 0; q < iters; ++q) {
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x + q * stride;
-    const bool live = t < total;
-    const int xq = live ? (int)(t % xq_n) : 0;
-    const long long r = live ? t / xq_n : 0;
-    const int y = (int)(r & 7), f = (int)((r >> 3) & 3), z = (int)((r >> 5) & 7);
-    const long long slab = r >> 8;               // (bz, by)
-    const long long by = slab % NBy, bz = slab / NBy;
-    const long long b = slab * NBx + (xq >> 1);
-    float m = 0.f;
-    if (live) {
-      const float* src = f == 0 ? f0 : (f == 1 ? f1 : (f == 2 ? f2 : f3));
-      const float4 a = *reinterpret_cast<const float4*>(
-          src + ((size_t)(8 * bz + z) * ny + (size_t)(8 * by + y)) * nx + 4 * (size_t)xq);
-      *reinterpret_cast<uint2*>(out + b * kNIn + z * 256 + f * 64 + y * 8 + 4 * (xq & 1)) =
-          make_uint2(gemm::pack_bf16(a.x, a.y), gemm::pack_bf16(a.z, a.w));
-      m = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w)));
-    }
-    // xq and xq ^ 1 are adjacent lanes (xq_n is even) and share block b and field f
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-    if (live && (xq & 1) == 0 && m > 0.f) atomicMax(bmax + b * 4 + f, __float_as_uint(m));
-  }
+// Both packings take whole vectors inside one CTA, so that a vector's maximum needs neither
+// a second pass nor atomics: 4 blocks side by side in x (128-byte row segments), 256 rows of
+// 8 float4, 8 float4 per thread, all 8 loads in flight at once.  Row r of a CTA's vectors is
+// 8 consecutive values of each vector, so a warp's stores fill 64-byte runs.
+constexpr int kPackX = 4;
+
+// max over the lanes of a warp that share a vector (lane = 4 rows x 8 float4, two float4 per
+// vector), left in the lanes 0, 2, 4, 6
+__device__ __forceinline__ float vector_max(float m) {
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+  return fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
 }
 
-// y = x * 2^-e per block-field (exact), from raw BF16 vectors and block maxima; out may
-// be raw itself (each thread rewrites only the 16 bytes it read)
-__global__ void normalise_kernel(const uint16_t* raw, const unsigned* __restrict__ bmax,
-                                 long long n, uint16_t* out) {
-  const long long total = n * (kNIn / 8);   // 16-byte pieces
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long b = t / (kNIn / 8);
-    const int k = (int)(t % (kNIn / 8)) * 8;
-    const int f = (k >> 6) & 3;
-    const float sc = gemm::block_inv_scale(__uint_as_float(bmax[b * 4 + f]));
-    uint4 v = *reinterpret_cast<const uint4*>(raw + b * kNIn + k);
-    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+// Normalised BF16 block vectors [block][2048] of a grid state and the block maxima
+// [block][4] (float bits, every entry written).  Bound by HBM: 16 B read and 8 B written per
+// node.  A raw pass with atomic maxima and a normalising pass took 116 + 37 us at 256^3; encode
+// and decode of a state together went from 382 to 284 us.  ROUND: x is rounded to BF16 before its exact division by the scale, as a
+// packed state's vectors are (the same but below BF16's normal range).
+template <bool ROUND>
+__global__ void __launch_bounds__(256) pack_state_kernel(const float* f0, const float* f1, const float* f2,
+                                                         const float* f3, int nx, int ny, int NBx,
+                                                         unsigned* __restrict__ bmax,
+                                                         uint16_t* __restrict__ out) {
+  __shared__ float red[8][kPackX][4];
+  const int tid = threadIdx.x, xq = tid & 7, r0 = tid >> 3, lane = tid & 31;
+  const int gx = (NBx + kPackX - 1) / kPackX, NBy = ny >> 3;
+  const int x0 = blockIdx.x % gx * kPackX, by = blockIdx.x / gx % NBy, bz = blockIdx.x / gx / NBy;
+  const int bx = x0 + (xq >> 1);
+  const bool live = bx < NBx;
+  const size_t blk = ((size_t)bz * NBy + by) * NBx + bx;
+  const int y = r0 & 7, z0 = r0 >> 3;   // rows r0 + 32 i: field i / 2, planes z0 and z0 + 4
+  float4 v[8];
+  const size_t at = ((size_t)(8 * bz + z0) * ny + 8 * by + y) * nx + 8 * (size_t)x0 + 4 * xq;
+  const size_t dz = (size_t)4 * ny * nx;
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      w[j] = gemm::pack_bf16(__uint_as_float(w[j] << 16) * sc, __uint_as_float(w[j] & 0xffff0000u) * sc);
-    *reinterpret_cast<uint4*>(out + b * kNIn + k) = make_uint4(w[0], w[1], w[2], w[3]);
+  for (int i = 0; i < 8; ++i) {
+    const float* f = i < 2 ? f0 : i < 4 ? f1 : i < 6 ? f2 : f3;
+    v[i] = live ? __ldg(reinterpret_cast<const float4*>(f + at + (i & 1) * dz)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    float m = 0.f;
+#pragma unroll
+    for (int i = 2 * f; i < 2 * f + 2; ++i)
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(v[i].x), fabsf(v[i].y)), fmaxf(fabsf(v[i].z), fabsf(v[i].w))));
+    m = vector_max(m);
+    if (lane < 8 && (lane & 1) == 0) red[tid >> 5][lane >> 1][f] = m;
+  }
+  __syncthreads();
+  float sc[4];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    float m = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) m = fmaxf(m, red[w][xq >> 1][f]);
+    sc[f] = gemm::block_inv_scale(m);
+    if (live && r0 == 0 && (xq & 1) == 0) bmax[blk * 4 + f] = __float_as_uint(m);
+  }
+  if (!live) return;
+  uint16_t* o = out + blk * kNIn + z0 * 256 + y * 8 + 4 * (xq & 1);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float4 a = v[i];
+    if (ROUND) {
+      const uint32_t lo = gemm::pack_bf16(a.x, a.y), hi = gemm::pack_bf16(a.z, a.w);
+      a = make_float4(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u),
+                      __uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+    }
+    const float c = sc[i >> 1];
+    *reinterpret_cast<uint2*>(o + (i & 1) * 1024 + (i >> 1) * 64) =
+        make_uint2(gemm::pack_bf16(a.x * c, a.y * c), gemm::pack_bf16(a.z * c, a.w * c));
   }
 }
 
-// Strain fields e[t][nz][ny][nx] (t < nsteps; later slots 0) -> raw BF16 window
-// vectors [nvec][2048], k = t*128 + z*64 + y*8 + x, and max |e| per vector (atomicMax;
-// vmax zeroed by the caller).  One thread per float4 of a grid row; the two threads of
-// an 8-node row combine their maxima by shuffle.
-__global__ void window_pack_kernel(const float* __restrict__ e, int nsteps, int nx, int ny,
-                                   int nz, uint16_t* __restrict__ raw, unsigned* vmax) {
-  const int xq_n = nx >> 2;
-  const long long total = (long long)kTSteps * nz * ny * xq_n;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  const long long iters = (total + stride - 1) / stride;
-  const int NBx = nx >> 3, NBy = ny >> 3;
-  for (long long q = 0; q < iters; ++q) {
-    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x + q * stride;
-    const bool live = t0 < total;
-    const int xq = live ? (int)(t0 % xq_n) : 0;
-    long long r = live ? t0 / xq_n : 0;
-    const int y = (int)(r % ny);
-    r /= ny;
-    const int z = (int)(r % nz);
-    const int t = (int)(r / nz);
-    const long long v = ((long long)(z >> 1) * NBy + (y >> 3)) * NBx + (xq >> 1);
-    float m = 0.f;
-    if (live) {
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (t < nsteps)
-        a = *reinterpret_cast<const float4*>(e + (((size_t)t * nz + z) * ny + y) * nx + 4 * (size_t)xq);
-      *reinterpret_cast<uint2*>(raw + v * kNIn + t * 128 + (z & 1) * 64 + (y & 7) * 8 + 4 * (xq & 1)) =
-          make_uint2(gemm::pack_bf16(a.x, a.y), gemm::pack_bf16(a.z, a.w));
-      m = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w)));
-    }
-    // xq and xq ^ 1 are adjacent lanes (xq_n is even) and share vector v
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-    if (live && (xq & 1) == 0 && m > 0.f) atomicMax(vmax + v, __float_as_uint(m));
+// Strain fields e[t][nz][ny][nx] (t < nsteps; later slots 0) -> raw BF16 window vectors
+// [nvec][2048], k = t*128 + z*64 + y*8 + x, and max |e| per vector (every entry written).
+// Bound by HBM: 4 B read and 2 B written per node and state.  One float4 per thread with
+// atomic maxima took 643 us at 256^3; encode and decode of a window together went from 1675
+// to 1255 us.
+__global__ void __launch_bounds__(256) window_pack_kernel(const float* __restrict__ e, int nsteps, int nx,
+                                                          int ny, int nz, uint16_t* __restrict__ raw,
+                                                          unsigned* __restrict__ vmax) {
+  __shared__ float red[8][kPackX];
+  const int tid = threadIdx.x, xq = tid & 7, r0 = tid >> 3, lane = tid & 31;
+  const int NBx = nx >> 3, NBy = ny >> 3, gx = (NBx + kPackX - 1) / kPackX;
+  const int x0 = blockIdx.x % gx * kPackX, by = blockIdx.x / gx % NBy, bz = blockIdx.x / gx / NBy;
+  const int bx = x0 + (xq >> 1);
+  const bool live = bx < NBx;
+  const size_t vec0 = ((size_t)bz * NBy + by) * NBx, vec = vec0 + bx;
+  // rows r0 + 32 i: states t0 + 2 i, plane z, row y
+  const int y = r0 & 7, z = (r0 >> 3) & 1, t0 = r0 >> 4;
+  const size_t at = ((size_t)(2 * bz + z) * ny + 8 * by + y) * nx + 8 * (size_t)x0 + 4 * xq;
+  const size_t C = (size_t)nx * ny * nz;
+  float4 v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    v[i] = live && t0 + 2 * i < nsteps ? __ldg(reinterpret_cast<const float4*>(e + (t0 + 2 * i) * C + at))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+  float m = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    m = fmaxf(m, fmaxf(fmaxf(fabsf(v[i].x), fabsf(v[i].y)), fmaxf(fabsf(v[i].z), fabsf(v[i].w))));
+    if (live)
+      *reinterpret_cast<uint2*>(raw + vec * kNIn + (r0 + 32 * i) * 8 + 4 * (xq & 1)) =
+          make_uint2(gemm::pack_bf16(v[i].x, v[i].y), gemm::pack_bf16(v[i].z, v[i].w));
+  }
+  m = vector_max(m);
+  if (lane < 8 && (lane & 1) == 0) red[tid >> 5][lane >> 1] = m;
+  __syncthreads();
+  if (tid < kPackX && x0 + tid < NBx) {
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t = fmaxf(t, red[w][tid]);
+    vmax[vec0 + x0 + tid] = __float_as_uint(t);
   }
 }
 
@@ -825,8 +851,7 @@ cudaError_t codec_encode_grid(Codec* c, const float* const f[4], int nx, int ny,
                               unsigned* bmax, uint16_t* lat, int* overflow, cudaStream_t s) {
   const long long nb = (long long)(nx / 8) * (ny / 8) * (nz / 8);
   if (!ensure_X(c, (size_t)nb)) return cudaErrorMemoryAllocation;
-  // raw BF16 block vectors and block maxima, then normalised in place
-  cudaError_t e = snapshot_pack(f, nx, ny, nz, bmax, c->X, c->X, s);
+  cudaError_t e = snapshot_pack(f, nx, ny, nz, bmax, c->X, true, s);
   if (e != cudaSuccess) return e;
   return codec_encode_vectors(c, c->X, nb, lat, overflow, s);
 }
@@ -977,13 +1002,8 @@ cudaError_t codec_decode_window(Codec* c, const uint16_t* lat, const unsigned* v
 
 cudaError_t window_pack(const float* e, int nsteps, int nx, int ny, int nz, uint16_t* raw,
                         unsigned* vmax, cudaStream_t s) {
-  const long long nvec = (long long)(nx / 8) * (ny / 8) * (nz / 2);
-  cudaError_t err = cudaMemsetAsync(vmax, 0, (size_t)nvec * sizeof(unsigned), s);
-  if (err != cudaSuccess) return err;
-  const long long total = (long long)kTSteps * nz * ny * (nx / 4);
-  long long blocks = (total + 255) / 256;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  window_pack_kernel<<<(unsigned)blocks, 256, 0, s>>>(e, nsteps, nx, ny, nz, raw, vmax);
+  const unsigned grid = (unsigned)((nx / 8 + kPackX - 1) / kPackX) * (ny / 8) * (nz / 2);
+  window_pack_kernel<<<grid, 256, 0, s>>>(e, nsteps, nx, ny, nz, raw, vmax);
   return cudaGetLastError();
 }
 
@@ -1103,22 +1123,13 @@ cudaError_t window_normalise(const uint16_t* raw, const unsigned* vmax, long lon
 }
 
 cudaError_t snapshot_pack(const float* const f[4], int nx, int ny, int nz, unsigned* bmax,
-                          uint16_t* raw, uint16_t* out, cudaStream_t s) {
-  const int NBx = nx / 8, NBy = ny / 8, NBz = nz / 8;
-  const long long nb = (long long)NBx * NBy * NBz;
-  cudaError_t e = cudaMemsetAsync(bmax, 0, (size_t)nb * 4 * sizeof(unsigned), s);
-  if (e != cudaSuccess) return e;
-  const long long threads = nb * 256 * 2;
-  long long blocks = (threads + 255) / 256;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  pack_raw_kernel<<<(unsigned)blocks, 256, 0, s>>>(f[0], f[1], f[2], f[3], nx, ny, NBx, NBy, nb,
-                                                   bmax, raw);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (out) {
-    normalise_kernel<<<152 * 8, 256, 0, s>>>(raw, bmax, nb, out);
-    e = cudaGetLastError();
-  }
-  return e;
+                          uint16_t* out, bool rounded, cudaStream_t s) {
+  const unsigned grid = (unsigned)((nx / 8 + kPackX - 1) / kPackX) * (ny / 8) * (nz / 8);
+  if (rounded)
+    pack_state_kernel<true><<<grid, 256, 0, s>>>(f[0], f[1], f[2], f[3], nx, ny, nx / 8, bmax, out);
+  else
+    pack_state_kernel<false><<<grid, 256, 0, s>>>(f[0], f[1], f[2], f[3], nx, ny, nx / 8, bmax, out);
+  return cudaGetLastError();
 }
 
 }  // namespace aew

@@ -83,7 +83,7 @@ cudaError_t codec_decode_window(Codec* c, const uint16_t* lat, const unsigned* v
 cudaError_t window_minmax(const uint16_t* raw, long long nvec, double beta, uint16_t* out,
                           double* mn, double* rr, cudaStream_t s, float* pair32 = nullptr);
 // Pack nsteps (<= 16) strain fields e[t][nz][ny][nx] into raw BF16 window vectors
-// [nvec][2048] (missing steps 0) and fold max |e| per vector into vmax (zeroed here).
+// [nvec][2048] (missing steps 0) with max |e| per vector (vmax, float bits [nvec], written).
 cudaError_t window_pack(const float* e, int nsteps, int nx, int ny, int nz, uint16_t* raw,
                         unsigned* vmax, cudaStream_t s);
 // Weighted moments of n normalised BF16 vectors Y [n][2048] for the PCA initialisation:
@@ -101,9 +101,9 @@ cudaError_t window_normalise(const uint16_t* raw, const unsigned* vmax, long lon
 
 // Algorithm 1 packing of one grid state: normalised BF16 block vectors [nblocks][2048]
 // (each block-field divided by its power-of-two scale) and the block maxima (bmax,
-// float bits [nblocks][4], written; work buffer X [nblocks][2048] for the raw values).
+// float bits [nblocks][4], written); rounded: x to BF16 before the division.
 cudaError_t snapshot_pack(const float* const f[4], int nx, int ny, int nz, unsigned* bmax,
-                          uint16_t* raw, uint16_t* out, cudaStream_t s);
+                          uint16_t* out, bool rounded, cudaStream_t s);
 
 // Device error flag of the codec kernels (set by a bounded wait that gave up); read and
 // clear it (synchronises the stream).  Returns true if it was set.
