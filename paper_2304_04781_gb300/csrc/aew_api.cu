@@ -1162,8 +1162,40 @@ int snapshots_time(aew_handle* h, int every, uint16_t* out, long long max_vector
     AEW_CK(cudaMemsetAsync(out + (size_t)at[0] * aew::kNIn, 0, nv * aew::kNIn * sizeof(uint16_t), s));
     AEW_CK(cudaMemsetAsync(vm(0), 0, nv * sizeof(unsigned), s));
   }
+  // the window whose last state is in: normalised in place
+  auto finish = [&](int tb) -> int {
+    uint16_t* tp = out + (size_t)at[tb] * aew::kNIn;
+    if (mm)   // offsets and ranges out as FP32 pairs
+      AEW_CK(aew::window_minmax(tp, (long long)nv, aew::codec_beta(h->codec), tp, nullptr, nullptr, s,
+                                vmax_dev ? vmax_dev + 2 * (size_t)at[tb] : nullptr));
+    else
+      AEW_CK(aew::window_normalise(tp, vm(tb), (long long)nv, tp, s));
+    ++h->stats.kernel_launches;
+    return AEW_OK;
+  };
   int cur = 0;
-  for (int n = 0; n < T * last + T - 1; ++n) {
+  for (int tb = 0, n = 0; h->brick && tb <= last; ++tb) {
+    if (at[tb] < 0) continue;
+    // one launch up to the window's first state - 1, one for the window itself
+    const int m0 = std::max(T * tb, 1), ends[2] = {m0 - 1, T * tb + T - 1};
+    for (int i = 0; i < 2; ++i) {
+      if (ends[i] <= n) continue;
+      aew::BrickFwd a = brick_fwd_args(h, n ? h->st[cur] : nullptr, h->st[cur ^ 1], ends[i] - n,
+                                       h->dts + n, nullptr);
+      if (i == 1) {
+        if (tb > 0) AEW_CK(cudaMemsetAsync(vm(tb), 0, nv * sizeof(unsigned), s));
+        a.npack = a.nsteps;
+        a.tpack = out + (size_t)at[tb] * aew::kNIn;
+        a.vmax = vm(tb);
+        a.tslot = m0 - T * tb;
+      }
+      if ((rc = brick_fwd(h, a, s))) return rc;
+      cur ^= 1;
+      n = ends[i];
+    }
+    if ((rc = finish(tb))) return rc;
+  }
+  for (int n = 0; !h->brick && n < T * last + T - 1; ++n) {
     const int m = n + 1, tb = m / T, slot = m % T;
     uint16_t* tp = nullptr;
     unsigned* vq = nullptr;
@@ -1176,14 +1208,7 @@ int snapshots_time(aew_handle* h, int every, uint16_t* out, long long max_vector
                        nullptr, nullptr, tp, slot, vq)))
       return rc;
     cur ^= 1;
-    if (tp && slot == T - 1) {
-      if (aew::codec_minmax(h->codec))   // offsets and ranges out as FP32 pairs
-        AEW_CK(aew::window_minmax(tp, (long long)nv, aew::codec_beta(h->codec), tp, nullptr, nullptr, s,
-                                  vmax_dev ? vmax_dev + 2 * (size_t)at[tb] : nullptr));
-      else
-        AEW_CK(aew::window_normalise(tp, vq, (long long)nv, tp, s));
-      ++h->stats.kernel_launches;
-    }
+    if (tp && slot == T - 1 && (rc = finish(tb))) return rc;
   }
   AEW_CK(cudaStreamSynchronize(s));
   *n_written = w;
@@ -2201,6 +2226,20 @@ int aew_snapshots(aew_handle* h, const float* c_dev, int every, uint16_t* out_de
     return block_max_dev ? reinterpret_cast<unsigned*>(block_max_dev) + (size_t)w * 4
                          : h->bm_tmp + ((size_t)(w / (long long)nb) & 1) * nb * 4;
   };
+  if (h->brick) {   // on chip from one packed state to the next
+    for (int n = 0, m = every; packs(m, written); n = m, m += every, cur ^= 1) {
+      if ((rc = brick_fwd(h, brick_fwd_args(h, n ? h->st[cur] : nullptr, h->st[cur ^ 1], m - n,
+                                            h->dts + n, nullptr), s)))
+        return rc;
+      AEW_CK(aew::snapshot_pack(h->st[cur ^ 1], h->cfg.nx, h->cfg.ny, h->cfg.nz, bm_at(written),
+                                out_dev + (size_t)written * aew::kNIn, false, s));
+      ++h->stats.kernel_launches;
+      written += (long long)nb;
+    }
+    AEW_CK(cudaStreamSynchronize(s));
+    *n_written = written;
+    return AEW_OK;
+  }
   for (int n = 0; n < nt; ++n) {
     const bool pack = packs(n, written);
     if (n + 1 == nt && !pack) break;

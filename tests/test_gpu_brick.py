@@ -91,6 +91,21 @@ def test_time_codec_equals_the_streaming_kernels(shape, nt, norm, monkeypatch):
     same(*both(monkeypatch, make, run))
 
 
+@pytest.mark.parametrize("codec,every,room", [("space", 1, 4), ("space", 7, 99), ("time", 1, 99),
+                                              ("time", 2, 99)])
+@pytest.mark.parametrize("shape", [(8, 8, 8), (24, 40, 72), (96, 96, 96)])
+def test_snapshots_equal_the_streaming_kernels(shape, codec, every, room, monkeypatch):
+    """Algorithm 1: packed vectors and maxima, with room for some or all of the states."""
+    prob, c, _ = setup(shape, 67, 1, seed=9)
+
+    def run(s):
+        unit = s.nvec if codec == "time" else s.nblocks
+        v, m = s.snapshots(cuda(c), every, room * unit + 1, with_scales=True)
+        return [v, m, s.snapshots(cuda(c), every, room * unit)]
+
+    same(*both(monkeypatch, lambda: solver(prob, storage="revolve", n_checkpoints=0, codec=codec), run))
+
+
 def test_smoothed_source_and_window_of_one(monkeypatch):
     """A source spread over many bricks, and an FP64 flush in every step."""
     shape = (48, 52, 56)
