@@ -10,10 +10,14 @@
 // products.  Arithmetic is FP32 -- GB300's FP64 rate is a small fraction of its FP32
 // rate -- with FP64 only in the reductions.
 //
-// Prior solve A x = w: conjugate gradients whose scalars never leave the device.  Each
-// kernel that needs rr or p^T A p sums the previous kernel's per-block FP64 partials
-// itself (every block in the same order, so all blocks agree), so an iteration is three
-// launches and the host reads the residual only every 8 iterations.
+// Prior solve A x = w: conjugate gradients whose scalars never leave the device, in two
+// passes over the vectors per iteration: (1) p' = r + b p with the partials of p'.Ap',
+// (2) x += a p', r -= a Ap' with the partials of r.r.  A p' is not stored: both passes take
+// it from a tile of p' planes (neighbouring rows in shared memory, planes in registers).
+// Each kernel sums the previous one's per-block FP64 partials itself (every block in the
+// same order, so all blocks agree).  The residual is tested on the device every 8
+// iterations; once it passes, the kernels already enqueued return at once, so the host
+// stays a batch of launches ahead of the test.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -200,46 +204,275 @@ __global__ void dot_kernel(const float* __restrict__ a, const float* __restrict_
   block_store(acc, part);
 }
 
-// CG for A x = w, FP32 vectors, scalars from FP64 partials (see the file comment).
-// update: a = rr / pAp; x += a p; r -= a Ap; partials of r.r into prr_new
-__global__ void cg_update_kernel(float* __restrict__ x, float* __restrict__ r,
-                                 const float* __restrict__ p, const float* __restrict__ Ap,
-                                 size_t n, const double* ppap, const double* prr, int nblk,
-                                 double* prr_new) {
-  const double pap = block_sum_of(ppap, nblk);
-  const double rr = block_sum_of(prr, nblk);
-  const float a = pap > 0.0 ? (float)(rr / pap) : 0.f;
-  float4* x4 = reinterpret_cast<float4*>(x);
-  float4* r4 = reinterpret_cast<float4*>(r);
-  const float4* p4 = reinterpret_cast<const float4*>(p);
-  const float4* q4 = reinterpret_cast<const float4*>(Ap);
-  Acc acc;
-  for (size_t i = blockIdx.x * (size_t)NT + threadIdx.x; i < n / 4; i += (size_t)gridDim.x * NT) {
-    const float4 pi = p4[i], qi = q4[i];
-    float4 xi = x4[i], ri = r4[i];
-    xi.x += a * pi.x; xi.y += a * pi.y; xi.z += a * pi.z; xi.w += a * pi.w;
-    ri.x -= a * qi.x; ri.y -= a * qi.y; ri.z -= a * qi.z; ri.w -= a * qi.w;
-    x4[i] = xi;
-    r4[i] = ri;
-    acc.add(dot4(ri, ri));
+// ---- CG for A x = w, FP32 vectors, scalars from FP64 partials (see the file comment) ----
+// A block takes a column of 128 x kCgRows nodes through kz planes: warp w holds row
+// y0 + w - 1 (the first and the last warp only feed their neighbours), lane l four nodes; the
+// next two planes are in flight in registers.  Bound by HBM: 12 B (r, p in, p' out) and 20 B
+// (p', r, x in, r, x out) per node; passes of alternating direction find the last planes of
+// the pass before in L2.  One iteration at 256^3 takes 131 us, where apply, update and
+// direction passes (8 + 24 + 12 B, the apply through L1 / L2) took 190.
+constexpr int kCgWarps = 12, kCgRows = kCgWarps - 2, kCgThreads = 32 * kCgWarps;
+
+struct CgTile {
+  int lane, x, y, z0, z1;   // the thread's nodes x .. x + 3 of row y; planes z0 .. z1 - 1
+  bool in, own, hx0, hx1;   // inside the grid; a row of the block's own; x neighbours exist
+  size_t i;                 // index of the nodes in plane z0
+  __device__ __forceinline__ CgTile(const Grid& g, int kz, bool reverse) {
+    lane = threadIdx.x & 31;
+    const int w = threadIdx.x >> 5, tx = (g.nx + 127) / 128, ty = (g.ny + kCgRows - 1) / kCgRows;
+    const int b = reverse ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    x = b % tx * 128 + 4 * lane;
+    y = b / tx % ty * kCgRows + w - 1;
+    z0 = b / tx / ty * kz;
+    z1 = min(z0 + kz, g.nz);
+    in = x < g.nx && y >= 0 && y < g.ny;
+    own = in && w >= 1 && w <= kCgRows;
+    hx0 = x > 0;
+    hx1 = x + 4 < g.nx;
+    i = ((size_t)z0 * g.ny + (in ? y : 0)) * g.nx + (in ? x : 0);
   }
-  block_store(acc.total(), prr_new);
+};
+
+// FP64 sums of the CG passes.  An FP64 add takes the SM 16 cycles per warp, so few warps do
+// them: one warp sums a kernel's partials (any order would do, but all blocks agree), and one
+// the threads' totals.
+// Within a thread the terms are summed in FP32 with the rounding errors kept (Knuth's two-sum),
+// since FP64 instructions slow the walk even where they are skipped.
+struct CgAcc {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
+    s = t;
+  }
+  __device__ __forceinline__ double total() const { return (double)s + (double)c; }
+};
+__device__ __forceinline__ double cg_warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// the sums of two arrays of partials, by warps 0 and 1
+__device__ __forceinline__ void cg_sums_of(const double* __restrict__ p0, int n0, const double* __restrict__ p1,
+                                           int n1, double* out) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w < 2) {
+    const double* p = w ? p1 : p0;
+    const int n = w ? n1 : n0;
+    double v = 0.0;
+    for (int i = lane; i < n; i += 32) v += p[i];
+    v = cg_warp_sum(v);
+    if (lane == 0) out[w] = v;
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ void cg_store_sum(double v, double* all, double* part) {
+  all[threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < kCgThreads; i += 32) s += all[i];
+    s = cg_warp_sum(s);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+  }
 }
 
-// direction: p = r + (rr_new / rr_old) p
-__global__ void cg_dir_kernel(float* __restrict__ p, const float* __restrict__ r, size_t n,
-                              const double* prr_old, const double* prr_new, int nblk) {
-  const double ro = block_sum_of(prr_old, nblk);
-  const double rn = block_sum_of(prr_new, nblk);
-  const float b = ro > 0.0 ? (float)(rn / ro) : 0.f;
-  float4* p4 = reinterpret_cast<float4*>(p);
-  const float4* r4 = reinterpret_cast<const float4*>(r);
-  for (size_t i = blockIdx.x * (size_t)NT + threadIdx.x; i < n / 4; i += (size_t)gridDim.x * NT) {
-    const float4 ri = r4[i];
-    float4 pi = p4[i];
-    pi.x = ri.x + b * pi.x; pi.y = ri.y + b * pi.y; pi.z = ri.z + b * pi.z; pi.w = ri.w + b * pi.w;
-    p4[i] = pi;
+// A x at four nodes from the plane's values c, the planes below and above, the rows on both
+// sides and the x neighbours, in the order of prior_kernel
+__device__ __forceinline__ float4 cg_apply(const Grid& g, const CgTile& t, int k, float4 c, float4 zm, float4 zp,
+                                           float4 ym, float4 yp, float xl, float xr, float alpha, float at) {
+  float v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float xn = f4c(c, q);
+    float lap = 0.f;
+    if (q > 0 || t.hx0) lap += (q == 0 ? xl : f4c(c, q - 1)) - xn;
+    if (q < 3 || t.hx1) lap += (q == 3 ? xr : f4c(c, q + 1)) - xn;
+    if (t.y > 0) lap += f4c(ym, q) - xn;
+    if (t.y + 1 < g.ny) lap += f4c(yp, q) - xn;
+    if (k > 0) lap += f4c(zm, q) - xn;
+    if (k + 1 < g.nz) lap += f4c(zp, q) - xn;
+    v[q] = alpha * xn - at * lap;
   }
+  return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// The planes of one field F as a block walks them: F.load(k) issues plane k's loads, F.get()
+// returns the oldest one's value.  edge: the x neighbour of lane 0 (node x - 1) or 31 (x + 4).
+struct CgRaw {
+  float4 a, b;
+  float ea, eb;
+};
+// walk the planes; body(k, c, v = A c) runs for the block's own nodes
+template <class Load, class Value, class Edge, class Body>
+__device__ __forceinline__ void cg_walk(const Grid& g, const CgTile& t, float alpha, float at, Load load,
+                                        Value value, Edge edge, Body body) {
+  __shared__ float4 sm[2][kCgWarps][32];
+  const int w = threadIdx.x >> 5;
+  CgRaw r0 = load(t.z0 - 1);
+  CgRaw r1 = load(t.z0);
+  CgRaw r2 = load(t.z0 + 1);
+  float4 zm = value(r0), c = value(r1);
+  float ec = edge(r1);
+  r1 = r2;
+  sm[t.z0 & 1][w][t.lane] = c;
+  for (int k = t.z0; k < t.z1; ++k) {
+    r2 = load(k + 2);   // in flight for two planes
+    const float4 n = value(r1);
+    const float en = edge(r1);
+    __syncthreads();
+    sm[(k + 1) & 1][w][t.lane] = n;
+    float xl = __shfl_up_sync(0xffffffffu, c.w, 1), xr = __shfl_down_sync(0xffffffffu, c.x, 1);
+    if (t.lane == 0) xl = ec;
+    if (t.lane == 31) xr = ec;
+    if (t.own) body(k, c, cg_apply(g, t, k, c, zm, n, sm[k & 1][w - 1][t.lane], sm[k & 1][w + 1][t.lane], xl, xr,
+                                   alpha, at));
+    zm = c;
+    c = n;
+    ec = en;
+    r1 = r2;
+  }
+}
+
+// (1) p' = r + b p, b = rr_new / rr_old (first: p' = r), partials of p'.Ap' into ppap.  With
+// check the residual test comes first: rr_new <= tol2 ends the solve after `it` iterations.
+__global__ void __launch_bounds__(kCgThreads, 2)
+    cg_dir_kernel(const float* __restrict__ r, const float* __restrict__ p, float* __restrict__ pn, Grid g,
+                  float alpha, float at, int kz, const double* prr_old, int nold, const double* prr_new, int nblk,
+                  bool first, bool check, double tol2, int it, int* done, double* ppap) {
+  __shared__ double sums[2], all[kCgThreads];
+  if (*reinterpret_cast<volatile int*>(done) >= 0) return;
+  float b = 0.f;
+  if (!first) {
+    cg_sums_of(prr_new, nblk, prr_old, nold, sums);
+    const double rn = sums[0], ro = sums[1];
+    if (check && rn <= tol2) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) *done = it;
+      return;
+    }
+    b = ro > 0.0 ? (float)(rn / ro) : 0.f;
+  }
+  const CgTile t(g, kz, false);
+  const size_t P = (size_t)g.nx * g.ny;
+  CgAcc acc;
+  cg_walk(
+      g, t, alpha, at,
+      [&](int k) {
+        CgRaw q{make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), 0.f, 0.f};
+        if (t.in && k >= 0 && k < g.nz && k <= t.z1) {
+          const size_t i = t.i + (ptrdiff_t)(k - t.z0) * (ptrdiff_t)P;
+          q.a = *reinterpret_cast<const float4*>(r + i);
+          if (!first) q.b = *reinterpret_cast<const float4*>(p + i);
+          const bool l = t.lane == 0 && t.hx0, h = t.lane == 31 && t.hx1;
+          if (l || h) {
+            const size_t j = l ? i - 1 : i + 4;
+            q.ea = r[j];
+            if (!first) q.eb = p[j];
+          }
+        }
+        return q;
+      },
+      [&](const CgRaw& q) {
+        return make_float4(fmaf(b, q.b.x, q.a.x), fmaf(b, q.b.y, q.a.y), fmaf(b, q.b.z, q.a.z),
+                           fmaf(b, q.b.w, q.a.w));
+      },
+      [&](const CgRaw& q) { return fmaf(b, q.eb, q.ea); },
+      [&](int k, float4 c, float4 v) {
+        *reinterpret_cast<float4*>(pn + t.i + (size_t)(k - t.z0) * P) = c;
+        acc.add(dot4(c, v));
+      });
+  cg_store_sum(acc.total(), all, ppap);
+}
+
+// (2) a = rr / p.Ap; x += a p; r -= a Ap; partials of r.r into prr_new
+__global__ void __launch_bounds__(kCgThreads, 2)
+    cg_update_kernel(float* __restrict__ x, float* __restrict__ r, const float* __restrict__ p, Grid g,
+                     float alpha, float at, int kz, const double* ppap, int npap, const double* prr, int nblk,
+                     const int* done, double* prr_new) {
+  __shared__ double sums[2], all[kCgThreads];
+  if (*reinterpret_cast<const volatile int*>(done) >= 0) return;
+  cg_sums_of(ppap, npap, prr, nblk, sums);
+  const double pap = sums[0], rr = sums[1];
+  const float a = pap > 0.0 ? (float)(rr / pap) : 0.f;
+  const CgTile t(g, kz, true);
+  const size_t P = (size_t)g.nx * g.ny;
+  CgAcc acc;
+  // x and r of the own rows travel with the plane of p they belong to
+  struct Own {
+    float4 x, r;
+  };
+  Own o0{}, o1{};
+  auto own_at = [&](int k) {
+    Own o{make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    if (t.own && k < t.z1) {
+      const size_t i = t.i + (size_t)(k - t.z0) * P;
+      o.x = *reinterpret_cast<const float4*>(x + i);
+      o.r = *reinterpret_cast<const float4*>(r + i);
+    }
+    return o;
+  };
+  o0 = own_at(t.z0);
+  cg_walk(
+      g, t, alpha, at,
+      [&](int k) {
+        CgRaw q{make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), 0.f, 0.f};
+        if (t.in && k >= 0 && k < g.nz && k <= t.z1) {
+          const size_t i = t.i + (ptrdiff_t)(k - t.z0) * (ptrdiff_t)P;
+          q.a = *reinterpret_cast<const float4*>(p + i);
+          const bool l = t.lane == 0 && t.hx0, h = t.lane == 31 && t.hx1;
+          if (l || h) q.ea = p[l ? i - 1 : i + 4];
+        }
+        if (k >= t.z0 + 2) o1 = own_at(k - 1);   // plane k - 1 is two walks away
+        return q;
+      },
+      [&](const CgRaw& q) { return q.a; }, [&](const CgRaw& q) { return q.ea; },
+      [&](int k, float4 c, float4 v) {
+        const size_t i = t.i + (size_t)(k - t.z0) * P;
+        float4 xi = o0.x, ri = o0.r;
+        xi.x += a * c.x; xi.y += a * c.y; xi.z += a * c.z; xi.w += a * c.w;
+        ri.x -= a * v.x; ri.y -= a * v.y; ri.z -= a * v.z; ri.w -= a * v.w;
+        *reinterpret_cast<float4*>(x + i) = xi;
+        *reinterpret_cast<float4*>(r + i) = ri;
+        acc.add(dot4(ri, ri));
+        o0 = o1;
+      });
+  cg_store_sum(acc.total(), all, prr_new);
+}
+
+// the residual test after the last iteration allowed
+__global__ void cg_check_kernel(const double* prr, int nblk, double tol2, int it, int* done) {
+  if (*done >= 0) return;
+  const double rr = block_sum_of(prr, nblk);
+  if (threadIdx.x == 0 && rr <= tol2) *done = it;
+}
+
+// r = sc w, x = 0
+__global__ void cg_start_kernel(const float* __restrict__ w, float sc, float* __restrict__ r,
+                                float* __restrict__ x, size_t n) {
+  const float4* w4 = reinterpret_cast<const float4*>(w);
+  for (size_t i = blockIdx.x * (size_t)NT + threadIdx.x; i < n / 4; i += (size_t)gridDim.x * NT) {
+    const float4 u = w4[i];
+    reinterpret_cast<float4*>(r)[i] = make_float4(sc * u.x, sc * u.y, sc * u.z, sc * u.w);
+    reinterpret_cast<float4*>(x)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
+
+// planes per block of the CG passes: whole waves of two blocks per SM with the least planes
+// walked (a block walks two more than it owns)
+int cg_planes(const Grid& g, int sms, int* blocks) {
+  const long long cols = (long long)((g.nx + 127) / 128) * ((g.ny + kCgRows - 1) / kCgRows);
+  int best = g.nz;
+  double cost = 0.0;
+  for (int kz = 4; kz <= 64; ++kz) {
+    const long long n = cols * ((g.nz + kz - 1) / kz);
+    if (n > 16384) continue;
+    const double c = (double)((n + 2 * sms - 1) / (2 * sms)) * (std::min(kz, g.nz) + 2);
+    if (cost == 0.0 || c < cost) {
+      cost = c;
+      best = kz;
+    }
+  }
+  *blocks = (int)(cols * ((g.nz + best - 1) / best));
+  return best;
 }
 
 // projection: partial dots of v with the r rows of W1, part[k][nblk]
@@ -371,9 +604,22 @@ __global__ void combine_kernel(const float* __restrict__ G, int N, size_t n,
 
 // device buffers of one call, freed when it returns
 struct Work {
-  std::vector<void*> ptrs;
+  std::vector<void*> ptrs, hosts;
   ~Work() {
     for (void* p : ptrs) cudaFree(p);
+    for (void* p : hosts) cudaFreeHost(p);
+  }
+  template <class T>
+  bool alloc_host(T** p, size_t count) {
+    void* q = nullptr;
+    if (cudaMallocHost(&q, count * sizeof(T)) != cudaSuccess) {
+      cudaGetLastError();
+      *p = nullptr;
+      return false;
+    }
+    hosts.push_back(q);
+    *p = static_cast<T*>(q);
+    return true;
   }
   template <class T>
   bool alloc(T** p, size_t count) {
@@ -454,21 +700,26 @@ int prior_args_ok(aew_handle* h, double alpha, double theta) {
 // CG on A x = w (device scalars); x_dev written
 int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta,
              const float* w, float* x, double rtol, int max_iter, int* iters, cudaStream_t s) {
+  int dev = 0, sms = 0, cb = 0;
+  NW_CK(cudaGetDevice(&dev));
+  NW_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int kz = cg_planes(g, sms > 0 ? sms : 1, &cb), nb = vec_grid(g.C);
+  const int np = std::max(cb, nb);   // partials per reduction
   Work ws;
-  float *r, *p, *Ap;
-  double* part;   // [3][kVecBlocks]: p.Ap, rr (two parities)
-  if (!ws.alloc(&r, g.C) || !ws.alloc(&p, g.C) || !ws.alloc(&Ap, g.C) ||
-      !ws.alloc(&part, 3 * (size_t)kVecBlocks))
+  float *r, *p[2];
+  double* part;   // [3][np]: p.Ap, rr (two parities)
+  int *done, *seen;
+  if (!ws.alloc(&r, g.C) || !ws.alloc(&p[0], g.C) || !ws.alloc(&p[1], g.C) ||
+      !ws.alloc(&part, 3 * (size_t)np) || !ws.alloc(&done, 1) || !ws.alloc_host(&seen, 2))
     return set_error(h, AEW_E_NOMEM, "prior solve: work vectors do not fit");
-  const int nb = vec_grid(g.C);
   double* ppap = part;
-  double* prr[2] = {part + kVecBlocks, part + 2 * kVecBlocks};
+  double* prr[2] = {part + np, part + 2 * (size_t)np};
   const float fa = (float)alpha, fat = (float)(alpha * theta / (hh * hh));
-  dot_kernel<<<nb, NT, 0, s>>>(w, w, g.C, prr[0]);
-  NW_CK(cudaGetLastError());
   std::vector<double> hp(nb);
-  auto host_sum = [&](const double* dpart, double* out) -> int {
-    NW_CK(cudaMemcpyAsync(hp.data(), dpart, nb * sizeof(double), cudaMemcpyDeviceToHost, s));
+  auto host_dot = [&](const float* v, double* out) -> int {   // v.v; partials left in prr[0]
+    dot_kernel<<<nb, NT, 0, s>>>(v, v, g.C, prr[0]);
+    NW_CK(cudaGetLastError());
+    NW_CK(cudaMemcpyAsync(hp.data(), prr[0], nb * sizeof(double), cudaMemcpyDeviceToHost, s));
     NW_CK(cudaStreamSynchronize(s));
     double a = 0.0;
     for (int i = 0; i < nb; ++i) a += hp[i];
@@ -476,7 +727,7 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
     return AEW_OK;
   };
   double ww = 0.0;
-  int rc = host_sum(prr[0], &ww);
+  int rc = host_dot(w, &ww);
   if (rc) return rc;
   if (iters) *iters = 0;
   if (ww == 0.0) {   // w = 0: x = 0
@@ -486,36 +737,51 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   // solve for the unit-rms right-hand side sc w (the iteration's FP32 squares then stay
   // far from FP32's range limits), and scale x back at the end
   const double sc = std::sqrt((double)g.C / ww);
-  NW_CK(cudaMemsetAsync(x, 0, g.C * sizeof(float), s));
-  axpby_kernel<<<nb, NT, 0, s>>>((float)sc, w, 0.f, w, r, g.C);
-  axpby_kernel<<<nb, NT, 0, s>>>((float)sc, w, 0.f, w, p, g.C);
+  cg_start_kernel<<<nb, NT, 0, s>>>(w, (float)sc, r, x, g.C);
+  NW_CK(cudaMemsetAsync(done, 0xff, sizeof(int), s));   // -1: not yet
   NW_CK(cudaGetLastError());
-  dot_kernel<<<nb, NT, 0, s>>>(r, r, g.C, prr[0]);
-  NW_CK(cudaGetLastError());
-  if ((rc = host_sum(prr[0], &ww))) return rc;
+  if ((rc = host_dot(r, &ww))) return rc;
   const double tol2 = rtol * rtol * ww;
-  int it = 0;
-  for (; it < max_iter; ++it) {
-    const int cur = it & 1, nxt = cur ^ 1;
-    prior_kernel<<<nb, NT, 0, s>>>(p, Ap, nullptr, g, fa, fat, p, ppap);
-    cg_update_kernel<<<nb, NT, 0, s>>>(x, r, p, Ap, g.C, ppap, prr[cur], nb, prr[nxt]);
-    cg_dir_kernel<<<nb, NT, 0, s>>>(p, r, g.C, prr[cur], prr[nxt], nb);
+  // batches of 8 iterations; the host reads batch j's flag after enqueueing batch j + 1
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  struct Events {
+    cudaEvent_t* e;
+    ~Events() {
+      for (int i = 0; i < 2; ++i)
+        if (e[i]) cudaEventDestroy(e[i]);
+    }
+  } guard{ev};
+  for (auto& e : ev) NW_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  int it = 0, at = -1, last = nb;   // last: partials of the newest r.r
+  for (int batch = 0; it < max_iter && at < 0; ++batch) {
+    for (int q = 0; q < 8 && it < max_iter; ++q, ++it) {
+      const int cur = it & 1, nxt = cur ^ 1;   // prr[cur]: the newest r.r, prr[nxt]: the one before
+      cg_dir_kernel<<<cb, kCgThreads, 0, s>>>(r, p[cur], p[nxt], g, fa, fat, kz, prr[nxt], it == 1 ? nb : cb, prr[cur], cb,
+                                              it == 0, q == 0, tol2, it, done, ppap);
+      cg_update_kernel<<<cb, kCgThreads, 0, s>>>(x, r, p[nxt], g, fa, fat, kz, ppap, cb, prr[cur], last, done,
+                                                 prr[nxt]);
+      last = cb;
+    }
     NW_CK(cudaGetLastError());
-    if ((it & 7) == 7 || it + 1 == max_iter) {
-      double rr = 0.0;
-      if ((rc = host_sum(prr[nxt], &rr))) return rc;
-      if (rr <= tol2) {
-        ++it;
-        if (iters) *iters = it;
-        axpby_kernel<<<nb, NT, 0, s>>>((float)(1.0 / sc), x, 0.f, x, x, g.C);
-        NW_CK(cudaGetLastError());
-        return AEW_OK;
-      }
+    NW_CK(cudaMemcpyAsync(seen + (batch & 1), done, sizeof(int), cudaMemcpyDeviceToHost, s));
+    NW_CK(cudaEventRecord(ev[batch & 1], s));
+    if (batch > 0) {
+      NW_CK(cudaEventSynchronize(ev[(batch - 1) & 1]));
+      at = seen[(batch - 1) & 1];
     }
   }
-  if (iters) *iters = it;
+  if (at < 0) {
+    cg_check_kernel<<<1, NT, 0, s>>>(prr[it & 1], last, tol2, it, done);
+    NW_CK(cudaGetLastError());
+    NW_CK(cudaMemcpyAsync(seen, done, sizeof(int), cudaMemcpyDeviceToHost, s));
+    NW_CK(cudaStreamSynchronize(s));
+    at = seen[0];
+  }
+  if (iters) *iters = at >= 0 ? at : it;
   axpby_kernel<<<nb, NT, 0, s>>>((float)(1.0 / sc), x, 0.f, x, x, g.C);
   NW_CK(cudaGetLastError());
+  NW_CK(cudaStreamSynchronize(s));   // the work vectors are freed on return
+  if (at >= 0) return AEW_OK;
   char buf[160];
   std::snprintf(buf, sizeof buf, "prior solve: relative residual above %.3g after %d iterations",
                 rtol, max_iter);
