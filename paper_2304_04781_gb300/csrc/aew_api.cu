@@ -24,6 +24,7 @@
 #include "aew_pca.h"
 #include "aew_revolve.h"
 #include "aew_solver.h"
+#include "aew_twostep.h"
 
 using aew::Codec;
 
@@ -113,6 +114,8 @@ struct aew_handle {
   // grids that fit the SMs run their time loops on chip (aew_brick.h): the cut, the halo
   // exchange buffer with its running tag, and dt s^n of the default and of a given wavelet
   bool brick = false;
+  bool two = false;   // larger grids: two steps per pass (aew_twostep.h)
+  int sms = 0;
   aew::BrickPlan bp;
   unsigned char* halo = nullptr;
   uint32_t halo_tag = 0;
@@ -425,6 +428,95 @@ int brick_adj(aew_handle* h, int n0, int nsteps, float* const in[4], float* cons
   return AEW_OK;
 }
 
+// ---------------------------------------------------------------------------------
+// Two steps per pass (aew_twostep.h)
+// ---------------------------------------------------------------------------------
+// the window slot of a state (null tp: the state is not packed)
+struct PackAt {
+  uint16_t* tp = nullptr;
+  unsigned* vm = nullptr;
+  int slot = 0;
+};
+// forward steps n and n + 1: in -> out, e^{n+1} to e1 (null: not kept), receiver rows from
+// d_row on (null: none)
+aew::TwoFwd two_fwd_args(aew_handle* h, int n, float* const in[4], float* const out[4], float* e1,
+                         const float* wav, float* d_row) {
+  aew::TwoFwd a{};
+  a.m = h->m;
+  a.e = in[0];
+  a.vx = in[1];
+  a.vy = in[2];
+  a.vz = in[3];
+  a.e1 = e1;
+  a.e2 = out[0];
+  a.vx2 = out[1];
+  a.vy2 = out[2];
+  a.vz2 = out[3];
+  a.nx = h->cfg.nx;
+  a.ny = h->cfg.ny;
+  a.nz = h->cfg.nz;
+  a.dth = h->dth;
+  for (int i = 0; i < 2; ++i) a.dts[i] = wav ? (float)(h->dt * (double)wav[n + i]) : 0.f;
+  a.si = h->cfg.src[0];
+  a.sj = h->cfg.src[1];
+  a.sk = wav ? h->cfg.src[2] : -1;
+  a.src_w = h->src_w;
+  a.sr = h->src_r;
+  a.krec = d_row ? h->krec : -1;
+  a.rec_map = h->rec_map;
+  a.d[0] = d_row;
+  a.d[1] = d_row ? d_row + h->nrow : nullptr;
+  a.err = aew::codec_err_flag(h->codec);
+  return a;
+}
+void two_pack(aew::TwoFwd& a, int i, const PackAt& p) {
+  a.tpack[i] = p.tp;
+  a.vmax[i] = p.vm;
+  a.tslot[i] = p.slot;
+}
+int two_fwd(aew_handle* h, const aew::TwoFwd& a, cudaStream_t s) {
+  AEW_CK(aew::launch_two_fwd(a, h->sms, s));
+  ++h->stats.kernel_launches;
+  return AEW_OK;
+}
+// reverse steps n and n - 1; en / en16: e^n and e^{n-1} (null: zero)
+int two_adj(aew_handle* h, int n, float* const in[4], float* const out[4], const float* resid,
+            const float* en0, const float* en1, const uint16_t* e16_0, const uint16_t* e16_1,
+            cudaStream_t s) {
+  aew::TwoAdj a{};
+  a.m = h->m;
+  a.mu = in[0];
+  a.lx = in[1];
+  a.ly = in[2];
+  a.lz = in[3];
+  a.mu2 = out[0];
+  a.lx2 = out[1];
+  a.ly2 = out[2];
+  a.lz2 = out[3];
+  a.nx = h->cfg.nx;
+  a.ny = h->cfg.ny;
+  a.nz = h->cfg.nz;
+  a.dth = h->dth;
+  a.en[0] = en0;
+  a.en[1] = en1;
+  a.en16[0] = e16_0;
+  a.en16[1] = e16_1;
+  a.acc32 = h->acc32;
+  a.acc64 = h->acc64;
+  const int W = h->cfg.accum_window, w = (h->cfg.nt - 1 - n) % W;
+  a.open = w == 0;
+  a.close[0] = w == W - 1;
+  a.close[1] = (w + 1) % W == W - 1 || n - 1 == 0;
+  a.krec = h->krec;
+  a.rec_map = h->rec_map;
+  for (int i = 0; i < 2; ++i)
+    a.resid[i] = (resid && h->nrow) ? resid + (size_t)(n + 1 - i) * h->nrow : nullptr;
+  a.err = aew::codec_err_flag(h->codec);
+  AEW_CK(aew::launch_two_adj(a, h->sms, s));
+  ++h->stats.kernel_launches;
+  return AEW_OK;
+}
+
 // reverse step n: (lam, mu) in ad[cur] -> ad[cur ^ 1]
 int adj_step(aew_handle* h, int n, int cur, const float* resid, const float* en,
              cudaStream_t s) {
@@ -577,10 +669,15 @@ int adjoint_full(aew_handle* h, const float* resid, cudaStream_t s) {
                      nt > 1 ? h->estore + (size_t)(nt - 1) * h->C : nullptr, nullptr, s);
   }
   if ((rc = begin_adjoint(h, s))) return rc;
-  for (int n = nt - 1; n >= 0; --n) {
-    const float* en = n > 0 ? h->estore + (size_t)n * h->C : nullptr;
-    if ((rc = adj_step(h, n, cur, resid, en, s))) return rc;
-    cur ^= 1;
+  auto en = [&](int n) { return n > 0 ? h->estore + (size_t)n * h->C : nullptr; };
+  for (int n = nt - 1; n >= 0; --n, cur ^= 1) {
+    if (h->two && n >= 1) {
+      rc = two_adj(h, n, h->ad[cur], h->ad[cur ^ 1], resid, en(n), en(n - 1), nullptr, nullptr, s);
+      --n;
+    } else {
+      rc = adj_step(h, n, cur, resid, en(n), s);
+    }
+    if (rc) return rc;
   }
   return AEW_OK;
 }
@@ -607,13 +704,16 @@ int gradient_full(aew_handle* h, const float* d_obs, const float* wav, cudaStrea
   for (int i = 0; i < 3; ++i) AEW_CK(cudaMemsetAsync(vb[0][i], 0, h->C * sizeof(float), s));
   AEW_CK(cudaMemsetAsync(h->estore, 0, h->C * sizeof(float), s));
   AEW_CK(cudaMemsetAsync(h->d, 0, h->nrow * sizeof(float), s));
-  for (int n = 0; n < nt; ++n) {
-    const int a = n & 1;
-    float* eout = (n + 1 < nt) ? h->estore + (size_t)(n + 1) * h->C : h->st[0][0];
+  for (int n = 0, a = 0; n < nt; ++n, a ^= 1) {
+    const int step = h->two && n + 1 < nt ? 2 : 1;
+    float* eout = (n + step < nt) ? h->estore + (size_t)(n + step) * h->C : h->st[0][0];
     float* in[4] = {h->estore + (size_t)n * h->C, vb[a][0], vb[a][1], vb[a][2]};
     float* out[4] = {eout, vb[a ^ 1][0], vb[a ^ 1][1], vb[a ^ 1][2]};
-    int rc = fwd_step(h, n, in, out, wav, drow(h, h->d, n + 1), s);
+    int rc = step == 2 ? two_fwd(h, two_fwd_args(h, n, in, out, h->estore + (size_t)(n + 1) * h->C, wav,
+                                                 drow(h, h->d, n + 1)), s)
+                       : fwd_step(h, n, in, out, wav, drow(h, h->d, n + 1), s);
     if (rc) return rc;
+    n += step - 1;
   }
   int rc = residual_and_misfit(h, d_obs, s);
   if (rc) return rc;
@@ -671,20 +771,23 @@ int run_revolve(aew_handle* h, const float* d_obs, const float* resid, const flo
         for (int k = 0; k < act.arg; ++k) {
           float* out[4];
           int out_buf;
-          if (to_slot && k == act.arg - 1) {
+          const int step = h->two && k + 1 < act.arg ? 2 : 1;
+          if (to_slot && k + step == act.arg) {
             slot(plan[a + 1].arg, out);
             out_buf = -1;
           } else {
             out_buf = live_buf == 0 ? 1 : 0;
             for (int i = 0; i < 4; ++i) out[i] = h->st[out_buf][i];
           }
-          rc = fwd_step(h, live_n, live, out, wav, gradient ? drow(h, h->d, live_n + 1) : nullptr,
-                        s);
+          float* row = gradient ? drow(h, h->d, live_n + 1) : nullptr;
+          rc = step == 2 ? two_fwd(h, two_fwd_args(h, live_n, live, out, nullptr, wav, row), s)
+                         : fwd_step(h, live_n, live, out, wav, row, s);
           if (rc) return rc;
           for (int i = 0; i < 4; ++i) live[i] = out[i];
           live_buf = out_buf;
-          ++live_n;
-          ++fwd;
+          k += step - 1;
+          live_n += step;
+          fwd += step;
         }
         break;
       }
@@ -852,9 +955,15 @@ int time_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
       }
       AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
     }
-    if ((rc = adj_step_x(h, n, h->ad[acur], h->ad[acur ^ 1], resid, nullptr, h->acc32, h->acc64,
-                         nullptr, nullptr, nullptr, s, window_e16(h, n))))
+    if (h->two && n % 2 == 1) {   // both steps in the same window
+      if ((rc = two_adj(h, n, h->ad[acur], h->ad[acur ^ 1], resid, nullptr, nullptr, window_e16(h, n),
+                        window_e16(h, n - 1), s)))
+        return rc;
+      --n;
+    } else if ((rc = adj_step_x(h, n, h->ad[acur], h->ad[acur ^ 1], resid, nullptr, h->acc32, h->acc64,
+                                nullptr, nullptr, nullptr, s, window_e16(h, n)))) {
       return rc;
+    }
     acur ^= 1;
     if (n % T == 0) AEW_CK(cudaEventRecord(h->ev_a[tb & 1], s));
   }
@@ -913,24 +1022,36 @@ int gradient_ae_time(aew_handle* h, const float* d_obs, const float* wav, cudaSt
   };
   if (nt == 1 && (rc = window_done(0))) return rc;
   int cur = 0;
-  for (int n = 0; n < nt; ++n) {
-    const int m = n + 1;
-    uint16_t* tp = nullptr;
-    unsigned* vm = nullptr;
+  // where state m goes (nowhere past nt - 1); a window's buffer is made ready for its first
+  // state: the encoder of the window before last is done with it, a partial window is zero
+  auto pack_at = [&](int m, PackAt* p) -> int {
+    *p = PackAt{};
+    if (m > nt - 1) return AEW_OK;
     const int tb = m / T, slot = m % T;
-    if (m <= nt - 1) {
-      if (slot == 0) {
-        if (tb >= 2) AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
-        if (T * tb + T > nt) AEW_CK(cudaMemsetAsync(h->xt[tb & 1], 0, wbytes, s));   // tail 0
-      }
-      tp = h->xt[tb & 1];
-      vm = h->vmx + (size_t)tb * nv;
+    if (slot == 0) {
+      if (tb >= 2) AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
+      if (T * tb + T > nt) AEW_CK(cudaMemsetAsync(h->xt[tb & 1], 0, wbytes, s));   // tail 0
     }
-    rc = fwd_step(h, n, h->st[cur], h->st[cur ^ 1], wav, drow(h, h->d, n + 1), s, nullptr,
-                  nullptr, nullptr, tp, slot, vm);
+    *p = PackAt{h->xt[tb & 1], h->vmx + (size_t)tb * nv, slot};
+    return AEW_OK;
+  };
+  for (int n = 0; n < nt; ++n, cur ^= 1) {
+    const int step = h->two && n + 1 < nt ? 2 : 1;
+    PackAt p[2];
+    for (int i = 0; i < step; ++i)
+      if ((rc = pack_at(n + 1 + i, &p[i]))) return rc;
+    if (step == 2) {
+      aew::TwoFwd a = two_fwd_args(h, n, h->st[cur], h->st[cur ^ 1], nullptr, wav, drow(h, h->d, n + 1));
+      for (int i = 0; i < 2; ++i) two_pack(a, i, p[i]);
+      rc = two_fwd(h, a, s);
+    } else {
+      rc = fwd_step(h, n, h->st[cur], h->st[cur ^ 1], wav, drow(h, h->d, n + 1), s, nullptr, nullptr,
+                    nullptr, p[0].tp, p[0].slot, p[0].vm);
+    }
     if (rc) return rc;
-    cur ^= 1;
-    if (m <= nt - 1 && (slot == T - 1 || m == nt - 1) && (rc = window_done(tb))) return rc;
+    for (int m = n + 1; m <= n + step && m <= nt - 1; ++m)
+      if ((m % T == T - 1 || m == nt - 1) && (rc = window_done(m / T))) return rc;
+    n += step - 1;
   }
   if ((rc = join(h, h->side, s, h->ev_sync2))) return rc;
   if ((rc = residual_and_misfit(h, d_obs, s))) return rc;
@@ -991,13 +1112,24 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
       a.nhist = nt - 1;
       return brick_fwd(h, a, s);
     }
-    for (int n = 0; n < nt; ++n) {
+    auto en = [&](int n) { return n > 0 ? h->estore + (size_t)n * h->C : nullptr; };
+    for (int n = 0; n < nt; ++n, cur ^= 1) {
+      const int step = h->two && n + 1 < nt ? 2 : 1;
       float* in[4] = {h->desto + (size_t)n * h->C, h->ad[cur][1], h->ad[cur][2], h->ad[cur][3]};
-      float* eo = n + 1 < nt ? h->desto + (size_t)(n + 1) * h->C : h->ad[cur ^ 1][0];
+      float* eo = n + step < nt ? h->desto + (size_t)(n + step) * h->C : h->ad[cur ^ 1][0];
       float* out[4] = {eo, h->ad[cur ^ 1][1], h->ad[cur ^ 1][2], h->ad[cur ^ 1][3]};
-      const float* en = n > 0 ? h->estore + (size_t)n * h->C : nullptr;
-      if ((rc = incr_step(h, in, out, en, drow(h, h->dd, n + 1), s))) return rc;
-      cur ^= 1;
+      if (step == 2) {
+        aew::TwoFwd a = two_fwd_args(h, n, in, out, h->desto + (size_t)(n + 1) * h->C, nullptr,
+                                     drow(h, h->dd, n + 1));
+        a.dm = h->dm;
+        a.ef[0] = en(n);
+        a.ef[1] = en(n + 1);
+        rc = two_fwd(h, a, s);
+      } else {
+        rc = incr_step(h, in, out, en(n), drow(h, h->dd, n + 1), s);
+      }
+      if (rc) return rc;
+      n += step - 1;
     }
     return AEW_OK;
   }
@@ -1034,23 +1166,36 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
       }
       AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
     }
-    const int m = n + 1, to = m / T, slot = m % T;
-    uint16_t* tp = nullptr;
-    unsigned* vm = nullptr;
-    if (m <= nt - 1) {
-      if (slot == 0) {
+    const int step = h->two && n % 2 == 0 && n + 1 < nt ? 2 : 1;   // both steps in the same window
+    PackAt p[2];
+    for (int i = 0; i < step; ++i) {
+      const int m = n + 1 + i, to = m / T;
+      if (m > nt - 1) continue;
+      if (m % T == 0) {
         if (to >= 2) AEW_CK(cudaStreamWaitEvent(s, h->ev_d[to & 1], 0));
         if (T * to + T > nt) AEW_CK(cudaMemsetAsync(h->xt[to & 1], 0, wbytes, s));
       }
-      tp = h->xt[to & 1];
-      vm = h->vmx2 + (size_t)to * nv;
+      p[i] = PackAt{h->xt[to & 1], h->vmx2 + (size_t)to * nv, m % T};
     }
-    if ((rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], nullptr, drow(h, h->dd, n + 1), s,
-                        tp, slot, vm, window_e16(h, n))))
-      return rc;
+    if (step == 2) {
+      aew::TwoFwd a = two_fwd_args(h, n, h->ad[cur], h->ad[cur ^ 1], nullptr, nullptr,
+                                   drow(h, h->dd, n + 1));
+      a.dm = h->dm;
+      for (int i = 0; i < 2; ++i) {
+        a.ef16[i] = window_e16(h, n + i);
+        two_pack(a, i, p[i]);
+      }
+      rc = two_fwd(h, a, s);
+    } else {
+      rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], nullptr, drow(h, h->dd, n + 1), s, p[0].tp,
+                     p[0].slot, p[0].vm, window_e16(h, n));
+    }
+    if (rc) return rc;
     cur ^= 1;
+    n += step - 1;
     if (n % T == T - 1 || n == nt - 1) AEW_CK(cudaEventRecord(h->ev_a[tb & 1], s));
-    if (m <= nt - 1 && (slot == T - 1 || m == nt - 1) && (rc = encode_de(to))) return rc;
+    for (int m = n + 2 - step; m <= n + 1 && m <= nt - 1; ++m)
+      if ((m % T == T - 1 || m == nt - 1) && (rc = encode_de(m / T))) return rc;
   }
   return join(h, h->side, s, h->ev_sync2);
 }
@@ -1357,22 +1502,6 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
          dalloc(h, &h->xt[1], nv * aew::kNIn) && dalloc(h, &h->edt[0], aew::kTSteps * C) &&
          dalloc(h, &h->edt[1], aew::kTSteps * C);
   }
-  if (ok && c.storage == AEW_AE) {
-    // The codec GEMMs run on a high-priority side stream with half the SMs, so their
-    // CTAs are placed first and the concurrent stencil step keeps the other half
-    // (measured best at 256^3 among caps of 76-152 CTAs and 2-4 GEMM stages).
-    int lo = 0, hi = 0, sms = 0;
-    if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess) hi = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    h->overlap_ctas = sms > 1 ? sms / 2 : 0;
-    if (const char* env = getenv("AEW_GEMM_CTAS_OVERLAP")) h->overlap_ctas = atoi(env);   // tuning override
-    ok = ok && cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, hi) == cudaSuccess;
-    for (int i = 0; ok && i < 2; ++i)
-      ok = cudaEventCreateWithFlags(&h->ev_a[i], cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&h->ev_b[i], cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaEventCreateWithFlags(&h->ev_sync, cudaEventDisableTiming) == cudaSuccess &&
-         cudaEventCreateWithFlags(&h->ev_sync2, cudaEventDisableTiming) == cudaSuccess;
-  }
   // on-chip time loops where the grid fits; a z-chunk depth set by hand asks for the
   // streaming kernels it belongs to
   if (ok && !getenv("AEW_STENCIL_KC_FWD") && !getenv("AEW_STENCIL_KC_ADJ")) {
@@ -1380,6 +1509,10 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
     h->brick = coop && aew::brick_plan(c.nx, c.ny, c.nz, sms, &h->bp);
+    // faster than single steps on every larger grid: 160^3 20 us a step against 34, 256^3 69
+    // against 95, 512 x 512 x 256 302 against 350
+    h->two = !h->brick;
+    h->sms = sms;
     if (h->brick) {
       const size_t nb = aew::brick_halo_bytes(c.nx, h->bp);
       std::vector<float> dts(nt);
@@ -1388,6 +1521,25 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
            dalloc(h, &h->dts, nt) &&
            cudaMemcpy(h->dts, dts.data(), nt * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
     }
+  }
+  if (ok && c.storage == AEW_AE) {
+    // The codec GEMMs run on a high-priority side stream with half the SMs, so their
+    // CTAs are placed first and the concurrent stencil step keeps the other half
+    // (measured best at 256^3 among caps of 76-152 CTAs and 2-4 GEMM stages).
+    int lo = 0, hi = 0, sms = 0;
+    if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess) hi = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    h->overlap_ctas = sms > 1 ? sms / 2 : 0;
+    // two steps per pass: a pass holds every SM for 70-100 us, so the GEMMs take all SMs
+    // between passes (217 us per gradient step at 256^3 against 222 with half of them)
+    if (h->two) h->overlap_ctas = 0;
+    if (const char* env = getenv("AEW_GEMM_CTAS_OVERLAP")) h->overlap_ctas = atoi(env);   // tuning override
+    ok = ok && cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, hi) == cudaSuccess;
+    for (int i = 0; ok && i < 2; ++i)
+      ok = cudaEventCreateWithFlags(&h->ev_a[i], cudaEventDisableTiming) == cudaSuccess &&
+           cudaEventCreateWithFlags(&h->ev_b[i], cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&h->ev_sync, cudaEventDisableTiming) == cudaSuccess &&
+         cudaEventCreateWithFlags(&h->ev_sync2, cudaEventDisableTiming) == cudaSuccess;
   }
   if (!ok) {
     g_create_err = "device allocation failed (" + std::to_string(h->bytes) + " bytes held)";
@@ -1484,11 +1636,15 @@ int aew_forward(aew_handle* h, const float* c_dev, const float* wavelet_host, fl
   const float* wav = wav_or_default(h, wavelet_host);
   if ((rc = zero_state(h, h->st[0], s))) return rc;
   int cur = 0;
-  for (int n = 0; n < h->cfg.nt; ++n) {
-    rc = fwd_step(h, n, h->st[cur], h->st[cur ^ 1], wav, d_dev ? drow(h, d_dev, n + 1) : nullptr,
-                  s);
+  for (int n = 0; n < h->cfg.nt; ++n, cur ^= 1) {
+    float* row = d_dev ? drow(h, d_dev, n + 1) : nullptr;
+    if (h->two && n + 1 < h->cfg.nt) {
+      rc = two_fwd(h, two_fwd_args(h, n, h->st[cur], h->st[cur ^ 1], nullptr, wav, row), s);
+      ++n;
+    } else {
+      rc = fwd_step(h, n, h->st[cur], h->st[cur ^ 1], wav, row, s);
+    }
     if (rc) return rc;
-    cur ^= 1;
   }
   return AEW_OK;
 }
@@ -1537,11 +1693,16 @@ int aew_propagate(aew_handle* h, const float* c_dev, float* const state_dev[4], 
   std::vector<float> w(wavelet_host ? (size_t)nsteps + (size_t)n0 : 0, 0.f);
   for (int k = 0; wavelet_host && k < nsteps; ++k) w[(size_t)n0 + k] = wavelet_host[k];
   int cur = 0;
-  for (int k = 0; k < nsteps; ++k) {
-    rc = fwd_step(h, n0 + k, bufs[cur], bufs[cur ^ 1], wavelet_host ? w.data() : nullptr,
-                  d_dev ? drow(h, d_dev, k + 1) : nullptr, s);
+  for (int k = 0; k < nsteps; ++k, cur ^= 1) {
+    const float* wv = wavelet_host ? w.data() : nullptr;
+    float* row = d_dev ? drow(h, d_dev, k + 1) : nullptr;
+    if (h->two && k + 1 < nsteps) {
+      rc = two_fwd(h, two_fwd_args(h, n0 + k, bufs[cur], bufs[cur ^ 1], nullptr, wv, row), s);
+      ++k;
+    } else {
+      rc = fwd_step(h, n0 + k, bufs[cur], bufs[cur ^ 1], wv, row, s);
+    }
     if (rc) return rc;
-    cur ^= 1;
   }
   if (cur == 1) {
     if ((rc = copy_state(h, bufs[0], bufs[1], s))) return rc;
@@ -1664,12 +1825,22 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
         }
         AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
       }
-      if ((rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], nullptr, drow(h, dd_out, n + 1), s,
-                          nullptr, 0, nullptr, window_e16(h, n))))
-        return rc;
+      const int step = h->two && n % 2 == 0 && n + 1 < nt ? 2 : 1;   // both in the same window
+      if (step == 2) {
+        aew::TwoFwd a = two_fwd_args(h, n, h->ad[cur], h->ad[cur ^ 1], nullptr, nullptr,
+                                     drow(h, dd_out, n + 1));
+        a.dm = h->dm;
+        for (int i = 0; i < 2; ++i) a.ef16[i] = window_e16(h, n + i);
+        rc = two_fwd(h, a, s);
+      } else {
+        rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], nullptr, drow(h, dd_out, n + 1), s, nullptr, 0,
+                       nullptr, window_e16(h, n));
+      }
+      if (rc) return rc;
+      n += step - 1;
       if (n % T == T - 1 || n == nt - 1) AEW_CK(cudaEventRecord(h->ev_a[tb & 1], s));
       cur ^= 1;
-      ++*fwd;
+      *fwd += step;
     }
     return join(h, h->side, s, h->ev_sync2);
   }
@@ -1715,6 +1886,15 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
                                                 drow(h, dd_out, 1)), s)
                   : brick_fwd(h, brick_incr_args(h, h->ad[cur], h->ad[cur ^ 1], n, 1, en, nullptr,
                                                  drow(h, dd_out, n + 1)), s);
+    } else if (h->two && h->cfg.storage == AEW_FULL && n + 1 < nt) {
+      aew::TwoFwd a = two_fwd_args(h, n, h->ad[cur], h->ad[cur ^ 1], nullptr, nullptr,
+                                   drow(h, dd_out, n + 1));
+      a.dm = h->dm;
+      a.ef[0] = en;
+      a.ef[1] = h->estore + (size_t)(n + 1) * h->C;
+      rc = two_fwd(h, a, s);
+      ++n;
+      ++*fwd;
     } else {
       rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], en, drow(h, dd_out, n + 1), s);
     }

@@ -85,4 +85,54 @@ __device__ __forceinline__ bool sticky_error(const int* err) {
   return err && *reinterpret_cast<const volatile int*>(err) != 0;
 }
 
+// ---- four nodes as two pairs ---------------------------------------------------------
+namespace quad {
+// The paired FP32 instructions round each lane as the scalar ones do.
+struct F4 {
+  uint64_t a, b;
+};
+__device__ __forceinline__ F4 f4(float4 v) {
+  return F4{gemm::f2::make(v.x, v.y), gemm::f2::make(v.z, v.w)};
+}
+__device__ __forceinline__ float4 v4(F4 f) {
+  float4 v;
+  gemm::f2::split(f.a, v.x, v.y);
+  gemm::f2::split(f.b, v.z, v.w);
+  return v;
+}
+__device__ __forceinline__ F4 add(F4 x, F4 y) { return F4{gemm::f2::add(x.a, y.a), gemm::f2::add(x.b, y.b)}; }
+__device__ __forceinline__ F4 sub(F4 x, F4 y) { return F4{gemm::f2::sub(x.a, y.a), gemm::f2::sub(x.b, y.b)}; }
+__device__ __forceinline__ F4 mul(F4 x, F4 y) { return F4{gemm::f2::mul(x.a, y.a), gemm::f2::mul(x.b, y.b)}; }
+__device__ __forceinline__ F4 fma(F4 x, F4 y, F4 z) {
+  return F4{gemm::f2::fma(x.a, y.a, z.a), gemm::f2::fma(x.b, y.b, z.b)};
+}
+__device__ __forceinline__ F4 lds(const float4* p) { return f4(*p); }
+__device__ __forceinline__ void sts(float4* p, F4 v) { *p = v4(v); }
+}  // namespace quad
+
+__device__ __forceinline__ float4 ldg4(const float* p) {
+  return __ldg(reinterpret_cast<const float4*>(p));
+}
+__device__ __forceinline__ float4 bf4(uint2 b) {
+  return make_float4(__uint_as_float(b.x << 16), __uint_as_float(b.x & 0xffff0000u),
+                     __uint_as_float(b.y << 16), __uint_as_float(b.y & 0xffff0000u));
+}
+// some of four nodes carry a receiver (rec_map points at theirs)
+__device__ __forceinline__ bool has_rec(const int* rec_map) {
+  const int4 m = __ldg(reinterpret_cast<const int4*>(rec_map));
+  return m.x >= 0 || m.y >= 0 || m.z >= 0 || m.w >= 0;
+}
+// the face values of four nodes to the receiver row d
+__device__ __forceinline__ void record(const int* rec_map, float* d, float4 x, float4 y, float4 z) {
+  const int4 r = __ldg(reinterpret_cast<const int4*>(rec_map));
+  const int rr[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    if (rr[c] >= 0) {
+      d[3 * rr[c] + 0] = comp(x, c);
+      d[3 * rr[c] + 1] = comp(y, c);
+      d[3 * rr[c] + 2] = comp(z, c);
+    }
+}
+
 }  // namespace aew
