@@ -823,12 +823,17 @@ cudaError_t codec_refresh(Codec* c, cudaStream_t s) {
     t.tiles[m + 1] = t.tiles[m] + ((t.rows[m] + 31) / 32) * ((t.cols[m] + 31) / 32);
   transpose_multi_kernel<<<t.tiles[4], dim3(32, 8), 0, s>>>(t);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return codec_refresh_strain(c, s);
+}
+
+cudaError_t codec_refresh_strain(Codec* c, cudaStream_t s) {
   if (c->time) return cudaSuccess;
   strain_rows_kernel<<<512, 128, 0, s>>>(c->W4t, c->W4e);
   return cudaGetLastError();
 }
 
 cudaError_t codec_set_weights(Codec* c, const float* const w[8]) {
+  ++c->version;
   for (int i = 0; i < 8; ++i) {
     cudaError_t e = cudaMemcpy(c->w[i], w[i], c->wn[i] * sizeof(float), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;

@@ -39,6 +39,8 @@ cudaError_t codec_get_weights(const Codec* c, float* const w[8]);
 
 // Rebuild the tensor-core operand copies of the weights from the FP32 masters.
 cudaError_t codec_refresh(Codec* c, cudaStream_t s);
+// .. of them, the space codec's strain rows of W4t (all a fused update leaves to do)
+cudaError_t codec_refresh_strain(Codec* c, cudaStream_t s);
 
 // Encode one grid state: BF16 block vectors plus per-block, per-field maxima of |f|
 // (bmax, float bits [nblocks][4], written), normalised by the power-of-two block scales,

@@ -16,6 +16,7 @@ struct Codec {
   int act = 0;
   double beta = 1e-7;
   bool ready = false;
+  unsigned long long version = 0;   // counts replacements of the master weights from outside training
   // FP32 master weights: W1 [2048][nh], b1, W2 [nh][nl], b2, W3 [nl][nh], b3,
   // W4 [nh][2048], b4
   float* w[8] = {};

@@ -229,10 +229,13 @@ __device__ __forceinline__ void gelu_fast_pair(float& a0, float& a1) {
 // ---------------------------------------------------------------------------------
 // The kernel (persistent: each CTA walks tiles blockIdx.x, +gridDim.x, ...)
 // ---------------------------------------------------------------------------------
+// One product on CTAs cta = 0 .. ctas - 1 of the launch.  A launch may be a programmatic
+// dependent of the one before it (training chains products of a few microseconds): its set-up
+// then runs while that one drains, and griddepcontrol.wait holds it back until all of that
+// one's results are visible.
 template <int BN, bool BF16, bool SW, class EP>
-__global__ void __launch_bounds__(kThreads, 1)
-    gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-                int M, int N, int K, int ns, EP ep, int* err) {
+__device__ __forceinline__ void gemm_body(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K, int ns,
+                                          const EP& ep, int* err, int cta, int ctas) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -250,12 +253,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tslot = reinterpret_cast<uint32_t*>(acce + 2);
   int* abort_flag = reinterpret_cast<int*>(tslot + 1);
 
-  // a previous launch already failed: do nothing (the host reports the error)
-  if (*reinterpret_cast<volatile int*>(err) != 0) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nK = (K + kBK - 1) / kBK;
   const int tn = (N + BN - 1) / BN;
-  const int T = ((M + kBM - 1) / kBM) * tn;
+  const int tiles = ((M + kBM - 1) / kBM) * tn;
 
   if (warp == kMmaWarp) {
     tc::tmem_alloc(tc::smem_u32(tslot), TCOLS);
@@ -272,20 +273,25 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc::mbar_init(tc::smem_u32(&accf[a]), 1);
       tc::mbar_init(tc::smem_u32(&acce[a]), kEpiThreads);
     }
-    *abort_flag = 0;
     tc::mbar_fence_init();
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // a previous launch already failed: do nothing (the host reports the error)
+  if (tid == 0) *abort_flag = *reinterpret_cast<volatile int*>(err) != 0 ? 2 : 0;
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  // after the TMEM allocation: a dependent's waits for this one's release, never the reverse
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t tmem = *tslot;
+  const int T = *reinterpret_cast<volatile int*>(abort_flag) == 2 ? 0 : tiles;
 
   if (warp == kTmaWarp) {
     if (lane == 0) {
       // ----------------------------------------------------------- TMA producer
       int it = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < T && ok; t += gridDim.x) {
+      for (int t = cta; t < T && ok; t += ctas) {
         const int m0 = (t / tn) * kBM, n0 = (t % tn) * BN;
         for (int c = 0; c < nK; ++c, ++it) {
           const int s = it % ns;
@@ -319,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) {
       // ----------------------------------------------------------- MMA issuer
       int it = 0, tl = 0;
-      for (int t = blockIdx.x; t < T; t += gridDim.x, ++tl) {
+      for (int t = cta; t < T; t += ctas, ++tl) {
         const int a = tl & 1;
         if (tl >= 2 && !tc::mbar_wait(tc::smem_u32(&acce[a]), ((tl >> 1) - 1) & 1, kWaitNs)) {
           atomicExch(abort_flag, 1);
@@ -363,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3, cg = warp >> 2;
     constexpr int G = BN / 32;                   // 32-column groups per tile
     int tl = 0;
-    for (int t = blockIdx.x; t < T; t += gridDim.x, ++tl) {
+    for (int t = cta; t < T; t += ctas, ++tl) {
       const int a = tl & 1;
       const bool ok = tc::mbar_wait(tc::smem_u32(&accf[a]), (tl >> 1) & 1, kWaitNs);
       tc::fence_after_sync();
@@ -392,6 +398,28 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == kMmaWarp) tc::tmem_dealloc(tmem, TCOLS);
 }
 
+template <int BN, bool BF16, bool SW, class EP>
+__global__ void __launch_bounds__(kThreads, 1)
+    gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
+                int M, int N, int K, int ns, EP ep, int* err) {
+  gemm_body<BN, BF16, SW>(ta, tb, M, N, K, ns, ep, err, blockIdx.x, gridDim.x);
+}
+
+// Two independent products in one launch: the first on CTAs 0 .. c1 - 1, the second on the rest.
+struct Shape {
+  int M, N, K, ns;
+};
+template <int BN, bool BF16, bool SW, class EP1, class EP2>
+__global__ void __launch_bounds__(kThreads, 1)
+    gemm_dual_kernel(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CUtensorMap tb1, Shape s1,
+                     EP1 ep1, const __grid_constant__ CUtensorMap ta2, const __grid_constant__ CUtensorMap tb2,
+                     Shape s2, EP2 ep2, int c1, int* err) {
+  if ((int)blockIdx.x < c1)
+    gemm_body<BN, BF16, SW>(ta1, tb1, s1.M, s1.N, s1.K, s1.ns, ep1, err, blockIdx.x, c1);
+  else
+    gemm_body<BN, BF16, SW>(ta2, tb2, s2.M, s2.N, s2.K, s2.ns, ep2, err, blockIdx.x - c1, gridDim.x - c1);
+}
+
 // SM count of the current device, found once (thread-safe static initialisation).
 inline int sm_count() {
   static const int n = [] {
@@ -414,9 +442,27 @@ struct Mat {
 #define AEW_GEMM_SWIZZLE 1
 #endif
 
+// a launch that may start while the one before it on the stream drains (its kernel waits for
+// that one's results itself)
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                             const A&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 template <int BN, bool BF16, class EP>
 cudaError_t launch(long long M, int N, int K, const Mat& A, const Mat& B, const EP& ep, int* err,
-                   cudaStream_t s, int max_ctas = 0, int max_ns = 0) {
+                   cudaStream_t s, int max_ctas = 0, int max_ns = 0, bool dependent = false) {
   constexpr bool SW = AEW_GEMM_SWIZZLE != 0;
   auto kern = gemm_kernel<BN, BF16, SW, EP>;
   const int nK = (K + kBK - 1) / kBK;
@@ -438,8 +484,57 @@ cudaError_t launch(long long M, int N, int K, const Mat& A, const Mat& B, const 
   const long long tiles = ((M + kBM - 1) / kBM) * (long long)((N + BN - 1) / BN);
   const int cap = (max_ctas > 0 && max_ctas < sms) ? max_ctas : sms;
   const int grid = (int)(tiles < cap ? tiles : cap);
+  if (dependent) return launch_dependent(kern, dim3(grid), dim3(kThreads), smem, s, ta, tb, (int)M, N, K, ns, ep, err);
   kern<<<grid, kThreads, smem, s>>>(ta, tb, (int)M, N, K, ns, ep, err);
   return cudaGetLastError();
+}
+
+// Two products in one dependent launch; the SMs are dealt by the chunks of K each has to run.
+struct Product {
+  long long M;
+  int N, K;
+  Mat A, B;
+};
+template <int BN, bool BF16, class EP1, class EP2>
+cudaError_t launch_dual(const Product& p1, const EP1& ep1, const Product& p2, const EP2& ep2, int* err,
+                        cudaStream_t s, int max_ns) {
+  constexpr bool SW = AEW_GEMM_SWIZZLE != 0;
+  auto kern = gemm_dual_kernel<BN, BF16, SW, EP1, EP2>;
+  const Product* p[2] = {&p1, &p2};
+  CUtensorMap ta[2], tb[2];
+  Shape sh[2];
+  long long tiles[2], work[2];
+  int ns = 2;
+  for (int i = 0; i < 2; ++i) {
+    const int nK = (p[i]->K + kBK - 1) / kBK;
+    int n = max_stages<BN>();
+    if (n > nK + 2) n = nK + 2;
+    if (max_ns > 0 && n > max_ns) n = max_ns;
+    if (n < 2) n = 2;
+    if (n > ns) ns = n;
+    sh[i] = Shape{(int)p[i]->M, p[i]->N, p[i]->K, n};
+    tiles[i] = ((p[i]->M + kBM - 1) / kBM) * (long long)((p[i]->N + BN - 1) / BN);
+    work[i] = tiles[i] * (nK + 4);   // a tile's epilogue costs about four chunks
+    if (make_tmap(&ta[i], p[i]->A.p, !BF16, p[i]->A.rows, p[i]->K, p[i]->A.ld, kBM, SW) != CUDA_SUCCESS ||
+        make_tmap(&tb[i], p[i]->B.p, !BF16, p[i]->B.rows, p[i]->K, p[i]->B.ld, BN, SW) != CUDA_SUCCESS)
+      return cudaErrorInvalidValue;
+  }
+  const size_t smem = smem_bytes_for(stage_bytes<BN>(), ns);
+  // once per instantiation (thread-safe static initialisation)
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      (int)smem_bytes_for(stage_bytes<BN>(), max_stages<BN>()));
+  if (attr != cudaSuccess) return attr;
+  const int sms = sm_count();
+  long long c1 = tiles[0], c2 = tiles[1];
+  if (c1 + c2 > sms) {
+    c1 = (sms * work[0] + (work[0] + work[1]) / 2) / (work[0] + work[1]);
+    c1 = c1 < 1 ? 1 : c1 > sms - 1 ? sms - 1 : c1;
+    c1 = c1 > tiles[0] ? tiles[0] : c1;
+    c2 = sms - c1 > tiles[1] ? tiles[1] : sms - c1;
+  }
+  return launch_dependent(kern, dim3((unsigned)(c1 + c2)), dim3(kThreads), smem, s, ta[0], tb[0], sh[0], ep1,
+                          ta[1], tb[1], sh[1], ep2, (int)c1, err);
 }
 
 }  // namespace gemm

@@ -3,6 +3,13 @@
 // GELU layers with a straight-through FP16 latent, and the LAMB optimiser
 // (You et al. 2019) with one trust ratio per parameter tensor.
 //
+// A step at batch 512 is a chain of products of a few microseconds each, so launches and
+// their gaps bound it: every kernel is a programmatic dependent of the one before it (its
+// set-up runs while that one drains), the weight gradient of a layer shares a launch with the
+// activation gradient that comes next (they need the same input), and the optimiser's second
+// pass also writes the operand copies of the new weights.  Time codec, us per step: batch 512
+// 252 -> 219, batch 64 222 -> 199; space codec at 512 208 -> 151.
+//
 // Every product is a tcgen05 GEMM (aew_gemm.cuh) with BF16 operands and FP32
 // accumulation (the decoder's first forward product uses FP16 operands, as in
 // inference).  Activations are written both row-major and transposed by the producing
@@ -29,6 +36,7 @@ struct TrainState {
   int B = 0;       // batch capacity
   int nl = 64;
   int t = 0;       // LAMB step count
+  unsigned long long copies = ~0ull;   // Codec::version that W4b, W3b, W2b belong to
   size_t bytes = 0;
   // activations
   float *a1, *a3, *d1, *d2, *d3, *d4;
@@ -189,17 +197,23 @@ struct EpMse {
   // called by all 32 lanes of a warp together (rows m0 + 32 q + lane): the loss is
   // reduced across the warp before its one atomic
   __device__ __forceinline__ void operator()(long long row, int col, const float (&v)[32]) const {
-    double acc = 0.0;
+    // sum of wf diff^2 in FP32 with every rounding error kept (products by FMA, sums by
+    // Knuth's two-sum): as exact as FP64, whose rate here would cost a third of the kernel
+    float s1 = 0.f, s2 = 0.f;
+    float wf = 1.f;
     if (row < M) {
       // the 32 columns lie in one field's 64-column group: one weight
-      const float wf = w ? __ldg(w + row * 4 + ((col >> 6) & 3)) : 1.f;
+      if (w) wf = __ldg(w + row * 4 + ((col >> 6) & 3));
       uint32_t pk[16];
       float dd[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
         const float a = v[j] + __ldg(bias + col + j);
         const float diff = a - gemm::bf16_val(__ldg(Y + row * kNIn + col + j));
-        acc += (double)wf * (double)diff * (double)diff;
+        const float p = __fmul_rn(diff, diff), t = __fadd_rn(s1, p), z = __fsub_rn(t, s1);
+        s2 = __fadd_rn(s2, __fadd_rn(fmaf(diff, diff, -p),
+                                     __fadd_rn(__fsub_rn(s1, __fsub_rn(t, z)), __fsub_rn(p, z))));
+        s1 = t;
         dd[j] = scale * wf * diff;
         d4T[(size_t)(col + j) * M + row] = gemm::bf16_bits(dd[j]);
       }
@@ -208,6 +222,7 @@ struct EpMse {
       store_row32f(d4 + row * kNIn + col, dd);
       store_row16(d4b + row * kNIn + col, pk);
     }
+    double acc = (double)wf * ((double)s1 + (double)s2);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc);
@@ -258,6 +273,8 @@ struct EpStore {
 // ---------------------------------------------------------------------------------
 __global__ void transpose16_kernel(const uint16_t* __restrict__ src, int rows, int cols,
                                    uint16_t* __restrict__ dst) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __shared__ uint16_t tile[32][34];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
@@ -283,6 +300,8 @@ struct ColSums {
   int n;
 };
 __global__ void colsum_multi_kernel(ColSums cs, int rows) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __shared__ double part[8][33];
   int m = 0;
   while (m + 1 < cs.n && (int)blockIdx.x >= cs.tiles[m + 1]) ++m;
@@ -322,6 +341,8 @@ __global__ void to_bf16_multi_kernel(ToBf16 t) {
 }
 
 __global__ void loss_kernel(const double* red, double inv_n, float* out, double* acc) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const double l = red[0] * inv_n;
   if (out) out[0] = (float)l;
   if (acc) acc[0] += l;
@@ -459,6 +480,8 @@ __device__ __forceinline__ void block_add2(double x, double y, double* dst) {
 // pass 1: moments, u (written over g), norms |w|^2 and |u|^2 into norms[2 t], [2 t + 1]
 __global__ void lamb1_multi_kernel(LambArgs a, float b1, float b2, float c1, float c2, float eps,
                                    double* norms) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int t = lamb_tensor(a);
   const size_t n4 = a.n[t] / 4;
   const int nb = a.blk[t + 1] - a.blk[t];
@@ -487,25 +510,67 @@ __global__ void lamb1_multi_kernel(LambArgs a, float b1, float b2, float c1, flo
   block_add2((double)sw, (double)su, norms + 2 * t);
 }
 
-// pass 2: w -= lr * (|w| / |u|) * u
-__global__ void lamb2_multi_kernel(LambArgs a, float lr, const double* norms) {
-  const int t = lamb_tensor(a);
-  const size_t n4 = a.n[t] / 4;
-  const int nb = a.blk[t + 1] - a.blk[t];
+// pass 2: w -= lr * (|w| / |u|) * u, and the operand copies of the new weights: a block takes
+// one 32 x 32 tile of a weight matrix (natural BF16 rows for the backward products, transposed
+// BF16 or FP16 for the forward ones) or 1024 elements of a bias
+struct Lamb2 {
+  float* w[8];
+  const float* u[8];
+  uint16_t* nat[4];    // of W1 .. W4 (null: none)
+  uint16_t* tr[4];
+  int rows[4], cols[4], fp16[4];
+  int tiles[5];        // prefix per matrix
+  int bias[5];         // prefix of 1024-element blocks per bias, behind the tiles
+  int n[4];            // bias lengths
+};
+__global__ void __launch_bounds__(256) lamb2_multi_kernel(Lamb2 a, float lr, const double* norms) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  __shared__ float tile[32][33];
+  const int tid = threadIdx.x;
+  const bool isb = (int)blockIdx.x >= a.tiles[4];
+  int m = 0;
+  if (isb)
+    while (m < 3 && (int)blockIdx.x - a.tiles[4] >= a.bias[m + 1]) ++m;
+  else
+    while (m < 3 && (int)blockIdx.x >= a.tiles[m + 1]) ++m;
+  const int t = 2 * m + (isb ? 1 : 0);
   const double wn = sqrt(norms[2 * t]), un = sqrt(norms[2 * t + 1]);
   const float r = (wn > 0.0 && un > 0.0) ? (float)(wn / un) : 1.f;
-  float4* w = reinterpret_cast<float4*>(a.w[t]);
-  const float4* u = reinterpret_cast<const float4*>(a.g[t]);
-  for (size_t i = (size_t)(blockIdx.x - a.blk[t]) * blockDim.x + threadIdx.x; i < n4;
-       i += (size_t)nb * blockDim.x) {
-    float4 x = w[i];
-    const float4 y = u[i];
-    x.x -= lr * r * y.x;
-    x.y -= lr * r * y.y;
-    x.z -= lr * r * y.z;
-    x.w -= lr * r * y.w;
-    w[i] = x;
+  float* const w = a.w[t];
+  const float* const u = a.u[t];
+  if (isb) {
+    const int i0 = ((int)blockIdx.x - a.tiles[4] - a.bias[m]) * 1024;
+    for (int i = i0 + tid; i < min(i0 + 1024, a.n[m]); i += 256) w[i] -= lr * r * u[i];
+    return;
   }
+  // a thread takes four columns of one row (every size is a multiple of 32)
+  const int cols = a.cols[m], rows = a.rows[m], tx = cols / 32, b = blockIdx.x - a.tiles[m];
+  const int c0 = b % tx * 32, r0 = b / tx * 32, y = tid >> 3, x = (tid & 7) * 4;
+  const size_t i = (size_t)(r0 + y) * cols + c0 + x;
+  float4 v = *reinterpret_cast<const float4*>(w + i);
+  const float4 g = *reinterpret_cast<const float4*>(u + i);
+  v.x -= lr * r * g.x;
+  v.y -= lr * r * g.y;
+  v.z -= lr * r * g.z;
+  v.w -= lr * r * g.w;
+  *reinterpret_cast<float4*>(w + i) = v;
+  if (a.nat[m])
+    *reinterpret_cast<uint2*>(a.nat[m] + i) = make_uint2(gemm::pack_bf16(v.x, v.y), gemm::pack_bf16(v.z, v.w));
+  tile[y][x] = v.x;
+  tile[y][x + 1] = v.y;
+  tile[y][x + 2] = v.z;
+  tile[y][x + 3] = v.w;
+  __syncthreads();
+  const float q[4] = {tile[x][y], tile[x + 1][y], tile[x + 2][y], tile[x + 3][y]};
+  uint2 o;
+  if (a.fp16[m]) {
+    const __half2 h0 = __floats2half2_rn(q[0], q[1]), h1 = __floats2half2_rn(q[2], q[3]);
+    o = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+  } else {
+    o = make_uint2(gemm::pack_bf16(q[0], q[1]), gemm::pack_bf16(q[2], q[3]));
+  }
+  *reinterpret_cast<uint2*>(a.tr[m] + (size_t)(c0 + y) * rows + r0 + x) = o;
 }
 
 int nblk(size_t n) {
@@ -525,37 +590,31 @@ gemm::Mat ld(const uint16_t* p, long long ldim, long long rows, int K) {
     if (_e != cudaSuccess) return _e;       \
   } while (0)
 
-// a GEMM whose N is the latent width (32, 64, 256 or 512): the narrowest fitting tile
-template <bool BF16, class EP>
-cudaError_t launch_nl(long long M, int N, int K, const gemm::Mat& A, const gemm::Mat& B,
-                      const EP& ep, int* err, cudaStream_t st) {
-  if (N <= 32) return gemm::launch<32, BF16>(M, N, K, A, B, ep, err, st);
-  if (N <= 64) return gemm::launch<64, BF16>(M, N, K, A, B, ep, err, st);
-  return gemm::launch<256, BF16>(M, N, K, A, B, ep, err, st);
-}
+// stages of the training products' rings: few enough that a dependent launch's CTA fits
+// beside the one that drains
+constexpr int kTrainStages = 4;
 
-// a training GEMM (M rows of the batch or of a weight): the widest tile that still gives
-// every SM a tile, since one batch's products are too small to fill the GPU with
-// 128 x 256 tiles (AEW_TRAIN_BN = 64, 128 or 256 forces a width: tuning override)
+// a training GEMM (M rows of the batch or of a weight): 64-column tiles, since one batch's
+// products are too small to fill the GPU with wider ones (32 for the 32-wide latent)
 template <bool BF16, class EP>
 cudaError_t launch_t(long long M, int N, int K, const gemm::Mat& A, const gemm::Mat& B,
                      const EP& ep, int* err, cudaStream_t st) {
-  static const int forced = [] {
-    const char* env = getenv("AEW_TRAIN_BN");   // tuning override
-    return env ? atoi(env) : 0;
-  }();
+  if (N <= 32) return gemm::launch<32, BF16>(M, N, K, A, B, ep, err, st, 0, kTrainStages, true);
+  // wide batches: the widest tile that still gives every SM one
   const long long mt = (M + 127) / 128;
   const int sms = gemm::sm_count();
-  int bn = forced;
-  if (bn != 64 && bn != 128 && bn != 256) {
-    if (N < 128 || mt * ((N + 255) / 256) >= sms) bn = 256;
-    else if (mt * ((N + 127) / 128) >= sms || N < 256) bn = 128;
-    else bn = 64;
-  }
-  if (N <= 64) return launch_nl<BF16>(M, N, K, A, B, ep, err, st);
-  if (bn == 64) return gemm::launch<64, BF16>(M, N, K, A, B, ep, err, st);
-  if (bn == 128) return gemm::launch<128, BF16>(M, N, K, A, B, ep, err, st);
-  return gemm::launch<256, BF16>(M, N, K, A, B, ep, err, st);
+  if (N >= 256 && mt * (N / 256) >= sms) return gemm::launch<256, BF16>(M, N, K, A, B, ep, err, st, 0, 0, true);
+  if (N >= 128 && mt * (N / 128) >= sms) return gemm::launch<128, BF16>(M, N, K, A, B, ep, err, st, 0, 0, true);
+  return gemm::launch<64, BF16>(M, N, K, A, B, ep, err, st, 0, kTrainStages, true);
+}
+// a weight gradient and the activation gradient that needs the same input, in one launch
+template <class EP1, class EP2>
+cudaError_t launch_pair(long long M1, int N1, int K1, const gemm::Mat& A1, const gemm::Mat& B1, const EP1& e1,
+                        long long M2, int N2, int K2, const gemm::Mat& A2, const gemm::Mat& B2, const EP2& e2,
+                        int* err, cudaStream_t st) {
+  const gemm::Product p1{M1, N1, K1, A1, B1}, p2{M2, N2, K2, A2, B2};
+  if (N1 <= 32 || N2 <= 32) return gemm::launch_dual<32, true>(p1, e1, p2, e2, err, st, kTrainStages);
+  return gemm::launch_dual<64, true>(p1, e1, p2, e2, err, st, kTrainStages);
 }
 
 }  // namespace
@@ -587,12 +646,14 @@ cudaError_t codec_train_step(Codec* c, const uint16_t* Y, const float* wts, int 
   const int H = c->n_hid, I = kNIn;
   int* e = c->err;
   TCK(cudaMemsetAsync(s->red, 0, 32 * sizeof(double), st));
-  // backward weight copies of the current masters
-  {
+  // natural BF16 copies of the masters for the backward products: kept by the update below,
+  // made here after the weights were set from outside
+  if (s->copies != c->version) {
     const ToBf16 tb{{c->w[6], c->w[4], c->w[2]}, {s->W4b, s->W3b, s->W2b},
                     {(size_t)H * I, (size_t)nl * H, (size_t)H * nl}};
     to_bf16_multi_kernel<<<dim3(nblk((size_t)H * I / 4), 3), 256, 0, st>>>(tb);
     TCK(cudaGetLastError());
+    s->copies = c->version;
   }
   {
     dim3 grid((I + 31) / 32, (B + 31) / 32), block(32, 8);
@@ -611,18 +672,15 @@ cudaError_t codec_train_step(Codec* c, const uint16_t* Y, const float* wts, int 
                                      2.0f / (float)((double)B * I), Bm},
                                e, st)));
   // ---- backward
-  TCK((launch_t<true>((long long)H, I, B, ld(s->h3T, B, H, B), ld(s->d4T, B, I, B),
-                               EpStore{s->g[6], I, H}, e, st)));
-  TCK((launch_t<true>(Bm, H, I, ld(s->d4b, I, Bm, I), ld(s->W4b, I, H, I),
-                               EpBack{s->a3, s->d3, s->d3b, s->d3T, H, Bm, c->act}, e, st)));
-  TCK((launch_t<true>((long long)nl, H, B, ld(s->zbT, B, nl, B), ld(s->d3T, B, H, B),
-                               EpStore{s->g[4], H, nl}, e, st)));
-  TCK((launch_t<true>(Bm, nl, H, ld(s->d3b, H, Bm, H), ld(s->W3b, H, nl, H),
-                       EpBack{nullptr, s->d2, s->d2b, s->d2T, nl, Bm, c->act}, e, st)));
-  TCK((launch_t<true>((long long)H, nl, B, ld(s->h1T, B, H, B), ld(s->d2T, B, nl, B),
-                       EpStore{s->g[2], nl, H}, e, st)));
-  TCK((launch_t<true>(Bm, H, nl, ld(s->d2b, nl, Bm, nl), ld(s->W2b, nl, H, nl),
-                               EpBack{s->a1, s->d1, nullptr, s->d1T, H, Bm, c->act}, e, st)));
+  TCK(launch_pair((long long)H, I, B, ld(s->h3T, B, H, B), ld(s->d4T, B, I, B), EpStore{s->g[6], I, H},
+                  Bm, H, I, ld(s->d4b, I, Bm, I), ld(s->W4b, I, H, I),
+                  EpBack{s->a3, s->d3, s->d3b, s->d3T, H, Bm, c->act}, e, st));
+  TCK(launch_pair((long long)nl, H, B, ld(s->zbT, B, nl, B), ld(s->d3T, B, H, B), EpStore{s->g[4], H, nl},
+                  Bm, nl, H, ld(s->d3b, H, Bm, H), ld(s->W3b, H, nl, H),
+                  EpBack{nullptr, s->d2, s->d2b, s->d2T, nl, Bm, c->act}, e, st));
+  TCK(launch_pair((long long)H, nl, B, ld(s->h1T, B, H, B), ld(s->d2T, B, nl, B), EpStore{s->g[2], nl, H},
+                  Bm, H, nl, ld(s->d2b, nl, Bm, nl), ld(s->W2b, nl, H, nl),
+                  EpBack{s->a1, s->d1, nullptr, s->d1T, H, Bm, c->act}, e, st));
   TCK((launch_t<true>((long long)I, H, B, ld(s->YT, B, I, B), ld(s->d1T, B, H, B),
                                EpStore{s->g[0], H, I}, e, st)));
   // bias gradients
@@ -630,13 +688,11 @@ cudaError_t codec_train_step(Codec* c, const uint16_t* Y, const float* wts, int 
     ColSums cs{{s->d1, s->d2, s->d3, s->d4}, {s->g[1], s->g[3], s->g[5], s->g[7]}, {H, nl, H, I},
                {0, 0, 0, 0, 0}, 4};
     for (int q = 0; q < 4; ++q) cs.tiles[q + 1] = cs.tiles[q] + (cs.cols[q] + 31) / 32;
-    colsum_multi_kernel<<<cs.tiles[4], 256, 0, st>>>(cs, B);
-    TCK(cudaGetLastError());
+    TCK(gemm::launch_dependent(colsum_multi_kernel, dim3(cs.tiles[4]), dim3(256), 0, st, cs, B));
   }
-  if (loss_dev || loss_acc) {
-    loss_kernel<<<1, 1, 0, st>>>(s->red, 1.0 / ((double)B * I), loss_dev, loss_acc);
-    TCK(cudaGetLastError());
-  }
+  if (loss_dev || loss_acc)
+    TCK(gemm::launch_dependent(loss_kernel, dim3(1), dim3(1), 0, st, (const double*)s->red,
+                               1.0 / ((double)B * I), loss_dev, loss_acc));
   // ---- LAMB
   s->t += 1;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-6f;
@@ -658,11 +714,29 @@ cudaError_t codec_train_step(Codec* c, const uint16_t* Y, const float* wts, int 
     const int b = (int)std::max<size_t>(1, (size_t)((double)kLambBlocks * c->wn[i] / total + 0.5));
     la.blk[i + 1] = la.blk[i] + b;
   }
-  lamb1_multi_kernel<<<la.blk[8], 256, 0, st>>>(la, b1, b2, c1, c2, eps, s->red + 1);
-  TCK(cudaGetLastError());
-  lamb2_multi_kernel<<<la.blk[8], 256, 0, st>>>(la, lr, s->red + 1);
-  TCK(cudaGetLastError());
-  return codec_refresh(c, st);
+  TCK(gemm::launch_dependent(lamb1_multi_kernel, dim3(la.blk[8]), dim3(256), 0, st, la, b1, b2, c1, c2, eps,
+                             s->red + 1));
+  Lamb2 l2{};
+  const int rows[4] = {I, H, nl, H}, cols[4] = {H, nl, H, I}, blen[4] = {H, nl, H, I};
+  uint16_t* const nat[4] = {nullptr, s->W2b, s->W3b, s->W4b};
+  uint16_t* const tr[4] = {c->W1t, c->W2t, c->W3t, c->W4t};
+  for (int i = 0; i < 8; ++i) {
+    l2.w[i] = c->w[i];
+    l2.u[i] = s->g[i];
+  }
+  for (int m = 0; m < 4; ++m) {
+    l2.nat[m] = nat[m];
+    l2.tr[m] = tr[m];
+    l2.rows[m] = rows[m];
+    l2.cols[m] = cols[m];
+    l2.fp16[m] = m == 2;
+    l2.tiles[m + 1] = l2.tiles[m] + rows[m] / 32 * (cols[m] / 32);
+    l2.n[m] = blen[m];
+    l2.bias[m + 1] = l2.bias[m] + (blen[m] + 1023) / 1024;
+  }
+  TCK(gemm::launch_dependent(lamb2_multi_kernel, dim3(l2.tiles[4] + l2.bias[4]), dim3(256), 0, st, l2, lr,
+                             (const double*)(s->red + 1)));
+  return codec_refresh_strain(c, st);
 }
 
 cudaError_t codec_train(Codec* c, const uint16_t* Y, const float* maxima, long long n,
