@@ -391,8 +391,10 @@ aew::BrickFwd brick_incr_args(aew_handle* h, float* const in[4], float* const ou
 // reverse steps n0, n0 - 1, .., n0 - nsteps + 1: in (null: the zero state) -> out (null: not
 // kept); en (or en16): e^{n0}, the earlier states at - C each
 int brick_adj(aew_handle* h, int n0, int nsteps, float* const in[4], float* const out[4],
-              const float* resid, const float* en, const uint16_t* en16, cudaStream_t s) {
+              const float* resid, const float* en, const uint16_t* en16, cudaStream_t s,
+              const aew::BrickAdj* list = nullptr) {
   aew::BrickAdj a{};
+  if (list) a = *list;   // the strains step by step
   a.m = h->m;
   if (in) {
     a.mu = in[0];
@@ -724,6 +726,129 @@ int gradient_full(aew_handle* h, const float* d_obs, const float* wav, cudaStrea
   return AEW_OK;
 }
 
+// The plan on chip: a run of advances and stores is one launch (each checkpoint written by the
+// step that reaches it), and so is a run of reverse steps (each reading the strain of the
+// state restored for it); near its leaves the plan alternates single steps with stores and
+// restores, four launches of one step each for every launch here.  Launches of 10 us and more
+// bound it, whatever the grid: 72 x 100 x 148 with 20 slots 34 -> 20 us per step of the
+// gradient, 128^3 29.
+int run_revolve_brick(aew_handle* h, const std::vector<aew::RevAction>& plan, const float* d_obs,
+                      const float* resid, bool gradient, cudaStream_t s, long long* fwd_out) {
+  const int ns = h->cfg.n_checkpoints;
+  int rc;
+  if (gradient) AEW_CK(cudaMemsetAsync(h->d, 0, h->nrow * sizeof(float), s));
+  AEW_CK(cudaMemsetAsync(h->acc64, 0, h->C * sizeof(double), s));
+  auto slot = [&](int k) { return h->ckpt + (size_t)k * 4 * h->C; };
+  std::vector<int> slot_step(ns > 0 ? ns : 1, -1);
+  // the live state: e, vx, vy, vz one after the other from a slot, in st[0] / st[1], or zero
+  float* live[4] = {};
+  int live_n = 0, live_buf = -1;
+  bool zero = true;
+  auto to_slot = [&](int k) {
+    for (int i = 0; i < 4; ++i) live[i] = slot(k) + (size_t)i * h->C;
+    live_buf = -1;
+    zero = false;
+  };
+  const float* R = resid;
+  long long fwd = 0;
+  int acur = 0;
+  bool first_adj = true;
+  // reverse steps collected: the latest index and the strains
+  aew::BrickAdj rev{};
+  int rev_n = -1;
+  auto flush_reverse = [&]() -> int {
+    if (!rev.nlist) return AEW_OK;
+    const int n = rev.nlist;
+    rc = brick_adj(h, rev_n, n, first_adj ? nullptr : h->ad[acur], rev_n - n + 1 > 0 ? h->ad[acur ^ 1] : nullptr,
+                   R, nullptr, nullptr, s, &rev);
+    first_adj = false;
+    acur ^= 1;
+    rev.nlist = 0;
+    return rc;
+  };
+  for (size_t a = 0; a < plan.size();) {
+    const aew::RevAction& act = plan[a];
+    if (act.op == aew::kOpRestore) {
+      if (act.arg < 0) {
+        zero = true;
+        live_buf = -1;
+        live_n = 0;
+      } else {
+        to_slot(act.arg);
+        live_n = slot_step[act.arg];
+      }
+      ++a;
+    } else if (act.op == aew::kOpReverse) {
+      if (!rev.nlist) rev_n = act.arg;
+      rev.en_list[rev.nlist++] = act.arg > 0 ? live[0] : nullptr;
+      ++a;
+      if (rev.nlist == aew::kBrickList && (rc = flush_reverse())) return rc;
+    } else if (act.op == aew::kOpFinal) {
+      if (gradient) {   // last step: records d^{nt}, keeps state nt - 1 live
+        if ((rc = brick_fwd(h, brick_fwd_args(h, zero ? nullptr : live, nullptr, 1, h->dts + live_n,
+                                              drow(h, h->d, live_n + 1)), s)))
+          return rc;
+        ++fwd;
+        if ((rc = residual_and_misfit(h, d_obs, s))) return rc;
+        R = h->R;
+      }
+      ++a;
+    } else if (act.op == aew::kOpStore) {   // a state that no advance just reached
+      if ((rc = flush_reverse())) return rc;   // they may read the slot
+      if (zero)
+        AEW_CK(cudaMemsetAsync(slot(act.arg), 0, 4 * h->C * sizeof(float), s));
+      else if (live[0] != slot(act.arg))
+        for (int i = 0; i < 4; ++i)
+          AEW_CK(cudaMemcpyAsync(slot(act.arg) + (size_t)i * h->C, live[i], h->C * sizeof(float),
+                                 cudaMemcpyDeviceToDevice, s));
+      to_slot(act.arg);
+      slot_step[act.arg] = live_n;
+      ++a;
+    } else {   // advance
+      if ((rc = flush_reverse())) return rc;
+      aew::BrickFwd f = brick_fwd_args(h, zero ? nullptr : live, nullptr, 0, h->dts + live_n,
+                                       gradient ? drow(h, h->d, live_n + 1) : nullptr);
+      int last = -1;   // slot that holds the state reached, if one does
+      while (a < plan.size() && f.nstore < aew::kBrickList) {
+        if (plan[a].op == aew::kOpAdvance) {
+          f.nsteps += plan[a].arg;
+          if (plan[a].arg > 0) last = -1;
+        } else if (plan[a].op == aew::kOpStore && f.nsteps > 0 && slot(plan[a].arg) != f.e) {
+          f.store_at[f.nstore] = f.nsteps - 1;   // never onto the state being read
+          f.store[f.nstore++] = slot(plan[a].arg);
+          slot_step[plan[a].arg] = live_n + f.nsteps;
+          last = plan[a].arg;
+        } else {
+          break;
+        }
+        ++a;
+      }
+      if (f.nsteps > 0) {
+        const int buf = live_buf == 0 ? 1 : 0;
+        if (last < 0) {
+          f.e1 = h->st[buf][0];
+          f.vx1 = h->st[buf][1];
+          f.vy1 = h->st[buf][2];
+          f.vz1 = h->st[buf][3];
+        }
+        if ((rc = brick_fwd(h, f, s))) return rc;
+        live_n += f.nsteps;
+        fwd += f.nsteps;
+        if (last >= 0) {
+          to_slot(last);
+        } else {
+          for (int i = 0; i < 4; ++i) live[i] = h->st[buf][i];
+          live_buf = buf;
+          zero = false;
+        }
+      }
+    }
+  }
+  if ((rc = flush_reverse())) return rc;
+  *fwd_out = fwd;
+  return AEW_OK;
+}
+
 // Execute a checkpointing plan.  mode gradient: the first pass records d and the
 // 'final' action computes the misfit; otherwise (incremental adjoint of the GN-HVP) the
 // residual is given.  The live state is a set of field pointers: a restore just points
@@ -735,6 +860,7 @@ int run_revolve(aew_handle* h, const float* d_obs, const float* resid, const flo
   const int ns = h->cfg.n_checkpoints;
   std::vector<aew::RevAction> plan;
   aew::revolve_plan(nt, ns, plan);
+  if (h->brick) return run_revolve_brick(h, plan, d_obs, resid, gradient, s, fwd_out);
   int live_n = 0, acur = 0, rc;
   long long fwd = 0;
   auto slot = [&](int k, float** f) {
@@ -752,22 +878,6 @@ int run_revolve(aew_handle* h, const float* d_obs, const float* resid, const flo
     switch (act.op) {
       case aew::kOpAdvance: {
         const bool to_slot = a + 1 < plan.size() && plan[a + 1].op == aew::kOpStore;
-        if (h->brick && act.arg > 0) {
-          float* out[4];
-          if (to_slot) slot(plan[a + 1].arg, out);
-          const bool direct = to_slot && out[0] != live[0];   // never onto the state it reads
-          const int out_buf = direct ? -1 : (live_buf == 0 ? 1 : 0);
-          for (int i = 0; !direct && i < 4; ++i) out[i] = h->st[out_buf][i];
-          rc = brick_fwd(h, brick_fwd_args(h, live[0] == h->zst[0] ? nullptr : live, out, act.arg,
-                                           h->dts + live_n,
-                                           gradient ? drow(h, h->d, live_n + 1) : nullptr), s);
-          if (rc) return rc;
-          for (int i = 0; i < 4; ++i) live[i] = out[i];
-          live_buf = out_buf;
-          live_n += act.arg;
-          fwd += act.arg;
-          break;
-        }
         for (int k = 0; k < act.arg; ++k) {
           float* out[4];
           int out_buf;
@@ -818,11 +928,7 @@ int run_revolve(aew_handle* h, const float* d_obs, const float* resid, const flo
           float* out[4];
           const int ob = live_buf == 0 ? 1 : 0;
           for (int i = 0; i < 4; ++i) out[i] = h->st[ob][i];
-          if (h->brick)
-            rc = brick_fwd(h, brick_fwd_args(h, live[0] == h->zst[0] ? nullptr : live, nullptr, 1,
-                                             h->dts + live_n, drow(h, h->d, live_n + 1)), s);
-          else
-            rc = fwd_step(h, live_n, live, out, wav, drow(h, h->d, live_n + 1), s);
+          rc = fwd_step(h, live_n, live, out, wav, drow(h, h->d, live_n + 1), s);
           if (rc) return rc;
           ++fwd;
           if ((rc = residual_and_misfit(h, d_obs, s))) return rc;

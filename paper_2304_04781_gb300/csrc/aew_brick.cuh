@@ -416,6 +416,7 @@ __global__ void __launch_bounds__(tmax(BZ), 1) fwd_kernel(const __grid_constant_
     c.publish_z(g, f, 0, a.tag);
   }
 
+  int next_store = 0;
 #pragma unroll 1
   for (int n = 0; n < a.nsteps; ++n) {
     const int par = n & 1;
@@ -523,6 +524,18 @@ __global__ void __launch_bounds__(tmax(BZ), 1) fwd_kernel(const __grid_constant_
       }
     }
     if (more) c.publish_z(g, f, par ^ 1, tag + 1);
+    if (INCR == 0 && !TPACK && next_store < a.nstore && a.store_at[next_store] == n) {   // a checkpoint
+      float* const o = a.store[next_store++];
+#pragma unroll
+      for (int k = 0; k < BZ; ++k)
+        if (bits >> k & 1u) {
+          const uint32_t i = c.row + k * g.P;
+          st4(o, i, v4(e.get(f + X::oS + tid, k)));
+          st4(o, i + g.C, v4(vx[k]));
+          st4(o, i + 2 * g.C, fl & kLastY ? z4() : V[k * PV]);
+          st4(o, i + 3 * g.C, g.k0 + k == a.nz - 1 ? z4() : v4(vz[k]));
+        }
+    }
     if (bits & 0xff000000u) {   // receivers
 #pragma unroll
       for (int k = 0; k < BZ; ++k)
@@ -619,7 +632,8 @@ __global__ void __launch_bounds__(tmax(BZ), 1) adj_kernel(const __grid_constant_
     const int par = n & 1;
     const uint32_t tag = a.tag + n;
     const bool more = n + 1 < a.nsteps;
-    const bool has_e = n < a.en_steps;
+    const float* const en_n = B16 ? nullptr : a.nlist ? a.en_list[n] : a.en - (size_t)n * g.C;
+    const bool has_e = a.nlist ? en_n != nullptr : n < a.en_steps;
     const F4 below = c.template receive_halos<NC == 1>(g, f, a.by, a.py, par, tag, dead, a.err);
     const uint32_t tid = fresh_copy(threadIdx.x), fl = fresh_copy(c.fl), bits = fresh_copy(c.bits);
     float4* const E = f + X::oE + tid;
@@ -661,10 +675,9 @@ __global__ void __launch_bounds__(tmax(BZ), 1) adj_kernel(const __grid_constant_
           if (B16) {
             enb[z] = __ldg(reinterpret_cast<const uint2*>(a.en16 - (size_t)n * g.C + i));
           } else {
-            const float* p = a.en - (size_t)n * g.C + i;
-            en[z] = ldg4(p);
+            en[z] = ldg4(en_n + i);
             // the next step's strain comes from HBM: into L2 now
-            if (n + 1 < a.en_steps) asm volatile("prefetch.global.L2 [%0];" ::"l"(p - g.C));
+            if (n + 1 < a.en_steps) asm volatile("prefetch.global.L2 [%0];" ::"l"(en_n + i - g.C));
           }
         }
         const F4 mu_n = lds(E + (k + 1) * PE);

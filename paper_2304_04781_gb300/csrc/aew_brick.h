@@ -15,6 +15,9 @@ struct BrickPlan {
   int threads = 0;   // by * nx / 4 rounded up to whole warps
 };
 
+// entries of the per-step lists below
+constexpr int kBrickList = 32;
+
 // One launch: `nsteps` forward-type steps n = 0 .. nsteps - 1 (indices inside the launch).
 struct BrickFwd {
   const float* m;
@@ -38,6 +41,11 @@ struct BrickFwd {
   size_t nrow;
   float* hist;         // e^{n+1} of step n to hist + n C for n < nhist (null: none)
   int nhist;
+  // checkpoints: the state after step store_at[i] (increasing) also to store[i] (e, vx, vy, vz
+  // one after the other)
+  int nstore;
+  int store_at[kBrickList];
+  float* store[kBrickList];
   // incremental solve: step n adds G(dm e^n), e^n = ef + n C (FP32) or ef16 + n C (BF16);
   // ef_first: the first step that has it (the initial strain is 0)
   const float* dm;
@@ -75,6 +83,9 @@ struct BrickAdj {
   const float* en;
   const uint16_t* en16;
   int en_steps;
+  // .. or, with nlist = nsteps, en_list[n] (null: none)
+  int nlist;
+  const float* en_list[kBrickList];
   const float* resid;  // residual row of step 0; step n reads resid - n nrow (null: none)
   size_t nrow;
   int krec;

@@ -12,7 +12,8 @@ cudaError_t go(const BrickAdj& a, const BrickPlan& p, cudaStream_t s) {
 
 cudaError_t launch_brick_adj(BrickAdj a, const BrickPlan& p, unsigned char* halo, uint32_t* tag,
                              int* err, cudaStream_t s) {
-  if (!halo || !err || a.nsteps < 1) return cudaErrorInvalidValue;
+  if (!halo || !err || a.nsteps < 1 || (a.nlist && a.nlist != a.nsteps) || a.nlist > kBrickList)
+    return cudaErrorInvalidValue;
   a.by = p.by;
   a.bz = p.bz;
   a.py = p.py;

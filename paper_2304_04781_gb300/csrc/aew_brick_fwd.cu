@@ -46,7 +46,8 @@ cudaError_t go(const BrickFwd& a, const BrickPlan& p, cudaStream_t s) {
 
 cudaError_t launch_brick_fwd(BrickFwd a, const BrickPlan& p, unsigned char* halo, uint32_t* tag,
                              int* err, cudaStream_t s) {
-  if (!halo || !err || a.nsteps < 1) return cudaErrorInvalidValue;
+  if (!halo || !err || a.nsteps < 1 || a.nstore > kBrickList || (a.nstore && (a.dm || a.tpack)))
+    return cudaErrorInvalidValue;
   a.by = p.by;
   a.bz = p.bz;
   a.py = p.py;
