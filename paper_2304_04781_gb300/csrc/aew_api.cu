@@ -312,6 +312,28 @@ int adj_step_x(aew_handle* h, int n, float* const in[4], float* const out[4],
 // ---------------------------------------------------------------------------------
 // On-chip time loops (aew_brick.h): many steps per launch
 // ---------------------------------------------------------------------------------
+// The handle's solves run on chip.  Their buffers are made by the first one (about a millisecond
+// that handles used for the codec alone need not spend); without memory for them the grid takes
+// the kernels of the larger ones.
+bool on_chip(aew_handle* h) {
+  if (!h->brick || h->halo) return h->brick;
+  const size_t nb = aew::brick_halo_bytes(h->cfg.nx, h->bp), nt = (size_t)h->cfg.nt;
+  std::vector<float> dts(nt);
+  for (size_t n = 0; n < nt; ++n) dts[n] = (float)(h->dt * (double)h->wav[n]);
+  unsigned char* halo = nullptr;
+  if (dalloc(h, &h->dts, nt) && dalloc(h, &halo, nb) &&
+      cudaMemcpy(h->dts, dts.data(), nt * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
+      cudaMemset(halo, 0, nb) == cudaSuccess && cudaStreamSynchronize(0) == cudaSuccess) {
+    h->halo = halo;
+  } else {
+    cudaGetLastError();
+    h->brick = false;
+    h->two = true;
+  }
+  h->stats.device_bytes = h->bytes + aew::codec_device_bytes(h->codec);
+  return h->brick;
+}
+
 // dt s^n, n = 0 .. nt - 1, on the device: the default wavelet's, or wav's [count]
 int wavelet_on_device(aew_handle* h, const float* wav, size_t count, const float** out,
                       cudaStream_t s) {
@@ -522,7 +544,7 @@ int two_adj(aew_handle* h, int n, float* const in[4], float* const out[4], const
 // reverse step n: (lam, mu) in ad[cur] -> ad[cur ^ 1]
 int adj_step(aew_handle* h, int n, int cur, const float* resid, const float* en,
              cudaStream_t s) {
-  if (h->brick) return brick_adj(h, n, 1, h->ad[cur], h->ad[cur ^ 1], resid, en, nullptr, s);
+  if (on_chip(h)) return brick_adj(h, n, 1, h->ad[cur], h->ad[cur ^ 1], resid, en, nullptr, s);
   return adj_step_x(h, n, h->ad[cur], h->ad[cur ^ 1], resid, en, h->acc32, h->acc64, nullptr,
                     nullptr, nullptr, s);
 }
@@ -665,7 +687,7 @@ int ae_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
 int adjoint_full(aew_handle* h, const float* resid, cudaStream_t s) {
   const int nt = h->cfg.nt;
   int rc, cur = 0;
-  if (h->brick) {
+  if (on_chip(h)) {
     AEW_CK(cudaMemsetAsync(h->acc64, 0, h->C * sizeof(double), s));
     return brick_adj(h, nt - 1, nt, nullptr, nullptr, resid,
                      nt > 1 ? h->estore + (size_t)(nt - 1) * h->C : nullptr, nullptr, s);
@@ -686,7 +708,7 @@ int adjoint_full(aew_handle* h, const float* resid, cudaStream_t s) {
 
 int gradient_full(aew_handle* h, const float* d_obs, const float* wav, cudaStream_t s) {
   const int nt = h->cfg.nt;
-  if (h->brick) {
+  if (on_chip(h)) {
     AEW_CK(cudaMemsetAsync(h->estore, 0, h->C * sizeof(float), s));
     AEW_CK(cudaMemsetAsync(h->d, 0, h->nrow * sizeof(float), s));
     aew::BrickFwd a = brick_fwd_args(h, nullptr, nullptr, nt, h->dts, drow(h, h->d, 1));
@@ -860,7 +882,7 @@ int run_revolve(aew_handle* h, const float* d_obs, const float* resid, const flo
   const int ns = h->cfg.n_checkpoints;
   std::vector<aew::RevAction> plan;
   aew::revolve_plan(nt, ns, plan);
-  if (h->brick) return run_revolve_brick(h, plan, d_obs, resid, gradient, s, fwd_out);
+  if (on_chip(h)) return run_revolve_brick(h, plan, d_obs, resid, gradient, s, fwd_out);
   int live_n = 0, acur = 0, rc;
   long long fwd = 0;
   auto slot = [&](int k, float** f) {
@@ -993,7 +1015,7 @@ int encode_window(aew_handle* h, int tb, cudaStream_t s) {
   const bool mm = aew::codec_minmax(h->codec);
   cudaError_t e = aew::codec_encode_window(h->codec, h->xt[tb & 1], h->vmx + (size_t)tb * nv,
                                            (long long)nv, h->lat + (size_t)tb * nv * h->cfg.n_lat,
-                                           h->ovf, s, h->brick ? 0 : h->overlap_ctas,
+                                           h->ovf, s, on_chip(h) ? 0 : h->overlap_ctas,
                                            mm ? h->wmn + (size_t)tb * nv : nullptr,
                                            mm ? h->wr + (size_t)tb * nv : nullptr);
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_encode_window");
@@ -1009,7 +1031,7 @@ int decode_window(aew_handle* h, int tb, cudaStream_t s, bool bf16 = false) {
   cudaError_t e = aew::codec_decode_window(h->codec, h->lat + (size_t)tb * nv * h->cfg.n_lat,
                                            h->vmx + (size_t)tb * nv, h->cfg.nx, h->cfg.ny,
                                            h->cfg.nz, h->edt[tb & 1], s,
-                                           h->brick ? 0 : h->overlap_ctas,
+                                           on_chip(h) ? 0 : h->overlap_ctas,
                                            mm ? h->wmn + (size_t)tb * nv : nullptr,
                                            mm ? h->wr + (size_t)tb * nv : nullptr, bf16);
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_decode_window");
@@ -1035,7 +1057,7 @@ const uint16_t* window_e16(aew_handle* h, int n) {
 int time_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
   const int nt = h->cfg.nt, W = nwin_of(h), T = aew::kTSteps;
   int rc;
-  if (h->brick) {   // the on-chip loops fill the GPU: decode and sweep each window in turn
+  if (on_chip(h)) {   // the on-chip loops fill the GPU: decode and sweep each window in turn
     AEW_CK(cudaMemsetAsync(h->acc64, 0, h->C * sizeof(double), s));
     for (int tb = W - 1, cur = 0; tb >= 0; --tb, cur ^= 1) {
       if ((rc = decode_window(h, tb, s, true))) return rc;
@@ -1089,7 +1111,7 @@ int gradient_ae_time(aew_handle* h, const float* d_obs, const float* wav, cudaSt
   AEW_CK(cudaMemsetAsync(h->xt[0], 0, wbytes, s));   // slot 0 of window 0 is e^0 = 0
   AEW_CK(cudaMemsetAsync(h->ovf, 0, sizeof(int), s));
   AEW_CK(cudaMemsetAsync(h->d, 0, h->nrow * sizeof(float), s));
-  if (h->brick) {   // the on-chip loops fill the GPU: run and encode each window in turn
+  if (on_chip(h)) {   // the on-chip loops fill the GPU: run and encode each window in turn
     // window tb's states m = T tb .. min(T tb + T, nt) - 1 come from steps m - 1; the last
     // launch also runs step nt - 1, whose state nt is not stored
     for (int tb = 0, cur = 0, n = 0; tb < W; ++tb, cur ^= 1) {
@@ -1211,7 +1233,7 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
   int cur = 0;
   if (h->cfg.storage == AEW_FULL) {
     AEW_CK(cudaMemsetAsync(h->desto, 0, h->C * sizeof(float), s));
-    if (h->brick) {
+    if (on_chip(h)) {
       aew::BrickFwd a = brick_incr_args(h, nullptr, nullptr, 0, nt, h->estore, nullptr,
                                         drow(h, h->dd, 1));
       a.hist = h->desto + h->C;
@@ -1425,7 +1447,7 @@ int snapshots_time(aew_handle* h, int every, uint16_t* out, long long max_vector
     return AEW_OK;
   };
   int cur = 0;
-  for (int tb = 0, n = 0; h->brick && tb <= last; ++tb) {
+  for (int tb = 0, n = 0; on_chip(h) && tb <= last; ++tb) {
     if (at[tb] < 0) continue;
     // one launch up to the window's first state - 1, one for the window itself
     const int m0 = std::max(T * tb, 1), ends[2] = {m0 - 1, T * tb + T - 1};
@@ -1446,7 +1468,7 @@ int snapshots_time(aew_handle* h, int every, uint16_t* out, long long max_vector
     }
     if ((rc = finish(tb))) return rc;
   }
-  for (int n = 0; !h->brick && n < T * last + T - 1; ++n) {
+  for (int n = 0; !on_chip(h) && n < T * last + T - 1; ++n) {
     const int m = n + 1, tb = m / T, slot = m % T;
     uint16_t* tp = nullptr;
     unsigned* vq = nullptr;
@@ -1619,14 +1641,6 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
     // against 95, 512 x 512 x 256 302 against 350
     h->two = !h->brick;
     h->sms = sms;
-    if (h->brick) {
-      const size_t nb = aew::brick_halo_bytes(c.nx, h->bp);
-      std::vector<float> dts(nt);
-      for (size_t n = 0; n < nt; ++n) dts[n] = (float)(h->dt * (double)h->wav[n]);
-      ok = dalloc(h, &h->halo, nb) && cudaMemset(h->halo, 0, nb) == cudaSuccess &&
-           dalloc(h, &h->dts, nt) &&
-           cudaMemcpy(h->dts, dts.data(), nt * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
-    }
   }
   if (ok && c.storage == AEW_AE) {
     // The codec GEMMs run on a high-priority side stream with half the SMs, so their
@@ -1733,7 +1747,7 @@ int aew_forward(aew_handle* h, const float* c_dev, const float* wavelet_host, fl
   if (rc) return rc;
   h->have_grad = false;  // m changed: stored history no longer matches
   if (d_dev && h->nrow) AEW_CK(cudaMemsetAsync(d_dev, 0, h->nrow * sizeof(float), s));
-  if (h->brick) {
+  if (on_chip(h)) {
     const float* dts = nullptr;
     if ((rc = wavelet_on_device(h, wavelet_host, (size_t)h->cfg.nt, &dts, s))) return rc;
     return brick_fwd(h, brick_fwd_args(h, nullptr, nullptr, h->cfg.nt, dts,
@@ -1788,7 +1802,7 @@ int aew_propagate(aew_handle* h, const float* c_dev, float* const state_dev[4], 
   float* tmp[4] = {h->st[0][0], h->st[0][1], h->st[0][2], h->st[0][3]};
   float* bufs[2][4] = {{state_dev[0], state_dev[1], state_dev[2], state_dev[3]},
                        {tmp[0], tmp[1], tmp[2], tmp[3]}};
-  if (h->brick && nsteps > 0) {
+  if (on_chip(h) && nsteps > 0) {
     const float* dts = nullptr;
     if (wavelet_host && (rc = wavelet_on_device(h, wavelet_host, (size_t)nsteps, &dts, s))) return rc;
     if ((rc = brick_fwd(h, brick_fwd_args(h, bufs[0], bufs[1], nsteps, dts,
@@ -1891,12 +1905,12 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
   if (h->nrow) AEW_CK(cudaMemsetAsync(dd_out, 0, h->nrow * sizeof(float), s));
   int cur = 0, fcur = 0;
   *fwd = 0;
-  if (h->brick && h->cfg.storage == AEW_FULL) {
+  if (on_chip(h) && h->cfg.storage == AEW_FULL) {
     *fwd = nt;
     return brick_fwd(h, brick_incr_args(h, nullptr, nullptr, 0, nt, h->estore, nullptr,
                                         drow(h, dd_out, 1)), s);
   }
-  if (h->brick && h->cfg.storage == AEW_AE && h->tcodec) {
+  if (on_chip(h) && h->cfg.storage == AEW_AE && h->tcodec) {
     const int W = nwin_of(h), T = aew::kTSteps;
     *fwd = nt;
     for (int tb = 0; tb < W; ++tb, cur ^= 1) {
@@ -1976,7 +1990,7 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
     }
     if (h->cfg.storage == AEW_REVOLVE) {
       if (n > 0) {  // lockstep forward recompute: state n from state n-1
-        if (h->brick)
+        if (on_chip(h))
           rc = brick_fwd(h, brick_fwd_args(h, h->st[fcur], h->st[fcur ^ 1], 1, h->dts + n - 1,
                                            nullptr), s);
         else
@@ -1987,7 +2001,7 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
         en = h->st[fcur][0];
       }
     }
-    if (h->brick && h->cfg.storage == AEW_REVOLVE) {
+    if (on_chip(h) && h->cfg.storage == AEW_REVOLVE) {
       rc = n == 0 ? brick_fwd(h, brick_fwd_args(h, h->ad[cur], h->ad[cur ^ 1], 1, nullptr,
                                                 drow(h, dd_out, 1)), s)
                   : brick_fwd(h, brick_incr_args(h, h->ad[cur], h->ad[cur ^ 1], n, 1, en, nullptr,
@@ -2512,7 +2526,7 @@ int aew_snapshots(aew_handle* h, const float* c_dev, int every, uint16_t* out_de
     return block_max_dev ? reinterpret_cast<unsigned*>(block_max_dev) + (size_t)w * 4
                          : h->bm_tmp + ((size_t)(w / (long long)nb) & 1) * nb * 4;
   };
-  if (h->brick) {   // on chip from one packed state to the next
+  if (on_chip(h)) {   // on chip from one packed state to the next
     for (int n = 0, m = every; packs(m, written); n = m, m += every, cur ^= 1) {
       if ((rc = brick_fwd(h, brick_fwd_args(h, n ? h->st[cur] : nullptr, h->st[cur ^ 1], m - n,
                                             h->dts + n, nullptr), s)))
@@ -2615,6 +2629,14 @@ GridInfo grid_of(const aew_handle* h) {
 }
 
 int set_error(aew_handle* h, int code, const std::string& msg) { return fail(h, code, msg); }
+
+bool brick_of(aew_handle* h, BrickRef* b) {
+  if (!on_chip(h)) return false;
+  *b = BrickRef{&h->bp, h->halo, &h->halo_tag, codec_err_flag(h->codec)};
+  return true;
+}
+
+bool take_timeout(aew_handle* h, cudaStream_t s) { return codec_take_error(h->codec, s); }
 
 int gradient_gated(aew_handle* h, const float* c_dev, const float* d_obs_dev, float* g_dev,
                    double gate, double* misfit, bool* accepted, cudaStream_t s) {

@@ -100,6 +100,24 @@ struct BrickAdj {
   int* err;
 };
 
+// CG for A x = w of the prior's operator (aew_newton.cu), one launch for the whole solve:
+// r = sc w at the start, x scaled by 1 / sc at the end; the residual test every 8 iterations
+// (and after the last): r.r <= tol2.
+struct BrickCg {
+  const float* w;
+  float* x;
+  int nx, ny, nz;
+  float alpha, at, sc, inv_sc;
+  float rr_hi, rr_lo;      // r.r at the start, as a pair of floats
+  float tol_hi, tol_lo;    // tol2
+  int max_iter;
+  int* result;             // device [2]: iterations, 1 if the test passed
+  int by, bz, py, pz;
+  unsigned char* halo;
+  uint32_t tag;
+  int* err;
+};
+
 // false where the grid does not fit (or sms is not known)
 bool brick_plan(int nx, int ny, int nz, int sms, BrickPlan* p);
 // bytes of the halo exchange buffer (zeroed once by its owner)
@@ -109,6 +127,12 @@ cudaError_t launch_brick_fwd(BrickFwd a, const BrickPlan& p, unsigned char* halo
                              int* err, cudaStream_t s);
 cudaError_t launch_brick_adj(BrickAdj a, const BrickPlan& p, unsigned char* halo, uint32_t* tag,
                              int* err, cudaStream_t s);
+cudaError_t launch_brick_cg(BrickCg a, const BrickPlan& p, unsigned char* halo, uint32_t* tag,
+                            int* err, cudaStream_t s);
+// before a launch that uses up to `steps` tags: where they would wrap, the buffer is cleared and
+// they start over
+cudaError_t brick_tags(uint32_t* tag, uint32_t steps, int nx, const BrickPlan& p, unsigned char* halo,
+                       cudaStream_t s);
 // per kernel family (internal to the launchers)
 cudaError_t launch_brick_incr(const BrickFwd& a, const BrickPlan& p, cudaStream_t s);
 

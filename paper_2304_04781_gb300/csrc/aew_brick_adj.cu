@@ -14,6 +14,8 @@ cudaError_t launch_brick_adj(BrickAdj a, const BrickPlan& p, unsigned char* halo
                              int* err, cudaStream_t s) {
   if (!halo || !err || a.nsteps < 1 || (a.nlist && a.nlist != a.nsteps) || a.nlist > kBrickList)
     return cudaErrorInvalidValue;
+  const cudaError_t e = brick_tags(tag, (uint32_t)a.nsteps, a.nx, p, halo, s);
+  if (e != cudaSuccess) return e;
   a.by = p.by;
   a.bz = p.bz;
   a.py = p.py;

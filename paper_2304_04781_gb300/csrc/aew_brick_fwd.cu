@@ -33,7 +33,15 @@ bool brick_plan(int nx, int ny, int nz, int sms, BrickPlan* p) {
 
 size_t brick_halo_bytes(int nx, const BrickPlan& p) {
   const size_t ctas = (size_t)p.py * p.pz;
-  return 2 * ctas * 2 * 2 * ((size_t)brick::tmax(p.bz) + (size_t)p.bz * (nx / 4)) * 16;
+  return 2 * ctas * 2 * 2 * ((size_t)brick::tmax(p.bz) + (size_t)p.bz * (nx / 4)) * 16 +
+         4 * ctas * 16;   // two sums of two parities per CTA
+}
+
+cudaError_t brick_tags(uint32_t* tag, uint32_t steps, int nx, const BrickPlan& p, unsigned char* halo,
+                       cudaStream_t s) {
+  if ((uint64_t)*tag + steps + 4 <= 0xffffffffull) return cudaSuccess;
+  *tag = 0;
+  return cudaMemsetAsync(halo, 0, brick_halo_bytes(nx, p), s);
 }
 
 namespace {
@@ -48,6 +56,8 @@ cudaError_t launch_brick_fwd(BrickFwd a, const BrickPlan& p, unsigned char* halo
                              int* err, cudaStream_t s) {
   if (!halo || !err || a.nsteps < 1 || a.nstore > kBrickList || (a.nstore && (a.dm || a.tpack)))
     return cudaErrorInvalidValue;
+  const cudaError_t e = brick_tags(tag, (uint32_t)a.nsteps, a.nx, p, halo, s);
+  if (e != cudaSuccess) return e;
   a.by = p.by;
   a.bz = p.bz;
   a.py = p.py;

@@ -17,7 +17,8 @@
 // Each kernel sums the previous one's per-block FP64 partials itself (every block in the
 // same order, so all blocks agree).  The residual is tested on the device every 8
 // iterations; once it passes, the kernels already enqueued return at once, so the host
-// stays a batch of launches ahead of the test.
+// stays a batch of launches ahead of the test.  Grids that fit the SMs: one launch for the
+// whole solve (aew_brick_cg.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -28,6 +29,7 @@
 #include <vector>
 
 #include "../../include/aewave.h"
+#include "aew_brick.h"
 #include "aew_internal.cuh"
 #include "aew_pca.h"
 #include "aew_solver.h"
@@ -697,6 +699,12 @@ int prior_args_ok(aew_handle* h, double alpha, double theta) {
   return AEW_OK;
 }
 
+int no_convergence(aew_handle* h, double rtol, int iters) {
+  char buf[160];
+  std::snprintf(buf, sizeof buf, "prior solve: relative residual above %.3g after %d iterations", rtol, iters);
+  return set_error(h, AEW_E_NOCONVERGE, buf);
+}
+
 // CG on A x = w (device scalars); x_dev written
 int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta,
              const float* w, float* x, double rtol, int max_iter, int* iters, cudaStream_t s) {
@@ -709,8 +717,10 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   float *r, *p[2];
   double* part;   // [3][np]: p.Ap, rr (two parities)
   int *done, *seen;
-  if (!ws.alloc(&r, g.C) || !ws.alloc(&p[0], g.C) || !ws.alloc(&p[1], g.C) ||
-      !ws.alloc(&part, 3 * (size_t)np) || !ws.alloc(&done, 1) || !ws.alloc_host(&seen, 2))
+  BrickRef br;
+  const bool chip = brick_of(h, &br);
+  if ((!chip && (!ws.alloc(&r, g.C) || !ws.alloc(&p[0], g.C) || !ws.alloc(&p[1], g.C))) ||
+      !ws.alloc(&part, 3 * (size_t)np) || !ws.alloc(&done, 2) || (!chip && !ws.alloc_host(&seen, 2)))
     return set_error(h, AEW_E_NOMEM, "prior solve: work vectors do not fit");
   double* ppap = part;
   double* prr[2] = {part + np, part + 2 * (size_t)np};
@@ -737,6 +747,35 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   // solve for the unit-rms right-hand side sc w (the iteration's FP32 squares then stay
   // far from FP32's range limits), and scale x back at the end
   const double sc = std::sqrt((double)g.C / ww);
+  // on chip where the grid fits: 128^3 45 -> 17 us per iteration, 64^3 37 -> 12
+  if (chip) {
+    const double rr = ww * (double)(float)sc * (double)(float)sc, t2 = rtol * rtol * rr;
+    BrickCg a{};
+    a.w = w;
+    a.x = x;
+    a.nx = g.nx;
+    a.ny = g.ny;
+    a.nz = g.nz;
+    a.alpha = fa;
+    a.at = fat;
+    a.sc = (float)sc;
+    a.inv_sc = (float)(1.0 / sc);
+    a.rr_hi = (float)rr;
+    a.rr_lo = (float)(rr - (double)a.rr_hi);
+    a.tol_hi = (float)t2;
+    a.tol_lo = (float)(t2 - (double)a.tol_hi);
+    a.max_iter = max_iter;
+    a.result = done;
+    NW_CK(cudaMemsetAsync(done, 0, 2 * sizeof(int), s));
+    NW_CK(launch_brick_cg(a, *br.plan, br.halo, br.tag, br.err, s));
+    int got[2] = {0, 0};
+    NW_CK(cudaMemcpyAsync(got, done, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    const bool timeout = take_timeout(h, s);   // synchronises
+    *br.tag += (uint32_t)std::max(got[0], 0) + 3;   // no CTA is more than an iteration ahead
+    if (timeout) return set_error(h, AEW_E_TIMEOUT, "a kernel gave up waiting (bounded halo wait)");
+    if (iters) *iters = got[0];
+    return got[1] ? AEW_OK : no_convergence(h, rtol, got[0]);
+  }
   cg_start_kernel<<<nb, NT, 0, s>>>(w, (float)sc, r, x, g.C);
   NW_CK(cudaMemsetAsync(done, 0xff, sizeof(int), s));   // -1: not yet
   NW_CK(cudaGetLastError());
@@ -781,11 +820,7 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   axpby_kernel<<<nb, NT, 0, s>>>((float)(1.0 / sc), x, 0.f, x, x, g.C);
   NW_CK(cudaGetLastError());
   NW_CK(cudaStreamSynchronize(s));   // the work vectors are freed on return
-  if (at >= 0) return AEW_OK;
-  char buf[160];
-  std::snprintf(buf, sizeof buf, "prior solve: relative residual above %.3g after %d iterations",
-                rtol, max_iter);
-  return set_error(h, AEW_E_NOCONVERGE, buf);
+  return at >= 0 ? AEW_OK : no_convergence(h, rtol, max_iter);
 }
 
 }  // namespace

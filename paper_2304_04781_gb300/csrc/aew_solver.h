@@ -8,6 +8,7 @@
 #include <string>
 
 #include "../../include/aewave.h"
+#include "aew_brick.h"
 
 namespace aew {
 
@@ -18,6 +19,17 @@ struct GridInfo {
 };
 
 GridInfo grid_of(const aew_handle* h);
+
+// where the handle's grid runs on chip: its cut, halo buffer, running tag and error flag
+struct BrickRef {
+  const BrickPlan* plan;
+  unsigned char* halo;
+  uint32_t* tag;
+  int* err;
+};
+bool brick_of(aew_handle* h, BrickRef* b);
+// a bounded wait of the handle's kernels gave up since the last look (synchronises)
+bool take_timeout(aew_handle* h, cudaStream_t s);
 
 // set the handle's error message; returns code
 int set_error(aew_handle* h, int code, const std::string& msg);
