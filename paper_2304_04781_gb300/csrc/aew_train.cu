@@ -8,7 +8,7 @@
 // set-up runs while that one drains), the weight gradient of a layer shares a launch with the
 // activation gradient that comes next (they need the same input), and the optimiser's second
 // pass also writes the operand copies of the new weights.  Time codec, us per step: batch 512
-// 252 -> 219, batch 64 222 -> 199; space codec at 512 208 -> 151.
+// 252 -> 166, batch 64 222 -> 146; space codec at 512 208 -> 130.
 //
 // Every product is a tcgen05 GEMM (aew_gemm.cuh) with BF16 operands and FP32
 // accumulation (the decoder's first forward product uses FP16 operands, as in
@@ -510,9 +510,11 @@ __global__ void lamb1_multi_kernel(LambArgs a, float b1, float b2, float c1, flo
   block_add2((double)sw, (double)su, norms + 2 * t);
 }
 
-// pass 2: w -= lr * (|w| / |u|) * u, and the operand copies of the new weights: a block takes
-// one 32 x 32 tile of a weight matrix (natural BF16 rows for the backward products, transposed
-// BF16 or FP16 for the forward ones) or 1024 elements of a bias
+// pass 2: w -= lr * (|w| / |u|) * u, and the operand copies of the new weights: 32 x 32 tiles
+// of the weight matrices (natural BF16 rows for the backward products, transposed BF16 or FP16
+// for the forward ones) and stretches of 1024 elements of the biases, dealt to the blocks.  A
+// block takes the eight ratios in FP64 once, in one warp; every thread of a block per tile did
+// before, and FP64 square roots were 55 of the kernel's 70 us (5.2 M weights; 14 us now).
 struct Lamb2 {
   float* w[8];
   const float* u[8];
@@ -526,51 +528,72 @@ struct Lamb2 {
 __global__ void __launch_bounds__(256) lamb2_multi_kernel(Lamb2 a, float lr, const double* norms) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  __shared__ float tile[32][33];
-  const int tid = threadIdx.x;
-  const bool isb = (int)blockIdx.x >= a.tiles[4];
-  int m = 0;
-  if (isb)
-    while (m < 3 && (int)blockIdx.x - a.tiles[4] >= a.bias[m + 1]) ++m;
-  else
-    while (m < 3 && (int)blockIdx.x >= a.tiles[m + 1]) ++m;
-  const int t = 2 * m + (isb ? 1 : 0);
-  const double wn = sqrt(norms[2 * t]), un = sqrt(norms[2 * t + 1]);
-  const float r = (wn > 0.0 && un > 0.0) ? (float)(wn / un) : 1.f;
-  float* const w = a.w[t];
-  const float* const u = a.u[t];
-  if (isb) {
-    const int i0 = ((int)blockIdx.x - a.tiles[4] - a.bias[m]) * 1024;
-    for (int i = i0 + tid; i < min(i0 + 1024, a.n[m]); i += 256) w[i] -= lr * r * u[i];
-    return;
+  __shared__ float tile[2][32][33];
+  __shared__ float ratio[8];
+  const int tid = threadIdx.x, ntiles = a.tiles[4], total = ntiles + a.bias[4];
+  // the tile's matrix and the thread's place in it: four columns of one row (every size is a
+  // multiple of 32)
+  const int y = tid >> 3, x = (tid & 7) * 4;
+  struct At {
+    int m, c0, r0;
+    size_t i;
+    float4 w, u;
+  };
+  auto load = [&](int b) {
+    At p{};
+    if (b >= ntiles) return p;
+    while (p.m < 3 && b >= a.tiles[p.m + 1]) ++p.m;
+    const int cols = a.cols[p.m], tx = cols / 32, t = b - a.tiles[p.m];
+    p.c0 = t % tx * 32;
+    p.r0 = t / tx * 32;
+    p.i = (size_t)(p.r0 + y) * cols + p.c0 + x;
+    p.w = *reinterpret_cast<const float4*>(a.w[2 * p.m] + p.i);
+    p.u = *reinterpret_cast<const float4*>(a.u[2 * p.m] + p.i);
+    return p;
+  };
+  At p = load(blockIdx.x);
+  if (tid < 8) {
+    const double wn = sqrt(norms[2 * tid]), un = sqrt(norms[2 * tid + 1]);
+    ratio[tid] = (wn > 0.0 && un > 0.0) ? (float)(wn / un) : 1.f;
   }
-  // a thread takes four columns of one row (every size is a multiple of 32)
-  const int cols = a.cols[m], rows = a.rows[m], tx = cols / 32, b = blockIdx.x - a.tiles[m];
-  const int c0 = b % tx * 32, r0 = b / tx * 32, y = tid >> 3, x = (tid & 7) * 4;
-  const size_t i = (size_t)(r0 + y) * cols + c0 + x;
-  float4 v = *reinterpret_cast<const float4*>(w + i);
-  const float4 g = *reinterpret_cast<const float4*>(u + i);
-  v.x -= lr * r * g.x;
-  v.y -= lr * r * g.y;
-  v.z -= lr * r * g.z;
-  v.w -= lr * r * g.w;
-  *reinterpret_cast<float4*>(w + i) = v;
-  if (a.nat[m])
-    *reinterpret_cast<uint2*>(a.nat[m] + i) = make_uint2(gemm::pack_bf16(v.x, v.y), gemm::pack_bf16(v.z, v.w));
-  tile[y][x] = v.x;
-  tile[y][x + 1] = v.y;
-  tile[y][x + 2] = v.z;
-  tile[y][x + 3] = v.w;
   __syncthreads();
-  const float q[4] = {tile[x][y], tile[x + 1][y], tile[x + 2][y], tile[x + 3][y]};
-  uint2 o;
-  if (a.fp16[m]) {
-    const __half2 h0 = __floats2half2_rn(q[0], q[1]), h1 = __floats2half2_rn(q[2], q[3]);
-    o = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
-  } else {
-    o = make_uint2(gemm::pack_bf16(q[0], q[1]), gemm::pack_bf16(q[2], q[3]));
+  int par = 0;
+  for (int b = blockIdx.x; b < total; b += gridDim.x, par ^= 1) {
+    const At next = load(b + gridDim.x);
+    if (b >= ntiles) {
+      int m = 0;
+      while (m < 3 && b - ntiles >= a.bias[m + 1]) ++m;
+      const float r = ratio[2 * m + 1];
+      const int i0 = (b - ntiles - a.bias[m]) * 1024;
+      for (int i = i0 + tid; i < min(i0 + 1024, a.n[m]); i += 256) a.w[2 * m + 1][i] -= lr * r * a.u[2 * m + 1][i];
+      continue;
+    }
+    const float r = ratio[2 * p.m];
+    float4 v = p.w;
+    v.x -= lr * r * p.u.x;
+    v.y -= lr * r * p.u.y;
+    v.z -= lr * r * p.u.z;
+    v.w -= lr * r * p.u.w;
+    *reinterpret_cast<float4*>(a.w[2 * p.m] + p.i) = v;
+    if (a.nat[p.m])
+      *reinterpret_cast<uint2*>(a.nat[p.m] + p.i) = make_uint2(gemm::pack_bf16(v.x, v.y), gemm::pack_bf16(v.z, v.w));
+    float(*const t)[33] = tile[par];   // two: one barrier per tile
+    t[y][x] = v.x;
+    t[y][x + 1] = v.y;
+    t[y][x + 2] = v.z;
+    t[y][x + 3] = v.w;
+    __syncthreads();
+    const float q[4] = {t[x][y], t[x + 1][y], t[x + 2][y], t[x + 3][y]};
+    uint2 o;
+    if (a.fp16[p.m]) {
+      const __half2 h0 = __floats2half2_rn(q[0], q[1]), h1 = __floats2half2_rn(q[2], q[3]);
+      o = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+    } else {
+      o = make_uint2(gemm::pack_bf16(q[0], q[1]), gemm::pack_bf16(q[2], q[3]));
+    }
+    *reinterpret_cast<uint2*>(a.tr[p.m] + (size_t)(p.c0 + y) * a.rows[p.m] + p.r0 + x) = o;
+    p = next;
   }
-  *reinterpret_cast<uint2*>(a.tr[m] + (size_t)(c0 + y) * rows + r0 + x) = o;
 }
 
 int nblk(size_t n) {
@@ -734,7 +757,7 @@ cudaError_t codec_train_step(Codec* c, const uint16_t* Y, const float* wts, int 
     l2.n[m] = blen[m];
     l2.bias[m + 1] = l2.bias[m] + (blen[m] + 1023) / 1024;
   }
-  TCK(gemm::launch_dependent(lamb2_multi_kernel, dim3(l2.tiles[4] + l2.bias[4]), dim3(256), 0, st, l2, lr,
+  TCK(gemm::launch_dependent(lamb2_multi_kernel, dim3(std::min(l2.tiles[4] + l2.bias[4], 152 * 6)), dim3(256), 0, st, l2, lr,
                              (const double*)(s->red + 1)));
   return codec_refresh_strain(c, st);
 }
