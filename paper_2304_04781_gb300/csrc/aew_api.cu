@@ -115,7 +115,7 @@ struct aew_handle {
   // exchange buffer with its running tag, and dt s^n of the default and of a given wavelet
   bool brick = false;
   bool two = false;   // larger grids: two steps per pass (aew_twostep.h)
-  int sms = 0;
+  aew::TwoCut cut;
   aew::BrickPlan bp;
   unsigned char* halo = nullptr;
   uint32_t halo_tag = 0;
@@ -499,7 +499,7 @@ void two_pack(aew::TwoFwd& a, int i, const PackAt& p) {
   a.tslot[i] = p.slot;
 }
 int two_fwd(aew_handle* h, const aew::TwoFwd& a, cudaStream_t s) {
-  AEW_CK(aew::launch_two_fwd(a, h->sms, s));
+  AEW_CK(aew::launch_two_fwd(a, h->cut, s));
   ++h->stats.kernel_launches;
   return AEW_OK;
 }
@@ -536,7 +536,7 @@ int two_adj(aew_handle* h, int n, float* const in[4], float* const out[4], const
   for (int i = 0; i < 2; ++i)
     a.resid[i] = (resid && h->nrow) ? resid + (size_t)(n + 1 - i) * h->nrow : nullptr;
   a.err = aew::codec_err_flag(h->codec);
-  AEW_CK(aew::launch_two_adj(a, h->sms, s));
+  AEW_CK(aew::launch_two_adj(a, h->cut, s));
   ++h->stats.kernel_launches;
   return AEW_OK;
 }
@@ -1637,10 +1637,10 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
     h->brick = coop && aew::brick_plan(c.nx, c.ny, c.nz, sms, &h->bp);
-    // faster than single steps on every larger grid: 160^3 20 us a step against 34, 256^3 69
-    // against 95, 512 x 512 x 256 302 against 350
+    // faster than single steps on every larger grid: 160^3 18 us a step against 34, 256^3 57
+    // against 95, 512 x 512 x 256 276 against 350
     h->two = !h->brick;
-    h->sms = sms;
+    h->cut = aew::two_cut(c.nx, c.ny, c.nz, sms > 0 ? sms : 1);
   }
   if (ok && c.storage == AEW_AE) {
     // The codec GEMMs run on a high-priority side stream with half the SMs, so their
@@ -1651,7 +1651,7 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     h->overlap_ctas = sms > 1 ? sms / 2 : 0;
     // two steps per pass: a pass holds every SM for 70-100 us, so the GEMMs take all SMs
-    // between passes (217 us per gradient step at 256^3 against 222 with half of them)
+    // between passes (217 us per gradient step at 256^3, 222 with half of them)
     if (h->two) h->overlap_ctas = 0;
     if (const char* env = getenv("AEW_GEMM_CTAS_OVERLAP")) h->overlap_ctas = atoi(env);   // tuning override
     ok = ok && cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, hi) == cudaSuccess;

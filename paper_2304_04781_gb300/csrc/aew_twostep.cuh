@@ -8,18 +8,18 @@
 // each side of the x tile) take part in the first step only; they are recomputed by the
 // neighbouring CTA, by the identical expressions, so results are bitwise those of two
 // single steps.  z chunks overlap by two planes the same way.
-//   256^3, us per step: forward 95 -> 69 (44 for its bytes at the copy rate), forward and
-//   adjoint with the whole history 225 -> 167, with the time codec 274 -> 217; 160^3 34 -> 20
-//   forward; 512 x 512 x 256 350 -> 302.  What is left is latency: with one CTA per SM one
-//   plane of loads (about 40 KB) is in flight.
+//   256^3, us per step: forward 95 -> 57 (44 for its bytes at the copy rate), forward and
+//   adjoint with the whole history 225 -> 153, with the time codec 274 -> 214; 160^3 34 -> 18
+//   forward; 512 x 512 x 256 350 -> 276.
 //
 // Layout.  Thread (j, q) owns four nodes of row j.  The state of the two planes in flight is
 // in its registers (the next plane's loads too); y neighbours go through four plane buffers
 // in shared memory, x neighbours by shuffle, z neighbours are the thread's own.  Per plane:
 //   A  faces of plane k (step 1) and x-, y-faces of plane k - 1 (step 2)
 //   B  nodes of plane k (step 1), z-faces and nodes of plane k - 1 (step 2), stores
-// with a barrier after each.  The rows beyond the column (one m e row, and one y-face row
-// below) come by cp.async into a small ring, so that they cost no registers.
+// with a barrier after each (forward_kernel: one barrier per plane).  The rows beyond the
+// column (one m e row, and one y-face row below) come by cp.async into a small ring, so that
+// they cost no registers.
 #pragma once
 
 #include "aew_stencil.cuh"
@@ -33,12 +33,12 @@ using namespace quad;
 constexpr int kThreads = 512;
 constexpr int kMaxTileQ = 64;   // float4 per x tile
 constexpr int kRing = 4;        // extra rows: planes in the cp.async ring
+// forward_kernel: planes of the threads' own nodes in their ring: e and m, which are first used
+// one plane early, and the faces; two iterations of loads are in flight
+constexpr int kEarly = 4, kLate = 3;
+constexpr int kOwnRing = 2 * kEarly + 3 * kLate;
 
-// the cut: x tiles of nqt float4 (plus halo columns), columns of `rows` thread rows (rows - 2
-// of their own), z chunks of kc planes
-struct Cut {
-  int nq, nqt, ntx, W, rows, nty, kc, ntz;
-};
+using Cut = TwoCut;
 
 __device__ __forceinline__ void cp16(float4* dst, const float* src, bool ok) {
   const uint32_t d = tc::smem_u32(dst);
@@ -131,7 +131,221 @@ __device__ __forceinline__ void fold_table(unsigned* table, unsigned* vmax, cons
   atomicMax(vmax + ((size_t)(k >> 1) * (ny >> 3) + yb) * (nx >> 3) + xb, m);
 }
 
-// INCR 0: forward; 1: + G(dm e) with FP32 e; 2: with BF16 e.  TP: window packing.
+// Forward steps.  One barrier per plane: a thread computes the faces below and left of its nodes
+// itself, from the neighbours' old faces in their ring slots (step 1) or their faces after step 1
+// (step 2), by the expressions of the thread that owns them.
+//   me: m e of the plane, rows -1 .. R; me1, vy1: after step 1, rows 0 .. R - 1; all in two
+//   buffers by the plane's parity.
+template <bool TP>
+__global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_constant__ TwoFwd a,
+                                                              const __grid_constant__ Cut cut) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (sticky_error(a.err)) return;
+  const Place p(cut, a.ny, a.nz);
+  const int W = cut.W, R = cut.rows, tid = threadIdx.x, warp = tid >> 5, N = kThreads + 2 * W;
+  float4* const ring = reinterpret_cast<float4*>(smem) + tid;   // [kOwnRing][kThreads]
+  float4* const me_s = reinterpret_cast<float4*>(smem) + kOwnRing * kThreads + tid;   // [2][N]: row j - 1
+  float4* const me1_s = me_s + 2 * N;
+  float4* const vy1_s = me1_s + 2 * N;
+  float4* const ex = vy1_s - tid + 2 * N;      // [kRing][3][W] e, m, vy of the row below ..
+  float4* const eh = ex + kRing * 3 * W;       // [kRing][2][W] e, m of the row above
+  float* const sx = reinterpret_cast<float*>(eh + kRing * 2 * W);   // [2][warps]: lane 31's last x-face
+  unsigned* const table = reinterpret_cast<unsigned*>(sx + 2 * (kThreads / 32));   // [2][kTable]
+  if (TP && tid < 2 * kTable) table[tid] = 0;
+  const F4 dth = f4(make_float4(a.dth, a.dth, a.dth, a.dth));
+  const size_t P = (size_t)a.nx * a.ny;
+  const size_t i0 = p.valid ? (size_t)p.y * a.nx + p.i0 : 0;
+  const int nz = a.nz;
+  const bool live_q = p.gq >= 0 && p.gq < cut.nq;
+  // rare work: the columns meet the source box; the quad has receivers
+  const bool src = a.sk >= 0 && p.valid && abs(p.y - a.sj) <= a.sr && p.i0 + 3 >= a.si - a.sr &&
+                   p.i0 <= a.si + a.sr;
+  const int krec = p.inner && a.krec >= p.kb && a.krec < p.ke && (a.d[0] || a.d[1]) &&
+                           has_rec(a.rec_map + i0)
+                       ? a.krec
+                       : -1;
+
+  auto ok = [&](int k) { return p.valid && k >= 0 && k < nz; };
+  auto em_at = [&](int k) { return ring + (size_t)((k & (kEarly - 1)) * 2) * kThreads; };
+  auto v_at = [&](int k) { return ring + (size_t)(2 * kEarly + k % kLate * 3) * kThreads; };
+  auto issue_em = [&](int k) {
+    const bool v = ok(k) && k <= p.ke + 1;
+    const size_t i = v ? i0 + (size_t)k * P : 0;
+    cp16(em_at(k), a.e + i, v);
+    cp16(em_at(k) + kThreads, a.m + i, v);
+  };
+  auto issue_v = [&](int k) {
+    const bool v = ok(k) && k <= p.ke;
+    const size_t i = v ? i0 + (size_t)k * P : 0;
+    cp16(v_at(k), a.vx + i, v);
+    cp16(v_at(k) + kThreads, a.vy + i, v);
+    cp16(v_at(k) + 2 * kThreads, a.vz + i, v);
+  };
+  // the extra rows of plane k into slot k % kRing, and the end of the plane's group
+  auto ex_at = [&](int k) { return (p.bot ? ex + k % kRing * 3 * W : eh + k % kRing * 2 * W) + p.q; };
+  auto issue_extra = [&](int k) {
+    if (p.bot || p.top) {
+      const int ye = p.bot ? p.y - 1 : p.y + 1;
+      const bool v = k <= p.ke + 1 && live_q && ye >= 0 && ye < a.ny && k < nz;
+      const size_t i = v ? (size_t)ye * a.nx + p.i0 + (size_t)k * P : 0;
+      cp16(ex_at(k), a.e + i, v);
+      cp16(ex_at(k) + W, a.m + i, v);
+      if (p.bot) cp16(ex_at(k) + 2 * W, a.vy + i, v);
+    }
+    cp_commit();
+  };
+  // m e of the own row and the extra ones into plane k's buffer
+  auto put_me = [&](int k, F4 me) {
+    float4* const d = me_s + (k & 1) * N;
+    if (p.j < R) d[W] = v4(me);
+    if (p.bot) d[0] = v4(mul_rn(ex_at(k)[W], ex_at(k)[0]));
+    if (p.top) d[2 * W] = v4(mul_rn(ex_at(k)[W], ex_at(k)[0]));
+  };
+
+  const int k0 = max(p.kb - 1, 0);
+  issue_em(k0);
+  issue_em(k0 + 1);
+  issue_v(k0);
+  issue_extra(k0);
+  issue_em(k0 + 2);
+  issue_v(k0 + 1);
+  issue_extra(k0 + 1);
+  F4 vzl1 = f4(z4());   // z-face below plane k0 after step 1
+  float4 eb = z4(), mb = z4(), vb = z4();
+  if (k0 >= 1) {
+    const size_t i = i0 + (size_t)(k0 - 1) * P;
+    eb = ldz(a.e + i, p.valid);
+    mb = ldz(a.m + i, p.valid);
+    vb = ldz(a.vz + i, p.valid);
+  }
+  cp_wait<1>();
+  F4 e_c = lds(em_at(k0)), me_c = mul(lds(em_at(k0) + kThreads), e_c);
+  if (k0 >= 1) {
+    vzl1 = fma(dth, sub(me_c, mul_rn(mb, eb)), f4(vb));
+    if (src && abs(k0 - 1 - a.sk) <= a.sr) {
+      float4 v = v4(vzl1);
+      add_source(v, k0 - 1, p.y, p.i0, a, a.dts[0]);
+      vzl1 = f4(v);
+    }
+  }
+  put_me(k0, me_c);
+  __syncthreads();
+
+  F4 vx1p = f4(z4()), vy1p = vx1p, vz1p = vzl1, e1p = vx1p, me1p = vx1p, vz2p = vx1p;
+  Pack pk1{0.f, 0}, pk2{0.f, 0};
+  if (TP && p.inner) {
+    const int by = blockIdx.x / cut.ntx % cut.nty, bx = blockIdx.x % cut.ntx, vx = cut.nqt >> 1;
+    pk1.cell = pk2.cell = ((p.y >> 3) - (by * (R - 2) >> 3)) * vx + (p.gq >> 1) - bx * vx;
+  }
+
+  for (int k = k0; k <= p.ke; ++k) {
+    const int cur = (k & 1) * N, old = N - cur;
+    // ---- loads of the planes ahead, into the slots of plane k - 1
+    issue_em(k + 3);
+    issue_v(k + 2);
+    issue_extra(k + 2);
+    const F4 e_n = lds(em_at(k + 1)), me_n = mul(lds(em_at(k + 1) + kThreads), e_n);
+    if (TP && k > k0) {   // the pairs of planes that the last iteration ended
+      if (a.tpack[0] && !(k & 1) && k - 1 >= p.kb) fold_table(table, a.vmax[0], cut, a.nx, a.ny, k - 1);
+      if (a.tpack[1] && (k & 1) && k - 2 >= p.kb) fold_table(table + kTable, a.vmax[1], cut, a.nx, a.ny, k - 2);
+    }
+    // ---- step 1 of plane k
+    F4 vx1, vy1, vz1, e1, me1;
+    {
+      const float4* const me = me_s + cur;
+      const float4* const v = v_at(k);
+      const float4 m = v4(me_c);
+      float mx1 = __shfl_down_sync(0xffffffffu, m.x, 1);
+      if (p.p31) mx1 = me[W + 1].x;
+      float4 x = v4(fma(dth, f4(make_float4(__fsub_rn(m.y, m.x), __fsub_rn(m.z, m.y), __fsub_rn(m.w, m.z),
+                                            __fsub_rn(mx1, m.w))),
+                        lds(v)));
+      if (p.last_x) x.w = 0.f;
+      vx1 = f4(x);
+      float vxl = __shfl_up_sync(0xffffffffu, x.w, 1);
+      if (p.p0) vxl = __fmaf_rn(a.dth, __fsub_rn(m.x, me[W - 1].w), v[-1].w);
+      if (p.first_x) vxl = 0.f;
+      vy1 = fma(dth, sub(lds(me + 2 * W), me_c), lds(v + kThreads));
+      if (p.last_y) vy1 = f4(z4());
+      const F4 vyl = fma(dth, sub(me_c, lds(me)), lds(p.bot ? ex_at(k) + 2 * W : v + kThreads - W));
+      vz1 = fma(dth, sub(me_n, me_c), lds(v + 2 * kThreads));
+      if (k >= nz - 1) vz1 = f4(z4());
+      if (src && abs(k - a.sk) <= a.sr) {
+        float4 z = v4(vz1);
+        add_source(z, k, p.y, p.i0, a, a.dts[0]);
+        vz1 = f4(z);
+      }
+      const F4 dx = f4(make_float4(x.x - vxl, x.y - x.x, x.z - x.y, x.w - x.z));
+      const F4 s = add(add(dx, sub(vy1, vyl)), sub(vz1, vz1p));
+      e1 = bounded(fma(dth, s, e_c), p, k == 0 || k >= nz - 1);
+      me1 = mul(lds(em_at(k) + kThreads), e1);
+      if ((tid & 31) == 31) sx[(k & 1) * (kThreads / 32) + warp] = x.w;
+    }
+    if (p.inner && k >= p.kb && k < p.ke) {
+      if (a.e1) st4(a.e1, i0 + (size_t)k * P, v4(e1));
+      if (k == krec && a.d[0]) record(a.rec_map + i0, a.d[0], v4(vx1), v4(vy1), v4(vz1));
+    }
+    if (TP && a.tpack[0] && k >= p.kb && k < p.ke)
+      pk1.plane(e1, table, a.tpack[0], a.tslot[0], a.nx, a.ny, k, p);
+    // ---- step 2 of plane k - 1
+    F4 vz2 = fma(dth, sub(me1, me1p), vz1p);
+    if (k - 1 >= nz - 1) vz2 = f4(z4());
+    if (src && abs(k - 1 - a.sk) <= a.sr && k > k0) {
+      float4 z = v4(vz2);
+      add_source(z, k - 1, p.y, p.i0, a, a.dts[1]);
+      vz2 = f4(z);
+    }
+    if (k - 1 >= p.kb && k > k0) {
+      const float4* const me = me1_s + old;
+      const float4 m = v4(me1p);
+      float mx1 = __shfl_down_sync(0xffffffffu, m.x, 1);
+      if (p.p31) mx1 = me[W + 1].x;
+      float4 x = v4(fma(dth, f4(make_float4(__fsub_rn(m.y, m.x), __fsub_rn(m.z, m.y), __fsub_rn(m.w, m.z),
+                                            __fsub_rn(mx1, m.w))),
+                        vx1p));
+      if (p.last_x) x.w = 0.f;
+      float vxl = __shfl_up_sync(0xffffffffu, x.w, 1);
+      if (p.p0)
+        vxl = __fmaf_rn(a.dth, __fsub_rn(m.x, me[W - 1].w), sx[((k - 1) & 1) * (kThreads / 32) + warp - 1]);
+      if (p.first_x) vxl = 0.f;
+      F4 vy2 = fma(dth, sub(lds(me + 2 * W), me1p), vy1p);
+      if (p.last_y) vy2 = f4(z4());
+      const F4 vyl = fma(dth, sub(me1p, lds(me)), lds(vy1_s + old));
+      const F4 dx = f4(make_float4(x.x - vxl, x.y - x.x, x.z - x.y, x.w - x.z));
+      const F4 s = add(add(dx, sub(vy2, vyl)), sub(vz2, vz2p));
+      const F4 e2 = bounded(fma(dth, s, e1p), p, k - 1 == 0 || k - 1 >= nz - 1);
+      const size_t i = i0 + (size_t)(k - 1) * P;
+      if (p.inner) {
+        st4(a.e2, i, v4(e2));
+        st4(a.vx2, i, x);
+        st4(a.vy2, i, v4(vy2));
+        st4(a.vz2, i, v4(vz2));
+        if (k - 1 == krec && a.d[1]) record(a.rec_map + i0, a.d[1], x, v4(vy2), v4(vz2));
+      }
+      if (TP && a.tpack[1]) pk2.plane(e2, table + kTable, a.tpack[1], a.tslot[1], a.nx, a.ny, k - 1, p);
+    }
+    // ---- the next plane
+    me1_s[cur + W] = v4(me1);
+    vy1_s[cur + W] = v4(vy1);
+    cp_wait<1>();   // what the last iteration asked for
+    put_me(k + 1, me_n);
+    vz2p = vz2;
+    vx1p = vx1;
+    vy1p = vy1;
+    vz1p = vz1;
+    e1p = e1;
+    me1p = me1;
+    me_c = me_n;
+    e_c = e_n;
+    __syncthreads();
+  }
+  if (TP) {   // the last pairs: planes ke - 1 of step 1 (ended one iteration ago) and of step 2
+    if (a.tpack[0] && p.ke - 1 >= k0 && (p.ke & 1)) fold_table(table, a.vmax[0], cut, a.nx, a.ny, p.ke - 1);
+    if (a.tpack[1]) fold_table(table + kTable, a.vmax[1], cut, a.nx, a.ny, p.ke - 1);
+  }
+}
+
+// Incremental steps: + G(dm e) with FP32 (INCR 1) or BF16 e (2).  TP: window packing.
 template <int INCR, bool TP>
 __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant__ TwoFwd a,
                                                           const __grid_constant__ Cut cut) {

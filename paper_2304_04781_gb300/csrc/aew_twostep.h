@@ -10,6 +10,13 @@
 
 namespace aew {
 
+// how a grid is cut: x tiles of nqt float4 (W with the halo columns), columns of `rows` thread
+// rows (rows - 2 of their own), z chunks of kc planes
+struct TwoCut {
+  int nq, nqt, ntx, W, rows, nty, kc, ntz;
+};
+TwoCut two_cut(int nx, int ny, int nz, int sms);
+
 // steps n and n + 1 of a forward-type solve: state n -> state n + 2
 struct TwoFwd {
   const float* m;
@@ -67,7 +74,7 @@ struct TwoAdj {
   int* err;
 };
 
-cudaError_t launch_two_fwd(const TwoFwd& a, int sms, cudaStream_t s);
-cudaError_t launch_two_adj(const TwoAdj& a, int sms, cudaStream_t s);
+cudaError_t launch_two_fwd(const TwoFwd& a, const TwoCut& cut, cudaStream_t s);
+cudaError_t launch_two_adj(const TwoAdj& a, const TwoCut& cut, cudaStream_t s);
 
 }  // namespace aew
