@@ -74,8 +74,10 @@ cudaError_t launch_two_adj(const TwoAdj& a, const TwoCut& cut, cudaStream_t s) {
   if (!a.err || (a.en[0] && a.en16[0]) || (a.en[1] && a.en16[1])) return cudaErrorInvalidValue;
   const bool close = a.close[0] || a.close[1];
   if (a.en16[0] || a.en16[1])
-    return close ? go<two::adj_kernel<true, true>>(a, cut, 0, 4, 3, s) : go<two::adj_kernel<true, false>>(a, cut, 0, 4, 3, s);
-  return close ? go<two::adj_kernel<false, true>>(a, cut, 0, 4, 3, s) : go<two::adj_kernel<false, false>>(a, cut, 0, 4, 3, s);
+    return close ? go<two::adjoint_kernel<true, true>>(a, cut, two::kAdjRing, 6, 3, s)
+                 : go<two::adjoint_kernel<true, false>>(a, cut, two::kAdjRing, 6, 3, s);
+  return close ? go<two::adjoint_kernel<false, true>>(a, cut, two::kAdjRing, 6, 3, s)
+               : go<two::adjoint_kernel<false, false>>(a, cut, two::kAdjRing, 6, 3, s);
 }
 
 }  // namespace aew

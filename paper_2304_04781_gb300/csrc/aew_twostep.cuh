@@ -9,7 +9,7 @@
 // neighbouring CTA, by the identical expressions, so results are bitwise those of two
 // single steps.  z chunks overlap by two planes the same way.
 //   256^3, us per step: forward 95 -> 57 (44 for its bytes at the copy rate), forward and
-//   adjoint with the whole history 225 -> 153, with the time codec 274 -> 214; 160^3 34 -> 18
+//   adjoint with the whole history 225 -> 148, with the time codec 274 -> 213; 160^3 34 -> 18
 //   forward; 512 x 512 x 256 350 -> 276.
 //
 // Layout.  Thread (j, q) owns four nodes of row j.  The state of the two planes in flight is
@@ -17,7 +17,7 @@
 // in shared memory, x neighbours by shuffle, z neighbours are the thread's own.  Per plane:
 //   A  faces of plane k (step 1) and x-, y-faces of plane k - 1 (step 2)
 //   B  nodes of plane k (step 1), z-faces and nodes of plane k - 1 (step 2), stores
-// with a barrier after each (forward_kernel: one barrier per plane).  The rows beyond the
+// with a barrier after each (forward_kernel and adjoint_kernel: one per plane).  The rows beyond the
 // column (one m e row, and one y-face row below) come by cp.async into a small ring, so that
 // they cost no registers.
 #pragma once
@@ -37,6 +37,7 @@ constexpr int kRing = 4;        // extra rows: planes in the cp.async ring
 // one plane early, and the faces; two iterations of loads are in flight
 constexpr int kEarly = 4, kLate = 3;
 constexpr int kOwnRing = 2 * kEarly + 3 * kLate;
+constexpr int kAdjRing = kEarly + 2 * kLate;   // mu, and lx and ly
 
 using Cut = TwoCut;
 
@@ -616,47 +617,70 @@ __device__ __forceinline__ F4 injected(F4 f, const int* rec_map, const float* r)
   return f4(l);
 }
 
-// Two adjoint steps with gradient accumulation.  B16: the strain is BF16.  CLOSE: a window
-// ends with one of the steps (FP64 instructions slow the loop even where they are skipped:
-// 238 us instead of 140 at 256^3, so the other launches are built without them).
+// Two adjoint steps with gradient accumulation, one barrier per plane as in forward_kernel.
+// B16: the strain is BF16.  CLOSE: a window ends with one of the steps (FP64 instructions slow
+// the loop even where they are skipped: 238 us instead of 140 at 256^3, so the other launches
+// are built without them).  mu, lx and ly, which neighbours read, come through the ring; the
+// fields that only their own thread uses stay in registers, one plane ahead (through the ring
+// too the pass was 15% slower).  Full gradient at 256^3: 153 us per step with two barriers, 148.5
+// now; 52 B per node and pass bound it from 128 us a pass, issue slots at about 175.
 template <bool B16, bool CLOSE>
-__global__ void __launch_bounds__(kThreads, 1) adj_kernel(const __grid_constant__ TwoAdj a,
-                                                          const __grid_constant__ Cut cut) {
+__global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(const __grid_constant__ TwoAdj a,
+                                                              const __grid_constant__ Cut cut) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (sticky_error(a.err)) return;
   const Place p(cut, a.ny, a.nz);
-  const int W = cut.W, R = cut.rows, tid = threadIdx.x, warp = tid >> 5;
-  float4* const sa = reinterpret_cast<float4*>(smem);   // mu [R + 1]
-  float4* const sb = sa + kThreads + 2 * W;             // ly1 [1 + R]
-  float4* const sc = sb + kThreads + 2 * W;             // mu1 [R]
-  float4* const sd = sc + kThreads + 2 * W;             // ly2 [1 + R]
-  float4* const ex = sd + kThreads + 2 * W;             // [kRing][2][W] mu, ly of the row below
-  float4* const eh = ex + kRing * 2 * W;                // [kRing][W] mu of the row above
-  float* const sx1 = reinterpret_cast<float*>(eh + kRing * W);
-  float* const sx2 = sx1 + kThreads / 32;
+  const int W = cut.W, R = cut.rows, tid = threadIdx.x, warp = tid >> 5, N = kThreads + 2 * W;
+  float4* const ring = reinterpret_cast<float4*>(smem) + tid;   // [kAdjRing][kThreads]
+  float4* const mu_s = reinterpret_cast<float4*>(smem) + kAdjRing * kThreads + tid;   // [2][N]: row j - 1
+  float4* const mu1_s = mu_s + 2 * N;
+  float4* const ly1_s = mu1_s + 2 * N;
+  float4* const ex = ly1_s - tid + 2 * N;      // [kRing][2][W] mu, ly of the row below ..
+  float4* const eh = ex + kRing * 2 * W;       // [kRing][W] mu of the row above
+  float* const sx = reinterpret_cast<float*>(eh + kRing * W);   // [2][warps]: lane 31's last x-face
   const F4 dth = f4(make_float4(a.dth, a.dth, a.dth, a.dth));
   const F4 ndth = f4(make_float4(-a.dth, -a.dth, -a.dth, -a.dth));
   const size_t P = (size_t)a.nx * a.ny;
   const size_t i0 = p.valid ? (size_t)p.y * a.nx + p.i0 : 0;
   const int nz = a.nz;
   const bool live_q = p.gq >= 0 && p.gq < cut.nq;
+  // receivers on the own nodes, on those of the row below, on the node left of them
   const int* const map = a.rec_map + i0;
-  const bool rz = a.krec >= 0 && (a.resid[0] || a.resid[1]) && a.krec >= p.kb - 2 && a.krec <= p.ke;
-  const bool rec = rz && p.valid && has_rec(map);
-  const bool rec_low = rz && p.bot && live_q && p.y - 1 >= 0 && has_rec(a.rec_map + (size_t)(p.y - 1) * a.nx + p.i0);
+  const bool rz = p.valid && a.krec >= 0 && (a.resid[0] || a.resid[1]) && a.krec >= p.kb - 2 && a.krec <= p.ke;
+  const bool rec = rz && has_rec(map), rec_y = rz && p.y > 0 && has_rec(map - a.nx);
+  const int rec_x = rz && p.p0 && p.gq > 0 ? __ldg(map - 1) : -1;
   const bool open = a.open, close1 = CLOSE && a.close[0], close2 = CLOSE && a.close[1];
 
   auto ok = [&](int k) { return p.valid && k >= 0 && k < nz; };
-  auto issue_extra = [&](int k, bool want) {
+  auto mu_at = [&](int k) { return ring + (size_t)(k & (kEarly - 1)) * kThreads; };
+  auto l_at = [&](int k) { return ring + (size_t)(kEarly + k % kLate * 2) * kThreads; };
+  auto issue_mu = [&](int k) {
+    const bool v = ok(k) && k <= p.ke + 1;
+    cp16(mu_at(k), a.mu + (v ? i0 + (size_t)k * P : 0), v);
+  };
+  auto issue_l = [&](int k) {
+    const bool v = ok(k) && k <= p.ke;
+    const size_t i = v ? i0 + (size_t)k * P : 0;
+    cp16(l_at(k), a.lx + i, v);
+    cp16(l_at(k) + kThreads, a.ly + i, v);
+  };
+  // the extra rows of plane k into slot k % kRing, and the end of the plane's group
+  auto ex_at = [&](int k) { return (p.bot ? ex + k % kRing * 2 * W : eh + k % kRing * W) + p.q; };
+  auto issue_extra = [&](int k) {
     if (p.bot || p.top) {
       const int ye = p.bot ? p.y - 1 : p.y + 1;
-      const bool v = want && live_q && p.j < R && ye >= 0 && ye < a.ny && k >= 0 && k < nz;
+      const bool v = k <= p.ke + 1 && live_q && ye >= 0 && ye < a.ny && k < nz;
       const size_t i = v ? (size_t)ye * a.nx + p.i0 + (size_t)k * P : 0;
-      const int s = k % kRing;
-      cp16((p.bot ? ex + s * 2 * W : eh + s * W) + p.q, a.mu + i, v);
-      if (p.bot) cp16(ex + (s * 2 + 1) * W + p.q, a.ly + i, v);
+      cp16(ex_at(k), a.mu + i, v);
+      if (p.bot) cp16(ex_at(k) + W, a.ly + i, v);
     }
     cp_commit();
+  };
+  auto put_mu = [&](int k, F4 mu) {
+    float4* const d = mu_s + (k & 1) * N;
+    if (p.j < R) d[W] = v4(mu);
+    if (p.bot) d[0] = ex_at(k)[0];
+    if (p.top) d[2 * W] = ex_at(k)[0];
   };
   // strain of step s in plane k (own nodes)
   struct Strain {
@@ -675,6 +699,11 @@ __global__ void __launch_bounds__(kThreads, 1) adj_kernel(const __grid_constant_
     }
     return e;
   };
+  auto load_w = [&](int k) {
+    return !open && p.inner && k >= p.kb && k < p.ke
+               ? *reinterpret_cast<const float4*>(a.acc32 + (i0 + (size_t)k * P))
+               : z4();
+  };
   auto flush = [&](size_t i, F4 f) {
     const float4 v = v4(f);
     double2* p64 = reinterpret_cast<double2*>(a.acc64 + i);
@@ -689,133 +718,131 @@ __global__ void __launch_bounds__(kThreads, 1) adj_kernel(const __grid_constant_
   auto val = [&](const Strain& e) { return f4(B16 ? bf4(e.f16) : e.f32); };
 
   const int k0 = max(p.kb - 1, 0);
-  F4 mu_c = f4(ldz(a.mu + (i0 + (size_t)k0 * P), ok(k0)));
-  F4 lzl1 = f4(z4());   // z-face below plane k0 after the first step
+  issue_mu(k0);
+  issue_mu(k0 + 1);
+  issue_l(k0);
+  issue_extra(k0);
+  issue_mu(k0 + 2);
+  issue_l(k0 + 1);
+  issue_extra(k0 + 1);
+  float4 mub = z4(), lzb = z4();
   if (k0 >= 1) {
     const size_t i = i0 + (size_t)(k0 - 1) * P;
-    F4 l = f4(ldz(a.lz + i, ok(k0 - 1)));
-    if (rec && a.krec == k0 - 1 && a.resid[0]) l = injected(l, map, a.resid[0] + 2);
-    lzl1 = fma(dth, sub(f4(ldz(a.mu + i, ok(k0 - 1))), mu_c), l);
+    mub = ldz(a.mu + i, p.valid);
+    lzb = ldz(a.lz + i, p.valid);
   }
-  float4 mur = ldz(a.mu + (i0 + (size_t)(k0 + 1) * P), ok(k0 + 1));
   const size_t ik = i0 + (size_t)k0 * P;
-  float4 lxr = ldz(a.lx + ik, ok(k0)), lyr = ldz(a.ly + ik, ok(k0)), lzr = ldz(a.lz + ik, ok(k0)),
-         mr = ldz(a.m + ik, ok(k0));
+  float4 lzr = ldz(a.lz + ik, ok(k0)), mr = ldz(a.m + ik, ok(k0));
   Strain e1r = load_en(0, k0), e2r = load_en(1, k0);
-  auto load_w = [&](int k) {
-    return !open && p.inner && k >= p.kb && k < p.ke
-               ? *reinterpret_cast<const float4*>(a.acc32 + (i0 + (size_t)k * P))
-               : z4();
-  };
   float4 wr = load_w(k0);
-  issue_extra(k0, true);
-  issue_extra(k0 + 1, true);
   cp_wait<1>();
-  const int at = tid;
-  if (p.j < R) sa[at] = v4(mu_c);
-  if (p.top && p.j < R) sa[R * W + p.q] = eh[(k0 % kRing) * W + p.q];
+  F4 mu_c = lds(mu_at(k0));
+  F4 lzl1 = f4(z4());   // z-face below plane k0 after the first step
+  if (k0 >= 1) {
+    F4 l = f4(lzb);
+    if (rec && a.krec == k0 - 1 && a.resid[0]) l = injected(l, map, a.resid[0] + 2);
+    lzl1 = fma(dth, sub(f4(mub), mu_c), l);
+  }
+  put_mu(k0, mu_c);
   __syncthreads();
 
   F4 lx1p = f4(z4()), ly1p = lx1p, lz1p = lzl1, mu1p = lx1p, lz2p = lx1p, mp = lx1p, gp = lx1p;
   Strain e2p{z4(), make_uint2(0u, 0u)};
 
   for (int k = k0; k <= p.ke; ++k) {
-    const F4 mu_n = f4(mur);
+    const int cur = (k & 1) * N, old = N - cur;
+    // ---- loads of the planes ahead, into the slots of plane k - 1
+    issue_mu(k + 3);
+    issue_l(k + 2);
+    issue_extra(k + 2);
+    const F4 mu_n = lds(mu_at(k + 1));
     const F4 m_c = f4(mr), w_c = f4(wr);
     const Strain e1c = e1r, e2c = e2r;
-    F4 lx1 = f4(lxr), ly1 = f4(lyr), lz1 = f4(lzr);
-    // ---- loads of the planes ahead
-    mur = ldz(a.mu + (i0 + (size_t)(k + 2) * P), ok(k + 2) && k + 2 <= p.ke + 1);
-    const bool vv = ok(k + 1) && k + 1 <= p.ke;
-    const size_t in = i0 + (size_t)(k + 1) * P;
-    lxr = ldz(a.lx + in, vv);
-    lyr = ldz(a.ly + in, vv);
-    lzr = ldz(a.lz + in, vv);
-    mr = ldz(a.m + in, vv);
-    e1r = load_en(0, k + 1);
-    e2r = load_en(1, k + 1);
-    wr = load_w(k + 1);
-    issue_extra(k + 2, k + 2 <= p.ke + 1);
-    // ---- A: faces of plane k after the first step
+    F4 lz1 = f4(lzr);
     {
-      if (rec && k == a.krec && a.resid[0]) {
-        lx1 = injected(lx1, map, a.resid[0]);
-        ly1 = injected(ly1, map, a.resid[0] + 1);
-        lz1 = injected(lz1, map, a.resid[0] + 2);
+      const bool vv = ok(k + 1) && k + 1 <= p.ke;
+      const size_t in = i0 + (size_t)(k + 1) * P;
+      lzr = ldz(a.lz + in, vv);
+      mr = ldz(a.m + in, vv);
+      e1r = load_en(0, k + 1);
+      e2r = load_en(1, k + 1);
+      wr = load_w(k + 1);
+    }
+    // ---- the first step of plane k
+    F4 lx1, ly1, mu1, g;
+    {
+      const float4* const me = mu_s + cur;
+      const float4* const l = l_at(k);
+      lx1 = lds(l);
+      ly1 = lds(l + kThreads);
+      F4 lyl = lds(p.bot ? ex_at(k) + W : l + kThreads - W);
+      float lxl_old = p.p0 ? l[-1].w : 0.f;
+      if (k == a.krec && a.resid[0]) {
+        if (rec) {
+          lx1 = injected(lx1, map, a.resid[0]);
+          ly1 = injected(ly1, map, a.resid[0] + 1);
+          lz1 = injected(lz1, map, a.resid[0] + 2);
+        }
+        if (rec_y) lyl = injected(lyl, map - a.nx, a.resid[0] + 1);
+        if (rec_x >= 0) lxl_old += __ldg(a.resid[0] + 3 * rec_x);
       }
-      const F4 mu_yp = lds(sa + at + W);
       const float4 m = v4(mu_c);
       float mx1 = __shfl_down_sync(0xffffffffu, m.x, 1);
-      if (p.p31) mx1 = sa[at + 1].x;
+      if (p.p31) mx1 = me[W + 1].x;
       float4 x = v4(fma(dth, f4(make_float4(m.x - m.y, m.y - m.z, m.z - m.w, m.w - mx1)), lx1));
       if (p.last_x) x.w = 0.f;
       lx1 = f4(x);
-      if ((tid & 31) == 31) sx1[warp] = x.w;
-      ly1 = fma(dth, sub(mu_c, mu_yp), ly1);
+      float lxl = __shfl_up_sync(0xffffffffu, x.w, 1);
+      if (p.p0) lxl = __fmaf_rn(a.dth, __fsub_rn(me[W - 1].w, m.x), lxl_old);
+      if (p.first_x) lxl = 0.f;
+      ly1 = fma(dth, sub(mu_c, lds(me + 2 * W)), ly1);
       if (p.last_y) ly1 = f4(z4());
+      lyl = fma(dth, sub(lds(me), mu_c), lyl);
       lz1 = fma(dth, sub(mu_c, mu_n), lz1);
       if (k >= nz - 1) lz1 = f4(z4());
-      sts(sb + at + W, ly1);
-      if (p.bot) {   // the y-face below the column, as its owner computes it
-        const float4* d = ex + (k % kRing) * 2 * W + p.q;
-        F4 l = lds(d + W);
-        if (rec_low && k == a.krec && a.resid[0])
-          l = injected(l, a.rec_map + (size_t)(p.y - 1) * a.nx + p.i0, a.resid[0] + 1);
-        sts(sb + p.q, fma(dth, sub(lds(d), mu_c), l));
-      }
-    }
-    // ---- A: x- and y-faces of plane k - 1 after the second step
-    F4 lx2 = lx1p, ly2 = ly1p;
-    {
-      if (rec && k - 1 == a.krec && k > k0 && a.resid[1]) {
-        lx2 = injected(lx2, map, a.resid[1]);
-        ly2 = injected(ly2, map, a.resid[1] + 1);
-      }
-      const F4 mu_yp = lds(sc + at + W);
-      const float4 m = v4(mu1p);
-      float mx1 = __shfl_down_sync(0xffffffffu, m.x, 1);
-      if (p.p31) mx1 = sc[at + 1].x;
-      float4 x = v4(fma(dth, f4(make_float4(m.x - m.y, m.y - m.z, m.z - m.w, m.w - mx1)), lx2));
-      if (p.last_x) x.w = 0.f;
-      lx2 = f4(x);
-      if ((tid & 31) == 31) sx2[warp] = x.w;
-      ly2 = fma(dth, sub(mu1p, mu_yp), ly2);
-      if (p.last_y) ly2 = f4(z4());
-      sts(sd + at + W, ly2);
-    }
-    cp_wait<1>();
-    __syncthreads();
-    // ---- B: nodes of plane k after the first step
-    F4 mu1, g;
-    {
-      const float4 x = v4(lx1);
-      float lxl = __shfl_up_sync(0xffffffffu, x.w, 1);
-      if (p.p0) lxl = sx1[warp - 1];
-      if (p.first_x) lxl = 0.f;
       const F4 dx = f4(make_float4(x.x - lxl, x.y - x.x, x.z - x.y, x.w - x.z));
-      const F4 s = add(add(dx, sub(ly1, lds(sb + at))), sub(lz1, lz1p));
+      const F4 s = add(add(dx, sub(ly1, lyl)), sub(lz1, lz1p));
       const F4 dq = bounded(mul(ndth, s), p, k == 0 || k >= nz - 1);
       mu1 = fma(m_c, dq, mu_c);
       g = fma(val(e1c), dq, w_c);
+      if ((tid & 31) == 31) sx[(k & 1) * (kThreads / 32) + warp] = x.w;
     }
-    sts(sc + at, mu1);
-    // ---- B: z-faces and nodes of plane k - 1 after the second step
+    // ---- the second step of plane k - 1
     F4 lz2 = lz1p;
-    if (rec && k - 1 == a.krec && k > k0 && a.resid[1]) lz2 = injected(lz2, map, a.resid[1] + 2);
+    const bool rec2 = k - 1 == a.krec && k > k0 && a.resid[1];
+    if (rec2 && rec) lz2 = injected(lz2, map, a.resid[1] + 2);
     lz2 = fma(dth, sub(mu1p, mu1), lz2);
     if (k - 1 >= nz - 1) lz2 = f4(z4());
-    {
-      const float4 x = v4(lx2);
+    if (k - 1 >= p.kb && k > k0) {
+      const float4* const me = mu1_s + old;
+      F4 lx2 = lx1p, ly2 = ly1p, lyl = lds(ly1_s + old);
+      float lxl_old = p.p0 ? sx[((k - 1) & 1) * (kThreads / 32) + warp - 1] : 0.f;
+      if (rec2) {
+        if (rec) {
+          lx2 = injected(lx2, map, a.resid[1]);
+          ly2 = injected(ly2, map, a.resid[1] + 1);
+        }
+        if (rec_y) lyl = injected(lyl, map - a.nx, a.resid[1] + 1);
+        if (rec_x >= 0) lxl_old += __ldg(a.resid[1] + 3 * rec_x);
+      }
+      const float4 m = v4(mu1p);
+      float mx1 = __shfl_down_sync(0xffffffffu, m.x, 1);
+      if (p.p31) mx1 = me[W + 1].x;
+      float4 x = v4(fma(dth, f4(make_float4(m.x - m.y, m.y - m.z, m.z - m.w, m.w - mx1)), lx2));
+      if (p.last_x) x.w = 0.f;
       float lxl = __shfl_up_sync(0xffffffffu, x.w, 1);
-      if (p.p0) lxl = sx2[warp - 1];
+      if (p.p0) lxl = __fmaf_rn(a.dth, __fsub_rn(me[W - 1].w, m.x), lxl_old);
       if (p.first_x) lxl = 0.f;
+      ly2 = fma(dth, sub(mu1p, lds(me + 2 * W)), ly2);
+      if (p.last_y) ly2 = f4(z4());
+      lyl = fma(dth, sub(lds(me), mu1p), lyl);
       const F4 dx = f4(make_float4(x.x - lxl, x.y - x.x, x.z - x.y, x.w - x.z));
-      const F4 s = add(add(dx, sub(ly2, lds(sd + at))), sub(lz2, lz2p));
+      const F4 s = add(add(dx, sub(ly2, lyl)), sub(lz2, lz2p));
       const F4 dq = bounded(mul(ndth, s), p, k - 1 == 0 || k - 1 >= nz - 1);
-      if (p.inner && k - 1 >= p.kb && k > k0) {
+      if (p.inner) {
         const size_t i = i0 + (size_t)(k - 1) * P;
         st4(a.mu2, i, v4(fma(mp, dq, mu1p)));
-        st4(a.lx2, i, v4(lx2));
+        st4(a.lx2, i, x);
         st4(a.ly2, i, v4(ly2));
         st4(a.lz2, i, v4(lz2));
         // dJ/dm += dt e q of both steps; a window that ends is flushed
@@ -826,8 +853,10 @@ __global__ void __launch_bounds__(kThreads, 1) adj_kernel(const __grid_constant_
       }
     }
     // ---- the next plane
-    if (p.j < R) sa[at] = v4(mu_n);
-    if (p.top && p.j < R) sa[R * W + p.q] = eh[((k + 1) % kRing) * W + p.q];
+    mu1_s[cur + W] = v4(mu1);
+    ly1_s[cur + W] = v4(ly1);
+    cp_wait<1>();   // what the last iteration asked for
+    put_mu(k + 1, mu_n);
     lz2p = lz2;
     lx1p = lx1;
     ly1p = ly1;
