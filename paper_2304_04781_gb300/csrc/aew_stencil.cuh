@@ -85,6 +85,33 @@ __device__ __forceinline__ bool sticky_error(const int* err) {
   return err && *reinterpret_cast<const volatile int*>(err) != 0;
 }
 
+// The same value in FP64, by integer instructions: GB300 converts at its FP64 rate, which made
+// the conversions half of a window's flush into the FP64 sum (a 256^3 two-step adjoint pass
+// that ends a window: 249 -> 216 us; the on-chip loops, short of registers, gain nothing by it
+// and convert by instruction).
+__device__ __forceinline__ double widen(float v) {
+  uint32_t u = __float_as_uint(v);
+  int bias = 1023 - 127;
+  if ((u & 0x7f800000u) == 0) {   // subnormal or zero: exact as 2^64 v
+    u = __float_as_uint(v * 18446744073709551616.f);
+    bias -= 64;
+  }
+  const int e = (int)(u >> 23 & 0xffu);
+  const uint32_t ed = e == 255 ? 2047u : e == 0 ? 0u : (uint32_t)(e + bias);
+  return __hiloint2double((int)((u & 0x80000000u) | ed << 20 | (u & 0x7fffffu) >> 3), (int)(u << 29));
+}
+// acc[0 .. 3] += v
+__device__ __forceinline__ void add_wide(double* acc, float4 v) {
+  double2* p = reinterpret_cast<double2*>(acc);
+  double2 lo = p[0], hi = p[1];
+  lo.x += widen(v.x);
+  lo.y += widen(v.y);
+  hi.x += widen(v.z);
+  hi.y += widen(v.w);
+  p[0] = lo;
+  p[1] = hi;
+}
+
 // ---- four nodes as two pairs ---------------------------------------------------------
 namespace quad {
 // The paired FP32 instructions round each lane as the scalar ones do.

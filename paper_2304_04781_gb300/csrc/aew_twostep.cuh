@@ -9,7 +9,7 @@
 // neighbouring CTA, by the identical expressions, so results are bitwise those of two
 // single steps.  z chunks overlap by two planes the same way.
 //   256^3, us per step: forward 95 -> 57 (44 for its bytes at the copy rate), forward and
-//   adjoint with the whole history 225 -> 148, with the time codec 274 -> 213; 160^3 34 -> 18
+//   adjoint with the whole history 225 -> 144, with the time codec 274 -> 208; 160^3 34 -> 18
 //   forward; 512 x 512 x 256 350 -> 276.
 //
 // Layout.  Thread (j, q) owns four nodes of row j.  The state of the two planes in flight is
@@ -107,19 +107,19 @@ __device__ __forceinline__ float4 ldz16(const uint16_t* p, bool ok) {
 constexpr int kTable = 128;
 struct Pack {
   float m;         // max |e| of the thread's nodes in the current pair of planes
-  int cell;        // the thread's vector in the table
-  __device__ __forceinline__ void plane(F4 f, unsigned* table, uint16_t* tpack, int slot, int nx, int ny, int k,
-                                        const Place& p) {
+  // at: the thread's row of its vector in the pair k / 2, this slot
+  __device__ __forceinline__ void plane(F4 f, unsigned* cell, uint16_t* at, int k) {
     const float4 v = v4(f);
-    const int NBx = nx >> 3, NBy = ny >> 3;
-    const size_t vec = ((size_t)(k >> 1) * NBy + (p.y >> 3)) * NBx + (p.i0 >> 3);
-    if (!p.inner) return;
-    *reinterpret_cast<uint2*>(tpack + vec * 2048 + slot * 128 + (k & 1) * 64 + (p.y & 7) * 8 + (p.i0 & 7)) =
-        make_uint2(pack2bf(v.x, v.y), pack2bf(v.z, v.w));
+    *reinterpret_cast<uint2*>(at + (k & 1) * 64) = make_uint2(pack2bf(v.x, v.y), pack2bf(v.z, v.w));
     m = fmaxf(k & 1 ? m : 0.f, hmax4(v));
-    if ((k & 1) && m > 0.f) atomicMax(table + cell, __float_as_uint(m));
+    if ((k & 1) && m > 0.f) atomicMax(cell, __float_as_uint(m));
   }
 };
+// the place of four nodes of plane 0 in the packed window (slot 0); planes 2 apart are
+// nx * ny / 64 vectors apart
+__device__ __forceinline__ size_t pack_place(int nx, const Place& p) {
+  return ((size_t)(p.y >> 3) * (nx >> 3) + (p.i0 >> 3)) * 2048 + (p.y & 7) * 8 + (p.i0 & 7);
+}
 // after the barrier that ends a pair's last plane: the table of planes k - 1, k into vmax
 __device__ __forceinline__ void fold_table(unsigned* table, unsigned* vmax, const Cut& c, int nx, int ny, int k) {
   const int t = threadIdx.x;
@@ -233,10 +233,12 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
   __syncthreads();
 
   F4 vx1p = f4(z4()), vy1p = vx1p, vz1p = vzl1, e1p = vx1p, me1p = vx1p, vz2p = vx1p;
-  Pack pk1{0.f, 0}, pk2{0.f, 0};
+  Pack pk1{0.f}, pk2{0.f};
+  unsigned* cell = table;
+  const size_t pk0 = TP && p.inner ? pack_place(a.nx, p) : 0, pair = P / 64 * 2048;
   if (TP && p.inner) {
     const int by = blockIdx.x / cut.ntx % cut.nty, bx = blockIdx.x % cut.ntx, vx = cut.nqt >> 1;
-    pk1.cell = pk2.cell = ((p.y >> 3) - (by * (R - 2) >> 3)) * vx + (p.gq >> 1) - bx * vx;
+    cell += ((p.y >> 3) - (by * (R - 2) >> 3)) * vx + (p.gq >> 1) - bx * vx;
   }
 
   for (int k = k0; k <= p.ke; ++k) {
@@ -286,8 +288,8 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
       if (a.e1) st4(a.e1, i0 + (size_t)k * P, v4(e1));
       if (k == krec && a.d[0]) record(a.rec_map + i0, a.d[0], v4(vx1), v4(vy1), v4(vz1));
     }
-    if (TP && a.tpack[0] && k >= p.kb && k < p.ke)
-      pk1.plane(e1, table, a.tpack[0], a.tslot[0], a.nx, a.ny, k, p);
+    if (TP && a.tpack[0] && p.inner && k >= p.kb && k < p.ke)
+      pk1.plane(e1, cell, a.tpack[0] + (k >> 1) * pair + a.tslot[0] * 128 + pk0, k);
     // ---- step 2 of plane k - 1
     F4 vz2 = fma(dth, sub(me1, me1p), vz1p);
     if (k - 1 >= nz - 1) vz2 = f4(z4());
@@ -323,7 +325,8 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
         st4(a.vz2, i, v4(vz2));
         if (k - 1 == krec && a.d[1]) record(a.rec_map + i0, a.d[1], x, v4(vy2), v4(vz2));
       }
-      if (TP && a.tpack[1]) pk2.plane(e2, table + kTable, a.tpack[1], a.tslot[1], a.nx, a.ny, k - 1, p);
+      if (TP && a.tpack[1] && p.inner)
+        pk2.plane(e2, cell + kTable, a.tpack[1] + (k - 1 >> 1) * pair + a.tslot[1] * 128 + pk0, k - 1);
     }
     // ---- the next plane
     me1_s[cur + W] = v4(me1);
@@ -469,10 +472,12 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
   __syncthreads();
 
   F4 vx1p = f4(z4()), vy1p = vx1p, vz1p = vzl1, e1p = vx1p, me1p = vx1p, vz2p = vx1p;
-  Pack pk1{0.f, 0}, pk2{0.f, 0};
+  Pack pk1{0.f}, pk2{0.f};
+  unsigned* cell = table;
+  const size_t pk0 = TP && p.inner ? pack_place(a.nx, p) : 0, pair = P / 64 * 2048;
   if (TP && p.inner) {
     const int by = blockIdx.x / cut.ntx % cut.nty, bx = blockIdx.x % cut.ntx, vx = cut.nqt >> 1;
-    pk1.cell = pk2.cell = ((p.y >> 3) - (by * (R - 2) >> 3)) * vx + (p.gq >> 1) - bx * vx;
+    cell += ((p.y >> 3) - (by * (R - 2) >> 3)) * vx + (p.gq >> 1) - bx * vx;
   }
 
   for (int k = k0; k <= p.ke; ++k) {
@@ -554,8 +559,8 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
       if (a.e1) st4(a.e1, i0 + (size_t)k * P, v4(e1));
       if (k == krec && a.d[0]) record(a.rec_map + i0, a.d[0], v4(vx1), v4(vy1), v4(vz1));
     }
-    if (TP && a.tpack[0] && k >= p.kb && k < p.ke)
-      pk1.plane(e1, table, a.tpack[0], a.tslot[0], a.nx, a.ny, k, p);
+    if (TP && a.tpack[0] && p.inner && k >= p.kb && k < p.ke)
+      pk1.plane(e1, cell, a.tpack[0] + (k >> 1) * pair + a.tslot[0] * 128 + pk0, k);
     // ---- B: z-faces and nodes of plane k - 1 after step 2
     F4 vz2 = fma(dth, sub(me1, me1p), vz1p);
     if (k - 1 >= nz - 1) vz2 = f4(z4());
@@ -581,7 +586,8 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
           st4(a.vz2, i, v4(vz2));
           if (k - 1 == krec && a.d[1]) record(a.rec_map + i0, a.d[1], v4(vx2), v4(vy2), v4(vz2));
         }
-        if (TP && a.tpack[1]) pk2.plane(e2, table + kTable, a.tpack[1], a.tslot[1], a.nx, a.ny, k - 1, p);
+        if (TP && a.tpack[1] && p.inner)
+          pk2.plane(e2, cell + kTable, a.tpack[1] + (k - 1 >> 1) * pair + a.tslot[1] * 128 + pk0, k - 1);
       }
     }
     // ---- the next plane
@@ -622,8 +628,8 @@ __device__ __forceinline__ F4 injected(F4 f, const int* rec_map, const float* r)
 // the loop even where they are skipped: 238 us instead of 140 at 256^3, so the other launches
 // are built without them).  mu, lx and ly, which neighbours read, come through the ring; the
 // fields that only their own thread uses stay in registers, one plane ahead (through the ring
-// too the pass was 15% slower).  Full gradient at 256^3: 153 us per step with two barriers, 148.5
-// now; 52 B per node and pass bound it from 128 us a pass, issue slots at about 175.
+// too the pass was 15% slower).  Full gradient at 256^3: 153 us per step with two barriers, 148
+// with one; 52 B per node and pass bound it from 128 us a pass, issue slots at about 175.
 template <bool B16, bool CLOSE>
 __global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(const __grid_constant__ TwoAdj a,
                                                               const __grid_constant__ Cut cut) {
@@ -704,17 +710,7 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(const __grid_const
                ? *reinterpret_cast<const float4*>(a.acc32 + (i0 + (size_t)k * P))
                : z4();
   };
-  auto flush = [&](size_t i, F4 f) {
-    const float4 v = v4(f);
-    double2* p64 = reinterpret_cast<double2*>(a.acc64 + i);
-    double2 lo = p64[0], hi = p64[1];
-    lo.x += (double)v.x;
-    lo.y += (double)v.y;
-    hi.x += (double)v.z;
-    hi.y += (double)v.w;
-    p64[0] = lo;
-    p64[1] = hi;
-  };
+  auto flush = [&](size_t i, F4 f) { add_wide(a.acc64 + i, v4(f)); };
   auto val = [&](const Strain& e) { return f4(B16 ? bf4(e.f16) : e.f32); };
 
   const int k0 = max(p.kb - 1, 0);
