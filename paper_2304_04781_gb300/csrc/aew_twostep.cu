@@ -42,11 +42,15 @@ TwoCut two_cut(int nx, int ny, int nz, int sms) {
 
 namespace {
 
+// shared memory: own ring, plane buffers, `planes` planes of `extra_rows` rows beyond the
+// column, edge words and maxima tables, the packed strain's stage
 template <auto kernel, class A>
-cudaError_t go(const A& a, const TwoCut& c, int ring, int buffers, int extra_rows, cudaStream_t s) {
+cudaError_t go(const A& a, const TwoCut& c, int ring, int buffers, int planes, int extra_rows, bool stage,
+               cudaStream_t s) {
   const size_t smem = ((size_t)ring * two::kThreads + buffers * (size_t)(two::kThreads + 2 * c.W) +
-                       (size_t)two::kRing * extra_rows * c.W) * 16 +
-                      2 * two::kThreads / 32 * 4 + 2 * two::kTable * 4;
+                       (size_t)planes * extra_rows * c.W) * 16 +
+                      2 * two::kThreads / 32 * 4 + 2 * two::kTable * 4 +
+                      (stage ? 4 * (size_t)c.rows * (c.nqt + 2) * 8 : 0);
   // once per instantiation (thread-safe static initialisation)
   static const cudaError_t attr =
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
@@ -63,21 +67,21 @@ cudaError_t launch_two_fwd(const TwoFwd& a, const TwoCut& cut, cudaStream_t s) {
   if (!a.err || (a.ef[0] && a.ef16[0]) || (a.ef[1] && a.ef16[1])) return cudaErrorInvalidValue;
   if (a.dm) {
     const bool b16 = a.ef16[0] || a.ef16[1];
-    if (tp) return b16 ? go<two::fwd_kernel<2, true>>(a, cut, 0, 4, 9, s) : cudaErrorInvalidValue;
-    return b16 ? go<two::fwd_kernel<2, false>>(a, cut, 0, 4, 9, s) : go<two::fwd_kernel<1, false>>(a, cut, 0, 4, 9, s);
+    if (tp) return b16 ? go<two::fwd_kernel<2, true>>(a, cut, 0, 4, two::kRing, 9, false, s) : cudaErrorInvalidValue;
+    return b16 ? go<two::fwd_kernel<2, false>>(a, cut, 0, 4, two::kRing, 9, false, s) : go<two::fwd_kernel<1, false>>(a, cut, 0, 4, two::kRing, 9, false, s);
   }
-  return tp ? go<two::forward_kernel<true>>(a, cut, two::kOwnRing, 6, 5, s)
-            : go<two::forward_kernel<false>>(a, cut, two::kOwnRing, 6, 5, s);
+  return tp ? go<two::forward_pack_kernel>(a, cut, two::kPackRing, 6, two::kExtra, 5, true, s)
+            : go<two::forward_kernel>(a, cut, two::kOwnRing, 6, two::kRing, 5, false, s);
 }
 
 cudaError_t launch_two_adj(const TwoAdj& a, const TwoCut& cut, cudaStream_t s) {
   if (!a.err || (a.en[0] && a.en16[0]) || (a.en[1] && a.en16[1])) return cudaErrorInvalidValue;
   const bool close = a.close[0] || a.close[1];
   if (a.en16[0] || a.en16[1])
-    return close ? go<two::adjoint_kernel<true, true>>(a, cut, two::kAdjRing, 6, 3, s)
-                 : go<two::adjoint_kernel<true, false>>(a, cut, two::kAdjRing, 6, 3, s);
-  return close ? go<two::adjoint_kernel<false, true>>(a, cut, two::kAdjRing, 6, 3, s)
-               : go<two::adjoint_kernel<false, false>>(a, cut, two::kAdjRing, 6, 3, s);
+    return close ? go<two::adjoint_kernel<true, true>>(a, cut, two::kAdjRing, 6, two::kRing, 3, false, s)
+                 : go<two::adjoint_kernel<true, false>>(a, cut, two::kAdjRing, 6, two::kRing, 3, false, s);
+  return close ? go<two::adjoint_kernel<false, true>>(a, cut, two::kAdjRing, 6, two::kRing, 3, false, s)
+               : go<two::adjoint_kernel<false, false>>(a, cut, two::kAdjRing, 6, two::kRing, 3, false, s);
 }
 
 }  // namespace aew

@@ -9,7 +9,7 @@
 // neighbouring CTA, by the identical expressions, so results are bitwise those of two
 // single steps.  z chunks overlap by two planes the same way.
 //   256^3, us per step: forward 95 -> 57 (44 for its bytes at the copy rate), forward and
-//   adjoint with the whole history 225 -> 144, with the time codec 274 -> 208; 160^3 34 -> 18
+//   adjoint with the whole history 225 -> 144, with the time codec 274 -> 202; 160^3 34 -> 18
 //   forward; 512 x 512 x 256 350 -> 276.
 //
 // Layout.  Thread (j, q) owns four nodes of row j.  The state of the two planes in flight is
@@ -17,7 +17,7 @@
 // in shared memory, x neighbours by shuffle, z neighbours are the thread's own.  Per plane:
 //   A  faces of plane k (step 1) and x-, y-faces of plane k - 1 (step 2)
 //   B  nodes of plane k (step 1), z-faces and nodes of plane k - 1 (step 2), stores
-// with a barrier after each (forward_kernel and adjoint_kernel: one per plane).  The rows beyond the
+// with a barrier after each (forward_kernel, forward_pack_kernel and adjoint_kernel: one per plane).  The rows beyond the
 // column (one m e row, and one y-face row below) come by cp.async into a small ring, so that
 // they cost no registers.
 #pragma once
@@ -33,10 +33,12 @@ using namespace quad;
 constexpr int kThreads = 512;
 constexpr int kMaxTileQ = 64;   // float4 per x tile
 constexpr int kRing = 4;        // extra rows: planes in the cp.async ring
-// forward_kernel: planes of the threads' own nodes in their ring: e and m, which are first used
-// one plane early, and the faces; two iterations of loads are in flight
+// Planes of the threads' own nodes in the rings of forward_kernel and adjoint_kernel: fields that
+// are used in two iterations (m, mu) and the others; two iterations of loads are in flight.
 constexpr int kEarly = 4, kLate = 3;
-constexpr int kOwnRing = 2 * kEarly + 3 * kLate;
+constexpr int kOwnRing = 2 * kEarly + 3 * kLate;   // forward_kernel: m and e, and the faces
+constexpr int kPackRing = kEarly + 4 * kLate;      // forward_pack_kernel: m, and e and the faces
+constexpr int kExtra = 3;                          // planes of the extra rows there
 constexpr int kAdjRing = kEarly + 2 * kLate;   // mu, and lx and ly
 
 using Cut = TwoCut;
@@ -107,10 +109,9 @@ __device__ __forceinline__ float4 ldz16(const uint16_t* p, bool ok) {
 constexpr int kTable = 128;
 struct Pack {
   float m;         // max |e| of the thread's nodes in the current pair of planes
-  // at: the thread's row of its vector in the pair k / 2, this slot
-  __device__ __forceinline__ void plane(F4 f, unsigned* cell, uint16_t* at, int k) {
+  __device__ __forceinline__ void plane(F4 f, unsigned* cell, uint2* at, int k) {
     const float4 v = v4(f);
-    *reinterpret_cast<uint2*>(at + (k & 1) * 64) = make_uint2(pack2bf(v.x, v.y), pack2bf(v.z, v.w));
+    *at = make_uint2(pack2bf(v.x, v.y), pack2bf(v.z, v.w));
     m = fmaxf(k & 1 ? m : 0.f, hmax4(v));
     if ((k & 1) && m > 0.f) atomicMax(cell, __float_as_uint(m));
   }
@@ -137,7 +138,6 @@ __device__ __forceinline__ void fold_table(unsigned* table, unsigned* vmax, cons
 // (step 2), by the expressions of the thread that owns them.
 //   me: m e of the plane, rows -1 .. R; me1, vy1: after step 1, rows 0 .. R - 1; all in two
 //   buffers by the plane's parity.
-template <bool TP>
 __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_constant__ TwoFwd a,
                                                               const __grid_constant__ Cut cut) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -151,8 +151,6 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
   float4* const ex = vy1_s - tid + 2 * N;      // [kRing][3][W] e, m, vy of the row below ..
   float4* const eh = ex + kRing * 3 * W;       // [kRing][2][W] e, m of the row above
   float* const sx = reinterpret_cast<float*>(eh + kRing * 2 * W);   // [2][warps]: lane 31's last x-face
-  unsigned* const table = reinterpret_cast<unsigned*>(sx + 2 * (kThreads / 32));   // [2][kTable]
-  if (TP && tid < 2 * kTable) table[tid] = 0;
   const F4 dth = f4(make_float4(a.dth, a.dth, a.dth, a.dth));
   const size_t P = (size_t)a.nx * a.ny;
   const size_t i0 = p.valid ? (size_t)p.y * a.nx + p.i0 : 0;
@@ -233,14 +231,6 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
   __syncthreads();
 
   F4 vx1p = f4(z4()), vy1p = vx1p, vz1p = vzl1, e1p = vx1p, me1p = vx1p, vz2p = vx1p;
-  Pack pk1{0.f}, pk2{0.f};
-  unsigned* cell = table;
-  const size_t pk0 = TP && p.inner ? pack_place(a.nx, p) : 0, pair = P / 64 * 2048;
-  if (TP && p.inner) {
-    const int by = blockIdx.x / cut.ntx % cut.nty, bx = blockIdx.x % cut.ntx, vx = cut.nqt >> 1;
-    cell += ((p.y >> 3) - (by * (R - 2) >> 3)) * vx + (p.gq >> 1) - bx * vx;
-  }
-
   for (int k = k0; k <= p.ke; ++k) {
     const int cur = (k & 1) * N, old = N - cur;
     // ---- loads of the planes ahead, into the slots of plane k - 1
@@ -248,10 +238,6 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
     issue_v(k + 2);
     issue_extra(k + 2);
     const F4 e_n = lds(em_at(k + 1)), me_n = mul(lds(em_at(k + 1) + kThreads), e_n);
-    if (TP && k > k0) {   // the pairs of planes that the last iteration ended
-      if (a.tpack[0] && !(k & 1) && k - 1 >= p.kb) fold_table(table, a.vmax[0], cut, a.nx, a.ny, k - 1);
-      if (a.tpack[1] && (k & 1) && k - 2 >= p.kb) fold_table(table + kTable, a.vmax[1], cut, a.nx, a.ny, k - 2);
-    }
     // ---- step 1 of plane k
     F4 vx1, vy1, vz1, e1, me1;
     {
@@ -288,8 +274,6 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
       if (a.e1) st4(a.e1, i0 + (size_t)k * P, v4(e1));
       if (k == krec && a.d[0]) record(a.rec_map + i0, a.d[0], v4(vx1), v4(vy1), v4(vz1));
     }
-    if (TP && a.tpack[0] && p.inner && k >= p.kb && k < p.ke)
-      pk1.plane(e1, cell, a.tpack[0] + (k >> 1) * pair + a.tslot[0] * 128 + pk0, k);
     // ---- step 2 of plane k - 1
     F4 vz2 = fma(dth, sub(me1, me1p), vz1p);
     if (k - 1 >= nz - 1) vz2 = f4(z4());
@@ -325,8 +309,6 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
         st4(a.vz2, i, v4(vz2));
         if (k - 1 == krec && a.d[1]) record(a.rec_map + i0, a.d[1], x, v4(vy2), v4(vz2));
       }
-      if (TP && a.tpack[1] && p.inner)
-        pk2.plane(e2, cell + kTable, a.tpack[1] + (k - 1 >> 1) * pair + a.tslot[1] * 128 + pk0, k - 1);
     }
     // ---- the next plane
     me1_s[cur + W] = v4(me1);
@@ -343,10 +325,253 @@ __global__ void __launch_bounds__(kThreads, 1) forward_kernel(const __grid_const
     e_c = e_n;
     __syncthreads();
   }
-  if (TP) {   // the last pairs: planes ke - 1 of step 1 (ended one iteration ago) and of step 2
-    if (a.tpack[0] && p.ke - 1 >= k0 && (p.ke & 1)) fold_table(table, a.vmax[0], cut, a.nx, a.ny, p.ke - 1);
-    if (a.tpack[1]) fold_table(table + kTable, a.vmax[1], cut, a.nx, a.ny, p.ke - 1);
+}
+
+// The same with window packing (time codec), a kernel of its own: e^{n+1} and e^{n+2} as BF16 go
+// through a stage in shared memory, so that the 16-byte rows of a vector leave together (a thread's
+// own 8 bytes would touch 16 lines per warp), and their maxima through the tables above.  256^3:
+// 147 us a pass with the stores of each thread, 137 now (111 without packing).  Room for the
+// stage: e and the extra rows in three planes; with that layout the kernel above is 5% slower.
+__global__ void __launch_bounds__(kThreads, 1) forward_pack_kernel(const __grid_constant__ TwoFwd a,
+                                                                   const __grid_constant__ Cut cut) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (sticky_error(a.err)) return;
+  const Place p(cut, a.ny, a.nz);
+  const int W = cut.W, R = cut.rows, tid = threadIdx.x, warp = tid >> 5, N = kThreads + 2 * W;
+  float4* const ring = reinterpret_cast<float4*>(smem) + tid;   // [kPackRing][kThreads]
+  float4* const me_s = reinterpret_cast<float4*>(smem) + kPackRing * kThreads + tid;   // [2][N]: row j - 1
+  float4* const me1_s = me_s + 2 * N;
+  float4* const vy1_s = me1_s + 2 * N;
+  float4* const ex = vy1_s - tid + 2 * N;      // [kExtra][3][W] e, m, vy of the row below ..
+  float4* const eh = ex + kExtra * 3 * W;      // [kExtra][2][W] e, m of the row above
+  float* const sx = reinterpret_cast<float*>(eh + kExtra * 2 * W);   // [2][warps]: lane 31's last x-face
+  unsigned* const table = reinterpret_cast<unsigned*>(sx + 2 * (kThreads / 32));   // [2][kTable]
+  // packed strain on its way out: [2][step][R][pitch] quads of the tile's own columns
+  const int pitch = cut.nqt + 2, SB = R * pitch;   // + 16 bytes per row: conflict-free columns
+  uint2* const stage = reinterpret_cast<uint2*>(table + 2 * kTable);
+  if (tid < 2 * kTable) table[tid] = 0;
+  const F4 dth = f4(make_float4(a.dth, a.dth, a.dth, a.dth));
+  const size_t P = (size_t)a.nx * a.ny;
+  const size_t i0 = p.valid ? (size_t)p.y * a.nx + p.i0 : 0;
+  const int nz = a.nz;
+  const bool live_q = p.gq >= 0 && p.gq < cut.nq;
+  // rare work: the columns meet the source box; the quad has receivers
+  const bool src = a.sk >= 0 && p.valid && abs(p.y - a.sj) <= a.sr && p.i0 + 3 >= a.si - a.sr &&
+                   p.i0 <= a.si + a.sr;
+  const int krec = p.inner && a.krec >= p.kb && a.krec < p.ke && (a.d[0] || a.d[1]) &&
+                           has_rec(a.rec_map + i0)
+                       ? a.krec
+                       : -1;
+
+  auto ok = [&](int k) { return p.valid && k >= 0 && k < nz; };
+  // the thread's slots: m; by c, the plane's number modulo 3 counted from k0, e and vx, vy, vz
+  auto m_at = [&](int k) { return ring + (k & (kEarly - 1)) * kThreads; };
+  auto e_at = [&](int c) { return ring + (kEarly + c) * kThreads; };
+  auto v_at = [&](int c) { return ring + (kEarly + (c + 1) * kLate) * kThreads; };
+  auto issue_em = [&](int k, int c) {
+    const bool v = ok(k) && k <= p.ke + 1;
+    const size_t i = v ? i0 + (size_t)k * P : 0;
+    cp16(e_at(c), a.e + i, v);
+    cp16(m_at(k), a.m + i, v);
+  };
+  auto issue_v = [&](int k, int c) {
+    const bool v = ok(k) && k <= p.ke;
+    const size_t i = v ? i0 + (size_t)k * P : 0;
+    cp16(v_at(c), a.vx + i, v);
+    cp16(v_at(c) + kThreads, a.vy + i, v);
+    cp16(v_at(c) + 2 * kThreads, a.vz + i, v);
+  };
+  // the extra rows of plane k into their slot, and the end of the plane's group
+  auto ex_at = [&](int c) { return (p.bot ? ex + c * 3 * W : eh + c * 2 * W) + p.q; };
+  auto issue_extra = [&](int k, int c) {
+    if (p.bot || p.top) {
+      const int ye = p.bot ? p.y - 1 : p.y + 1;
+      const bool v = k <= p.ke + 1 && live_q && ye >= 0 && ye < a.ny && k < nz;
+      const size_t i = v ? (size_t)ye * a.nx + p.i0 + (size_t)k * P : 0;
+      cp16(ex_at(c), a.e + i, v);
+      cp16(ex_at(c) + W, a.m + i, v);
+      if (p.bot) cp16(ex_at(c) + 2 * W, a.vy + i, v);
+    }
+    cp_commit();
+  };
+  // m e of the own row and the extra ones into plane k's buffer
+  auto put_me = [&](int k, int c, F4 me) {
+    float4* const d = me_s + (k & 1) * N;
+    if (p.j < R) d[W] = v4(me);
+    if (p.bot) d[0] = v4(mul_rn(ex_at(c)[W], ex_at(c)[0]));
+    if (p.top) d[2 * W] = v4(mul_rn(ex_at(c)[W], ex_at(c)[0]));
+  };
+
+  const int k0 = max(p.kb - 1, 0);
+  int c0 = 0, c1 = 1, c2 = 2;   // slots of planes k, k + 1, k + 2
+  issue_em(k0, c0);
+  issue_em(k0 + 1, c1);
+  issue_v(k0, c0);
+  issue_extra(k0, c0);
+  issue_em(k0 + 2, c2);
+  issue_v(k0 + 1, c1);
+  issue_extra(k0 + 1, c1);
+  F4 vzl1 = f4(z4());   // z-face below plane k0 after step 1
+  float4 eb = z4(), mb = z4(), vb = z4();
+  if (k0 >= 1) {
+    const size_t i = i0 + (size_t)(k0 - 1) * P;
+    eb = ldz(a.e + i, p.valid);
+    mb = ldz(a.m + i, p.valid);
+    vb = ldz(a.vz + i, p.valid);
   }
+  cp_wait<1>();
+  F4 e_c = lds(e_at(c0)), me_c = mul(lds(m_at(k0)), e_c);
+  if (k0 >= 1) {
+    vzl1 = fma(dth, sub(me_c, mul_rn(mb, eb)), f4(vb));
+    if (src && abs(k0 - 1 - a.sk) <= a.sr) {
+      float4 v = v4(vzl1);
+      add_source(v, k0 - 1, p.y, p.i0, a, a.dts[0]);
+      vzl1 = f4(v);
+    }
+  }
+  put_me(k0, c0, me_c);
+  __syncthreads();
+
+  F4 vx1p = f4(z4()), vy1p = vx1p, vz1p = vzl1, e1p = vx1p, me1p = vx1p, vz2p = vx1p;
+  Pack pk1{0.f}, pk2{0.f};
+  unsigned* cell = table;
+  uint2* put = stage;   // the thread's quad in the stage
+  // Write-out: half of the threads take a row of 8 nodes of one vector each for step 1, half for
+  // step 2; consecutive lanes take the rows of a vector, whose 16-byte rows are contiguous.
+  const int which = tid >> 8;
+  const size_t pair = P / 64 * 2048;   // a pair of planes further in the window
+  uint16_t* to = nullptr;
+  const uint2* from = stage;
+  const int bx = blockIdx.x % cut.ntx, by = blockIdx.x / cut.ntx % cut.nty, vx = cut.nqt >> 1;
+  const int item = tid & 255, v = item / (R - 2), r = item - v * (R - 2), y = by * (R - 2) + r;
+  uint16_t* const window = which ? a.tpack[1] : a.tpack[0];
+  if (window && 2 * v < min(cut.nqt, cut.nq - bx * cut.nqt) && y < a.ny)
+    to = window + (which ? a.tslot[1] : a.tslot[0]) * 128 +
+         ((size_t)(y >> 3) * (a.nx >> 3) + bx * vx + v) * 2048 + (y & 7) * 8;
+  from += which * SB + (r + 1) * pitch + 2 * v;
+  if (p.inner) {
+    cell += ((p.y >> 3) - (by * (R - 2) >> 3)) * vx + (p.gq >> 1) - bx * vx;
+    put += p.j * pitch + p.gq - bx * cut.nqt;
+  }
+  // what iteration k - 1 staged: plane k - 1 after step 1, plane k - 2 after step 2
+  auto write_out = [&](int k) {
+    const int w = k - 1 - which;
+    if (to && w >= p.kb && w < p.ke)
+      *reinterpret_cast<uint4*>(to + (w >> 1) * pair + (w & 1) * 64) =
+          *reinterpret_cast<const uint4*>(from + (k - 1 & 1) * 2 * SB);
+  };
+
+  for (int k = k0; k <= p.ke; ++k) {
+    const int cur = (k & 1) * N, old = N - cur;
+    // ---- loads of the planes ahead, into the slots of plane k - 1
+    issue_em(k + 3, c0);
+    issue_v(k + 2, c2);
+    issue_extra(k + 2, c2);
+    const F4 e_n = lds(e_at(c1)), me_n = mul(lds(m_at(k + 1)), e_n);
+    if (k > k0) {   // the pairs of planes that the last iteration ended
+      write_out(k);
+      if (a.tpack[0] && !(k & 1) && k - 1 >= p.kb) fold_table(table, a.vmax[0], cut, a.nx, a.ny, k - 1);
+      if (a.tpack[1] && (k & 1) && k - 2 >= p.kb) fold_table(table + kTable, a.vmax[1], cut, a.nx, a.ny, k - 2);
+    }
+    // ---- step 1 of plane k
+    F4 vx1, vy1, vz1, e1, me1;
+    {
+      const float4* const me = me_s + cur;
+      const float4* const v = v_at(c0);
+      const float4 m = v4(me_c);
+      float mx1 = __shfl_down_sync(0xffffffffu, m.x, 1);
+      if (p.p31) mx1 = me[W + 1].x;
+      float4 x = v4(fma(dth, f4(make_float4(__fsub_rn(m.y, m.x), __fsub_rn(m.z, m.y), __fsub_rn(m.w, m.z),
+                                            __fsub_rn(mx1, m.w))),
+                        lds(v)));
+      if (p.last_x) x.w = 0.f;
+      vx1 = f4(x);
+      float vxl = __shfl_up_sync(0xffffffffu, x.w, 1);
+      if (p.p0) vxl = __fmaf_rn(a.dth, __fsub_rn(m.x, me[W - 1].w), v[-1].w);
+      if (p.first_x) vxl = 0.f;
+      vy1 = fma(dth, sub(lds(me + 2 * W), me_c), lds(v + kThreads));
+      if (p.last_y) vy1 = f4(z4());
+      const F4 vyl = fma(dth, sub(me_c, lds(me)), lds(p.bot ? ex_at(c0) + 2 * W : v + kThreads - W));
+      vz1 = fma(dth, sub(me_n, me_c), lds(v + 2 * kThreads));
+      if (k >= nz - 1) vz1 = f4(z4());
+      if (src && abs(k - a.sk) <= a.sr) {
+        float4 z = v4(vz1);
+        add_source(z, k, p.y, p.i0, a, a.dts[0]);
+        vz1 = f4(z);
+      }
+      const F4 dx = f4(make_float4(x.x - vxl, x.y - x.x, x.z - x.y, x.w - x.z));
+      const F4 s = add(add(dx, sub(vy1, vyl)), sub(vz1, vz1p));
+      e1 = bounded(fma(dth, s, e_c), p, k == 0 || k >= nz - 1);
+      me1 = mul(lds(m_at(k)), e1);
+      if ((tid & 31) == 31) sx[(k & 1) * (kThreads / 32) + warp] = x.w;
+    }
+    if (p.inner && k >= p.kb && k < p.ke) {
+      if (a.e1) st4(a.e1, i0 + (size_t)k * P, v4(e1));
+      if (k == krec && a.d[0]) record(a.rec_map + i0, a.d[0], v4(vx1), v4(vy1), v4(vz1));
+    }
+    if (a.tpack[0] && p.inner && k >= p.kb && k < p.ke)
+      pk1.plane(e1, cell, put + (k & 1) * 2 * SB, k);
+    // ---- step 2 of plane k - 1
+    F4 vz2 = fma(dth, sub(me1, me1p), vz1p);
+    if (k - 1 >= nz - 1) vz2 = f4(z4());
+    if (src && abs(k - 1 - a.sk) <= a.sr && k > k0) {
+      float4 z = v4(vz2);
+      add_source(z, k - 1, p.y, p.i0, a, a.dts[1]);
+      vz2 = f4(z);
+    }
+    if (k - 1 >= p.kb && k > k0) {
+      const float4* const me = me1_s + old;
+      const float4 m = v4(me1p);
+      float mx1 = __shfl_down_sync(0xffffffffu, m.x, 1);
+      if (p.p31) mx1 = me[W + 1].x;
+      float4 x = v4(fma(dth, f4(make_float4(__fsub_rn(m.y, m.x), __fsub_rn(m.z, m.y), __fsub_rn(m.w, m.z),
+                                            __fsub_rn(mx1, m.w))),
+                        vx1p));
+      if (p.last_x) x.w = 0.f;
+      float vxl = __shfl_up_sync(0xffffffffu, x.w, 1);
+      if (p.p0)
+        vxl = __fmaf_rn(a.dth, __fsub_rn(m.x, me[W - 1].w), sx[((k - 1) & 1) * (kThreads / 32) + warp - 1]);
+      if (p.first_x) vxl = 0.f;
+      F4 vy2 = fma(dth, sub(lds(me + 2 * W), me1p), vy1p);
+      if (p.last_y) vy2 = f4(z4());
+      const F4 vyl = fma(dth, sub(me1p, lds(me)), lds(vy1_s + old));
+      const F4 dx = f4(make_float4(x.x - vxl, x.y - x.x, x.z - x.y, x.w - x.z));
+      const F4 s = add(add(dx, sub(vy2, vyl)), sub(vz2, vz2p));
+      const F4 e2 = bounded(fma(dth, s, e1p), p, k - 1 == 0 || k - 1 >= nz - 1);
+      const size_t i = i0 + (size_t)(k - 1) * P;
+      if (p.inner) {
+        st4(a.e2, i, v4(e2));
+        st4(a.vx2, i, x);
+        st4(a.vy2, i, v4(vy2));
+        st4(a.vz2, i, v4(vz2));
+        if (k - 1 == krec && a.d[1]) record(a.rec_map + i0, a.d[1], x, v4(vy2), v4(vz2));
+      }
+      if (a.tpack[1] && p.inner)
+        pk2.plane(e2, cell + kTable, put + ((k & 1) * 2 + 1) * SB, k - 1);
+    }
+    // ---- the next plane
+    me1_s[cur + W] = v4(me1);
+    vy1_s[cur + W] = v4(vy1);
+    cp_wait<1>();   // what the last iteration asked for
+    put_me(k + 1, c1, me_n);
+    const int c = c0;
+    c0 = c1;
+    c1 = c2;
+    c2 = c;
+    vz2p = vz2;
+    vx1p = vx1;
+    vy1p = vy1;
+    vz1p = vz1;
+    e1p = e1;
+    me1p = me1;
+    me_c = me_n;
+    e_c = e_n;
+    __syncthreads();
+  }
+  write_out(p.ke + 1);
+  // the last pairs: planes ke - 1 of step 1 (ended one iteration ago) and of step 2
+  if (a.tpack[0] && p.ke - 1 >= k0 && (p.ke & 1)) fold_table(table, a.vmax[0], cut, a.nx, a.ny, p.ke - 1);
+  if (a.tpack[1]) fold_table(table + kTable, a.vmax[1], cut, a.nx, a.ny, p.ke - 1);
 }
 
 // Incremental steps: + G(dm e) with FP32 (INCR 1) or BF16 e (2).  TP: window packing.
@@ -560,7 +785,8 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
       if (k == krec && a.d[0]) record(a.rec_map + i0, a.d[0], v4(vx1), v4(vy1), v4(vz1));
     }
     if (TP && a.tpack[0] && p.inner && k >= p.kb && k < p.ke)
-      pk1.plane(e1, cell, a.tpack[0] + (k >> 1) * pair + a.tslot[0] * 128 + pk0, k);
+      pk1.plane(e1, cell,
+                reinterpret_cast<uint2*>(a.tpack[0] + (k >> 1) * pair + a.tslot[0] * 128 + (k & 1) * 64 + pk0), k);
     // ---- B: z-faces and nodes of plane k - 1 after step 2
     F4 vz2 = fma(dth, sub(me1, me1p), vz1p);
     if (k - 1 >= nz - 1) vz2 = f4(z4());
@@ -587,7 +813,10 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
           if (k - 1 == krec && a.d[1]) record(a.rec_map + i0, a.d[1], v4(vx2), v4(vy2), v4(vz2));
         }
         if (TP && a.tpack[1] && p.inner)
-          pk2.plane(e2, cell + kTable, a.tpack[1] + (k - 1 >> 1) * pair + a.tslot[1] * 128 + pk0, k - 1);
+          pk2.plane(e2, cell + kTable,
+                    reinterpret_cast<uint2*>(a.tpack[1] + (k - 1 >> 1) * pair + a.tslot[1] * 128 +
+                                             (k - 1 & 1) * 64 + pk0),
+                    k - 1);
       }
     }
     // ---- the next plane
@@ -659,16 +888,16 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(const __grid_const
 
   auto ok = [&](int k) { return p.valid && k >= 0 && k < nz; };
   auto mu_at = [&](int k) { return ring + (size_t)(k & (kEarly - 1)) * kThreads; };
-  auto l_at = [&](int k) { return ring + (size_t)(kEarly + k % kLate * 2) * kThreads; };
+  auto l_at = [&](int c) { return ring + (kEarly + c * 2) * kThreads; };   // by slot
   auto issue_mu = [&](int k) {
     const bool v = ok(k) && k <= p.ke + 1;
     cp16(mu_at(k), a.mu + (v ? i0 + (size_t)k * P : 0), v);
   };
-  auto issue_l = [&](int k) {
+  auto issue_l = [&](int k, int c) {
     const bool v = ok(k) && k <= p.ke;
     const size_t i = v ? i0 + (size_t)k * P : 0;
-    cp16(l_at(k), a.lx + i, v);
-    cp16(l_at(k) + kThreads, a.ly + i, v);
+    cp16(l_at(c), a.lx + i, v);
+    cp16(l_at(c) + kThreads, a.ly + i, v);
   };
   // the extra rows of plane k into slot k % kRing, and the end of the plane's group
   auto ex_at = [&](int k) { return (p.bot ? ex + k % kRing * 2 * W : eh + k % kRing * W) + p.q; };
@@ -716,10 +945,11 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(const __grid_const
   const int k0 = max(p.kb - 1, 0);
   issue_mu(k0);
   issue_mu(k0 + 1);
-  issue_l(k0);
+  int c0 = 0, c1 = 1, c2 = 2;   // slots of planes k, k + 1, k + 2 (modulo 3)
+  issue_l(k0, c0);
   issue_extra(k0);
   issue_mu(k0 + 2);
-  issue_l(k0 + 1);
+  issue_l(k0 + 1, c1);
   issue_extra(k0 + 1);
   float4 mub = z4(), lzb = z4();
   if (k0 >= 1) {
@@ -749,7 +979,7 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(const __grid_const
     const int cur = (k & 1) * N, old = N - cur;
     // ---- loads of the planes ahead, into the slots of plane k - 1
     issue_mu(k + 3);
-    issue_l(k + 2);
+    issue_l(k + 2, c2);
     issue_extra(k + 2);
     const F4 mu_n = lds(mu_at(k + 1));
     const F4 m_c = f4(mr), w_c = f4(wr);
@@ -768,7 +998,7 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(const __grid_const
     F4 lx1, ly1, mu1, g;
     {
       const float4* const me = mu_s + cur;
-      const float4* const l = l_at(k);
+      const float4* const l = l_at(c0);
       lx1 = lds(l);
       ly1 = lds(l + kThreads);
       F4 lyl = lds(p.bot ? ex_at(k) + W : l + kThreads - W);
@@ -853,6 +1083,10 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(const __grid_const
     ly1_s[cur + W] = v4(ly1);
     cp_wait<1>();   // what the last iteration asked for
     put_mu(k + 1, mu_n);
+    const int c = c0;
+    c0 = c1;
+    c1 = c2;
+    c2 = c;
     lz2p = lz2;
     lx1p = lx1;
     ly1p = ly1;
