@@ -562,8 +562,8 @@ def run_ours(args):
                                                      f"summed by one all-reduce") if world > 1
                            else "one shot on one GPU"),
             "accuracy": accuracy,
-            "roofline": {"kernel": "adjoint step (adj_tma_kernel), the longest per-step kernel "
-                                   "of the AE gradient" + (", reading its decoded strain as BF16 "
+            "roofline": {"kernel": "single adjoint step (adj_tma_kernel, the kernel of odd last "
+                                   "steps; the solves take two steps per pass)" + (", reading its decoded strain as BF16 "
                                                            "(48 B/node)" if args.codec == "time"
                                                            else ""), "bound": "hbm",
                          "achieved": dom["achieved_gbs"], "peak": hbm_peak, "unit": "GB/s",
@@ -778,7 +778,7 @@ def run_map(args):
     solve_ms = a.elapsed_time(b)
     alpha_s = float(x1.double().std()) / args.prior_std
     # the prior's HBM-bound kernels alone: A q (8 B per node: read q, write A q) and one
-    # CG iteration (apply 8 + update 24 + direction 12 = 44 B per node)
+    # CG iteration (direction 12 + update 20 = 32 B per node)
     peaks = load_peaks()
     y1 = torch.empty_like(w)
     for _ in range(3):
@@ -803,7 +803,7 @@ def run_map(args):
                      "solve_ms": solve_ms, "solve_cg_iters": its,
                      "apply_ms": apply_ms,
                      "apply_gbs": 8.0 * c0.numel() / (apply_ms * 1e-3) / 1e9,
-                     "cg_iter_gbs": 44.0 * c0.numel() * its / (solve_ms * 1e-3) / 1e9,
+                     "cg_iter_gbs": 32.0 * c0.numel() * its / (solve_ms * 1e-3) / 1e9,
                      "hbm_peak_gbs": peaks[0]},
            "initial_mean_rel_err": mean_rel(c0)}
     del x1, w

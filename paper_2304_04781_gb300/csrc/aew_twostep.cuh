@@ -17,9 +17,9 @@
 // in shared memory, x neighbours by shuffle, z neighbours are the thread's own.  Per plane:
 //   A  faces of plane k (step 1) and x-, y-faces of plane k - 1 (step 2)
 //   B  nodes of plane k (step 1), z-faces and nodes of plane k - 1 (step 2), stores
-// with a barrier after each (forward_kernel, forward_pack_kernel and adjoint_kernel: one per plane).  The rows beyond the
-// column (one m e row, and one y-face row below) come by cp.async into a small ring, so that
-// they cost no registers.
+// with a barrier after each (forward_kernel, forward_pack_kernel and adjoint_kernel: one per
+// plane).  The rows beyond the column (one m e row, and one y-face row below) come by cp.async
+// into a small ring, so that they cost no registers.
 #pragma once
 
 #include "aew_stencil.cuh"
