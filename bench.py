@@ -441,16 +441,18 @@ def run_ours(args):
     if args.codec == "time":
         fl = codec_flops_per_window(ae.nvec, n_lat, ae.n_hid)
         sms = torch.cuda.get_device_properties(local).multi_processor_count
-        share = (sms // 2) / sms      # the codec GEMMs' CTA cap beside a stencil step
+        # the codec GEMMs' CTA cap: none between two-step passes (grids beyond the SMs)
+        ctas = sms if C > 4_000_000 else sms // 2
+        share = ctas / sms
         for kind, prof in (("encode_window", "encode_window"), ("decode_window", "decode_window_bf16")):
             kms = ae.profile(c, prof, 8)
             tf = fl[kind] / kms / 1e9
             kernels[kind] = {"ms_per_launch": kms, "flops_per_launch": fl[kind],
-                             "achieved_tflops": tf, "ctas": sms // 2,
+                             "achieved_tflops": tf, "ctas": ctas,
                              "frac_of_bf16_burst_share": tf / (tf_peak * share),
                              "note": f"both layers of one window (two tcgen05 GEMMs on SM pairs) "
-                                     f"on {sms // 2} CTAs, the cap they run with beside the "
-                                     f"stencil; frac against that share of the measured peak"
+                                     f"on {ctas} CTAs; frac against that share of the "
+                                     f"measured peak"
                                      + ("; the decoder writes BF16 strain, as for the adjoint "
                                         "sweeps" if kind == "decode_window" else "")}
     del ae
