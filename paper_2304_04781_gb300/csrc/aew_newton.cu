@@ -337,18 +337,21 @@ __device__ __forceinline__ void cg_walk(const Grid& g, const CgTile& t, float al
 
 // (1) p' = r + b p, b = rr_new / rr_old (first: p' = r), partials of p'.Ap' into ppap.  With
 // check the residual test comes first: rr_new <= tol2 ends the solve after `it` iterations.
+// Only a launch with check writes `done`, and there only the thread that writes it reads it: the
+// others go by the sums, which no launch changes once the test has passed, so all threads of all
+// blocks take the same way.  A launch without check reads what an earlier one wrote.
 __global__ void __launch_bounds__(kCgThreads, 2)
     cg_dir_kernel(const float* __restrict__ r, const float* __restrict__ p, float* __restrict__ pn, Grid g,
                   float alpha, float at, int kz, const double* prr_old, int nold, const double* prr_new, int nblk,
                   bool first, bool check, double tol2, int it, int* done, double* ppap) {
   __shared__ double sums[2], all[kCgThreads];
-  if (*reinterpret_cast<volatile int*>(done) >= 0) return;
+  if (!check && *done >= 0) return;
   float b = 0.f;
   if (!first) {
     cg_sums_of(prr_new, nblk, prr_old, nold, sums);
     const double rn = sums[0], ro = sums[1];
     if (check && rn <= tol2) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) *done = it;
+      if (blockIdx.x == 0 && threadIdx.x == 0 && *done < 0) *done = it;
       return;
     }
     b = ro > 0.0 ? (float)(rn / ro) : 0.f;
