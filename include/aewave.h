@@ -188,6 +188,12 @@ const char* aew_last_error(const aew_handle* h);
 /* Counters and memory of the handle (host struct filled in). */
 int aew_stats(const aew_handle* h, aew_stats_t* out);
 
+/* Which kernels ran the handle's time steps: counts_host[3] receives the launches since
+ * creation of single steps, of passes of two steps, and of on-chip runs of many steps (the
+ * library chooses by grid size and by how many steps follow one another).  AEW_E_ARG for NULL
+ * pointers. */
+int aew_routes(const aew_handle* h, long long* counts_host);
+
 /* ---------------------------------------------------------------------------------
  * Codec: the autoencoder of Sec. 3.1-3.3 (dense layers sigma(yW+b), Eq. (5)).
  * Encoder 2048 -> n_hid (GELU) -> n_lat; decoder n_lat -> n_hid (GELU) -> 2048, with

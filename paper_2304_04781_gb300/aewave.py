@@ -92,6 +92,7 @@ _SIGS = [
     ("aew_destroy", None, [c_void_p]),
     ("aew_last_error", ctypes.c_char_p, [c_void_p]),
     ("aew_stats", c_int, [c_void_p, POINTER(aew_stats_t)]),
+    ("aew_routes", c_int, [c_void_p, POINTER(c_longlong)]),
     ("aew_codec_set", c_int, [c_void_p] + [c_void_p] * 8),
     ("aew_codec_get", c_int, [c_void_p] + [c_void_p] * 8),
     ("aew_codec_encode", c_int, [c_void_p, POINTER(c_void_p), c_void_p, c_void_p, c_void_p]),
@@ -438,6 +439,12 @@ class Solver:
         s = aew_stats_t()
         self._check(lib().aew_stats(self._h, byref(s)))
         return {k: getattr(s, k) for k, _ in aew_stats_t._fields_}
+
+    def routes(self) -> dict:
+        """Launches since creation of single time steps, two-step passes and on-chip runs."""
+        n = (c_longlong * 3)()
+        self._check(lib().aew_routes(self._h, n))
+        return {"single": n[0], "two": n[1], "chip": n[2]}
 
     # ------------------------------------------------------------------ codec
     def codec_set(self, W: dict):

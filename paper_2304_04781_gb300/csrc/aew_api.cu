@@ -115,6 +115,7 @@ struct aew_handle {
   // exchange buffer with its running tag, and dt s^n of the default and of a given wavelet
   bool brick = false;
   bool two = false;   // larger grids: two steps per pass (aew_twostep.h)
+  long long routes[3] = {};   // launches of single steps, two-step passes, on-chip runs
   aew::TwoCut cut;
   aew::BrickPlan bp;
   unsigned char* halo = nullptr;
@@ -229,6 +230,7 @@ int fwd_step(aew_handle* h, int n, float* const in[4], float* const out[4], cons
   a.err = aew::codec_err_flag(h->codec);
   AEW_CK(aew::launch_fwd_step(a, false, s));
   ++h->stats.kernel_launches;
+  ++h->routes[0];
   return AEW_OK;
 }
 
@@ -266,6 +268,7 @@ int incr_step(aew_handle* h, float* const in[4], float* const out[4], const floa
   a.err = aew::codec_err_flag(h->codec);
   AEW_CK(aew::launch_fwd_step(a, incr, s));
   ++h->stats.kernel_launches;
+  ++h->routes[0];
   return AEW_OK;
 }
 
@@ -306,6 +309,7 @@ int adj_step_x(aew_handle* h, int n, float* const in[4], float* const out[4],
   a.err = aew::codec_err_flag(h->codec);
   AEW_CK(aew::launch_adj_step(a, s));
   ++h->stats.kernel_launches;
+  ++h->routes[0];
   return AEW_OK;
 }
 
@@ -396,6 +400,7 @@ aew::BrickFwd brick_fwd_args(aew_handle* h, float* const in[4], float* const out
 int brick_fwd(aew_handle* h, const aew::BrickFwd& a, cudaStream_t s) {
   AEW_CK(aew::launch_brick_fwd(a, h->bp, h->halo, &h->halo_tag, aew::codec_err_flag(h->codec), s));
   ++h->stats.kernel_launches;
+  ++h->routes[2];
   return AEW_OK;
 }
 
@@ -449,6 +454,7 @@ int brick_adj(aew_handle* h, int n0, int nsteps, float* const in[4], float* cons
   a.last = n0 - nsteps + 1 == 0;
   AEW_CK(aew::launch_brick_adj(a, h->bp, h->halo, &h->halo_tag, aew::codec_err_flag(h->codec), s));
   ++h->stats.kernel_launches;
+  ++h->routes[2];
   return AEW_OK;
 }
 
@@ -501,6 +507,7 @@ void two_pack(aew::TwoFwd& a, int i, const PackAt& p) {
 int two_fwd(aew_handle* h, const aew::TwoFwd& a, cudaStream_t s) {
   AEW_CK(aew::launch_two_fwd(a, h->cut, s));
   ++h->stats.kernel_launches;
+  ++h->routes[1];
   return AEW_OK;
 }
 // reverse steps n and n - 1; en / en16: e^n and e^{n-1} (null: zero)
@@ -538,13 +545,17 @@ int two_adj(aew_handle* h, int n, float* const in[4], float* const out[4], const
   a.err = aew::codec_err_flag(h->codec);
   AEW_CK(aew::launch_two_adj(a, h->cut, s));
   ++h->stats.kernel_launches;
+  ++h->routes[1];
   return AEW_OK;
 }
 
-// reverse step n: (lam, mu) in ad[cur] -> ad[cur ^ 1]
+// reverse step n: (lam, mu) in ad[cur] -> ad[cur ^ 1], the streaming kernel on every grid.  The
+// space codec's sweep decodes state n - 1 beside it: a cooperative launch of one step would wait
+// until the decoder's CTAs leave it all its SMs, and load, store and clear its state for one step
+// (gradient at 128^3, 40 steps: 2.83 ms with this kernel, 3.30 with on-chip steps; 96^3 2.41 and
+// 2.61; up to 64^3 no difference).
 int adj_step(aew_handle* h, int n, int cur, const float* resid, const float* en,
              cudaStream_t s) {
-  if (on_chip(h)) return brick_adj(h, n, 1, h->ad[cur], h->ad[cur ^ 1], resid, en, nullptr, s);
   return adj_step_x(h, n, h->ad[cur], h->ad[cur ^ 1], resid, en, h->acc32, h->acc64, nullptr,
                     nullptr, nullptr, s);
 }
@@ -1735,6 +1746,12 @@ int aew_stats(const aew_handle* h, aew_stats_t* out) {
       cudaEventElapsedTime(&ms, h->th[0], h->th[1]) == cudaSuccess)
     out->last_hessvec_ms = ms;
   cudaGetLastError();   // a query of an unfinished event is not an error of the handle
+  return AEW_OK;
+}
+
+int aew_routes(const aew_handle* h, long long* counts_host) {
+  if (!h || !counts_host) return AEW_E_ARG;
+  for (int i = 0; i < 3; ++i) counts_host[i] = h->routes[i];
   return AEW_OK;
 }
 

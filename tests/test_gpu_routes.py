@@ -1,0 +1,32 @@
+"""Which kernels run the time steps: on-chip runs and two-step passes only where they are
+the faster ones (the lines and both sides' times stand at the rules)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2304_04781_gb300 import inputs
+
+from .helpers import cuda, setup, solver
+
+pytestmark = pytest.mark.gpu
+
+
+def routes_of(s, run):
+    """Launches of (single steps, two-step passes, on-chip runs) made by run()."""
+    a = s.routes()
+    run()
+    b = s.routes()
+    return tuple(b[k] - a[k] for k in ("single", "two", "chip"))
+
+
+@pytest.mark.parametrize("shape", [(32, 32, 32), (96, 96, 96)])
+def test_space_codec_steps_beside_the_codec_are_single(shape):
+    """A cooperative launch would wait for the decoder beside it to leave it all its SMs."""
+    nt = 6
+    prob, c, _ = setup(shape, nt, 16, seed=5)
+    cc, dc = cuda(c), cuda(np.ones(shape))
+    d_obs = torch.zeros((nt + 1, prob.nrec, 3), device="cuda")
+    s = solver(prob, storage="ae")
+    s.codec_set(inputs.codec_init(seed=4))
+    assert routes_of(s, lambda: s.gradient(cc, d_obs)) == (2 * nt, 0, 0)
+    assert routes_of(s, lambda: s.hessvec(dc)) == (2 * nt, 0, 0)
