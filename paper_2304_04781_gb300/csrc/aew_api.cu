@@ -66,7 +66,9 @@ struct aew_handle {
   // AE mode: side stream running the codec GEMMs concurrently with the stencil steps,
   // double-buffered packed inputs and decoded strains, and the events ordering them
   cudaStream_t side = nullptr;
-  int overlap_ctas = 0;   // CTA cap of the codec GEMMs that run beside a stencil step
+  // CTA caps of the codec GEMMs that run beside single steps and beside two-step passes
+  int overlap_ctas = 0;
+  int overlap_two = 0;
   cudaEvent_t ev_a[2] = {}, ev_b[2] = {}, ev_sync = nullptr, ev_sync2 = nullptr;
   uint16_t* xpk[2] = {};
   float* edb[2] = {};
@@ -635,12 +637,22 @@ float* drow(aew_handle* h, float* d, int n) {
 // ---------------------------------------------------------------------------------
 // AE helpers
 // ---------------------------------------------------------------------------------
+// what runs beside a codec call, and the call's CTA cap for it (0: none)
+enum Beside { kAlone, kBesideSingle, kBesideTwo };
+int codec_ctas(const aew_handle* h, Beside b) {
+  return b == kAlone ? 0 : b == kBesideTwo ? h->overlap_two : h->overlap_ctas;
+}
+// .. the time codec beside steps on the handle's grid, two per pass where it takes them.  (The full
+// Newton HVP's adjoints are single steps on every grid; a cap beside them on the larger grids made
+// the product 0.5-0.9% slower at 136^3, 160^3 and 192^3: two windows' decodes are due at once.)
+Beside beside_steps(const aew_handle* h) { return h->two ? kBesideTwo : kBesideSingle; }
+
 // encoder GEMMs of the packed, normalised state n (xpk[n % 2]) into latents[n]
 int encode_packed(aew_handle* h, int n, cudaStream_t s) {
   const size_t nb = nblocks_of(h);
   cudaError_t e = aew::codec_encode_vectors(h->codec, h->xpk[n & 1], (long long)nb,
                                             h->lat + (size_t)n * nb * h->cfg.n_lat, h->ovf, s,
-                                            h->overlap_ctas);
+                                            codec_ctas(h, kBesideSingle));
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_encode_vectors");
   h->stats.kernel_launches += 2;
   return AEW_OK;
@@ -651,7 +663,8 @@ int decode_e(aew_handle* h, int n, float* buf, cudaStream_t s) {
   const size_t nb = nblocks_of(h);
   cudaError_t e = aew::codec_decode_grid_e(h->codec, h->lat + (size_t)n * nb * h->cfg.n_lat,
                                            h->cfg.nx, h->cfg.ny, h->cfg.nz,
-                                           h->bmx + (size_t)n * nb * 4, buf, s, h->overlap_ctas);
+                                           h->bmx + (size_t)n * nb * 4, buf, s,
+                                           codec_ctas(h, kBesideSingle));
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_decode_grid_e");
   h->stats.kernel_launches += 1;   // the fused two-layer decoder
   return AEW_OK;
@@ -1021,12 +1034,12 @@ int gradient_ae(aew_handle* h, const float* d_obs, const float* wav, cudaStream_
 // Compression in time: windows of 16 strain states per 2 x 8 x 8-node block
 // ---------------------------------------------------------------------------------
 // encoder of window tb (raw vectors in xt[tb % 2], maxima vmx[tb]) into its latents
-int encode_window(aew_handle* h, int tb, cudaStream_t s) {
+int encode_window(aew_handle* h, int tb, cudaStream_t s, Beside beside) {
   const size_t nv = nvec_of(h);
   const bool mm = aew::codec_minmax(h->codec);
   cudaError_t e = aew::codec_encode_window(h->codec, h->xt[tb & 1], h->vmx + (size_t)tb * nv,
                                            (long long)nv, h->lat + (size_t)tb * nv * h->cfg.n_lat,
-                                           h->ovf, s, on_chip(h) ? 0 : h->overlap_ctas,
+                                           h->ovf, s, codec_ctas(h, beside),
                                            mm ? h->wmn + (size_t)tb * nv : nullptr,
                                            mm ? h->wr + (size_t)tb * nv : nullptr);
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_encode_window");
@@ -1036,13 +1049,13 @@ int encode_window(aew_handle* h, int tb, cudaStream_t s) {
 
 // decoder of window tb into its 16 strain slices edt[tb % 2]: BF16 for every sweep (their
 // e^n boxes then carry half the bytes), FP32 for the profiling hook's FP32 kind
-int decode_window(aew_handle* h, int tb, cudaStream_t s, bool bf16 = false) {
+int decode_window(aew_handle* h, int tb, cudaStream_t s, Beside beside, bool bf16 = true) {
   const size_t nv = nvec_of(h);
   const bool mm = aew::codec_minmax(h->codec);
   cudaError_t e = aew::codec_decode_window(h->codec, h->lat + (size_t)tb * nv * h->cfg.n_lat,
                                            h->vmx + (size_t)tb * nv, h->cfg.nx, h->cfg.ny,
                                            h->cfg.nz, h->edt[tb & 1], s,
-                                           on_chip(h) ? 0 : h->overlap_ctas,
+                                           codec_ctas(h, beside),
                                            mm ? h->wmn + (size_t)tb * nv : nullptr,
                                            mm ? h->wr + (size_t)tb * nv : nullptr, bf16);
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_decode_window");
@@ -1071,7 +1084,7 @@ int time_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
   if (on_chip(h)) {   // the on-chip loops fill the GPU: decode and sweep each window in turn
     AEW_CK(cudaMemsetAsync(h->acc64, 0, h->C * sizeof(double), s));
     for (int tb = W - 1, cur = 0; tb >= 0; --tb, cur ^= 1) {
-      if ((rc = decode_window(h, tb, s, true))) return rc;
+      if ((rc = decode_window(h, tb, s, kAlone))) return rc;
       const int n0 = std::min(nt - 1, T * tb + T - 1);
       if ((rc = brick_adj(h, n0, n0 - T * tb + 1, tb == W - 1 ? nullptr : h->ad[cur],
                           tb > 0 ? h->ad[cur ^ 1] : nullptr, resid, nullptr, window_e16(h, n0), s)))
@@ -1081,7 +1094,7 @@ int time_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
   }
   if ((rc = begin_adjoint(h, s))) return rc;
   if ((rc = join(h, s, h->side, h->ev_sync))) return rc;
-  if ((rc = decode_window(h, W - 1, h->side, true))) return rc;
+  if ((rc = decode_window(h, W - 1, h->side, beside_steps(h)))) return rc;
   AEW_CK(cudaEventRecord(h->ev_b[(W - 1) & 1], h->side));
   int acur = 0;
   for (int n = nt - 1; n >= 0; --n) {
@@ -1089,7 +1102,7 @@ int time_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
     if (n == nt - 1 || n % T == T - 1) {
       if (tb >= 1) {
         if (tb + 1 <= W - 1) AEW_CK(cudaStreamWaitEvent(h->side, h->ev_a[(tb + 1) & 1], 0));
-        if ((rc = decode_window(h, tb - 1, h->side, true))) return rc;
+        if ((rc = decode_window(h, tb - 1, h->side, beside_steps(h)))) return rc;
         AEW_CK(cudaEventRecord(h->ev_b[(tb - 1) & 1], h->side));
       }
       AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
@@ -1140,7 +1153,7 @@ int gradient_ae_time(aew_handle* h, const float* d_obs, const float* wav, cudaSt
         if ((rc = brick_fwd(h, a, s))) return rc;
         n += steps;
       }
-      if ((rc = encode_window(h, tb, s))) return rc;
+      if ((rc = encode_window(h, tb, s, kAlone))) return rc;
     }
     if ((rc = residual_and_misfit(h, d_obs, s))) return rc;
     if ((rc = misfit_gate(h, s))) return rc;
@@ -1154,7 +1167,7 @@ int gradient_ae_time(aew_handle* h, const float* d_obs, const float* wav, cudaSt
   auto window_done = [&](int tb) -> int {
     AEW_CK(cudaEventRecord(h->ev_a[tb & 1], s));
     AEW_CK(cudaStreamWaitEvent(h->side, h->ev_a[tb & 1], 0));
-    int r = encode_window(h, tb, h->side);
+    int r = encode_window(h, tb, h->side, beside_steps(h));
     if (r) return r;
     AEW_CK(cudaEventRecord(h->ev_b[tb & 1], h->side));
     return AEW_OK;
@@ -1284,7 +1297,7 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
     const bool mm = aew::codec_minmax(h->codec);
     cudaError_t e = aew::codec_encode_window(h->codec, h->xt[tb & 1], h->vmx2 + (size_t)tb * nv,
                                              (long long)nv, h->lat2 + (size_t)tb * nv * h->cfg.n_lat,
-                                             h->ovf, h->side, h->overlap_ctas,
+                                             h->ovf, h->side, codec_ctas(h, beside_steps(h)),
                                              mm ? h->wmn2 + (size_t)tb * nv : nullptr,
                                              mm ? h->wr2 + (size_t)tb * nv : nullptr);
     if (e != cudaSuccess) return cuda_fail(h, e, "codec_encode_window");
@@ -1292,7 +1305,7 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
     AEW_CK(cudaEventRecord(h->ev_d[tb & 1], h->side));
     return AEW_OK;
   };
-  if ((rc = decode_window(h, 0, h->side, true))) return rc;
+  if ((rc = decode_window(h, 0, h->side, beside_steps(h)))) return rc;
   AEW_CK(cudaEventRecord(h->ev_b[0], h->side));
   if (nt == 1 && (rc = encode_de(0))) return rc;
   for (int n = 0; n < nt; ++n) {
@@ -1300,7 +1313,7 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
     if (n % T == 0) {
       if (tb + 1 <= W - 1) {
         if (tb >= 1) AEW_CK(cudaStreamWaitEvent(h->side, h->ev_a[(tb + 1) & 1], 0));
-        if ((rc = decode_window(h, tb + 1, h->side, true))) return rc;
+        if ((rc = decode_window(h, tb + 1, h->side, beside_steps(h)))) return rc;
         AEW_CK(cudaEventRecord(h->ev_b[(tb + 1) & 1], h->side));
       }
       AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
@@ -1345,7 +1358,7 @@ int decode_de_window(aew_handle* h, int tb, cudaStream_t s) {
   const bool mm = aew::codec_minmax(h->codec);
   cudaError_t e = aew::codec_decode_window(h->codec, h->lat2 + (size_t)tb * nv * h->cfg.n_lat,
                                            h->vmx2 + (size_t)tb * nv, h->cfg.nx, h->cfg.ny,
-                                           h->cfg.nz, h->edt2[tb & 1], s, h->overlap_ctas,
+                                           h->cfg.nz, h->edt2[tb & 1], s, codec_ctas(h, beside_steps(h)),
                                            mm ? h->wmn2 + (size_t)tb * nv : nullptr,
                                            mm ? h->wr2 + (size_t)tb * nv : nullptr, true);
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_decode_window");
@@ -1368,7 +1381,7 @@ int newton_adjoint_sweep(aew_handle* h, cudaStream_t s) {
   const bool ae = h->cfg.storage == AEW_AE;
   const int W = nwin_of(h);
   auto decode_both = [&](int tb) -> int {
-    int r = decode_window(h, tb, h->side, true);
+    int r = decode_window(h, tb, h->side, beside_steps(h));
     if (!r) r = decode_de_window(h, tb, h->side);
     return r;
   };
@@ -1661,10 +1674,12 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
     if (cudaDeviceGetStreamPriorityRange(&lo, &hi) != cudaSuccess) hi = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     h->overlap_ctas = sms > 1 ? sms / 2 : 0;
-    // two steps per pass: a pass holds every SM for 70-100 us, so the GEMMs take all SMs
-    // between passes (217 us per gradient step at 256^3, 222 with half of them)
-    if (h->two) h->overlap_ctas = 0;
-    if (const char* env = getenv("AEW_GEMM_CTAS_OVERLAP")) h->overlap_ctas = atoi(env);   // tuning override
+    // A two-step pass holds every SM for 110 us and more at 256^3, so beside those the GEMMs take
+    // all SMs between passes (217 us per gradient step at 256^3 without a cap, 222 with half of
+    // them; 202 now that the passes are faster)
+    h->overlap_two = 0;
+    if (const char* env = getenv("AEW_GEMM_CTAS_OVERLAP"))   // tuning override of both
+      h->overlap_ctas = h->overlap_two = atoi(env);
     ok = ok && cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, hi) == cudaSuccess;
     for (int i = 0; ok && i < 2; ++i)
       ok = cudaEventCreateWithFlags(&h->ev_a[i], cudaEventDisableTiming) == cudaSuccess &&
@@ -1931,7 +1946,7 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
     const int W = nwin_of(h), T = aew::kTSteps;
     *fwd = nt;
     for (int tb = 0; tb < W; ++tb, cur ^= 1) {
-      if ((rc = decode_window(h, tb, s, true))) return rc;
+      if ((rc = decode_window(h, tb, s, kAlone))) return rc;
       const int n = T * tb;
       const uint16_t* e16 = reinterpret_cast<const uint16_t*>(h->edt[tb & 1]);
       if ((rc = brick_fwd(h, brick_incr_args(h, tb ? h->ad[cur] : nullptr,
@@ -1950,14 +1965,14 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
     // ev_b[w % 2]: window w decoded, ev_a[w % 2]: window w's incremental steps done
     const int W = nwin_of(h), T = aew::kTSteps;
     if ((rc = join(h, s, h->side, h->ev_sync))) return rc;
-    if ((rc = decode_window(h, 0, h->side, true))) return rc;
+    if ((rc = decode_window(h, 0, h->side, beside_steps(h)))) return rc;
     AEW_CK(cudaEventRecord(h->ev_b[0], h->side));
     for (int n = 0; n < nt; ++n) {
       const int tb = n / T;
       if (n % T == 0) {
         if (tb + 1 <= W - 1) {
           if (tb >= 1) AEW_CK(cudaStreamWaitEvent(h->side, h->ev_a[(tb + 1) & 1], 0));
-          if ((rc = decode_window(h, tb + 1, h->side, true))) return rc;
+          if ((rc = decode_window(h, tb + 1, h->side, beside_steps(h)))) return rc;
           AEW_CK(cudaEventRecord(h->ev_b[(tb + 1) & 1], h->side));
         }
         AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
@@ -2435,6 +2450,7 @@ int aew_profile_steps(aew_handle* h, const float* c_dev, int kind, int nsteps, d
   if (rc) return rc;
   h->have_grad = false;
   const int nt = h->cfg.nt, T = aew::kTSteps;
+  const Beside beside = on_chip(h) ? kAlone : beside_steps(h);   // as in the time codec's solves
   cudaEvent_t e0, e1;
   AEW_CK(cudaEventCreate(&e0));
   AEW_CK(cudaEventCreate(&e1));
@@ -2458,10 +2474,10 @@ int aew_profile_steps(aew_handle* h, const float* c_dev, int kind, int nsteps, d
         rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], h->st[0][0], nullptr, s);
         break;
       case 4:
-        rc = encode_window(h, 0, s);
+        rc = encode_window(h, 0, s, beside);
         break;
       case 5:
-        rc = decode_window(h, 0, s);
+        rc = decode_window(h, 0, s, beside, false);
         break;
       case 6:   // the adjoint step reading its strain field as BF16 (time-codec sweeps)
         rc = adj_step_x(h, nt - 1 - n, h->ad[cur], h->ad[cur ^ 1], h->R, nullptr, h->acc32,
@@ -2469,7 +2485,7 @@ int aew_profile_steps(aew_handle* h, const float* c_dev, int kind, int nsteps, d
                         reinterpret_cast<const uint16_t*>(h->st[0][0]));
         break;
       case 7:
-        rc = decode_window(h, 0, s, true);
+        rc = decode_window(h, 0, s, beside);
         break;
       case 8:   // the incremental forward step reading its strain field as BF16
         rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], nullptr, nullptr, s, nullptr, 0, nullptr,

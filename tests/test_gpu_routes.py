@@ -30,3 +30,25 @@ def test_space_codec_steps_beside_the_codec_are_single(shape):
     s.codec_set(inputs.codec_init(seed=4))
     assert routes_of(s, lambda: s.gradient(cc, d_obs)) == (2 * nt, 0, 0)
     assert routes_of(s, lambda: s.hessvec(dc)) == (2 * nt, 0, 0)
+
+
+def test_space_codec_leaves_half_the_gpu_to_the_step_beside_it(monkeypatch):
+    """Its solves run single steps on every grid, so its decoder is capped at half the SMs
+    there too: 256 tiles take four rounds on 76 CTAs, two on 152."""
+    shape = (256, 256, 256)
+    prob, c, _ = setup(shape, 2, 4, seed=5)
+    cc = cuda(c)
+
+    def decode_ms(cap):
+        monkeypatch.delenv("AEW_GEMM_CTAS_OVERLAP", raising=False)
+        if cap is not None:
+            monkeypatch.setenv("AEW_GEMM_CTAS_OVERLAP", cap)
+        s = solver(prob, storage="ae")
+        s.codec_set(inputs.codec_init(seed=4))
+        s.profile(cc, "decode_state", 5)
+        ms = s.profile(cc, "decode_state", 50)
+        s.close()
+        return ms
+
+    free, capped = decode_ms("0"), decode_ms(None)
+    assert 1.4 * free < capped < 3.0 * free, (free, capped)
