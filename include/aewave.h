@@ -37,8 +37,8 @@
  *    a message.  A failed call leaves the handle usable.
  *  - Device waits are bounded.  A kernel whose wait gives up sets the handle's sticky
  *    device error flag and returns; later kernels of the handle see the flag and return
- *    at once.  Calls that synchronise (aew_gradient, aew_hessvec, the codec calls) and
- *    aew_sync_check read and clear the flag and report AEW_E_TIMEOUT; the asynchronous
+ *    at once.  Calls that synchronise (aew_gradient, aew_hessvec, aew_snapshots, the codec
+ *    calls) and aew_sync_check read and clear the flag and report AEW_E_TIMEOUT; the asynchronous
  *    solves (aew_forward, aew_propagate, aew_jvp) leave it for the next such call.
  *  - A handle is not thread-safe: one call at a time per handle.
  */
@@ -348,7 +348,8 @@ int aew_jvp(aew_handle* h, const float* dc_dev, float* dd_dev, void* stream);
  * block_max_dev (may be NULL): device FP32 [max_vectors][4], 16-byte aligned
  * (AEW_E_ARG otherwise), receiving the block maxima of each written vector (the forward
  * step that writes a state stores them).  The history storage of the handle is not
- * touched. */
+ * touched.  Synchronises the stream; AEW_E_TIMEOUT (and *n_written = 0) if a step kernel gave
+ * up waiting, or an earlier one had. */
 int aew_snapshots(aew_handle* h, const float* c_dev, int every, uint16_t* out_dev,
                   long long max_vectors, float* block_max_dev, long long* n_written,
                   void* stream);

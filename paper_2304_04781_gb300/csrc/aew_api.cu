@@ -1426,6 +1426,16 @@ int newton_adjoint_sweep(aew_handle* h, cudaStream_t s) {
   return AEW_OK;
 }
 
+// The end of aew_snapshots: synchronises.  After a step kernel that gave up waiting, or found the
+// error flag set, the packed vectors are void: none count as written.
+int snapshots_done(aew_handle* h, long long written, long long* n_written, cudaStream_t s) {
+  *n_written = 0;
+  if (aew::codec_take_error(h->codec, s))
+    return fail(h, AEW_E_TIMEOUT, "a step kernel gave up waiting (bounded wait)");
+  *n_written = written;
+  return AEW_OK;
+}
+
 // Algorithm 1 with the time codec: the complete windows tb = 0, every, 2 every, ... are
 // packed by the forward steps that write their states (raw BF16 plus per-vector
 // maxima), then normalised in place once their last state is in.
@@ -1507,9 +1517,7 @@ int snapshots_time(aew_handle* h, int every, uint16_t* out, long long max_vector
     cur ^= 1;
     if (tp && slot == T - 1 && (rc = finish(tb))) return rc;
   }
-  AEW_CK(cudaStreamSynchronize(s));
-  *n_written = w;
-  return AEW_OK;
+  return snapshots_done(h, w, n_written, s);
 }
 
 }  // namespace
@@ -2569,9 +2577,7 @@ int aew_snapshots(aew_handle* h, const float* c_dev, int every, uint16_t* out_de
       ++h->stats.kernel_launches;
       written += (long long)nb;
     }
-    AEW_CK(cudaStreamSynchronize(s));
-    *n_written = written;
-    return AEW_OK;
+    return snapshots_done(h, written, n_written, s);
   }
   for (int n = 0; n < nt; ++n) {
     const bool pack = packs(n, written);
@@ -2586,9 +2592,7 @@ int aew_snapshots(aew_handle* h, const float* c_dev, int every, uint16_t* out_de
     cur ^= 1;
     written = wnext;
   }
-  AEW_CK(cudaStreamSynchronize(s));
-  *n_written = written;
-  return AEW_OK;
+  return snapshots_done(h, written, n_written, s);
 }
 
 int aew_codec_train(aew_handle* h, const uint16_t* vectors_dev, const float* maxima_dev,
