@@ -340,6 +340,16 @@ bool on_chip(aew_handle* h) {
   return h->brick;
 }
 
+// Whether a run of `steps` steps that starts from and ends in a state in memory goes on chip.  A
+// launch loads, stores and clears its state whatever it runs, about one streaming step's time on
+// small bricks and more than one on large ones, so single steps go on chip up to 8192 nodes per
+// brick.  us per step, on chip / streaming (grid, nodes per brick): 32^3 256 6.5 / 9.5, 96^3 6144
+// 11.2 / 12.2, 148 x 100 x 72 7200 12.3 / 15.7, 104^3 7800 13.5 / 13.5, 112^3 9408 17.4 / 13.5,
+// 24 x 256 x 256 10752 19.6 / 14.3, 128^3 14336 25.0 / 19.7.  Runs of two gain on every grid.
+bool run_on_chip(aew_handle* h, int steps) {
+  return on_chip(h) && (steps > 1 || h->bp.by * h->bp.bz * h->cfg.nx <= 8192);
+}
+
 // dt s^n, n = 0 .. nt - 1, on the device: the default wavelet's, or wav's [count]
 int wavelet_on_device(aew_handle* h, const float* wav, size_t count, const float** out,
                       cudaStream_t s) {
@@ -2013,6 +2023,7 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
       AEW_CK(cudaEventRecord(h->ev_b[1], h->side));
     }
   }
+  const bool chip = h->cfg.storage == AEW_REVOLVE && run_on_chip(h, 1);
   for (int n = 0; n < nt; ++n) {
     const float* en = nullptr;
     if (ae) {
@@ -2030,7 +2041,7 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
     }
     if (h->cfg.storage == AEW_REVOLVE) {
       if (n > 0) {  // lockstep forward recompute: state n from state n-1
-        if (on_chip(h))
+        if (chip)
           rc = brick_fwd(h, brick_fwd_args(h, h->st[fcur], h->st[fcur ^ 1], 1, h->dts + n - 1,
                                            nullptr), s);
         else
@@ -2041,7 +2052,7 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
         en = h->st[fcur][0];
       }
     }
-    if (on_chip(h) && h->cfg.storage == AEW_REVOLVE) {
+    if (chip) {
       rc = n == 0 ? brick_fwd(h, brick_fwd_args(h, h->ad[cur], h->ad[cur ^ 1], 1, nullptr,
                                                 drow(h, dd_out, 1)), s)
                   : brick_fwd(h, brick_incr_args(h, h->ad[cur], h->ad[cur ^ 1], n, 1, en, nullptr,
@@ -2567,7 +2578,7 @@ int aew_snapshots(aew_handle* h, const float* c_dev, int every, uint16_t* out_de
     return block_max_dev ? reinterpret_cast<unsigned*>(block_max_dev) + (size_t)w * 4
                          : h->bm_tmp + ((size_t)(w / (long long)nb) & 1) * nb * 4;
   };
-  if (on_chip(h)) {   // on chip from one packed state to the next
+  if (run_on_chip(h, every)) {   // on chip from one packed state to the next
     for (int n = 0, m = every; packs(m, written); n = m, m += every, cur ^= 1) {
       if ((rc = brick_fwd(h, brick_fwd_args(h, n ? h->st[cur] : nullptr, h->st[cur ^ 1], m - n,
                                             h->dts + n, nullptr), s)))

@@ -52,3 +52,21 @@ def test_space_codec_leaves_half_the_gpu_to_the_step_beside_it(monkeypatch):
 
     free, capped = decode_ms("0"), decode_ms(None)
     assert 1.4 * free < capped < 3.0 * free, (free, capped)
+
+
+@pytest.mark.parametrize("shape,chip", [((32, 32, 32), True), ((104, 104, 104), True),
+                                        ((112, 112, 112), False), ((24, 256, 256), False)])
+def test_single_steps_go_on_chip_on_small_bricks_only(shape, chip):
+    """The JVP with checkpoints runs forward and incremental steps in turn, and data of every
+    state ends a run at each: runs of one step.  Runs of two and more stay on chip."""
+    nt = 9
+    prob, c, _ = setup(shape, nt, 16, seed=5)
+    cc, dc = cuda(c), cuda(np.ones(shape))
+    s = solver(prob, storage="revolve", n_checkpoints=2)
+    s.gradient(cc, torch.zeros((nt + 1, prob.nrec, 3), device="cuda"))
+    n = 2 * nt - 1
+    assert routes_of(s, lambda: s.jvp(dc)) == ((0, 0, n) if chip else (n, 0, 0))
+    room = nt * s.nblocks
+    one, _, many = routes_of(s, lambda: s.snapshots(cc, 1, room))
+    assert (one == 0 and many == nt - 1) if chip else (one >= nt - 1 and many == 0)
+    assert routes_of(s, lambda: s.snapshots(cc, 2, room)) == (0, 0, (nt - 1) // 2)
