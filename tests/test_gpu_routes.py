@@ -70,3 +70,29 @@ def test_single_steps_go_on_chip_on_small_bricks_only(shape, chip):
     one, _, many = routes_of(s, lambda: s.snapshots(cc, 1, room))
     assert (one == 0 and many == nt - 1) if chip else (one >= nt - 1 and many == 0)
     assert routes_of(s, lambda: s.snapshots(cc, 2, room)) == (0, 0, (nt - 1) // 2)
+
+
+@pytest.mark.parametrize("shape,least", [((20, 24, 28), 1), ((112, 112, 112), 3)])
+@pytest.mark.parametrize("nsteps", [1, 2, 3, 4, 8])
+def test_propagate_routes_and_bits(shape, least, nsteps, monkeypatch):
+    """On chip from `least` steps on, two launches that end in the caller's buffers; the same
+    bits as the streaming kernels either way."""
+    prob, c, _ = setup(shape, 10, 16, seed=5)
+    cc, rng = cuda(c), np.random.default_rng(3)
+    state = [cuda(rng.standard_normal(shape)) for _ in range(4)]
+    wav = rng.standard_normal(nsteps).astype(np.float32)
+    out = []
+    for kc in (None, "6"):
+        if kc:
+            monkeypatch.setenv("AEW_STENCIL_KC_FWD", kc)   # the streaming kernels
+        s = solver(prob)
+        for w in (None, wav):
+            st = [x.clone() for x in state]
+            rec = []
+            n = routes_of(s, lambda: rec.append(s.propagate(cc, st, 0, nsteps, wavelet=w, record=True)))
+            chip = not kc and nsteps >= least
+            assert n == ((0, 0, min(nsteps, 2)) if chip else (nsteps, 0, 0))
+            out.append([rec[0], *st])
+        s.close()
+    for a, b in zip(out[:2], out[2:]):
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
