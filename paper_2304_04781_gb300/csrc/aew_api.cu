@@ -318,26 +318,24 @@ int adj_step_x(aew_handle* h, int n, float* const in[4], float* const out[4],
 // ---------------------------------------------------------------------------------
 // On-chip time loops (aew_brick.h): many steps per launch
 // ---------------------------------------------------------------------------------
-// The handle's solves run on chip.  Their buffers are made by the first one (about a millisecond
-// that handles used for the codec alone need not spend); without memory for them the grid takes
+bool on_chip(const aew_handle* h) { return h->brick; }
+
+// The buffers of the on-chip loops, made with the handle; without memory for them the grid takes
 // the kernels of the larger ones.
-bool on_chip(aew_handle* h) {
-  if (!h->brick || h->halo) return h->brick;
+void make_brick_buffers(aew_handle* h) {
   const size_t nb = aew::brick_halo_bytes(h->cfg.nx, h->bp), nt = (size_t)h->cfg.nt;
   std::vector<float> dts(nt);
   for (size_t n = 0; n < nt; ++n) dts[n] = (float)(h->dt * (double)h->wav[n]);
-  unsigned char* halo = nullptr;
-  if (dalloc(h, &h->dts, nt) && dalloc(h, &halo, nb) &&
-      cudaMemcpy(h->dts, dts.data(), nt * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
-      cudaMemset(halo, 0, nb) == cudaSuccess && cudaStreamSynchronize(0) == cudaSuccess) {
-    h->halo = halo;
-  } else {
-    cudaGetLastError();
-    h->brick = false;
-    h->two = true;
+  if (dalloc(h, &h->halo, nb + nt * sizeof(float)) &&   // the words, then dt s^n
+      cudaMemset(h->halo, 0, nb) == cudaSuccess &&
+      cudaMemcpy(h->halo + nb, dts.data(), nt * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
+      cudaStreamSynchronize(0) == cudaSuccess) {   // solves run on other streams
+    h->dts = reinterpret_cast<float*>(h->halo + nb);
+    return;
   }
-  h->stats.device_bytes = h->bytes + aew::codec_device_bytes(h->codec);
-  return h->brick;
+  cudaGetLastError();
+  h->brick = false;
+  h->two = true;
 }
 
 // Whether a run of `steps` steps that starts from and ends in a state in memory goes on chip.  A
@@ -346,7 +344,7 @@ bool on_chip(aew_handle* h) {
 // brick.  us per step, on chip / streaming (grid, nodes per brick): 32^3 256 6.5 / 9.5, 96^3 6144
 // 11.2 / 12.2, 148 x 100 x 72 7200 12.3 / 15.7, 104^3 7800 13.5 / 13.5, 112^3 9408 17.4 / 13.5,
 // 24 x 256 x 256 10752 19.6 / 14.3, 128^3 14336 25.0 / 19.7.  Runs of two gain on every grid.
-bool run_on_chip(aew_handle* h, int steps) {
+bool run_on_chip(const aew_handle* h, int steps) {
   return on_chip(h) && (steps > 1 || h->bp.by * h->bp.bz * h->cfg.nx <= 8192);
 }
 
@@ -1731,6 +1729,7 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
       aew_destroy(h);
       return AEW_E_CUDA;
     }
+  if (h->brick) make_brick_buffers(h);   // last: the only buffers a handle can do without
   h->stats.device_bytes = h->bytes + aew::codec_device_bytes(h->codec);
   h->stats.latent_bytes =
       c.storage != AEW_AE ? 0
