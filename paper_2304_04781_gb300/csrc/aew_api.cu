@@ -124,7 +124,6 @@ struct aew_handle {
   uint32_t halo_tag = 0;
   float* dts = nullptr;
   float* dts_given = nullptr;
-  size_t dts_cap = 0;
   Codec* codec = nullptr;
   std::vector<void*> allocs;
   size_t bytes = 0;
@@ -326,11 +325,12 @@ void make_brick_buffers(aew_handle* h) {
   const size_t nb = aew::brick_halo_bytes(h->cfg.nx, h->bp), nt = (size_t)h->cfg.nt;
   std::vector<float> dts(nt);
   for (size_t n = 0; n < nt; ++n) dts[n] = (float)(h->dt * (double)h->wav[n]);
-  if (dalloc(h, &h->halo, nb + nt * sizeof(float)) &&   // the words, then dt s^n
+  if (dalloc(h, &h->halo, nb + 2 * nt * sizeof(float)) &&   // the words, then both dt s^n
       cudaMemset(h->halo, 0, nb) == cudaSuccess &&
       cudaMemcpy(h->halo + nb, dts.data(), nt * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
       cudaStreamSynchronize(0) == cudaSuccess) {   // solves run on other streams
     h->dts = reinterpret_cast<float*>(h->halo + nb);
+    h->dts_given = h->dts + nt;
     return;
   }
   cudaGetLastError();
@@ -348,25 +348,14 @@ bool run_on_chip(const aew_handle* h, int steps) {
   return on_chip(h) && (steps > 1 || h->bp.by * h->bp.bz * h->cfg.nx <= 8192);
 }
 
-// dt s^n, n = 0 .. nt - 1, on the device: the default wavelet's, or wav's [count]
-int wavelet_on_device(aew_handle* h, const float* wav, size_t count, const float** out,
-                      cudaStream_t s) {
-  if (!wav) {
-    *out = h->dts;
-    return AEW_OK;
-  }
-  if (h->dts_cap < count) {
-    float* p = nullptr;
-    if (!dalloc(h, &p, count)) return fail(h, AEW_E_NOMEM, "wavelet buffer");
-    h->dts_given = p;   // a smaller buffer stays with the handle until it is destroyed
-    h->dts_cap = count;
-    h->stats.device_bytes = h->bytes + aew::codec_device_bytes(h->codec);
-  }
-  std::vector<float> d(count);
-  for (size_t n = 0; n < count; ++n) d[n] = (float)(h->dt * (double)wav[n]);
-  AEW_CK(cudaMemcpyAsync(h->dts_given, d.data(), count * sizeof(float), cudaMemcpyHostToDevice, s));
-  AEW_CK(cudaStreamSynchronize(s));   // d is on this stack
-  *out = h->dts_given;
+// dt s^n of a caller's wavelet, n = 0 .. count - 1 (count <= nt), to dts_given on the device.  The
+// values travel as kernel arguments: the solves are asynchronous, and a copy from pageable memory
+// would make the host wait for all earlier work on the stream.
+int wavelet_to_device(aew_handle* h, const float* wav, int count, cudaStream_t s) {
+  std::vector<float> d((size_t)count);
+  for (int n = 0; n < count; ++n) d[n] = (float)(h->dt * (double)wav[n]);
+  AEW_CK(aew::launch_set_floats(h->dts_given, d.data(), d.size(), s));
+  ++h->stats.kernel_launches;
   return AEW_OK;
 }
 
@@ -1797,9 +1786,8 @@ int aew_forward(aew_handle* h, const float* c_dev, const float* wavelet_host, fl
   h->have_grad = false;  // m changed: stored history no longer matches
   if (d_dev && h->nrow) AEW_CK(cudaMemsetAsync(d_dev, 0, h->nrow * sizeof(float), s));
   if (on_chip(h)) {
-    const float* dts = nullptr;
-    if ((rc = wavelet_on_device(h, wavelet_host, (size_t)h->cfg.nt, &dts, s))) return rc;
-    return brick_fwd(h, brick_fwd_args(h, nullptr, nullptr, h->cfg.nt, dts,
+    if (wavelet_host && (rc = wavelet_to_device(h, wavelet_host, h->cfg.nt, s))) return rc;
+    return brick_fwd(h, brick_fwd_args(h, nullptr, nullptr, h->cfg.nt, wavelet_host ? h->dts_given : h->dts,
                                        d_dev ? drow(h, d_dev, 1) : nullptr), s);
   }
   const float* wav = wav_or_default(h, wavelet_host);
@@ -1855,14 +1843,18 @@ int aew_propagate(aew_handle* h, const float* c_dev, float* const state_dev[4], 
   // longer than copying the state back (128^3, about 20 us either way; smaller grids 7 and 18).
   // Large bricks gain from three steps on (an odd count of streaming steps copies the state too).
   if (on_chip(h) && nsteps >= (run_on_chip(h, 1) ? 1 : 3)) {
-    const float* dts = nullptr;
-    if (wavelet_host && (rc = wavelet_on_device(h, wavelet_host, (size_t)nsteps, &dts, s))) return rc;
+    // (an even number of launches; more than two where a given wavelet exceeds its buffer)
+    const int nt = h->cfg.nt;
+    const long long parts = nsteps == 1 ? 1 : wavelet_host ? 2 * (((long long)nsteps + 2LL * nt - 1) / (2LL * nt)) : 2;
     int cur = 0;
-    for (int k = 0, n; k < nsteps; k += n, cur ^= 1) {
-      n = k == 0 && nsteps > 1 ? nsteps / 2 : nsteps - k;
-      if ((rc = brick_fwd(h, brick_fwd_args(h, bufs[cur], bufs[cur ^ 1], n, dts ? dts + k : nullptr,
+    for (int k = 0, i = 0, n; k < nsteps; k += n, ++i) {
+      n = (int)((long long)nsteps * (i + 1) / parts) - k;
+      if (n == 0) continue;
+      if (wavelet_host && (rc = wavelet_to_device(h, wavelet_host + k, n, s))) return rc;
+      if ((rc = brick_fwd(h, brick_fwd_args(h, bufs[cur], bufs[cur ^ 1], n, wavelet_host ? h->dts_given : nullptr,
                                             d_dev ? drow(h, d_dev, k + 1) : nullptr), s)))
         return rc;
+      cur ^= 1;
     }
     return cur == 1 ? copy_state(h, bufs[0], bufs[1], s) : AEW_OK;
   }

@@ -118,6 +118,8 @@ struct FieldCheck {
   unsigned int cneg;        // count of c <= 0
 };
 // m = c^2 and checks; writes *chk (device)
+// n host values to device memory in stream order, without a copy: the host does not wait
+cudaError_t launch_set_floats(float* dst, const float* src_host, size_t n, cudaStream_t s);
 cudaError_t launch_prep_m(const float* c, float* m, size_t n, FieldCheck* chk, cudaStream_t s);
 // dm = 2 c dc and checks of dc
 cudaError_t launch_prep_dm(const float* c, const float* dc, float* dm, size_t n,

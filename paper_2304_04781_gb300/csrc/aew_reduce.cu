@@ -6,6 +6,7 @@
 // deterministic run to run.
 #include "aew_internal.cuh"
 
+#include <algorithm>
 #include <cmath>
 
 namespace aew {
@@ -132,7 +133,28 @@ int grid_for(size_t n) {
   return b < 1 ? 1 : (int)b;
 }
 
+// values that travel as kernel arguments (4 KB of them per launch)
+struct FloatChunk {
+  static constexpr int kMax = 960;
+  float v[kMax];
+};
+__global__ void set_floats_kernel(const __grid_constant__ FloatChunk c, float* __restrict__ dst, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = c.v[i];
+}
+
 }  // namespace
+
+cudaError_t launch_set_floats(float* dst, const float* src_host, size_t n, cudaStream_t s) {
+  for (size_t i = 0; i < n; i += FloatChunk::kMax) {
+    FloatChunk c;
+    const int m = (int)std::min<size_t>(FloatChunk::kMax, n - i);
+    std::copy(src_host + i, src_host + i + m, c.v);
+    set_floats_kernel<<<1, 320, 0, s>>>(c, dst + i, m);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
 
 cudaError_t launch_prep_m(const float* c, float* m, size_t n, FieldCheck* chk, cudaStream_t s) {
   prep_m_kernel<<<grid_for(n), RT, 0, s>>>(c, m, n, chk);
