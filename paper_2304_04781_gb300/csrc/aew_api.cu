@@ -116,7 +116,8 @@ struct aew_handle {
   // grids that fit the SMs run their time loops on chip (aew_brick.h): the cut, the halo
   // exchange buffer with its running tag, and dt s^n of the default and of a given wavelet
   bool brick = false;
-  bool two = false;   // larger grids: two steps per pass (aew_twostep.h)
+  bool two = false;   // larger grids: two incremental steps per pass (aew_twostep.h) ..
+  bool two_plain = false;   // .. and two forward or adjoint ones
   long long routes[3] = {};   // launches of single steps, two-step passes, on-chip runs
   aew::TwoCut cut;
   aew::BrickPlan bp;
@@ -319,6 +320,12 @@ int adj_step_x(aew_handle* h, int n, float* const in[4], float* const out[4],
 // ---------------------------------------------------------------------------------
 bool on_chip(const aew_handle* h) { return h->brick; }
 
+// Whether grids beyond the SMs take forward and adjoint steps two per pass (the line of
+// aew_twostep.cu; the time codec's share of a solve moves it)
+bool two_plain(const aew_handle* h) {
+  return h->cut.vs_single <= (h->cfg.storage == AEW_AE && h->cfg.codec == AEW_CODEC_TIME ? 1.1 : 1.0);
+}
+
 // The buffers of the on-chip loops, made with the handle; without memory for them the grid takes
 // the kernels of the larger ones.
 void make_brick_buffers(aew_handle* h) {
@@ -336,6 +343,7 @@ void make_brick_buffers(aew_handle* h) {
   cudaGetLastError();
   h->brick = false;
   h->two = true;
+  h->two_plain = two_plain(h);
 }
 
 // Whether a run of `steps` steps that starts from and ends in a state in memory goes on chip.  A
@@ -639,10 +647,12 @@ enum Beside { kAlone, kBesideSingle, kBesideTwo };
 int codec_ctas(const aew_handle* h, Beside b) {
   return b == kAlone ? 0 : b == kBesideTwo ? h->overlap_two : h->overlap_ctas;
 }
-// .. the time codec beside steps on the handle's grid, two per pass where it takes them.  (The full
-// Newton HVP's adjoints are single steps on every grid; a cap beside them on the larger grids made
-// the product 0.5-0.9% slower at 136^3, 160^3 and 192^3: two windows' decodes are due at once.)
-Beside beside_steps(const aew_handle* h) { return h->two ? kBesideTwo : kBesideSingle; }
+// .. the time codec beside steps on the handle's grid, two per pass where it takes them
+Beside beside_steps(const aew_handle* h) { return h->two_plain ? kBesideTwo : kBesideSingle; }
+// .. beside incremental steps.  (The full Newton HVP's adjoints are single steps on every grid; a
+// cap beside them on the larger grids made the product 0.5-0.9% slower at 136^3, 160^3 and 192^3:
+// two windows' decodes are due at once.)
+Beside beside_incr(const aew_handle* h) { return h->two ? kBesideTwo : kBesideSingle; }
 
 // encoder GEMMs of the packed, normalised state n (xpk[n % 2]) into latents[n]
 int encode_packed(aew_handle* h, int n, cudaStream_t s) {
@@ -716,7 +726,7 @@ int adjoint_full(aew_handle* h, const float* resid, cudaStream_t s) {
   if ((rc = begin_adjoint(h, s))) return rc;
   auto en = [&](int n) { return n > 0 ? h->estore + (size_t)n * h->C : nullptr; };
   for (int n = nt - 1; n >= 0; --n, cur ^= 1) {
-    if (h->two && n >= 1) {
+    if (h->two_plain && n >= 1) {
       rc = two_adj(h, n, h->ad[cur], h->ad[cur ^ 1], resid, en(n), en(n - 1), nullptr, nullptr, s);
       --n;
     } else {
@@ -750,7 +760,7 @@ int gradient_full(aew_handle* h, const float* d_obs, const float* wav, cudaStrea
   AEW_CK(cudaMemsetAsync(h->estore, 0, h->C * sizeof(float), s));
   AEW_CK(cudaMemsetAsync(h->d, 0, h->nrow * sizeof(float), s));
   for (int n = 0, a = 0; n < nt; ++n, a ^= 1) {
-    const int step = h->two && n + 1 < nt ? 2 : 1;
+    const int step = h->two_plain && n + 1 < nt ? 2 : 1;
     float* eout = (n + step < nt) ? h->estore + (size_t)(n + step) * h->C : h->st[0][0];
     float* in[4] = {h->estore + (size_t)n * h->C, vb[a][0], vb[a][1], vb[a][2]};
     float* out[4] = {eout, vb[a ^ 1][0], vb[a ^ 1][1], vb[a ^ 1][2]};
@@ -924,7 +934,7 @@ int run_revolve(aew_handle* h, const float* d_obs, const float* resid, const flo
         for (int k = 0; k < act.arg; ++k) {
           float* out[4];
           int out_buf;
-          const int step = h->two && k + 1 < act.arg ? 2 : 1;
+          const int step = h->two_plain && k + 1 < act.arg ? 2 : 1;
           if (to_slot && k + step == act.arg) {
             slot(plan[a + 1].arg, out);
             out_buf = -1;
@@ -1104,7 +1114,7 @@ int time_adjoint_sweep(aew_handle* h, const float* resid, cudaStream_t s) {
       }
       AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
     }
-    if (h->two && n % 2 == 1) {   // both steps in the same window
+    if (h->two_plain && n % 2 == 1) {   // both steps in the same window
       if ((rc = two_adj(h, n, h->ad[acur], h->ad[acur ^ 1], resid, nullptr, nullptr, window_e16(h, n),
                         window_e16(h, n - 1), s)))
         return rc;
@@ -1185,7 +1195,7 @@ int gradient_ae_time(aew_handle* h, const float* d_obs, const float* wav, cudaSt
     return AEW_OK;
   };
   for (int n = 0; n < nt; ++n, cur ^= 1) {
-    const int step = h->two && n + 1 < nt ? 2 : 1;
+    const int step = h->two_plain && n + 1 < nt ? 2 : 1;
     PackAt p[2];
     for (int i = 0; i < step; ++i)
       if ((rc = pack_at(n + 1 + i, &p[i]))) return rc;
@@ -1294,7 +1304,7 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
     const bool mm = aew::codec_minmax(h->codec);
     cudaError_t e = aew::codec_encode_window(h->codec, h->xt[tb & 1], h->vmx2 + (size_t)tb * nv,
                                              (long long)nv, h->lat2 + (size_t)tb * nv * h->cfg.n_lat,
-                                             h->ovf, h->side, codec_ctas(h, beside_steps(h)),
+                                             h->ovf, h->side, codec_ctas(h, beside_incr(h)),
                                              mm ? h->wmn2 + (size_t)tb * nv : nullptr,
                                              mm ? h->wr2 + (size_t)tb * nv : nullptr);
     if (e != cudaSuccess) return cuda_fail(h, e, "codec_encode_window");
@@ -1302,7 +1312,7 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
     AEW_CK(cudaEventRecord(h->ev_d[tb & 1], h->side));
     return AEW_OK;
   };
-  if ((rc = decode_window(h, 0, h->side, beside_steps(h)))) return rc;
+  if ((rc = decode_window(h, 0, h->side, beside_incr(h)))) return rc;
   AEW_CK(cudaEventRecord(h->ev_b[0], h->side));
   if (nt == 1 && (rc = encode_de(0))) return rc;
   for (int n = 0; n < nt; ++n) {
@@ -1310,7 +1320,7 @@ int newton_incremental_forward(aew_handle* h, cudaStream_t s) {
     if (n % T == 0) {
       if (tb + 1 <= W - 1) {
         if (tb >= 1) AEW_CK(cudaStreamWaitEvent(h->side, h->ev_a[(tb + 1) & 1], 0));
-        if ((rc = decode_window(h, tb + 1, h->side, beside_steps(h)))) return rc;
+        if ((rc = decode_window(h, tb + 1, h->side, beside_incr(h)))) return rc;
         AEW_CK(cudaEventRecord(h->ev_b[(tb + 1) & 1], h->side));
       }
       AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));
@@ -1355,7 +1365,7 @@ int decode_de_window(aew_handle* h, int tb, cudaStream_t s) {
   const bool mm = aew::codec_minmax(h->codec);
   cudaError_t e = aew::codec_decode_window(h->codec, h->lat2 + (size_t)tb * nv * h->cfg.n_lat,
                                            h->vmx2 + (size_t)tb * nv, h->cfg.nx, h->cfg.ny,
-                                           h->cfg.nz, h->edt2[tb & 1], s, codec_ctas(h, beside_steps(h)),
+                                           h->cfg.nz, h->edt2[tb & 1], s, codec_ctas(h, beside_incr(h)),
                                            mm ? h->wmn2 + (size_t)tb * nv : nullptr,
                                            mm ? h->wr2 + (size_t)tb * nv : nullptr, true);
   if (e != cudaSuccess) return cuda_fail(h, e, "codec_decode_window");
@@ -1378,7 +1388,7 @@ int newton_adjoint_sweep(aew_handle* h, cudaStream_t s) {
   const bool ae = h->cfg.storage == AEW_AE;
   const int W = nwin_of(h);
   auto decode_both = [&](int tb) -> int {
-    int r = decode_window(h, tb, h->side, beside_steps(h));
+    int r = decode_window(h, tb, h->side, beside_incr(h));
     if (!r) r = decode_de_window(h, tb, h->side);
     return r;
   };
@@ -1666,10 +1676,9 @@ int aew_create(const aew_config* cfg, aew_handle** out) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device);
     h->brick = coop && aew::brick_plan(c.nx, c.ny, c.nz, sms, &h->bp);
-    // faster than single steps on every larger grid: 160^3 18 us a step against 34, 256^3 57
-    // against 95, 512 x 512 x 256 276 against 350
-    h->two = !h->brick;
     h->cut = aew::two_cut(c.nx, c.ny, c.nz, sms > 0 ? sms : 1);
+    h->two = !h->brick;
+    h->two_plain = h->two && two_plain(h);
   }
   if (ok && c.storage == AEW_AE) {
     // The codec GEMMs run on a high-priority side stream with half the SMs, so their
@@ -1795,7 +1804,7 @@ int aew_forward(aew_handle* h, const float* c_dev, const float* wavelet_host, fl
   int cur = 0;
   for (int n = 0; n < h->cfg.nt; ++n, cur ^= 1) {
     float* row = d_dev ? drow(h, d_dev, n + 1) : nullptr;
-    if (h->two && n + 1 < h->cfg.nt) {
+    if (h->two_plain && n + 1 < h->cfg.nt) {
       rc = two_fwd(h, two_fwd_args(h, n, h->st[cur], h->st[cur ^ 1], nullptr, wav, row), s);
       ++n;
     } else {
@@ -1864,7 +1873,7 @@ int aew_propagate(aew_handle* h, const float* c_dev, float* const state_dev[4], 
   for (int k = 0; k < nsteps; ++k, cur ^= 1) {
     const float* wv = wavelet_host ? w.data() : nullptr;
     float* row = d_dev ? drow(h, d_dev, k + 1) : nullptr;
-    if (h->two && k + 1 < nsteps) {
+    if (h->two_plain && k + 1 < nsteps) {
       rc = two_fwd(h, two_fwd_args(h, n0 + k, bufs[cur], bufs[cur ^ 1], nullptr, wv, row), s);
       ++k;
     } else {
@@ -1981,14 +1990,14 @@ static int incremental_forward(aew_handle* h, float* dd_out, cudaStream_t s, lon
     // ev_b[w % 2]: window w decoded, ev_a[w % 2]: window w's incremental steps done
     const int W = nwin_of(h), T = aew::kTSteps;
     if ((rc = join(h, s, h->side, h->ev_sync))) return rc;
-    if ((rc = decode_window(h, 0, h->side, beside_steps(h)))) return rc;
+    if ((rc = decode_window(h, 0, h->side, beside_incr(h)))) return rc;
     AEW_CK(cudaEventRecord(h->ev_b[0], h->side));
     for (int n = 0; n < nt; ++n) {
       const int tb = n / T;
       if (n % T == 0) {
         if (tb + 1 <= W - 1) {
           if (tb >= 1) AEW_CK(cudaStreamWaitEvent(h->side, h->ev_a[(tb + 1) & 1], 0));
-          if ((rc = decode_window(h, tb + 1, h->side, beside_steps(h)))) return rc;
+          if ((rc = decode_window(h, tb + 1, h->side, beside_incr(h)))) return rc;
           AEW_CK(cudaEventRecord(h->ev_b[(tb + 1) & 1], h->side));
         }
         AEW_CK(cudaStreamWaitEvent(s, h->ev_b[tb & 1], 0));

@@ -11,6 +11,17 @@ namespace aew {
 // least planes times whole waves of one CTA per SM.  Tiles narrower than the grid have halo
 // columns and unaligned rows: a plane takes 1.2 times as long (256^3 forward 57 us per step in
 // one tile, 73 in two; 512 x 512 x 256 301, 283, 276 and 292 in two to five).
+//
+// Against single steps.  A pass takes about 1.5 us per plane of that cost in one wave, 1.15 in
+// more (a second wave's start hides).  Where rows are whole 128-node tiles of the single-step
+// kernels and the state (36 B per node) stays in L2, a single step takes 7.45 us per million
+// nodes and no less than 11.4, and passes of several x tiles lose.  us per forward step (nz x ny
+// x nx), single / two: 8 x 512 x 512 15.6 / 17.6, 8 x 256 x 1024 15.6 / 18.7, 16 x 256 x 512 15.6
+// / 16.7, 4 x 64 x 4096 11.4 / 12.4; but 64 x 64 x 512 15.6 / 14.6, 16 x 512 x 512 30.3 / 28.3,
+// and rows that fill no tile 40 x 200 x 320 20.8 / 17.2, one x tile 160^3 36 / 18.6.  Adjoint steps
+// divide alike; incremental ones gain on all but the first two (18.2 / 19.1, 18.4 / 19.6), and the
+// time codec's solves gain on 32 x 128 x 512, where forward steps lose (15.6 / 16.6; gradient step
+// 48.5 / 46.0).
 TwoCut two_cut(int nx, int ny, int nz, int sms) {
   TwoCut best{};
   double least = 0.0;
@@ -37,6 +48,10 @@ TwoCut two_cut(int nx, int ny, int nz, int sms) {
       }
     }
   }
+  const double m = (double)nx * ny * nz / 1e6;
+  const double pass = ((long long)best.ntx * best.nty * best.ntz <= sms ? 1.5 : 1.15) * least;
+  const bool close = best.ntx > 1 && nx % 128 == 0 && 36.0 * m <= 96.0;
+  best.vs_single = close ? pass / (2.0 * std::max(11.4, 7.45 * m)) : 0.0;
   return best;
 }
 

@@ -14,6 +14,9 @@ namespace aew {
 // rows (rows - 2 of their own), z chunks of kc planes
 struct TwoCut {
   int nq, nqt, ntx, W, rows, nty, kc, ntz;
+  // estimated time of a forward or adjoint pass by that of two single steps, where these may be
+  // the faster ones (otherwise 0)
+  double vs_single;
 };
 TwoCut two_cut(int nx, int ny, int nz, int sms);
 

@@ -96,3 +96,36 @@ def test_propagate_routes_and_bits(shape, least, nsteps, monkeypatch):
         s.close()
     for a, b in zip(out[:2], out[2:]):
         assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("shape,plain", [((8, 512, 512), False), ((4, 64, 4096), False),
+                                         ((64, 64, 512), True), ((100, 104, 260), True),
+                                         ((24, 256, 512), True), ((160, 112, 112), True)])
+def test_two_steps_per_pass_where_they_are_faster(shape, plain, monkeypatch):
+    """Grids beyond the SMs: single forward and adjoint steps where x needs several tiles,
+    rows are whole tiles of the single-step kernels and the state stays in L2; the same bits
+    as with single steps everywhere."""
+    nt = 6
+    prob, c, _ = setup(shape, nt, 1, seed=5)
+    cc, rng = cuda(c), np.random.default_rng(3)
+    d_obs = cuda(rng.standard_normal((nt + 1, prob.nrec, 3)) * 1e-6)
+    dc = cuda(rng.standard_normal(shape))
+    out = []
+    for kc in (None, "6"):
+        if kc:
+            monkeypatch.setenv("AEW_STENCIL_KC_FWD", kc)   # single steps
+        s = solver(prob)
+        res = []
+
+        def run():
+            res.extend([s.forward(cc), *s.gradient(cc, d_obs)[::-1], s.hessvec(dc)])
+
+        n = routes_of(s, run)
+        if kc:
+            assert n == (5 * nt, 0, 0)
+        else:
+            assert n == ((0, 5 * nt // 2, 0) if plain else (4 * nt, nt // 2, 0))
+        out.append(res)
+        s.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b) if isinstance(a, torch.Tensor) else a == b
