@@ -197,9 +197,9 @@ struct EpMse {
   // called by all 32 lanes of a warp together (rows m0 + 32 q + lane): the loss is
   // reduced across the warp before its one atomic
   __device__ __forceinline__ void operator()(long long row, int col, const float (&v)[32]) const {
-    // sum of wf diff^2 in FP32 with every rounding error kept (products by FMA, sums by
-    // Knuth's two-sum): as exact as FP64, whose rate here would cost a third of the kernel
-    float s1 = 0.f, s2 = 0.f;
+    // sum of diff^2 in FP64, whose range a diverging decoder needs: one conversion and one FMA per
+    // value, and the weight of the 32 values once
+    double acc = 0.0;
     float wf = 1.f;
     if (row < M) {
       // the 32 columns lie in one field's 64-column group: one weight
@@ -210,10 +210,7 @@ struct EpMse {
       for (int j = 0; j < 32; ++j) {
         const float a = v[j] + __ldg(bias + col + j);
         const float diff = a - gemm::bf16_val(__ldg(Y + row * kNIn + col + j));
-        const float p = __fmul_rn(diff, diff), t = __fadd_rn(s1, p), z = __fsub_rn(t, s1);
-        s2 = __fadd_rn(s2, __fadd_rn(fmaf(diff, diff, -p),
-                                     __fadd_rn(__fsub_rn(s1, __fsub_rn(t, z)), __fsub_rn(p, z))));
-        s1 = t;
+        acc = fma((double)diff, (double)diff, acc);
         dd[j] = scale * wf * diff;
         d4T[(size_t)(col + j) * M + row] = gemm::bf16_bits(dd[j]);
       }
@@ -222,7 +219,7 @@ struct EpMse {
       store_row32f(d4 + row * kNIn + col, dd);
       store_row16(d4b + row * kNIn + col, pk);
     }
-    double acc = (double)wf * ((double)s1 + (double)s2);
+    acc *= (double)wf;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc);
