@@ -524,7 +524,7 @@ int aew_prior_apply(aew_handle* h, double alpha, double theta, const float* q_de
                     float* out_dev, void* stream);
 
 /* x_dev = A^{-1} w_dev by conjugate gradients on FP32 vectors with FP64 inner products
- * (A is SPD with spectrum inside [alpha, alpha (1 + 12 theta / h^2)]), stopped when the
+ * (of FP32 sums of four products; A is SPD with spectrum inside [alpha, alpha (1 + 12 theta / h^2)]), stopped when the
  * recursive residual |r| <= rtol |w| (tolerances down to about 1e-7 are reached) or
  * after max_iter iterations; *iters_host (may be NULL) receives the iterations taken.
  * Prior samples are c + A^{-1} w for white noise w.  Synchronises `stream` (the

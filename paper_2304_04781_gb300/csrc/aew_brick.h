@@ -109,7 +109,7 @@ struct BrickCg {
   int nx, ny, nz;
   float alpha, at, sc, inv_sc;
   float rr_hi, rr_lo;      // r.r at the start, as a pair of floats
-  float tol_hi, tol_lo;    // tol2
+  double tol2;
   int max_iter;
   int* result;             // device [2]: iterations, 1 if the test passed
   int by, bz, py, pz;

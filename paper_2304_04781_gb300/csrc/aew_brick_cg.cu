@@ -4,79 +4,113 @@
 // registers and p in shared memory, with its halos exchanged as in the time loops
 // (aew_brick.cuh), and both inner products of an iteration are all-reduced through one
 // tagged word pair per CTA: three L2 round trips per iteration bound it, with the reductions'
-// dependent adds.  us per iteration, before -> now: 32^3 21 -> 8, 64^3 37 -> 12, 128^3
-// 45 -> 17.
+// dependent adds.  us per iteration, launch per pass -> now: 32^3 21 -> 9, 64^3 37 -> 10, 128^3
+// 45 -> 15.
 //
-// The sums are pairs of floats (value and accumulated rounding error, Knuth's two-sum), as
-// exact as FP64 here and without FP64 instructions, whose rate on this GPU would make the
-// reductions the longest part.  Every CTA adds the same pairs in the same order, so all take
-// the same steps and stop together.
+// The inner products: four products are summed by FP32 FMAs, as in the streaming passes; from
+// there a thread's and a warp's sums keep their rounding errors in two more floats (72 bits
+// against FP64's 53, and FP64 instructions in every warp would be the longest part of an
+// iteration), and one warp per CTA adds the warps' and the CTAs' parts in FP64.  Every CTA adds the
+// same parts in the same order, so all take the same steps and stop together.
 #include "aew_brick.cuh"
 
 namespace aew {
 namespace brick {
 
-struct Pair {
-  float s, c;
-  __device__ __forceinline__ void add(float x, float e = 0.f) {
-    const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
-    c = __fadd_rn(__fadd_rn(c, e), __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
-    s = t;
+// a sum in three floats: value, accumulated rounding errors (Knuth's two-sum), and theirs
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+  return t;
+}
+struct Sum3 {
+  float s, c, d;
+  __device__ __forceinline__ void add(float x) {
+    float e, f;
+    s = two_sum(s, x, e);
+    c = two_sum(c, e, f);
+    d = __fadd_rn(d, f);
   }
+  __device__ __forceinline__ void add(float x, float y, float z) {   // the same in either order
+    float e, f, g;
+    s = two_sum(s, x, e);
+    c = two_sum(c, y, f);
+    c = two_sum(c, e, g);
+    d = __fadd_rn(__fadd_rn(d, z), __fadd_rn(f, g));
+  }
+  __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)d); }
 };
-__device__ __forceinline__ Pair warp_sum(Pair p) {
+__device__ __forceinline__ Sum3 warp_sum(Sum3 p) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float s = __shfl_xor_sync(0xffffffffu, p.s, o), c = __shfl_xor_sync(0xffffffffu, p.c, o);
-    // both lanes add the lower lane's value first: the same result in both
-    const bool up = threadIdx.x & o;
-    Pair q{up ? s : p.s, up ? c : p.c};
-    q.add(up ? p.s : s, up ? p.c : c);
-    p = q;
-  }
+  for (int o = 16; o > 0; o >>= 1)
+    p.add(__shfl_xor_sync(0xffffffffu, p.s, o), __shfl_xor_sync(0xffffffffu, p.c, o),
+          __shfl_xor_sync(0xffffffffu, p.d, o));
   return p;
 }
-// the sum over all CTAs of the threads' pairs (slot: the words of this reduction)
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+constexpr int kParts = 5;   // CTAs per lane and round: one round on 152 SMs
+struct Shared {
+  Sum3 warp[32], total;
+  int pass, dead;
+};
+// the sum over all CTAs of the threads' sums (words: those of this reduction).  A CTA's sum travels
+// as one FP64 number; one warp per CTA fetches all of them, all missing ones in flight at once, and
+// adds them in FP64.  us per iteration, with every thread polling one word and FP32 pairs / so:
+// 16^3 7.8 / 9.8, 32^3 8.0 / 8.8, 64^3 12.3 / 10.1, 96^3 13.5 / 10.6, 128^3 17.1 / 15.2 (fewer pollers;
+// the small grids see the FP64 adds' latency).  sh.pass: the total is at most tol2.
 // (*stop: a wait gave up, the same for all threads)
-__device__ __forceinline__ Pair all_sum(Pair p, ulonglong2* words, int ctas, uint32_t tag, Pair* scr,
-                                        volatile int* dead, int* err, int* stop) {
+__device__ __forceinline__ Sum3 all_sum(Sum3 p, ulonglong2* words, int ctas, uint32_t tag, double tol2, Shared& sh,
+                                        int* err, int* stop) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  volatile int* const dead = &sh.dead;
   p = warp_sum(p);
-  if (lane == 0) scr[warp] = p;
+  if (lane == 0) sh.warp[warp] = p;
   __syncthreads();
   if (warp == 0) {
-    Pair q = lane < nw ? scr[lane] : Pair{0.f, 0.f};
-    q = warp_sum(q);
+    const Sum3 q = warp_sum(lane < nw ? sh.warp[lane] : Sum3{0.f, 0.f, 0.f});
     if (lane == 0) {
-      const unsigned long long t = (unsigned long long)tag << 32;
+      const unsigned long long t = (unsigned long long)tag << 32, b = __double_as_longlong(q.value());
       asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(words + blockIdx.x),
-                   "l"(t | __float_as_uint(q.s)), "l"(t | __float_as_uint(q.c))
+                   "l"(t | (b >> 32)), "l"(t | (b & 0xffffffffull))
                    : "memory");
     }
-  }
-  Pair q{0.f, 0.f};
-  for (int i = threadIdx.x; i < ctas; i += blockDim.x) {
-    uint32_t t0 = 0;
-    for (uint32_t it = 1; !*dead; ++it) {
-      const ulonglong2 v = ld_words(words + i);
-      if ((uint32_t)(v.x >> 32) == tag && (uint32_t)(v.y >> 32) == tag) {
-        q.add(__uint_as_float((uint32_t)v.x), __uint_as_float((uint32_t)v.y));
-        break;
+    double v = 0.0;
+    for (int i0 = lane; i0 < ctas; i0 += 32 * kParts) {
+      ulonglong2 w[kParts];
+      uint32_t need = 0, t0 = 0;
+#pragma unroll
+      for (int k = 0; k < kParts; ++k) {
+        w[k] = make_ulonglong2(0, 0);
+        if (i0 + 32 * k < ctas) need |= 1u << k;
       }
-      if ((it & 63u) == 0 && !keep_waiting(t0, dead, err)) break;
+      for (uint32_t it = 1; need && !*dead; ++it) {
+#pragma unroll
+        for (int k = 0; k < kParts; ++k)
+          if (need >> k & 1u) w[k] = ld_words(words + i0 + 32 * k);
+#pragma unroll
+        for (int k = 0; k < kParts; ++k)
+          if ((uint32_t)(w[k].x >> 32) == tag && (uint32_t)(w[k].y >> 32) == tag) need &= ~(1u << k);
+        if (need && (it & 63u) == 0 && !keep_waiting(t0, dead, err)) break;
+      }
+#pragma unroll
+      for (int k = 0; k < kParts; ++k) v += __longlong_as_double((long long)(w[k].x << 32 | (w[k].y & 0xffffffffull)));
+    }
+    v = warp_sum(v);
+    if (lane == 0) {
+      const float a = (float)v;
+      sh.total = Sum3{a, (float)(v - (double)a), 0.f};
+      sh.pass = v <= tol2;
     }
   }
-  q = warp_sum(q);
-  Pair* const scr2 = scr + 32;
-  if (lane == 0) scr2[warp] = q;
   *stop = __syncthreads_or(*dead);
-  Pair r = scr2[0];
-  const int n = min(nw, (ctas + 31) / 32);
-  for (int w = 1; w < n; ++w) r.add(scr2[w].s, scr2[w].c);
-  return r;
+  return sh.total;
 }
 // a / b in one rounding or so
-__device__ __forceinline__ float ratio(Pair a, Pair b) {
+__device__ __forceinline__ float ratio(const Sum3& a, const Sum3& b) {
   const float q = __fdiv_rn(a.s, b.s);
   return q + __fdiv_rn(fmaf(-q, b.s, a.s) + fmaf(-q, b.c, a.c), b.s);
 }
@@ -86,16 +120,14 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
   using X = Ctx<BZ>;
   constexpr int PE = X::PE;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int dead_s;
-  __shared__ Pair scr[64];
+  __shared__ Shared sh;
   if (sticky_error(a.err)) return;
   float4* const f = reinterpret_cast<float4*>(smem);
-  volatile int* dead = &dead_s;
+  volatile int* dead = &sh.dead;
   const Geo g(a);
   const X c(g, a.halo, a.by, a.py, a.pz, a.ny, a.nz);
   const int tid = g.tid, nq = g.nq, ctas = a.py * a.pz;
-  if (tid == 0) dead_s = 0;
-  if (tid < 64) scr[tid] = Pair{0.f, 0.f};
+  if (tid == 0) sh.dead = 0;
   c.clear(f);
   ulonglong2* const red = c.wd.base + (2 * (size_t)ctas * (4 * X::TP) + 2 * (size_t)ctas * 4 * BZ * nq);
   const bool y0 = g.y > 0, y1 = g.y + 1 < a.ny, x0 = g.q > 0, x1 = g.q < nq - 1;
@@ -113,7 +145,7 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
     }
   }
   c.publish_z(g, f, 0, a.tag);
-  Pair rr{a.rr_hi, a.rr_lo};
+  Sum3 rr{a.rr_hi, a.rr_lo, 0.f};
   int it = 0, ok = 0, stop = 0;
 #pragma unroll 1
   while (it < a.max_iter) {
@@ -121,7 +153,7 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
     const uint32_t tag = a.tag + it;
     const float4 below = v4(c.template receive_halos<true>(g, f, a.by, a.py, par, tag, dead, a.err));
     // ---- v = A p and p.v
-    Pair acc{0.f, 0.f};
+    Sum3 acc{0.f, 0.f, 0.f};
     float4 zm = below;
 #pragma unroll
     for (int k = 0; k < BZ; ++k) {
@@ -150,10 +182,10 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
         acc.add(fmaf(p.x, o[0], fmaf(p.y, o[1], fmaf(p.z, o[2], p.w * o[3]))));
       zm = p;
     }
-    const Pair pap = all_sum(acc, red + (size_t)par * ctas, ctas, tag, scr, dead, a.err, &stop);
+    const Sum3 pap = all_sum(acc, red + (size_t)par * ctas, ctas, tag, a.tol2, sh, a.err, &stop);
     const float al = pap.s > 0.f ? ratio(rr, pap) : 0.f;
     // ---- x += a p, r -= a A p and r.r
-    acc = Pair{0.f, 0.f};
+    acc = Sum3{0.f, 0.f, 0.f};
 #pragma unroll
     for (int k = 0; k < BZ; ++k) {
       if (!(c.bits >> k & 1u)) continue;
@@ -162,9 +194,9 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
       r[k].x -= al * v[k].x; r[k].y -= al * v[k].y; r[k].z -= al * v[k].z; r[k].w -= al * v[k].w;
       acc.add(fmaf(r[k].x, r[k].x, fmaf(r[k].y, r[k].y, fmaf(r[k].z, r[k].z, r[k].w * r[k].w))));
     }
-    const Pair rn = all_sum(acc, red + (size_t)(2 + par) * ctas, ctas, tag, scr, dead, a.err, &stop);
+    const Sum3 rn = all_sum(acc, red + (size_t)(2 + par) * ctas, ctas, tag, a.tol2, sh, a.err, &stop);
     const bool last = it + 1 == a.max_iter;
-    if (((it & 7) == 7 || last) && (rn.s - a.tol_hi) + (rn.c - a.tol_lo) <= 0.f) ok = 1;
+    if (((it & 7) == 7 || last) && sh.pass) ok = 1;
     const float be = rr.s > 0.f ? ratio(rn, rr) : 0.f;
     rr = rn;
     ++it;

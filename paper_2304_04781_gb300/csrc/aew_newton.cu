@@ -750,7 +750,7 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   // solve for the unit-rms right-hand side sc w (the iteration's FP32 squares then stay
   // far from FP32's range limits), and scale x back at the end
   const double sc = std::sqrt((double)g.C / ww);
-  // on chip where the grid fits: 128^3 45 -> 17 us per iteration, 64^3 37 -> 12
+  // on chip where the grid fits: 128^3 45 -> 15 us per iteration, 64^3 37 -> 10
   if (chip) {
     const double rr = ww * (double)(float)sc * (double)(float)sc, t2 = rtol * rtol * rr;
     BrickCg a{};
@@ -765,8 +765,7 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
     a.inv_sc = (float)(1.0 / sc);
     a.rr_hi = (float)rr;
     a.rr_lo = (float)(rr - (double)a.rr_hi);
-    a.tol_hi = (float)t2;
-    a.tol_lo = (float)(t2 - (double)a.tol_hi);
+    a.tol2 = t2;
     a.max_iter = max_iter;
     a.result = done;
     NW_CK(cudaMemsetAsync(done, 0, 2 * sizeof(int), s));
