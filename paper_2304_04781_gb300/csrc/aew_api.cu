@@ -2687,7 +2687,7 @@ int set_error(aew_handle* h, int code, const std::string& msg) { return fail(h, 
 
 bool brick_of(aew_handle* h, BrickRef* b) {
   if (!on_chip(h)) return false;
-  *b = BrickRef{&h->bp, h->halo, &h->halo_tag, codec_err_flag(h->codec)};
+  *b = BrickRef{&h->bp, h->halo, &h->halo_tag, codec_err_flag(h->codec), {h->st[0][0], h->st[0][1]}};
   return true;
 }
 

@@ -100,18 +100,22 @@ struct BrickAdj {
   int* err;
 };
 
-// CG for A x = w of the prior's operator (aew_newton.cu), one launch for the whole solve:
+// CG for A x = w of the prior's operator (aew_newton.cu), up to max_iter iterations in one launch:
 // r = sc w at the start, x scaled by 1 / sc at the end; the residual test every 8 iterations
-// (and after the last): r.r <= tol2.
+// (and after the last): r.r <= tol2.  Where more iterations may follow (more; max_iter is then a
+// multiple of 8) a launch that did not pass leaves x unscaled, r, p and r.r for the next one (resume).
 struct BrickCg {
   const float* w;
   float* x;
+  float* r;                // between launches
+  float* p;
+  bool resume, more;
   int nx, ny, nz;
   float alpha, at, sc, inv_sc;
   float rr_hi, rr_lo;      // r.r at the start, as a pair of floats
   double tol2;
   int max_iter;
-  int* result;             // device [2]: iterations, 1 if the test passed
+  int* result;             // device [4]: iterations, 1 if the test passed, r.r as a pair of floats
   int by, bz, py, pz;
   unsigned char* halo;
   uint32_t tag;

@@ -138,14 +138,26 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
   for (int k = 0; k < BZ; ++k) {
     x[k] = r[k] = z4();
     if (c.bits >> k & 1u) {
-      const float4 w = ldg4(a.w + (g.row + k * g.P));
-      r[k] = make_float4(a.sc * w.x, a.sc * w.y, a.sc * w.z, a.sc * w.w);
-      E[k * PE] = r[k];   // p = r
-      if (c.fl & (kLow | kHi)) c.publish_y(g, r[k], a.by, 0, a.tag, k);
+      const uint32_t i = g.row + k * g.P;
+      float4 p;
+      if (a.resume) {
+        x[k] = *reinterpret_cast<const float4*>(a.x + i);
+        r[k] = *reinterpret_cast<const float4*>(a.r + i);
+        p = *reinterpret_cast<const float4*>(a.p + i);
+      } else {
+        const float4 w = ldg4(a.w + i);
+        p = r[k] = make_float4(a.sc * w.x, a.sc * w.y, a.sc * w.z, a.sc * w.w);
+      }
+      E[k * PE] = p;
+      if (c.fl & (kLow | kHi)) c.publish_y(g, p, a.by, 0, a.tag, k);
     }
   }
   c.publish_z(g, f, 0, a.tag);
   Sum3 rr{a.rr_hi, a.rr_lo, 0.f};
+  if (a.resume) {
+    rr.s = __int_as_float(a.result[2]);
+    rr.c = __int_as_float(a.result[3]);
+  }
   int it = 0, ok = 0, stop = 0;
 #pragma unroll 1
   while (it < a.max_iter) {
@@ -200,7 +212,7 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
     const float be = rr.s > 0.f ? ratio(rn, rr) : 0.f;
     rr = rn;
     ++it;
-    if (ok || last || stop) break;   // stop: the values are void, and the error flag is set
+    if (ok || (last && !a.more) || stop) break;   // stop: the values are void, and the error flag is set
     // ---- p = r + b p
 #pragma unroll
     for (int k = 0; k < BZ; ++k) {
@@ -209,9 +221,26 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
       const float4 q = make_float4(fmaf(be, p.x, r[k].x), fmaf(be, p.y, r[k].y), fmaf(be, p.z, r[k].z),
                                    fmaf(be, p.w, r[k].w));
       E[k * PE] = q;
-      if (c.fl & (kLow | kHi)) c.publish_y(g, q, a.by, par ^ 1, tag + 1, k);
+      if (!last && (c.fl & (kLow | kHi))) c.publish_y(g, q, a.by, par ^ 1, tag + 1, k);
     }
-    c.publish_z(g, f, par ^ 1, tag + 1);
+    if (!last) c.publish_z(g, f, par ^ 1, tag + 1);
+  }
+  if (a.more && !ok) {   // to go on with
+#pragma unroll
+    for (int k = 0; k < BZ; ++k)
+      if (c.bits >> k & 1u) {
+        const uint32_t i = g.row + k * g.P;
+        st4(a.x, i, x[k]);
+        st4(a.r, i, r[k]);
+        st4(a.p, i, E[k * PE]);
+      }
+    if (blockIdx.x == 0 && tid == 0) {
+      a.result[0] = it;
+      a.result[1] = 0;
+      a.result[2] = __float_as_int(rr.s);
+      a.result[3] = __float_as_int(rr.c);
+    }
+    return;
   }
 #pragma unroll
   for (int k = 0; k < BZ; ++k)
@@ -227,7 +256,8 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
 
 cudaError_t launch_brick_cg(BrickCg a, const BrickPlan& p, unsigned char* halo, uint32_t* tag, int* err,
                             cudaStream_t s) {
-  if (!halo || !err || a.max_iter < 1) return cudaErrorInvalidValue;
+  if (!halo || !err || a.max_iter < 1 || (a.more && a.max_iter % 8) || ((a.more || a.resume) && (!a.r || !a.p)))
+    return cudaErrorInvalidValue;
   const cudaError_t e = brick_tags(tag, (uint32_t)a.max_iter, a.nx, p, halo, s);
   if (e != cudaSuccess) return e;
   a.by = p.by;
@@ -235,7 +265,8 @@ cudaError_t launch_brick_cg(BrickCg a, const BrickPlan& p, unsigned char* halo, 
   a.py = p.py;
   a.pz = p.pz;
   a.halo = halo;
-  a.tag = *tag + 1;   // the caller moves the tag on by the iterations taken
+  a.tag = *tag + 1;
+  *tag += (uint32_t)a.max_iter + 1;
   a.err = err;
   switch (p.bz) {
     case 1: return brick::launch_coop<brick::cg_kernel<1>>(a, p, s);

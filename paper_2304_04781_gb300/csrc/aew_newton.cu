@@ -25,6 +25,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
+#include <cstdlib>
 #include <string>
 #include <vector>
 
@@ -702,6 +703,14 @@ int prior_args_ok(aew_handle* h, double alpha, double theta) {
   return AEW_OK;
 }
 
+// iterations per launch of the on-chip solve, a multiple of 8
+constexpr int kCgRun = 1024;
+int cg_run() {
+  const char* env = getenv("AEW_PRIOR_RUN");   // tuning override
+  const int n = env ? atoi(env) : 0;
+  return n > 0 ? (n + 7) / 8 * 8 : kCgRun;
+}
+
 int no_convergence(aew_handle* h, double rtol, int iters) {
   char buf[160];
   std::snprintf(buf, sizeof buf, "prior solve: relative residual above %.3g after %d iterations", rtol, iters);
@@ -723,7 +732,7 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   BrickRef br;
   const bool chip = brick_of(h, &br);
   if ((!chip && (!ws.alloc(&r, g.C) || !ws.alloc(&p[0], g.C) || !ws.alloc(&p[1], g.C))) ||
-      !ws.alloc(&part, 3 * (size_t)np) || !ws.alloc(&done, 2) || (!chip && !ws.alloc_host(&seen, 2)))
+      !ws.alloc(&part, 3 * (size_t)np) || !ws.alloc(&done, 4) || (!chip && !ws.alloc_host(&seen, 2)))
     return set_error(h, AEW_E_NOMEM, "prior solve: work vectors do not fit");
   double* ppap = part;
   double* prr[2] = {part + np, part + 2 * (size_t)np};
@@ -766,17 +775,28 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
     a.rr_hi = (float)rr;
     a.rr_lo = (float)(rr - (double)a.rr_hi);
     a.tol2 = t2;
-    a.max_iter = max_iter;
+    a.r = br.scratch[0];
+    a.p = br.scratch[1];
     a.result = done;
-    NW_CK(cudaMemsetAsync(done, 0, 2 * sizeof(int), s));
-    NW_CK(launch_brick_cg(a, *br.plan, br.halo, br.tag, br.err, s));
-    int got[2] = {0, 0};
-    NW_CK(cudaMemcpyAsync(got, done, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-    const bool timeout = take_timeout(h, s);   // synchronises
-    *br.tag += (uint32_t)std::max(got[0], 0) + 3;   // no CTA is more than an iteration ahead
-    if (timeout) return set_error(h, AEW_E_TIMEOUT, "a kernel gave up waiting (bounded halo wait)");
-    if (iters) *iters = got[0];
-    return got[1] ? AEW_OK : no_convergence(h, rtol, got[0]);
+    NW_CK(cudaMemsetAsync(done, 0, 4 * sizeof(int), s));
+    // launches of kCgRun iterations, about 15 ms at most: a tolerance that is never reached does not
+    // hold the GPU for the whole of a large max_iter
+    int it = 0, ok = 0;
+    const int run = cg_run();
+    while (!ok && it < max_iter) {
+      a.max_iter = std::min(run, max_iter - it);
+      a.more = it + a.max_iter < max_iter;
+      a.resume = it > 0;
+      NW_CK(launch_brick_cg(a, *br.plan, br.halo, br.tag, br.err, s));
+      int got[2] = {0, 0};
+      NW_CK(cudaMemcpyAsync(got, done, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+      if (take_timeout(h, s))   // synchronises
+        return set_error(h, AEW_E_TIMEOUT, "a kernel gave up waiting (bounded halo wait)");
+      it += got[0];
+      ok = got[1];
+    }
+    if (iters) *iters = it;
+    return ok ? AEW_OK : no_convergence(h, rtol, it);
   }
   cg_start_kernel<<<nb, NT, 0, s>>>(w, (float)sc, r, x, g.C);
   NW_CK(cudaMemsetAsync(done, 0xff, sizeof(int), s));   // -1: not yet

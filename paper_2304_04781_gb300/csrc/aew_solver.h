@@ -20,12 +20,14 @@ struct GridInfo {
 
 GridInfo grid_of(const aew_handle* h);
 
-// where the handle's grid runs on chip: its cut, halo buffer, running tag and error flag
+// where the handle's grid runs on chip: its cut, halo buffer, running tag and error flag, and two
+// fields that are free between solves
 struct BrickRef {
   const BrickPlan* plan;
   unsigned char* halo;
   uint32_t* tag;
   int* err;
+  float* scratch[2];
 };
 bool brick_of(aew_handle* h, BrickRef* b);
 // a bounded wait of the handle's kernels gave up since the last look (synchronises)
