@@ -45,17 +45,28 @@ constexpr uint64_t kWaitNs = 2000000000ull;
 constexpr int kSmemMax = 232448;   // 227 KB
 constexpr int kMaxBz = 8;
 
-// thread limit of a BZ-plane kernel: two to three float4 of state per plane and about 45
-// working registers have to fit 65,536 / threads
+// Limits and layout by depth.  Each depth is compiled for itself, so the tables trade registers
+// (65,536 per SM), shared memory (smem_bytes below) and barriers; bytes spilled per thread are
+// -Xptxas -v's for the FP32 adjoint, the tightest kernel of each depth.
+// Threads: a kernel needs about 45 working registers and 8 to 12 per plane, so two planes fit
+// 65,536 / 640 = 102 registers, up to seven 128, eight 168.
 __host__ __device__ constexpr int tmax(int bz) {
   return bz <= 2 ? 640 : bz <= 7 ? 512 : 384;
 }
-// longest x row, in float4
+// Longest x row, in float4: the exchanged field holds two rows beyond the brick and the y faces one
+// in every plane.  128 (512 nodes) where that is a small part; 64 from five planes on; at seven only
+// 32 fits beside four shared planes of the third field (225,216 of 231,424 B; 64 would take 236,992).
 __host__ __device__ constexpr int nqmax(int bz) { return bz <= 4 ? 128 : bz == 7 ? 32 : 64; }
-// planes per chunk of the forward and the adjoint kernels
+// Planes per chunk of the forward and the adjoint kernels: a chunk is a barrier, so two where the
+// registers of a second plane's faces are there.  In the adjoint they are up to four planes (from
+// five on two would spill 64 B for 8, 204 for 72, 340 for 184, 48 for 0), in the forward kernel up to
+// five (six would spill 44 B for 20, seven 88 for 56), with dm e^n in flight up to four.
 __host__ __device__ constexpr int zc(int bz, bool incr) { return bz <= 2 ? bz : bz <= (incr ? 4 : 5) ? 2 : 1; }
 __host__ __device__ constexpr int zca(int bz) { return bz <= 1 ? bz : bz <= 4 ? 2 : 1; }
-// planes whose third register field (e, or the accumulator) lives in shared memory instead
+// Planes whose third register field (e, or the accumulator) lives in shared memory instead, each for
+// 16 B per thread and access: two at five planes (8 B spilled; 44 with none), three at six (72; 212
+// with none, 24 with a fourth, which was not timed), four at seven, as many as fit (184; 372 with
+// none), two at eight (0; 44 with none).
 __host__ __device__ constexpr int ks(int bz) { return bz == 5 || bz == 8 ? 2 : bz == 6 ? 3 : bz == 7 ? 4 : 0; }
 // row pitches (float4) of the exchanged field (a halo row on both sides), of the y faces (one
 // below) and of the private fields: constants, so that plane offsets are immediates

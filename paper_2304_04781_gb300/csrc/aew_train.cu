@@ -627,7 +627,9 @@ cudaError_t launch_t(long long M, int N, int K, const gemm::Mat& A, const gemm::
   if (N >= 128 && mt * (N / 128) >= sms) return gemm::launch<128, BF16>(M, N, K, A, B, ep, err, st, 0, 0, true);
   return gemm::launch<64, BF16>(M, N, K, A, B, ep, err, st, 0, kTrainStages, true);
 }
-// a weight gradient and the activation gradient that needs the same input, in one launch
+// a weight gradient and the activation gradient that needs the same input, in one launch of
+// 64-column tiles.  On wide batches too: with the activation gradient in a launch of its own on 256-
+// column tiles a step of the time codec takes 507 us for 502 at batch 4096, 901 for 876 at 8192.
 template <class EP1, class EP2>
 cudaError_t launch_pair(long long M1, int N1, int K1, const gemm::Mat& A1, const gemm::Mat& B1, const EP1& e1,
                         long long M2, int N2, int K2, const gemm::Mat& A2, const gemm::Mat& B2, const EP2& e2,

@@ -582,7 +582,8 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
   if (sticky_error(a.err)) return;
   const Place p(cut, a.ny, a.nz);
   const int W = cut.W, R = cut.rows, tid = threadIdx.x, warp = tid >> 5;
-  constexpr int NE = INCR ? 4 : 2;   // extra fields of the m e row: e, m (dm, e of the step)
+  static_assert(INCR == 1 || INCR == 2, "");
+  constexpr int NE = 4;   // extra fields of the m e row: e, m, dm, e of the step
   // plane buffers, rows W apart: me0 [R + 1], vy1 [1 + R], me1 [R], vy2 [1 + R]; every index is
   // rounded up to whole threads
   float4* const sa = reinterpret_cast<float4*>(smem);
@@ -600,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
   const size_t i0 = p.valid ? (size_t)p.y * a.nx + p.i0 : 0;
   const int nz = a.nz;
   const bool live_q = p.gq >= 0 && p.gq < cut.nq;
-  const bool has_ef0 = INCR && (a.ef[0] || a.ef16[0]), has_ef1 = INCR && (a.ef[1] || a.ef16[1]);
+  const bool has_ef0 = a.ef[0] || a.ef16[0], has_ef1 = a.ef[1] || a.ef16[1];
   // rare work: the columns meet the source box; the quad has receivers
   const bool src = a.sk >= 0 && p.valid && abs(p.y - a.sj) <= a.sr && p.i0 + 3 >= a.si - a.sr &&
                    p.i0 <= a.si + a.sr;
@@ -620,11 +621,9 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
     const bool v = ok(k);
     const size_t i = i0 + (size_t)k * P;
     r.m = ldz(a.m + i, v);
-    if (INCR) {
-      r.dm = ldz(a.dm + i, v);
-      if (INCR == 1) r.f32 = ldz(a.ef[s] + i, v && a.ef[s]);
-      else r.f16 = v && a.ef16[s] ? __ldg(reinterpret_cast<const uint2*>(a.ef16[s] + i)) : make_uint2(0u, 0u);
-    }
+    r.dm = ldz(a.dm + i, v);
+    if (INCR == 1) r.f32 = ldz(a.ef[s] + i, v && a.ef[s]);
+    else r.f16 = v && a.ef16[s] ? __ldg(reinterpret_cast<const uint2*>(a.ef16[s] + i)) : make_uint2(0u, 0u);
   };
   auto load_em = [&](int k) {
     Raw r;
@@ -633,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
     return r;
   };
   auto with_dm = [&](const Raw& r, F4 v, bool has) {
-    if (INCR && has) v = fma(f4(r.dm), f4(INCR == 2 ? bf4(r.f16) : r.f32), v);
+    if (has) v = fma(f4(r.dm), f4(INCR == 2 ? bf4(r.f16) : r.f32), v);
     return v;
   };
   auto me_of = [&](const Raw& r) { return with_dm(r, mul(f4(r.m), f4(r.e)), has_ef0); };
@@ -647,15 +646,13 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
       float4* d = (p.bot ? ex + s * (NE + 1) * W : eh + s * NE * W) + p.q;
       cp16(d, a.e + i, v);
       cp16(d + W, a.m + i, v);
-      if (INCR) {
-        cp16(d + 2 * W, a.dm + i, v);
-        if (has_ef0 && INCR == 1) cp16(d + 3 * W, a.ef[0] + i, v);
-        if (has_ef0 && INCR == 2) {   // BF16: 8 bytes
-          const uint32_t dd = tc::smem_u32(d + 3 * W);
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dd), "l"(a.ef16[0] + i),
-                       "r"(v ? 8 : 0)
-                       : "memory");
-        }
+      cp16(d + 2 * W, a.dm + i, v);
+      if (has_ef0 && INCR == 1) cp16(d + 3 * W, a.ef[0] + i, v);
+      if (has_ef0 && INCR == 2) {   // BF16: 8 bytes
+        const uint32_t dd = tc::smem_u32(d + 3 * W);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dd), "l"(a.ef16[0] + i),
+                     "r"(v ? 8 : 0)
+                     : "memory");
       }
       if (p.bot) cp16(d + NE * W, a.vy + i, v);
     }
@@ -665,7 +662,7 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
     const int s = (k + kRing) % kRing;
     const float4* d = (p.bot ? ex + s * (NE + 1) * W : eh + s * NE * W) + p.q;
     F4 v = mul_rn(d[W], d[0]);
-    if (INCR && has_ef0)
+    if (has_ef0)
       v = fma(lds(d + 2 * W), INCR == 2 ? f4(bf4(*reinterpret_cast<const uint2*>(d + 3 * W))) : lds(d + 3 * W), v);
     return v;
   };
