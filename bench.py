@@ -36,12 +36,12 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "gradients/hour at 256^3x2000 steps: AE vs checkpointing; stencil HBM GB/s"
-# DRAM bytes (read + write) of one adjoint-step launch at 256^3, from an ncu capture of
-# the current kernel (dram__bytes_read.sum + dram__bytes_write.sum, a window-middle step
-# without the FP64 flush); to be set to None when the kernel changes until it is
-# captured again
-ADJ_TRAFFIC_256 = 701.6e6     # FP32 e^n (full storage / checkpointing)
-ADJ16_TRAFFIC_256 = 665.5e6   # BF16 e^n (the time codec's adjoint sweeps)
+# DRAM bytes (read + write) of one adjoint launch at 256^3, from an ncu capture of the
+# current kernel (window-middle, without the FP64 flush); to be taken out when the kernel
+# changes until it is captured again
+TRAFFIC_256 = {"adjoint": 701.6e6,        # FP32 e^n (full storage / checkpointing)
+               "adjoint_bf16": 665.5e6,   # BF16 e^n (the time codec's adjoint sweeps)
+               "adjoint_bf16_two": 782.8e6}   # two steps per pass
 SHAPE = (256, 256, 256)
 NT = 2000
 NREC = 128
@@ -81,7 +81,9 @@ def parse():
     p.add_argument("--kernel", default="",
                    choices=["", "forward", "forward_pack", "adjoint", "incremental",
                             "encode_window", "decode_window", "adjoint_bf16",
-                            "decode_window_bf16", "incremental_bf16", "decode_state"],
+                            "decode_window_bf16", "incremental_bf16", "decode_state",
+                            "forward_two", "forward_pack_two", "adjoint_two", "adjoint_bf16_two",
+                            "incremental_bf16_two", "forward_chip", "adjoint_bf16_chip"],
                    help="instead of the benchmark: time one hot-path kernel alone "
                         "(aew_profile_steps) on an AE handle of --shape, for profiling")
     p.add_argument("--launches", type=int, default=16)
@@ -297,7 +299,40 @@ BYTES_PER_NODE = {
     "adjoint_bf16": 48.0,   # the same with e^n read as BF16 (the time codec's sweeps)
     "incremental": 44.0,    # forward + dm, e^n
     "incremental_bf16": 42.0,   # the same with e^n read as BF16 (the time codec's GN-HVP)
+    # passes of two steps
+    "forward_two": 36.0,
+    "forward_pack_two": 40.0,       # + both strains as BF16
+    "adjoint_two": 56.0,            # both e^n; the FP64 read-modify-write every 4 passes
+    "adjoint_bf16_two": 52.0,
+    "incremental_bf16_two": 44.0,   # + dm, both e^n
+    # on chip, 16 steps per launch: the state once in and out, m, and the strains
+    "forward_chip": 36.0,
+    "adjoint_bf16_chip": 100.0,     # 16 e^n, and two FP64 read-modify-writes
 }
+# the pass of a gradient that takes the longest, by the route of the solves and the codec, and
+# how its kernel is called
+DOMINANT = {
+    ("two", "time"): ("adjoint_bf16_two", "two::adjoint_kernel: two adjoint steps per pass, decoded strain as BF16"),
+    ("chip", "time"): ("adjoint_bf16_chip", "brick::adj_kernel: 16 adjoint steps per launch, the state on chip "
+                                            "(bound by its L2 exchanges, not by HBM)"),
+    ("single", "time"): ("adjoint_bf16", "adj_tma_kernel: one adjoint step, decoded strain as BF16"),
+    ("single", "space"): ("adjoint", "adj_tma_kernel: one adjoint step"),
+}
+
+
+def route_of(before: dict, after: dict) -> str:
+    """The kernels that ran the time steps between two Solver.routes(): 'two', 'chip' or
+    'single', whichever ran the most steps (an on-chip run is many)."""
+    n = {k: after[k] - before[k] for k in after}
+    if n["chip"]:
+        return "chip"
+    return "two" if n["two"] * 2 > n["single"] else "single"
+
+
+def codec_ctas(route: str, sms: int) -> int:
+    """CTAs of the codec's products in the solves: half the SMs beside single steps, all of them
+    between two-step passes and where the steps run on chip (then nothing runs beside them)."""
+    return sms // 2 if route == "single" else sms
 
 
 def codec_flops_per_window(nvec: int, n_lat: int, n_hid: int) -> dict:
@@ -344,6 +379,7 @@ def run_ours(args):
         shots(ae)
     torch.cuda.synchronize()
     l0 = ae.stats()["kernel_launches"]
+    routes0 = ae.routes()
     barrier(world)
     torch.cuda.synchronize()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -356,6 +392,7 @@ def run_ours(args):
     barrier(world)
     ms = e0.elapsed_time(e1) / args.steps
     launches = ae.stats()["kernel_launches"] - l0
+    route = route_of(routes0, ae.routes())
     ms_max = reduce_max(ms, world, torch.device("cuda", local))
     value = world * 3600e3 / ms_max
     g_ae = g.clone()
@@ -430,9 +467,15 @@ def run_ours(args):
     # ---- the hot-path kernels alone (CUDA events around back-to-back launches)
     nprof = min(nt, 200)
     kernels = {}
+    # single steps (odd last steps, the space codec's and the full Newton's solves), then the
+    # kernels of the timed gradients
     kinds = ["forward", "adjoint", "incremental"] + (["forward_pack", "adjoint_bf16",
                                                       "incremental_bf16"]
                                                      if args.codec == "time" else [])
+    if route == "two":
+        kinds += ["forward_two", "forward_pack_two", "adjoint_two", "adjoint_bf16_two", "incremental_bf16_two"]
+    if route == "chip" and nt >= 32:
+        kinds += ["forward_chip", "adjoint_bf16_chip"]
     for kind in kinds:
         kms = ae.profile(c, kind, nprof)
         b = BYTES_PER_NODE[kind] * C
@@ -441,8 +484,7 @@ def run_ours(args):
     if args.codec == "time":
         fl = codec_flops_per_window(ae.nvec, n_lat, ae.n_hid)
         sms = torch.cuda.get_device_properties(local).multi_processor_count
-        # the codec GEMMs' CTA cap: none between two-step passes (grids beyond the SMs)
-        ctas = sms if C > 4_000_000 else sms // 2
+        ctas = codec_ctas(route, sms)
         share = ctas / sms
         for kind, prof in (("encode_window", "encode_window"), ("decode_window", "decode_window_bf16")):
             kms = ae.profile(c, prof, 8)
@@ -552,7 +594,12 @@ def run_ours(args):
                "sample": what}
 
     if rank == 0:
-        dom = kernels["adjoint_bf16" if args.codec == "time" else "adjoint"]
+        kind, dom_name = DOMINANT[route, args.codec]
+        if kind not in kernels:   # an on-chip run shorter than the hook's 32 steps
+            kind, dom_name = DOMINANT["single", args.codec]
+        dom = kernels[kind]
+        steps_per_launch = {"two": 2, "chip": 16}.get(kind.rsplit("_", 1)[-1], 1)
+        fwd = kernels["forward" + {"two": "_two", "chip": "_chip"}.get(kind.rsplit("_", 1)[-1], "")]
         line = {
             "metric": METRIC, "value": value, "unit": "gradients/hour", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_max,
@@ -564,25 +611,17 @@ def run_ours(args):
                                                      f"summed by one all-reduce") if world > 1
                            else "one shot on one GPU"),
             "accuracy": accuracy,
-            "roofline": {"kernel": "single adjoint step (adj_tma_kernel, the kernel of odd last "
-                                   "steps; the solves take two steps per pass)" + (", reading its decoded strain as BF16 "
-                                                           "(48 B/node)" if args.codec == "time"
-                                                           else ""), "bound": "hbm",
+            "roofline": {"kernel": dom_name, "route": route, "steps_per_launch": steps_per_launch, "bound": "hbm",
                          "achieved": dom["achieved_gbs"], "peak": hbm_peak, "unit": "GB/s",
                          "frac": dom["achieved_gbs"] / hbm_peak,
                          "peak_kind": f"{peak_kind} copy bandwidth (burst: kernel timed alone)",
-                         "traffic": ((ADJ16_TRAFFIC_256 if args.codec == "time" else ADJ_TRAFFIC_256)
-                                     if shape == SHAPE else None),
-                         "traffic_source": "ncu capture of a window-middle adjoint step at 256^3 "
-                                           + ("(profiles/adj_tma_kernel_bf16_256cubed.md)"
-                                              if args.codec == "time" else
-                                              "(profiles/adj_tma_kernel_256cubed.md)"),
+                         "traffic": TRAFFIC_256.get(kind) if shape == SHAPE else None,
+                         "traffic_source": "ncu capture of a window-middle pass at 256^3 (profiles/)",
                          "bytes_per_launch": dom["bytes_per_launch"],
                          "timing": f"CUDA events around {nprof} back-to-back launches"},
             "kernels": kernels,
-            "stencil": {"cell_updates_per_s": C / (kernels["forward"]["ms_per_launch"] / 1e3),
-                        "gbs": kernels["forward"]["achieved_gbs"],
-                        "frac_of_8tbs": kernels["forward"]["achieved_gbs"] / 8000.0},
+            "stencil": {"cell_updates_per_s": steps_per_launch * C / (fwd["ms_per_launch"] / 1e3),
+                        "gbs": fwd["achieved_gbs"], "frac_of_8tbs": fwd["achieved_gbs"] / 8000.0},
             "revolve": {"gradients_per_hour": 3600e3 / rev_ms, "ms_per_gradient": rev_ms,
                         "forward_steps": rev_fwd, "slots": 20},
             "speedup_vs_revolve": rev_ms / ms_max,

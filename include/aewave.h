@@ -425,8 +425,13 @@ int aew_codec_init_pca(aew_handle* h, const uint16_t* vectors_dev, const float* 
  * (as the time codec's adjoint sweeps do; nx a multiple of 8), 7 decoder of one window
  * into BF16 strain slices, 8 incremental forward step reading its strain field as BF16,
  * 9 the space codec's fused strain decoder of one state (both layers, scattered to the
- * grid).  Kinds 1, 4, 5 and 7 need AE storage with the time codec, 9 with the space codec
- * (AEW_E_CONFIG otherwise), 4, 5, 7 and 9 codec weights.  Overwrites the handle's stored
+ * grid); passes of two steps per launch on grids beyond the on-chip ones: 10 forward, 11
+ * forward packing both strains into a window, 12 and 13 adjoint reading FP32 and BF16
+ * strain, 14 incremental reading BF16 strain; on chip 16 steps per launch: 15 forward, 16
+ * adjoint reading a decoded window (BF16).  Kinds 0-3, 6 and 8 are single steps whatever the
+ * solves take (aew_routes tells).  Kinds 1, 4, 5, 7, 11 and 16 need AE storage with the time
+ * codec, 9 with the space codec (AEW_E_CONFIG otherwise, as where the handle has no such
+ * passes), 4, 5, 7 and 9 codec weights.  Overwrites the handle's stored
  * history (a later aew_hessvec needs a new aew_gradient).  Synchronises the stream. */
 int aew_profile_steps(aew_handle* h, const float* c_dev, int kind, int nsteps, double* ms_host,
                       void* stream);

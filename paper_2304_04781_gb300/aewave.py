@@ -426,7 +426,10 @@ class Solver:
 
     PROFILE_KINDS = {"forward": 0, "forward_pack": 1, "adjoint": 2, "incremental": 3,
                      "encode_window": 4, "decode_window": 5, "adjoint_bf16": 6,
-                     "decode_window_bf16": 7, "incremental_bf16": 8, "decode_state": 9}
+                     "decode_window_bf16": 7, "incremental_bf16": 8, "decode_state": 9,
+                     "forward_two": 10, "forward_pack_two": 11, "adjoint_two": 12,
+                     "adjoint_bf16_two": 13, "incremental_bf16_two": 14, "forward_chip": 15,
+                     "adjoint_bf16_chip": 16}
 
     def profile(self, c: torch.Tensor, kind: str, nsteps: int) -> float:
         """aew_profile_steps: mean device ms per launch of one hot-path kernel."""

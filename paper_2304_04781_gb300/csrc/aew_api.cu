@@ -2460,15 +2460,19 @@ int aew_codec_init_pca(aew_handle* h, const uint16_t* vectors_dev, const float* 
 int aew_profile_steps(aew_handle* h, const float* c_dev, int kind, int nsteps, double* ms_host,
                       void* stream) {
   if (!h) return AEW_E_ARG;
-  if (kind < 0 || kind > 9 || nsteps < 1 || !ms_host) return fail(h, AEW_E_ARG, "bad argument");
+  if (kind < 0 || kind > 16 || nsteps < 1 || !ms_host) return fail(h, AEW_E_ARG, "bad argument");
   const bool tw = h->cfg.storage == AEW_AE && h->tcodec;
-  if ((kind == 1 || kind == 4 || kind == 5 || kind == 7) && !tw)
+  if ((kind == 1 || kind == 4 || kind == 5 || kind == 7 || kind == 11 || kind == 16) && !tw)
     return fail(h, AEW_E_CONFIG, "this kernel needs AE storage with the time codec");
   if (kind == 9 && !(h->cfg.storage == AEW_AE && !h->tcodec))
     return fail(h, AEW_E_CONFIG, "this kernel needs AE storage with the space codec");
   if ((kind == 4 || kind == 5 || kind == 7 || kind == 9) && !aew::codec_ready(h->codec))
     return fail(h, AEW_E_NOCODEC, "codec weights not set");
-  if ((kind == 6 || kind == 8) && h->cfg.nx % 8)
+  if (kind >= 10 && kind <= 14 && (!h->two || h->cfg.nt < 2))
+    return fail(h, AEW_E_CONFIG, "the grid takes no two-step passes (or nt < 2)");
+  if (kind >= 15 && (!on_chip(h) || h->cfg.nt < 2 * aew::kTSteps))
+    return fail(h, AEW_E_CONFIG, "the grid does not run on chip (or nt < 32)");
+  if ((kind == 6 || kind == 8 || kind == 13 || kind == 14) && h->cfg.nx % 8)
     return fail(h, AEW_E_CONFIG, "a BF16 strain field needs nx % 8 == 0");
   h->err.clear();
   cudaStream_t s = S(stream);
@@ -2476,6 +2480,7 @@ int aew_profile_steps(aew_handle* h, const float* c_dev, int kind, int nsteps, d
   if (rc) return rc;
   h->have_grad = false;
   const int nt = h->cfg.nt, T = aew::kTSteps;
+  const uint16_t* const st16 = reinterpret_cast<const uint16_t*>(h->st[0][0]);
   const Beside beside = on_chip(h) ? kAlone : beside_steps(h);   // as in the time codec's solves
   cudaEvent_t e0, e1;
   AEW_CK(cudaEventCreate(&e0));
@@ -2507,18 +2512,47 @@ int aew_profile_steps(aew_handle* h, const float* c_dev, int kind, int nsteps, d
         break;
       case 6:   // the adjoint step reading its strain field as BF16 (time-codec sweeps)
         rc = adj_step_x(h, nt - 1 - n, h->ad[cur], h->ad[cur ^ 1], h->R, nullptr, h->acc32,
-                        h->acc64, nullptr, nullptr, nullptr, s,
-                        reinterpret_cast<const uint16_t*>(h->st[0][0]));
+                        h->acc64, nullptr, nullptr, nullptr, s, st16);
         break;
       case 7:
         rc = decode_window(h, 0, s, beside);
         break;
       case 8:   // the incremental forward step reading its strain field as BF16
-        rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], nullptr, nullptr, s, nullptr, 0, nullptr,
-                       reinterpret_cast<const uint16_t*>(h->st[0][0]));
+        rc = incr_step(h, h->ad[cur], h->ad[cur ^ 1], nullptr, nullptr, s, nullptr, 0, nullptr, st16);
         break;
       case 9:   // the space codec's fused strain decoder, step 0's latents
         rc = decode_e(h, 0, h->st[1][0], s);
+        break;
+      case 10:   // two steps per pass: forward, forward with packing, ..
+      case 11: {
+        aew::TwoFwd a = two_fwd_args(h, 2 * (k % (nt / 2)), h->st[cur], h->st[cur ^ 1], nullptr, h->wav.data(),
+                                     nullptr);
+        for (int i = 0; kind == 11 && i < 2; ++i) two_pack(a, i, PackAt{h->xt[0], h->vmx, (2 * k + 1 + i) % T});
+        rc = two_fwd(h, a, s);
+        break;
+      }
+      case 12:   // .. adjoint reading FP32 and BF16 strain, ..
+        rc = two_adj(h, nt - 1 - 2 * (k % (nt / 2)), h->ad[cur], h->ad[cur ^ 1], h->R, h->st[0][0], h->st[0][1],
+                     nullptr, nullptr, s);
+        break;
+      case 13:
+        rc = two_adj(h, nt - 1 - 2 * (k % (nt / 2)), h->ad[cur], h->ad[cur ^ 1], h->R, nullptr, nullptr, st16,
+                     st16 + h->C, s);
+        break;
+      case 14: {   // .. incremental reading BF16 strain
+        aew::TwoFwd a = two_fwd_args(h, 0, h->ad[cur], h->ad[cur ^ 1], nullptr, nullptr, nullptr);
+        a.dm = h->dm;
+        a.ef16[0] = st16;
+        a.ef16[1] = st16 + h->C;
+        rc = two_fwd(h, a, s);
+        break;
+      }
+      case 15:   // on chip, a window's steps per launch: forward, ..
+        rc = brick_fwd(h, brick_fwd_args(h, h->st[cur], h->st[cur ^ 1], T, h->dts, nullptr), s);
+        break;
+      case 16:   // .. adjoint reading a decoded window
+        rc = brick_adj(h, 2 * T - 1, T, h->ad[cur], h->ad[cur ^ 1], h->R, nullptr,
+                       reinterpret_cast<const uint16_t*>(h->edt[0]) + (size_t)(T - 1) * h->C, s);
         break;
     }
     cur ^= 1;
