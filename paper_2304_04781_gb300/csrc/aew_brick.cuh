@@ -189,17 +189,6 @@ struct Geo {
   }
 };
 
-// l plus the residual row's component (r points at it) at the receivers of four nodes
-__device__ __forceinline__ F4 injected(F4 f, const int* rec_map, const float* r) {
-  const int4 m = __ldg(reinterpret_cast<const int4*>(rec_map));
-  float4 l = v4(f);
-  if (m.x >= 0) l.x += __ldg(r + 3 * m.x);
-  if (m.y >= 0) l.y += __ldg(r + 3 * m.y);
-  if (m.z >= 0) l.z += __ldg(r + 3 * m.z);
-  if (m.w >= 0) l.w += __ldg(r + 3 * m.w);
-  return f4(l);
-}
-
 // A field of BZ planes of which the first KS live in shared memory
 template <int BZ, int KS>
 struct Split {

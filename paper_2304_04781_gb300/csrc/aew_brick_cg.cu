@@ -17,12 +17,7 @@
 namespace aew {
 namespace brick {
 
-// a sum in three floats: value, accumulated rounding errors (Knuth's two-sum), and theirs
-__device__ __forceinline__ float two_sum(float a, float b, float& err) {
-  const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
-  err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
-  return t;
-}
+// a sum in three floats: value, accumulated rounding errors, and theirs
 struct Sum3 {
   float s, c, d;
   __device__ __forceinline__ void add(float x) {

@@ -112,14 +112,21 @@ int default_kc(int nx, int ny, int nz, bool adjoint);
 // ------------------------------------------------------------------------------
 // Reductions and elementwise helpers (aew_reduce.cu)
 // ------------------------------------------------------------------------------
+// fl(a + b), and its rounding error exactly (Knuth's two-sum)
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+  const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+  return t;
+}
+
+// n host values to device memory in stream order, without a copy: the host does not wait
+cudaError_t launch_set_floats(float* dst, const float* src_host, size_t n, cudaStream_t s);
 struct FieldCheck {
   unsigned int nonfinite;
   unsigned int cmax_bits;   // max c as float bits (c >= 0 expected)
   unsigned int cneg;        // count of c <= 0
 };
 // m = c^2 and checks; writes *chk (device)
-// n host values to device memory in stream order, without a copy: the host does not wait
-cudaError_t launch_set_floats(float* dst, const float* src_host, size_t n, cudaStream_t s);
 cudaError_t launch_prep_m(const float* c, float* m, size_t n, FieldCheck* chk, cudaStream_t s);
 // dm = 2 c dc and checks of dc
 cudaError_t launch_prep_dm(const float* c, const float* dc, float* dm, size_t n,

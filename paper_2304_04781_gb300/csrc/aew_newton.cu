@@ -244,9 +244,9 @@ struct CgTile {
 struct CgAcc {
   float s = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float x) {
-    const float t = __fadd_rn(s, x), z = __fsub_rn(t, s);
-    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
-    s = t;
+    float e;
+    s = two_sum(s, x, e);
+    c = __fadd_rn(c, e);
   }
   __device__ __forceinline__ double total() const { return (double)s + (double)c; }
 };

@@ -135,6 +135,16 @@ __device__ __forceinline__ F4 fma(F4 x, F4 y, F4 z) {
 }
 __device__ __forceinline__ F4 lds(const float4* p) { return f4(*p); }
 __device__ __forceinline__ void sts(float4* p, F4 v) { *p = v4(v); }
+// l plus the residual row's component (r points at it) at the receivers of four nodes
+__device__ __forceinline__ F4 injected(F4 f, const int* rec_map, const float* r) {
+  const int4 m = __ldg(reinterpret_cast<const int4*>(rec_map));
+  float4 l = v4(f);
+  if (m.x >= 0) l.x += __ldg(r + 3 * m.x);
+  if (m.y >= 0) l.y += __ldg(r + 3 * m.y);
+  if (m.z >= 0) l.z += __ldg(r + 3 * m.z);
+  if (m.w >= 0) l.w += __ldg(r + 3 * m.w);
+  return f4(l);
+}
 }  // namespace quad
 
 __device__ __forceinline__ float4 ldg4(const float* p) {

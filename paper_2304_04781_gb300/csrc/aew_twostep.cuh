@@ -838,17 +838,6 @@ __global__ void __launch_bounds__(kThreads, 1) fwd_kernel(const __grid_constant_
   }
 }
 
-// l plus the residual row's component (r points at it) at the receivers of four nodes
-__device__ __forceinline__ F4 injected(F4 f, const int* rec_map, const float* r) {
-  const int4 m = __ldg(reinterpret_cast<const int4*>(rec_map));
-  float4 l = v4(f);
-  if (m.x >= 0) l.x += __ldg(r + 3 * m.x);
-  if (m.y >= 0) l.y += __ldg(r + 3 * m.y);
-  if (m.z >= 0) l.z += __ldg(r + 3 * m.z);
-  if (m.w >= 0) l.w += __ldg(r + 3 * m.w);
-  return f4(l);
-}
-
 // Two adjoint steps with gradient accumulation, one barrier per plane as in forward_kernel.
 // B16: the strain is BF16.  CLOSE: a window ends with one of the steps (FP64 instructions slow
 // the loop even where they are skipped: 238 us instead of 140 at 256^3, so the other launches
