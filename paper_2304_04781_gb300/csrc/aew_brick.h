@@ -115,7 +115,9 @@ struct BrickCg {
   float rr_hi, rr_lo;      // r.r at the start, as a pair of floats
   double tol2;
   int max_iter;
-  int* result;             // device [4]: iterations, 1 if the test passed, r.r as a pair of floats
+  int* result;             // device [2]: iterations, 1 if the test passed
+  const float* rr_in;      // device [2] each: r.r as a pair of floats, from the launch before and
+  float* rr_out;           // for the next one (two places: all CTAs read the one, CTA 0 writes the other)
   int by, bz, py, pz;
   unsigned char* halo;
   uint32_t tag;

@@ -4,8 +4,8 @@
 // registers and p in shared memory, with its halos exchanged as in the time loops
 // (aew_brick.cuh), and both inner products of an iteration are all-reduced through one
 // tagged word pair per CTA: three L2 round trips per iteration bound it, with the reductions'
-// dependent adds.  us per iteration, launch per pass -> now: 32^3 21 -> 9, 64^3 37 -> 10, 128^3
-// 45 -> 15.
+// dependent adds.  us per iteration, launch per pass -> now: 32^3 21 -> 9, 64^3 37 -> 11, 128^3
+// 45 -> 16.
 //
 // The inner products: four products are summed by FP32 FMAs, as in the streaming passes; from
 // there a thread's and a warp's sums keep their rounding errors in two more floats (72 bits
@@ -55,7 +55,7 @@ struct Shared {
 // the sum over all CTAs of the threads' sums (words: those of this reduction).  A CTA's sum travels
 // as one FP64 number; one warp per CTA fetches all of them, all missing ones in flight at once, and
 // adds them in FP64.  us per iteration, with every thread polling one word and FP32 pairs / so:
-// 16^3 7.8 / 9.8, 32^3 8.0 / 8.8, 64^3 12.3 / 10.1, 96^3 13.5 / 10.6, 128^3 17.1 / 15.2 (fewer pollers;
+// 16^3 7.8 / 10.2, 32^3 8.0 / 9.3, 64^3 12.3 / 10.7, 96^3 13.5 / 9.9, 128^3 17.1 / 16.2 (fewer pollers;
 // the small grids see the FP64 adds' latency).  sh.pass: the total is at most tol2.
 // (*stop: a wait gave up, the same for all threads)
 __device__ __forceinline__ Sum3 all_sum(Sum3 p, ulonglong2* words, int ctas, uint32_t tag, double tol2, Shared& sh,
@@ -150,8 +150,8 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
   c.publish_z(g, f, 0, a.tag);
   Sum3 rr{a.rr_hi, a.rr_lo, 0.f};
   if (a.resume) {
-    rr.s = __int_as_float(a.result[2]);
-    rr.c = __int_as_float(a.result[3]);
+    rr.s = __ldg(a.rr_in);
+    rr.c = __ldg(a.rr_in + 1);
   }
   int it = 0, ok = 0, stop = 0;
 #pragma unroll 1
@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
     if (blockIdx.x == 0 && tid == 0) {
       a.result[0] = it;
       a.result[1] = 0;
-      a.result[2] = __float_as_int(rr.s);
-      a.result[3] = __float_as_int(rr.c);
+      a.rr_out[0] = rr.s;
+      a.rr_out[1] = rr.c;
     }
     return;
   }
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
 
 cudaError_t launch_brick_cg(BrickCg a, const BrickPlan& p, unsigned char* halo, uint32_t* tag, int* err,
                             cudaStream_t s) {
-  if (!halo || !err || a.max_iter < 1 || (a.more && a.max_iter % 8) || ((a.more || a.resume) && (!a.r || !a.p)))
+  if (!halo || !err || a.max_iter < 1 || (a.more && a.max_iter % 8) || ((a.more || a.resume) && (!a.r || !a.p || !a.rr_in || !a.rr_out || a.rr_in == a.rr_out)))
     return cudaErrorInvalidValue;
   const cudaError_t e = brick_tags(tag, (uint32_t)a.max_iter, a.nx, p, halo, s);
   if (e != cudaSuccess) return e;

@@ -27,6 +27,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/aewave.h"
@@ -732,7 +733,7 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   BrickRef br;
   const bool chip = brick_of(h, &br);
   if ((!chip && (!ws.alloc(&r, g.C) || !ws.alloc(&p[0], g.C) || !ws.alloc(&p[1], g.C))) ||
-      !ws.alloc(&part, 3 * (size_t)np) || !ws.alloc(&done, 4) || (!chip && !ws.alloc_host(&seen, 2)))
+      !ws.alloc(&part, 3 * (size_t)np) || !ws.alloc(&done, 6) || (!chip && !ws.alloc_host(&seen, 2)))
     return set_error(h, AEW_E_NOMEM, "prior solve: work vectors do not fit");
   double* ppap = part;
   double* prr[2] = {part + np, part + 2 * (size_t)np};
@@ -759,7 +760,7 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   // solve for the unit-rms right-hand side sc w (the iteration's FP32 squares then stay
   // far from FP32's range limits), and scale x back at the end
   const double sc = std::sqrt((double)g.C / ww);
-  // on chip where the grid fits: 128^3 45 -> 15 us per iteration, 64^3 37 -> 10
+  // on chip where the grid fits: 128^3 45 -> 16 us per iteration, 64^3 37 -> 11
   if (chip) {
     const double rr = ww * (double)(float)sc * (double)(float)sc, t2 = rtol * rtol * rr;
     BrickCg a{};
@@ -778,7 +779,8 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
     a.r = br.scratch[0];
     a.p = br.scratch[1];
     a.result = done;
-    NW_CK(cudaMemsetAsync(done, 0, 4 * sizeof(int), s));
+    float* rr_between[2] = {reinterpret_cast<float*>(done + 2), reinterpret_cast<float*>(done + 4)};
+    NW_CK(cudaMemsetAsync(done, 0, 6 * sizeof(int), s));
     // launches of kCgRun iterations, about 15 ms at most: a tolerance that is never reached does not
     // hold the GPU for the whole of a large max_iter
     int it = 0, ok = 0;
@@ -787,6 +789,9 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
       a.max_iter = std::min(run, max_iter - it);
       a.more = it + a.max_iter < max_iter;
       a.resume = it > 0;
+      a.rr_in = rr_between[0];
+      a.rr_out = rr_between[1];
+      std::swap(rr_between[0], rr_between[1]);
       NW_CK(launch_brick_cg(a, *br.plan, br.halo, br.tag, br.err, s));
       int got[2] = {0, 0};
       NW_CK(cudaMemcpyAsync(got, done, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
