@@ -1,4 +1,4 @@
-// The prior solve of grids that fit the SMs: all of its CG iterations in one launch.
+// The prior solve of grids that fit the SMs: up to 1024 CG iterations per launch.
 //
 // A launch per pass took 15 us and more however small the grid.  Here x, r and A p stay in
 // registers and p in shared memory, with its halos exchanged as in the time loops

@@ -17,8 +17,8 @@
 // Each kernel sums the previous one's per-block FP64 partials itself (every block in the
 // same order, so all blocks agree).  The residual is tested on the device every 8
 // iterations; once it passes, the kernels already enqueued return at once, so the host
-// stays a batch of launches ahead of the test.  Grids that fit the SMs: one launch for the
-// whole solve (aew_brick_cg.cu).
+// stays a batch of launches ahead of the test.  Grids that fit the SMs: up to 1024 iterations per
+// launch (aew_brick_cg.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
