@@ -4,14 +4,14 @@
 // registers and p in shared memory, with its halos exchanged as in the time loops
 // (aew_brick.cuh), and both inner products of an iteration are all-reduced through one
 // tagged word pair per CTA: three L2 round trips per iteration bound it, with the reductions'
-// dependent adds.  us per iteration, launch per pass -> now: 32^3 21 -> 9, 64^3 37 -> 11, 128^3
+// dependent adds.  us per iteration, launch per pass -> now: 32^3 21 -> 7, 64^3 37 -> 9, 128^3
 // 45 -> 16.
 //
 // The inner products: four products are summed by FP32 FMAs, as in the streaming passes; from
 // there a thread's and a warp's sums keep their rounding errors in two more floats (72 bits
 // against FP64's 53, and FP64 instructions in every warp would be the longest part of an
-// iteration), and one warp per CTA adds the warps' and the CTAs' parts in FP64.  Every CTA adds the
-// same parts in the same order, so all take the same steps and stop together.
+// iteration), and one warp per CTA adds the warps' and the CTAs' parts in as many bits or in FP64.
+// Every CTA adds the same parts in the same order, so all take the same steps and stop together.
 #include "aew_brick.cuh"
 
 namespace aew {
@@ -52,14 +52,17 @@ struct Shared {
   Sum3 warp[32], total;
   int pass, dead;
 };
-// the sum over all CTAs of the threads' sums (words: those of this reduction).  A CTA's sum travels
-// as one FP64 number; one warp per CTA fetches all of them, all missing ones in flight at once, and
-// adds them in FP64.  us per iteration, with every thread polling one word and FP32 pairs / so:
-// 16^3 7.8 / 10.2, 32^3 8.0 / 9.3, 64^3 12.3 / 10.7, 96^3 13.5 / 9.9, 128^3 17.1 / 16.2 (fewer pollers;
-// the small grids see the FP64 adds' latency).  sh.pass: the total is at most tol2.
+// The sum over all CTAs of the threads' sums (words: two per CTA of this reduction); one warp per CTA
+// fetches the CTAs' sums, all missing ones in flight at once.  They travel and are added as FP64
+// numbers, or on one-plane bricks (THREE) as the three floats, which saves the small grids the FP64
+// adds' latency and costs the large ones a second word per CTA.  us per iteration with every thread
+// polling a word of FP32 pairs / so: 16^3 7.8 / 8.0, 32^3 8.0 / 7.3, 64^3 12.3 / 8.6, 96^3 13.5 / 10.3,
+// 128^3 17.1 / 15.6; the other way round 32^3 9.3, 64^3 10.7, 128^3 18.6.
+// test: sh.pass tells whether the total is at most tol2 (in FP64).
 // (*stop: a wait gave up, the same for all threads)
-__device__ __forceinline__ Sum3 all_sum(Sum3 p, ulonglong2* words, int ctas, uint32_t tag, double tol2, Shared& sh,
-                                        int* err, int* stop) {
+template <bool THREE>
+__device__ __forceinline__ Sum3 all_sum(Sum3 p, ulonglong2* words, int ctas, uint32_t tag, bool test, double tol2,
+                                        Shared& sh, int* err, int* stop) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   volatile int* const dead = &sh.dead;
   p = warp_sum(p);
@@ -69,36 +72,56 @@ __device__ __forceinline__ Sum3 all_sum(Sum3 p, ulonglong2* words, int ctas, uin
     const Sum3 q = warp_sum(lane < nw ? sh.warp[lane] : Sum3{0.f, 0.f, 0.f});
     if (lane == 0) {
       const unsigned long long t = (unsigned long long)tag << 32, b = __double_as_longlong(q.value());
-      asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(words + blockIdx.x),
-                   "l"(t | (b >> 32)), "l"(t | (b & 0xffffffffull))
+      const unsigned long long x = THREE ? __float_as_uint(q.s) : b >> 32,
+                               y = THREE ? __float_as_uint(q.c) : b & 0xffffffffull;
+      asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(words + blockIdx.x), "l"(t | x), "l"(t | y)
                    : "memory");
+      if (THREE)
+        asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(words + ctas + blockIdx.x),
+                     "l"(t | __float_as_uint(q.d)), "l"(t)
+                     : "memory");
     }
     double v = 0.0;
+    Sum3 v3{0.f, 0.f, 0.f};
     for (int i0 = lane; i0 < ctas; i0 += 32 * kParts) {
-      ulonglong2 w[kParts];
+      ulonglong2 w[kParts], u[THREE ? kParts : 1];
       uint32_t need = 0, t0 = 0;
 #pragma unroll
       for (int k = 0; k < kParts; ++k) {
         w[k] = make_ulonglong2(0, 0);
+        if (THREE) u[THREE ? k : 0] = w[k];
         if (i0 + 32 * k < ctas) need |= 1u << k;
       }
       for (uint32_t it = 1; need && !*dead; ++it) {
 #pragma unroll
         for (int k = 0; k < kParts; ++k)
-          if (need >> k & 1u) w[k] = ld_words(words + i0 + 32 * k);
+          if (need >> k & 1u) {
+            w[k] = ld_words(words + i0 + 32 * k);
+            if (THREE) u[THREE ? k : 0] = ld_words(words + ctas + i0 + 32 * k);
+          }
 #pragma unroll
         for (int k = 0; k < kParts; ++k)
-          if ((uint32_t)(w[k].x >> 32) == tag && (uint32_t)(w[k].y >> 32) == tag) need &= ~(1u << k);
+          if (fresh(w[k], THREE ? u[THREE ? k : 0] : w[k], tag)) need &= ~(1u << k);
         if (need && (it & 63u) == 0 && !keep_waiting(t0, dead, err)) break;
       }
 #pragma unroll
-      for (int k = 0; k < kParts; ++k) v += __longlong_as_double((long long)(w[k].x << 32 | (w[k].y & 0xffffffffull)));
+      for (int k = 0; k < kParts; ++k) {
+        if (THREE)
+          v3.add(__uint_as_float((uint32_t)w[k].x), __uint_as_float((uint32_t)w[k].y),
+                 __uint_as_float((uint32_t)u[THREE ? k : 0].x));
+        else
+          v += __longlong_as_double((long long)(w[k].x << 32 | (w[k].y & 0xffffffffull)));
+      }
     }
-    v = warp_sum(v);
+    if (THREE) v3 = warp_sum(v3);
+    else v = warp_sum(v);
     if (lane == 0) {
-      const float a = (float)v;
-      sh.total = Sum3{a, (float)(v - (double)a), 0.f};
-      sh.pass = v <= tol2;
+      if (!THREE) {
+        v3.s = (float)v;
+        v3.c = (float)(v - (double)v3.s);
+      }
+      sh.total = v3;
+      if (test) sh.pass = (THREE ? v3.value() : v) <= tol2;
     }
   }
   *stop = __syncthreads_or(*dead);
@@ -189,7 +212,7 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
         acc.add(fmaf(p.x, o[0], fmaf(p.y, o[1], fmaf(p.z, o[2], p.w * o[3]))));
       zm = p;
     }
-    const Sum3 pap = all_sum(acc, red + (size_t)par * ctas, ctas, tag, a.tol2, sh, a.err, &stop);
+    const Sum3 pap = all_sum<BZ == 1>(acc, red + (size_t)par * 2 * ctas, ctas, tag, false, a.tol2, sh, a.err, &stop);
     const float al = pap.s > 0.f ? ratio(rr, pap) : 0.f;
     // ---- x += a p, r -= a A p and r.r
     acc = Sum3{0.f, 0.f, 0.f};
@@ -201,9 +224,9 @@ __global__ void __launch_bounds__(tmax(BZ), 1) cg_kernel(const __grid_constant__
       r[k].x -= al * v[k].x; r[k].y -= al * v[k].y; r[k].z -= al * v[k].z; r[k].w -= al * v[k].w;
       acc.add(fmaf(r[k].x, r[k].x, fmaf(r[k].y, r[k].y, fmaf(r[k].z, r[k].z, r[k].w * r[k].w))));
     }
-    const Sum3 rn = all_sum(acc, red + (size_t)(2 + par) * ctas, ctas, tag, a.tol2, sh, a.err, &stop);
-    const bool last = it + 1 == a.max_iter;
-    if (((it & 7) == 7 || last) && sh.pass) ok = 1;
+    const bool last = it + 1 == a.max_iter, test = (it & 7) == 7 || last;
+    const Sum3 rn = all_sum<BZ == 1>(acc, red + (size_t)(2 + par) * 2 * ctas, ctas, tag, test, a.tol2, sh, a.err, &stop);
+    if (test && sh.pass) ok = 1;
     const float be = rr.s > 0.f ? ratio(rn, rr) : 0.f;
     rr = rn;
     ++it;

@@ -34,7 +34,7 @@ bool brick_plan(int nx, int ny, int nz, int sms, BrickPlan* p) {
 size_t brick_halo_bytes(int nx, const BrickPlan& p) {
   const size_t ctas = (size_t)p.py * p.pz;
   return 2 * ctas * 2 * 2 * ((size_t)brick::tmax(p.bz) + (size_t)p.bz * (nx / 4)) * 16 +
-         4 * ctas * 16;   // two sums of two parities per CTA
+         8 * ctas * 16;   // two sums of two parities, two words each, per CTA
 }
 
 cudaError_t brick_tags(uint32_t* tag, uint32_t steps, int nx, const BrickPlan& p, unsigned char* halo,

@@ -760,7 +760,7 @@ int prior_cg(aew_handle* h, const Grid& g, double hh, double alpha, double theta
   // solve for the unit-rms right-hand side sc w (the iteration's FP32 squares then stay
   // far from FP32's range limits), and scale x back at the end
   const double sc = std::sqrt((double)g.C / ww);
-  // on chip where the grid fits: 128^3 45 -> 16 us per iteration, 64^3 37 -> 11
+  // on chip where the grid fits: 128^3 45 -> 16 us per iteration, 64^3 37 -> 9
   if (chip) {
     const double rr = ww * (double)(float)sc * (double)(float)sc, t2 = rtol * rtol * rr;
     BrickCg a{};
